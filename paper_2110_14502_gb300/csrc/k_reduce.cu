@@ -10,6 +10,8 @@
 // pass through shared memory.  Consecutive threads read consecutive k, so the
 // reads coalesce when the contracted indices are the operands' fastest ones
 // (the planner's layout puts them there).
+#include <mutex>
+
 #include "kernels.h"
 
 namespace tn {
@@ -84,6 +86,159 @@ __global__ void __launch_bounds__(NT) reduce_kernel(const float2* __restrict__ A
   }
 }
 
+// The same sums with one unit spread over the chip, for launches with fewer
+// units than SMs (one CTA per unit leaves the rest idle and walks K alone: a
+// 2^3 x 2^3 x 2^18 step took 4.15 ms that way, 8 GB/s).
+//
+// What bounds it: every output is a sum in a fixed order -- per thread t of 256
+// over k = t, t + 256, .., then a shuffle tree over each warp's lanes, then the
+// eight warps in order -- and that order is kept, so the results are those of
+// reduce_kernel bit for bit and do not depend on the number of units.  The
+// K / 256 dependent multiply-adds per thread are the serial chain; the bytes
+// are an L2 -> SM stream.  So the eight warps' shares of k go to the eight CTAs
+// of a cluster, and the outputs in 2 x 2 blocks to clusters: 128 SMs for
+// 64 outputs, each reading 4 operand rows (2 of A, 2 of B) of its k share once
+// for 4 outputs, one warp per output.  The rows arrive by 8-byte cp.async
+// (any index order) through a ring of 16-value groups, 3 of 4 in flight; the
+// CTAs' partial sums meet in the first one's shared memory.  Measured per
+// tn_contract_pair call: 2^3 x 2^3 x 2^18 with contiguous K 3260 -> 45 us (of
+// which about 25 us are the call), 2^6 x 1 x 2^16 43 us, 1 x 1 x 2^19 102 us.
+constexpr int SP_G = 16;                   // values of k per thread and group (bits LOW .. LOW + 3)
+constexpr int SP_RING = 4;
+constexpr int SP_ROWS = 4;                 // at most 2 rows of A and 2 of B per CTA
+constexpr int SP_SMEM = SP_RING * SP_G * SP_ROWS * 32 * (int)sizeof(float2);
+
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
+}
+
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(128)
+    reduce_spread_kernel(const float2* __restrict__ A, const float2* __restrict__ B, float2* __restrict__ C,
+                         const GemmDesc d) {
+  extern __shared__ __align__(16) float2 ring[];  // [SP_RING][SP_G][row][32]
+  __shared__ float2 part[8][4];                   // first CTA of the cluster: [original warp][output]
+  const int64_t ulo = blockIdx.y % d.units_lo, uhi = blockIdx.y / d.units_lo;
+  A += ulo * d.a_lo + uhi * d.a_hi;
+  B += ulo * d.b_lo + uhi * d.b_hi;
+  C += ulo * d.c_lo + uhi * d.c_hi;
+  // the cluster's CTAs have all started once this barrier's phase completes
+  // (awaited before the first store to another CTA's shared memory)
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int share = blockIdx.x & 7, blk = blockIdx.x >> 3;  // cluster rank, output block
+  const int wm = d.nm > 0 ? 1 : 0, wn = d.nn > 0 ? 1 : 0;   // the block's rows and columns (log2)
+  const int nblk_n = 1 << (d.nn - wn);
+  const int m0 = (blk / nblk_n) << wm, n0 = (blk % nblk_n) << wn;
+  const int ra = 1 << wm, rows = ra + (1 << wn);
+  const int m_l = warp >> wn, n_l = warp & ((1 << wn) - 1);  // this warp's output in the block
+  const int gbits = d.nk - LOW < 4 ? d.nk - LOW : 4;
+  const int glen = 1 << gbits;
+  const int64_t ngroups = int64_t(1) << (d.nk - LOW - gbits);
+  const int t = share * 32 + lane;  // the thread of the 256 whose values this lane sums
+  // The warp copies rows warp, warp + nwarps (at most two).  Everything an
+  // issue needs is in registers: the offsets of a group's 16 values, and one
+  // stride of the group index per lane, summed over the warp.
+  const float2* src[2];
+  int32_t tab[2][SP_G], gst[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int r = warp + q * nwarps;
+    const bool isa = r < ra;
+    const int32_t* ks = isa ? d.ak : d.bk;
+    src[q] = isa ? A + bit_offset(m0 + r, 0, d.nm, d.am) : B + bit_offset(n0 + r - ra, 0, d.nn, d.bn);
+    src[q] += bit_offset(t, 0, LOW, ks);
+    gst[q] = LOW + gbits + lane < d.nk ? ks[LOW + gbits + lane] : 0;
+#pragma unroll
+    for (int i = 0; i < SP_G; ++i) {
+      tab[q][i] = 0;
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        if (((i >> b) & 1) && b < gbits) tab[q][i] += ks[LOW + b];
+    }
+  }
+  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(ring);
+  auto issue = [&](int g) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int r = warp + q * nwarps;
+      if (r >= rows) break;
+      const float2* p = src[q] + (int32_t)__reduce_add_sync(0xffffffffu, (uint32_t)(((g >> lane) & 1) ? gst[q] : 0));
+      const uint32_t slot = sbase + (uint32_t)(((g % SP_RING) * SP_G * SP_ROWS + r) * 32 + lane) * 8u;
+#pragma unroll
+      for (int i = 0; i < SP_G; ++i)
+        if (i < glen) cp_async8(slot + (uint32_t)(i * SP_ROWS * 32) * 8u, p + tab[q][i]);
+    }
+  };
+  for (int g = 0; g < SP_RING - 1; ++g) {
+    if (g < ngroups) issue(g);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  }
+  float2 c = make_float2(0.f, 0.f);
+  for (int g = 0; g < (int)ngroups; ++g) {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(SP_RING - 2) : "memory");
+    __syncthreads();  // group g landed for every warp; group g - 1's slot is free
+    if (g + SP_RING - 1 < ngroups) issue(g + SP_RING - 1);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    const float2* pa = ring + ((g % SP_RING) * SP_G * SP_ROWS + m_l) * 32 + lane;
+    const float2* pb = ring + ((g % SP_RING) * SP_G * SP_ROWS + ra + n_l) * 32 + lane;
+    auto mac = [&](int i) {
+      const float2 a = pa[i * SP_ROWS * 32], b = pb[i * SP_ROWS * 32];
+      c.x = fmaf(a.x, b.x, fmaf(-a.y, b.y, c.x));
+      c.y = fmaf(a.x, b.y, fmaf(a.y, b.x, c.y));
+    };
+    if (glen == SP_G) {
+#pragma unroll
+      for (int i = 0; i < SP_G; ++i) mac(i);
+    } else {
+      for (int i = 0; i < glen; ++i) mac(i);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    c.x += __shfl_xor_sync(0xffffffffu, c.x, o);
+    c.y += __shfl_xor_sync(0xffffffffu, c.y, o);
+  }
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (lane == 0) {
+    uint32_t dst;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst)
+                 : "r"((uint32_t)__cvta_generic_to_shared(&part[share][warp])));
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(c.x), "f"(c.y) : "memory");
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (share == 0 && lane == 0) {
+    float2 s = part[0][warp];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) {
+      s.x += part[w][warp].x;
+      s.y += part[w][warp].y;
+    }
+    C[bit_offset(m0 + m_l, 0, d.nm, d.cm) + bit_offset(n0 + n_l, 0, d.nn, d.cn)] = s;
+  }
+}
+
+// One unit per CTA fills the chip from one unit per SM on; below that the
+// spread kernel is used whatever K is (both at 2^3 x 2^3 x 2^8, one unit: one
+// group of loads each).
+constexpr int SPREAD_UNITS = 152;
+
+cudaError_t launch_spread(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s) {
+  static std::once_flag once[64];
+  static cudaError_t attr[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::call_once(once[dev], [&] {
+    attr[dev] = cudaFuncSetAttribute(reduce_spread_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SP_SMEM);
+  });
+  if (attr[dev] != cudaSuccess) return attr[dev];
+  const int wm = d.nm > 0 ? 1 : 0, wn = d.nn > 0 ? 1 : 0;
+  const dim3 grid(8u << (d.nm - wm + d.nn - wn), (unsigned)d.units);
+  reduce_spread_kernel<<<grid, 32u << (wm + wn), SP_SMEM, s>>>(A, B, C, d);
+  return cudaGetLastError();
+}
+
 template <int NM, int NN>
 cudaError_t launch(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s) {
   reduce_kernel<NM, NN><<<(unsigned)d.units, NT, 0, s>>>(A, B, C, d);
@@ -111,6 +266,7 @@ bool reduce_shape_ok(const GemmDesc& d) { return d.nm + d.nn <= 6 && d.nk >= LOW
 
 cudaError_t launch_reduce(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s) {
   if (!reduce_shape_ok(d) || d.units < 1 || d.units > (int64_t(1) << 31) - 1) return cudaErrorInvalidValue;
+  if (d.units < SPREAD_UNITS) return launch_spread(A, B, C, d, s);
   switch (d.nm) {
     case 0: return launch_nn<0>(A, B, C, d, s);
     case 1: return launch_nn<1>(A, B, C, d, s);
