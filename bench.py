@@ -335,8 +335,7 @@ def run_ours(args):
         roof = {"bound": "alu", "achieved": round(achieved, 2), "peak": round(fp32, 1), "unit": "TFLOP/s",
                 "frac": round(achieved / fp32, 4), "peak_kind": "FP32 FFMA: 152 SMs x 128 lanes x 2 x max clock"}
     roof["kernel"] = {0: "gemm_simt_kernel", 1: "vector_kernel",
-                      2: "gemm_tma_chunked" if args.precision.startswith("split")
-                      else "gemm_tma_persistent / gemm_tma_kernel"}[dom]
+                      2: "gemm_tma_chunked"}[dom]
     roof["launches_per_step"] = cls_n[dom] / args.steps
     roof["share_of_device_time"] = round(cls_ms[dom] / sum(cls_ms), 4) if sum(cls_ms) else None
     if cls_n[3]:

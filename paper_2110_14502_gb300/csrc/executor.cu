@@ -126,7 +126,7 @@ struct Executor {
   struct Graph { int phase, precision, handover, gs, gb; cudaGraphExec_t exec; int64_t kernels; };
   std::vector<Graph> graphs;
   // autotuner choices per (precision, step): tensor-core tile width, raster group
-  struct Tune { int precision, step, tile_n, group_m, persistent; };
+  struct Tune { int precision, step, tile_n, group_m; };
   std::vector<Tune> tuned;
   bool tune_loaded = false;
   std::vector<GemmDesc> desc;  // per step, unit strides filled at launch
@@ -554,7 +554,6 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
       if (t.precision == c.precision && t.step == (int)s) {
         d.tile_n = t.tile_n;
         d.group_m = t.group_m;
-        d.persistent = t.persistent;
       }
     ScaleIO sio{};
     e = cudaSuccess;
@@ -619,16 +618,13 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
       // result; the last launch below leaves it in place) and keep the fastest
       const int def_n = d.nn >= 7 ? 128 : (1 << d.nn);
       float best = 1e30f;
-      int bt = 0, bg = 0, bp = 0;
+      int bt = 0, bg = 0;
       for (int tn : {128, 64}) {
         if (tn > def_n) continue;
-        for (int cand = 0; cand < 6; ++cand) {
-          const int gm = (cand % 3 == 0) ? 8 : (cand % 3 == 1) ? 16 : 32;
-          const int pers = cand < 3 ? 1 : 2;
+        for (int gm : {8, 16, 32}) {
           GemmDesc dc = d;
           dc.tile_n = tn;
           dc.group_m = gm;
-          dc.persistent = pers;
           cudaEvent_t t0, t1;
           cudaEventCreate(&t0);
           cudaEventCreate(&t1);
@@ -641,13 +637,12 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
           cudaEventDestroy(t0);
           cudaEventDestroy(t1);
           if (e != cudaSuccess) break;
-          if (ms < best) { best = ms; bt = tn; bg = gm; bp = pers; }
+          if (ms < best) { best = ms; bt = tn; bg = gm; }
         }
       }
-      E.tuned.push_back({c.precision, (int)s, bt, bg, bp});
+      E.tuned.push_back({c.precision, (int)s, bt, bg});
       d.tile_n = bt;
       d.group_m = bg;
-      d.persistent = bp;
     }
     if (e == cudaSuccess) e = launch_gemm_tma(pa, pb, C, c.planes_out[s] != 0, d, c.bf16, sio, E.err, c.st);
   }
@@ -961,9 +956,9 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
         if (FILE* f = fopen(path, "r")) {
           unsigned long long h;
           int pr, st_, tn, gm;
-          int pe;
+          int pe;  // a kernel variant of earlier files, no longer a choice
           while (fscanf(f, "%llx %d %d %d %d %d", &h, &pr, &st_, &tn, &gm, &pe) == 6)
-            if (h == P.hash) E.tuned.push_back({pr, st_, tn, gm, pe});
+            if (h == P.hash) E.tuned.push_back({pr, st_, tn, gm});
           fclose(f);
         }
       }
@@ -1084,8 +1079,8 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
         if (FILE* f = fopen(path, "a")) {
           for (auto& t : E.tuned)
             if (t.precision == c.precision)
-              fprintf(f, "%llx %d %d %d %d %d\n", (unsigned long long)P.hash, t.precision, t.step, t.tile_n,
-                      t.group_m, t.persistent);
+              fprintf(f, "%llx %d %d %d %d 1\n", (unsigned long long)P.hash, t.precision, t.step, t.tile_n,
+                      t.group_m);
           fclose(f);
         }
       }

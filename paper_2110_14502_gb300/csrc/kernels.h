@@ -27,7 +27,6 @@ struct GemmDesc {
   int nm, nn, nk;
   int units, units_lo;
   int tile_n, group_m;       // tensor-core tile width / raster group (0 = default; set by the autotuner)
-  int persistent;            // tensor-core GEMM: 0 auto, 1 persistent CTAs (double-buffered accumulators), 2 one tile per CTA
   int64_t a_lo, a_hi, b_lo, b_hi, c_lo, c_hi;
   int32_t am[kMaxBits], cm[kMaxBits];
   int32_t bn[kMaxBits], cn[kMaxBits];
