@@ -231,68 +231,61 @@ __device__ __forceinline__ int vec_bits(const GemmDesc& d) {
   return v;
 }
 
+// C offset of tile column j of 16 from the strides of its four bits.
+__device__ __forceinline__ int32_t col_offset(const int32_t (&cs)[4], int j) {
+  return ((j & 1) ? cs[0] : 0) + ((j & 2) ? cs[1] : 0) + ((j & 4) ? cs[2] : 0) + ((j & 8) ? cs[3] : 0);
+}
+
 // One thread's 16 consecutive tile columns of one row (packed elements, see
-// pack_planes) as NP 16-bit planes: each contiguous run of 2^vb columns goes
-// out as one store per plane (the run starts at a multiple of 2^vb elements:
-// every other index of C has a larger stride).
+// pack_planes) as NP 16-bit planes, P at the row and first column: each
+// contiguous run of 2^vb columns goes out as one store per plane (the run
+// starts at a multiple of 2^vb elements: every other index of C has a larger
+// stride).
 template <int NP>
 __device__ __forceinline__ uint32_t plane_pair(const uint32_t (&e)[NP / 2][16], int p, int j) {
   return __byte_perm(e[p >> 1][j], e[p >> 1][j + 1], (p & 1) ? 0x7632 : 0x5410);
 }
 template <int NP>
-__device__ __forceinline__ void store_planes(uint16_t* P, int64_t plane, int64_t ro, const int32_t* col, int vb,
+__device__ __forceinline__ void store_planes(uint16_t* P, int64_t plane, const int32_t (&cs)[4], int vb,
                                              const uint32_t (&e)[NP / 2][16]) {
   auto pk = [&](int p, int j) { return plane_pair<NP>(e, p, j); };
   if (vb >= 3) {
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int64_t o = ro + col[8 * r];
+    for (int r = 0; r < 2; ++r)
 #pragma unroll
       for (int p = 0; p < NP; ++p)
-        *reinterpret_cast<uint4*>(P + p * plane + o) =
+        *reinterpret_cast<uint4*>(P + p * plane + col_offset(cs, 8 * r)) =
             make_uint4(pk(p, 8 * r), pk(p, 8 * r + 2), pk(p, 8 * r + 4), pk(p, 8 * r + 6));
-    }
   } else if (vb == 2) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int64_t o = ro + col[4 * r];
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
       for (int p = 0; p < NP; ++p)
-        *reinterpret_cast<uint2*>(P + p * plane + o) = make_uint2(pk(p, 4 * r), pk(p, 4 * r + 2));
-    }
+        *reinterpret_cast<uint2*>(P + p * plane + col_offset(cs, 4 * r)) = make_uint2(pk(p, 4 * r), pk(p, 4 * r + 2));
   } else if (vb == 1) {
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const int64_t o = ro + col[2 * r];
+    for (int r = 0; r < 8; ++r)
 #pragma unroll
-      for (int p = 0; p < NP; ++p) *reinterpret_cast<uint32_t*>(P + p * plane + o) = pk(p, 2 * r);
-    }
+      for (int p = 0; p < NP; ++p) *reinterpret_cast<uint32_t*>(P + p * plane + col_offset(cs, 2 * r)) = pk(p, 2 * r);
   } else {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int64_t o = ro + col[j];
+    for (int j = 0; j < 16; ++j)
 #pragma unroll
       for (int p = 0; p < NP; ++p)
-        P[p * plane + o] = (uint16_t)((p & 1) ? e[p >> 1][j] >> 16 : e[p >> 1][j] & 0xffffu);
-    }
+        P[p * plane + col_offset(cs, j)] = (uint16_t)((p & 1) ? e[p >> 1][j] >> 16 : e[p >> 1][j] & 0xffffu);
   }
 }
 
-// The same for complex64 output (two complex values per 16-byte store).
-__device__ __forceinline__ void store_c64(float2* C, int64_t ro, const int32_t* col, int vb, const float* vr,
-                                          const float* vi) {
-  if (vb >= 1) {
-    const int run = vb >= 4 ? 16 : (1 << vb);
-#pragma unroll
-    for (int j = 0; j < 16; j += 2) {
-      // pairs (j, j + 1) are contiguous; a new run starts every `run` columns
-      float4* q = reinterpret_cast<float4*>(C + ro + col[j & ~(run - 1)]) + ((j & (run - 1)) >> 1);
-      *q = make_float4(vr[j], vi[j], vr[j + 1], vi[j + 1]);
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) C[ro + col[j]] = make_float2(vr[j], vi[j]);
-  }
+__device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y) {
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void sts32(uint32_t a, uint32_t x) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(x) : "memory");
+}
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
 }
 
 template <int NREG>
@@ -318,18 +311,15 @@ __device__ __forceinline__ void drain_loads(uint64_t* full, int ns, int64_t issu
     }
 }
 
-// Staged output of the chunked kernel.  A warp's 32 x 16 sub-tile (lanes =
-// tile row bits 0..4, columns = tile column bits 0..3) covers 512 elements of
-// C; sorted by their C stride these 9 bits give each element a C-order index.
-// When the output's fastest indices interleave row and column bits (neither
-// the lanes nor a thread's columns form long contiguous runs), the warp writes
-// its values to shared memory at their C-order index and reads them back in
-// C order, consecutive lanes taking consecutive 16-byte pieces (2 complex64
-// values, or 8 values of one 16-bit plane): the first `run` sorted strides
-// are 1, 2, 4, .., so each store instruction writes runs of 2^run values.
-// For 16-bit plane output the same staging also serves layouts whose
-// contiguous run lies along the lanes (rows fastest), where each thread would
-// otherwise store its values two bytes at a time.
+// Staged output.  A warp's 32 x 16 sub-tile (lanes = tile row bits 0..4,
+// columns = tile column bits 0..3) covers 512 elements of C; sorted by their C
+// stride these 9 bits give each element a C-order index.  The warp writes its
+// values to shared memory at their C-order index and reads them back in C
+// order, consecutive lanes taking consecutive 16-byte pieces (2 complex64
+// values, or 8 values of one 16-bit plane): the first `run` sorted strides are
+// 1, 2, 4, .., so each store instruction writes runs of 2^run values.  Only a
+// complex64 output whose lanes already cover consecutive elements, or one whose
+// fastest indices lie outside the sub-tile, goes out directly.
 constexpr int STAGE_SLOTS = 512 + 64;  // 8-byte slots per warp: 512 elements, 2 padding slots after every 16
 
 struct StageMap {
@@ -342,7 +332,7 @@ struct StageMap {
   int32_t step_pl;     // C offset added by the second plane read-back step
 };
 
-__device__ __forceinline__ StageMap stage_map(const GemmDesc& d, int lane, int vb, bool planes) {
+__device__ __forceinline__ StageMap stage_map(const GemmDesc& d, int lane, bool planes, bool wide) {
   StageMap m;
   int32_t st[9], sst[9];
   int rnk[9];
@@ -358,10 +348,7 @@ __device__ __forceinline__ StageMap stage_map(const GemmDesc& d, int lane, int v
   while (run < 9 && sst[run] == (1 << run)) ++run;
   int lane_run = 0;
   while (lane_run < 5 && d.cm[lane_run] == (1 << lane_run)) ++lane_run;
-  // complex64: staged only where it lengthens the contiguous runs; planes
-  // (2-byte values): also where it merely turns 2-, 4- or 8-byte stores into
-  // 16-byte ones (a thread's columns give fewer than 8 contiguous values)
-  m.on = planes ? run >= 3 && vb < 3 : run >= 3 && lane_run < 5 && vb < 4 && run > lane_run && run > vb;
+  m.on = planes ? run >= 3 : run >= 1 && lane_run < 5 && wide;
   m.lane_idx = 0;
   for (int b = 0; b < 5; ++b) m.lane_idx |= ((lane >> b) & 1) << rnk[b];
   for (int b = 0; b < 4; ++b) m.rank_c[b] = rnk[5 + b];
@@ -452,7 +439,7 @@ template <int TN, int NP, int ROWB, int EW>
 __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
     gemm_tma_chunked(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                      float2* __restrict__ C0, const GemmDesc d, int kp, int a_zlo, int a_zhi, int b_zlo, int b_zhi,
-                     int c_planes, const ScaleIO sio, int chunk, int fold, bool bf16, int* __restrict__ err,
+                     int out_flags, const ScaleIO sio, int chunk, int fold, bool bf16, int* __restrict__ err,
                      const BulkPlanes ba, const BulkPlanes bb) {
   using CC = ChunkCfg<TN, NP, ROWB, EW>;
   using CF = Cfg2<TN, NP, ROWB>;
@@ -467,9 +454,7 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   __shared__ uint64_t full[NS], empty[NS], acc_full[2], acc_empty[2], mma_done;
   __shared__ uint32_t tmem_slot;
-  __shared__ int32_t colC[TN];
   __shared__ volatile int abort_flag;
-  __shared__ volatile int epi_fail;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long wl = g_wait_limit;
@@ -505,7 +490,6 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
     for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], ET); }
     mbar_init(&mma_done, 1);
     abort_flag = 0;
-    epi_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapA)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapB)) : "memory");
@@ -701,81 +685,106 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
   } else if (warp >= 4) {
     // ---- epilogue: fold chunks 1.. into R; after the last one, store R.
     // Warp 4 + e reads TMEM lane quarter q = warp % 4 (the hardware's rule)
-    // and, with eight epilogue warps, every other 16-column chunk (h).
+    // and, with eight epilogue warps, every other 16-column chunk (h).  The
+    // warps share nothing but the accumulator barriers.  What bounds an
+    // output-bound step here is the warps' instruction latency, so every
+    // address is a sum of few terms set up once: shared-memory slots per
+    // column, C offsets per read-back step, and per tile the offsets of its
+    // upper row and column bits, each one warp sum over the bits' strides.
+    // Measured against column offsets in a shared table behind barriers and
+    // per-element scaling branches: 16-bit planes, (11, 10, 5) x 4096 units 20.1
+    // -> 12.4 ms; four planes, (15, 9, 7) x 128 units 7.2 -> 5.3 ms; complex64,
+    // (14, 14, 5) 832 -> 518 us.
     const int e = warp - 4, q = warp & 3, h = e >> 2;
     constexpr int CS = 16 * (EW / 4);  // column stride between a warp's chunks
-    const int tq = tid - 128;
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-    const StageMap sm = stage_map(d, lane, vec_bits(d), c_planes != 0);
-    float2* const slots = reinterpret_cast<float2*>(smem + NS * CF::STAGE) + e * STAGE_SLOTS;
-    // the C-order index of (lane, jj) is lane_idx | (jj's bits at their ranks);
-    // the two parts have disjoint bits, so their slots add
-    const bool slot4 = NP == 2 && c_planes;  // 4-byte slots
-    const int lane_slot = slot4 ? stage_slot4(sm.lane_idx) : stage_slot(sm.lane_idx);
-    int cs[4];  // slot offset of column bit b alone
-    for (int b = 0; b < 4; ++b) cs[b] = slot4 ? stage_slot4(1 << sm.rank_c[b]) : stage_slot(1 << sm.rank_c[b]);
-    auto col_slot = [&](int jj) {
-      return ((jj & 1) ? cs[0] : 0) + ((jj & 2) ? cs[1] : 0) + ((jj & 4) ? cs[2] : 0) + ((jj & 8) ? cs[3] : 0);
+    const bool planes = (out_flags & 1) != 0, wide = (out_flags & 2) != 0;
+    const StageMap sm = stage_map(d, lane, planes, wide);
+    const int vb = wide || planes ? vec_bits(d) : 0;
+    // this lane's slots: the C-order index of (lane, jj) is lane_idx | (jj's
+    // bits at their ranks); the two parts have disjoint bits, so their slots add
+    const bool slot4 = NP == 2 && planes;  // 4-byte slots
+    const uint32_t slots = smem_u32(smem + NS * CF::STAGE) + e * STAGE_SLOTS * 8;
+    auto slot_of = [&](int idx) { return (uint32_t)(slot4 ? stage_slot4(idx) * 4 : stage_slot(idx) * 8); };
+    uint32_t slot[16];
+    {
+      uint32_t cs[4];
+      for (int b = 0; b < 4; ++b) cs[b] = slot_of(1 << sm.rank_c[b]);
+#pragma unroll
+      for (int jj = 0; jj < 16; ++jj)
+        slot[jj] = slots + slot_of(sm.lane_idx) + ((jj & 1) ? cs[0] : 0) + ((jj & 2) ? cs[1] : 0) +
+                   ((jj & 4) ? cs[2] : 0) + ((jj & 8) ? cs[3] : 0);
+    }
+    const uint32_t rd = slots + slot_of(planes ? 8 * lane : 2 * lane);
+    int32_t back[8];  // C offset of this lane's piece in read-back step t
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+      back[t] = planes ? sm.off_pl + ((t & 1) ? sm.step_pl : 0)
+                       : sm.off_c64 + ((t & 1) ? sm.step_c64[0] : 0) + ((t & 2) ? sm.step_c64[1] : 0) +
+                             ((t & 4) ? sm.step_c64[2] : 0);
+    const int32_t lane_row = bit_offset(lane, 5, d.cm);  // direct stores: this lane's row
+    const int32_t cn_lo[4] = {d.cn[0], d.cn[1], d.cn[2], d.cn[3]};
+    // strides of the tile's row bits 5.. and column bits 7.. (lane b: bit b), and of column bits 4..6
+    const int32_t my_cm = lane >= 5 && lane < d.nm ? d.cm[lane] : 0;
+    const int32_t my_cn = lane >= 4 && lane < d.nn ? d.cn[lane] : 0;
+    const int32_t cn_mid[3] = {d.nn > 4 ? d.cn[4] : 0, d.nn > 5 ? d.cn[5] : 0, d.nn > 6 ? d.cn[6] : 0};
+    auto bit_sum = [&](int x, int32_t st) {
+      return (int32_t)__reduce_add_sync(0xffffffffu, (uint32_t)(((x >> lane) & 1) ? st : 0));
     };
-    // C offset of the thread's row: its bits 0..6 (q * 32 + lane) once, the
-    // tile's bits 7.. per item as a warp sum (lane b holds row bit b's stride)
-    const int32_t ro_lo = bit_offset(q * 32 + lane, min(7, d.nm), d.cm);
-    const int32_t my_cm = lane >= 7 && lane < d.nm ? d.cm[lane] : 0;
-    int last_n0 = -1;
-    // scaling and the maximum / filter tracking only where the formats need them
+    const int64_t plane = int64_t(1) << (d.nm + d.nn);
+    const int gw = fold > 1 ? nsub : TN;  // tile columns of one unit
+    // maximum / filter tracking only where the formats need it
     const bool track = sio.mc != nullptr || sio.flag != nullptr;
+    // Scaled formats: exponents of the operands of the tile's f-th unit (a
+    // folded tile holds `fold` hi units side by side, f = column / 2^nn, with A
+    // shared and B, C of their own) and the output shift r that keeps the
+    // predicted bound 2 K maxA maxB below 2^15.
+    float vmax = 0.f, fin[2] = {0.f, 0.f};
+    bool weak = false;
+    int ea = 0, eb = 0, r = 0, scaled_unit = -1;
+    Pow2 sc(0);
+    auto unit_scale = [&](int ulo, int uhi, int f) {
+      const int un = ulo + (uhi + f) * d.units_lo;
+      if (!sio.ea || un == scaled_unit) return;
+      scaled_unit = un;
+      const int za = (a_zlo ? ulo : 0) + (a_zhi ? uhi : 0) * (a_zlo ? d.units_lo : 1);
+      const int zb = (b_zlo ? ulo : 0) + (b_zhi ? uhi + f : 0) * (b_zlo ? d.units_lo : 1);
+      ea = sio.ea[za];
+      eb = sio.eb[zb];
+      const float ma = sio.ma[za], mb = sio.mb[zb];
+      weak = !(ma >= 0x1p-10f) || !(mb >= 0x1p-10f);
+      const float bound = 2.f * ldexpf(ma * mb, d.nk);
+      r = 0;
+      if (bound > 0.f && isfinite(bound)) {
+        int x;
+        frexpf(bound, &x);
+        r = x - 15;
+      }
+      sc = Pow2(planes ? -r : ea + eb);
+    };
     int64_t t = 0;
     uint32_t seen[2] = {0u, 0u};
-    for (int64_t it = first; it < items; it += stride, ++t) {
+    bool ok = true;
+    for (int64_t it = first; ok && it < items; it += stride, ++t) {
       int unit, m0, n0;
       decode(it, unit, m0, n0);
       const int ulo = unit % d.units_lo, uhi = (unit / d.units_lo) * fold;
-      // the column offsets change with the tile's first column only (the
-      // barriers around each item order these writes against every read)
-      if (n0 != last_n0) {
-        for (int jj = tq; jj < TN; jj += ET) colC[jj] = bit_offset(fold > 1 ? (jj & (nsub - 1)) : n0 + jj, d.nn, d.cn);
-        last_n0 = n0;
-      }
-      const int32_t ro = ro_lo + (int32_t)__reduce_add_sync(0xffffffffu, (uint32_t)(((m0 >> lane) & 1) ? my_cm : 0));
-      float2* Cu = C0 + (int64_t)ulo * d.c_lo + (int64_t)uhi * d.c_hi;
-      // Scaled formats: exponents of the operands of the tile's f-th unit (a
-      // folded tile holds `fold` hi units side by side, f = column / 2^nn,
-      // with A shared and B, C of their own) and the output shift r that keeps
-      // the predicted bound 2 K maxA maxB below 2^15.
-      auto unit_scale = [&](int f, int& ea, int& eb, int& r, bool& weak) {
-        ea = eb = r = 0;
-        weak = false;
-        if (!sio.ea) return;
-        const int za = (a_zlo ? ulo : 0) + (a_zhi ? uhi : 0) * (a_zlo ? d.units_lo : 1);
-        const int zb = (b_zlo ? ulo : 0) + (b_zhi ? uhi + f : 0) * (b_zlo ? d.units_lo : 1);
-        ea = sio.ea[za];
-        eb = sio.eb[zb];
-        const float ma = sio.ma[za], mb = sio.mb[zb];
-        weak = !(ma >= 0x1p-10f) || !(mb >= 0x1p-10f);
-        const float bound = 2.f * ldexpf(ma * mb, d.nk);
-        if (bound > 0.f && isfinite(bound)) {
-          int x;
-          frexpf(bound, &x);
-          r = x - 15;
-        }
-      };
-      const int vb = vec_bits(d);
-      const int gw = fold > 1 ? nsub : TN;  // tile columns of one unit
+      unit_scale(ulo, uhi, 0);  // (loads in flight while the accumulator fills)
+      float2* const Cu = C0 + ((int64_t)ulo * d.c_lo + (int64_t)uhi * d.c_hi);
+      const int32_t tile_off = bit_sum(m0 + q * 32, my_cm) + (fold > 1 ? 0 : bit_sum(n0, my_cn));
       const int rb = (int)(t & 1);
       const uint32_t R = tmem + lane_off + (uint32_t)rb * BUF, P = tmem + lane_off + (uint32_t)(1 - rb) * BUF;
       for (int c = 0; c < nch; ++c) {
         const int b = c == 0 ? rb : 1 - rb;
-        bool ok = mbar_wait(&acc_full[b], seen[b] & 1, wl);
+        ok = mbar_wait_warp(&acc_full[b], seen[b] & 1, wl);
         ++seen[b];
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok && lane == 0) {
-          atomicExch(err, 34);
-          abort_flag = 1;
-          epi_fail = 1;
+        if (!ok) {
+          if (lane == 0) {
+            atomicExch(err, 34);
+            abort_flag = 1;
+          }
+          break;
         }
-        // colC of this item and any failure visible to every epilogue warp
-        asm volatile("bar.sync 1, %0;" ::"r"(ET) : "memory");
-        if (epi_fail) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (c == 0) continue;  // the first chunk accumulated in R itself
 #pragma unroll 1
@@ -799,11 +808,7 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[1 - rb])) : "memory");
       }
-      if (epi_fail) break;
-      float vmax = 0.f;
-      bool bad = false, weak = false;
-      int ea = 0, eb = 0, r = 0;
-      Pow2 sc(0);
+      if (!ok) break;
 #pragma unroll 1
       for (int c0 = 16 * h; c0 < TN; c0 += CS) {
         // columns of a folded tile belong to hi unit uhi + c0 / 2^nn (N >= 16:
@@ -811,48 +816,56 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
         // last chunks among a unit's gw columns open and close its records
         const int f = fold > 1 ? (c0 >> d.nn) : 0;
         if (c0 % gw < CS) {
-          unit_scale(f, ea, eb, r, weak);
-          sc = Pow2(c_planes ? -r : ea + eb);
-          vmax = 0.f;
-          bad = false;
+          if (f > 0) unit_scale(ulo, uhi, f);
+          vmax = fin[0] = fin[1] = 0.f;
         }
-        float2* C = Cu + (int64_t)f * d.c_hi;
         uint32_t ur[16], ui[16];
         tmem_ld<16>(R + (uint32_t)c0, ur);
         tmem_ld<16>(R + (uint32_t)(TN + c0), ui);
+        const int cc = fold > 1 ? (c0 & (nsub - 1)) : c0;
+        float2* const C = Cu + (int64_t)f * d.c_hi;
+        const int32_t off = tile_off + ((cc & 16) ? cn_mid[0] : 0) + ((cc & 32) ? cn_mid[1] : 0) +
+                            ((cc & 64) ? cn_mid[2] : 0);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (c0 + CS >= TN) {
+          // R read out: the MMA warp may start a later tile's chunks in it
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[rb])) : "memory");
+        }
         float vr[16], vi[16];
-        if (sc.direct && sc.f == 1.f) {
+        if (sc.direct) {
 #pragma unroll
           for (int jj = 0; jj < 16; ++jj) {
-            vr[jj] = __uint_as_float(ur[jj]);
-            vi[jj] = __uint_as_float(ui[jj]);
+            vr[jj] = __uint_as_float(ur[jj]) * sc.f;
+            vi[jj] = __uint_as_float(ui[jj]) * sc.f;
           }
         } else {
 #pragma unroll
           for (int jj = 0; jj < 16; ++jj) {
-            vr[jj] = sc(__uint_as_float(ur[jj]));
-            vi[jj] = sc(__uint_as_float(ui[jj]));
+            vr[jj] = ldexpf(__uint_as_float(ur[jj]), sc.e);
+            vi[jj] = ldexpf(__uint_as_float(ui[jj]), sc.e);
           }
         }
-        if (c_planes) {
-          uint16_t* Pl = reinterpret_cast<uint16_t*>(C);
-          const int64_t plane = int64_t(1) << (d.nm + d.nn);
+        if (planes) {
+          uint16_t* const Pl = reinterpret_cast<uint16_t*>(C) + off;
           if (track) {
+            // 0 x is 0 for a finite x and NaN for an infinity or NaN, so `fin`
+            // stays 0 until a value turns non-finite
 #pragma unroll
             for (int jj = 0; jj < 16; ++jj) {
               vmax = fmaxf(vmax, fmaxf(fabsf(vr[jj]), fabsf(vi[jj])));
-              bad |= !isfinite(vr[jj]) || !isfinite(vi[jj]);
+              fin[0] = fmaf(vr[jj], 0.f, fin[0]);
+              fin[1] = fmaf(vi[jj], 0.f, fin[1]);
             }
           }
-          uint32_t e[NP / 2][16];
+          uint32_t x[NP / 2][16];
           auto pack = [&](bool fmt) {
 #pragma unroll
             for (int jj = 0; jj < 16; ++jj) {
-              uint32_t x[NP / 2];
-              pack_planes<NP>(fmt, vr[jj], vi[jj], x);
+              uint32_t y[NP / 2];
+              pack_planes<NP>(fmt, vr[jj], vi[jj], y);
 #pragma unroll
-              for (int u = 0; u < NP / 2; ++u) e[u][jj] = x[u];
+              for (int u = 0; u < NP / 2; ++u) x[u][jj] = y[u];
             }
           };
           if (bf16) pack(true);
@@ -861,86 +874,75 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
             // planes of one element packed in one slot (4 NP / 2 bytes), in C order
 #pragma unroll
             for (int jj = 0; jj < 16; ++jj) {
-              if constexpr (NP == 4)
-                reinterpret_cast<uint2*>(slots)[lane_slot + col_slot(jj)] = make_uint2(e[0][jj], e[1][jj]);
-              else
-                reinterpret_cast<uint32_t*>(slots)[lane_slot + col_slot(jj)] = e[0][jj];
+              if constexpr (NP == 4) sts64(slot[jj], x[0][jj], x[1][jj]);
+              else sts32(slot[jj], x[0][jj]);
             }
             __syncwarp();
-            const int64_t ob = (int64_t)__shfl_sync(0xffffffffu, ro, 0) + colC[c0] + sm.off_pl;
+            uint4 y2[2][NP];  // C-order values 8 (lane + 32 t2) .. + 7, one slot each
 #pragma unroll
-            for (int t = 0; t < 2; ++t) {
-              // C-order values 8 (lane + 32 t) .. + 7, one slot each
+            for (int t2 = 0; t2 < 2; ++t2)
+#pragma unroll
+              for (int u = 0; u < NP; ++u)
+                y2[t2][u] = lds128(rd + 16 * u + t2 * (NP == 4 ? (256 + 32) * 8 : (256 + 32) * 4));
+#pragma unroll
+            for (int t2 = 0; t2 < 2; ++t2) {
               uint32_t v[NP / 2][8];
-              if constexpr (NP == 4) {
-                const uint4* src = reinterpret_cast<const uint4*>(slots) + stage_slot(8 * (lane + 32 * t)) / 2;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  const uint4 x = src[u];
-                  v[0][2 * u] = x.x;
-                  v[1][2 * u] = x.y;
-                  v[0][2 * u + 1] = x.z;
-                  v[1][2 * u + 1] = x.w;
-                }
-              } else {
-                const uint4* src = reinterpret_cast<const uint4*>(slots) + stage_slot4(8 * (lane + 32 * t)) / 4;
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                  const uint4 x = src[u];
-                  v[0][4 * u] = x.x;
-                  v[0][4 * u + 1] = x.y;
-                  v[0][4 * u + 2] = x.z;
-                  v[0][4 * u + 3] = x.w;
+              for (int u = 0; u < NP; ++u) {
+                const uint4 y = y2[t2][u];
+                if constexpr (NP == 4) {
+                  v[0][2 * u] = y.x;
+                  v[NP / 2 - 1][2 * u] = y.y;
+                  v[0][2 * u + 1] = y.z;
+                  v[NP / 2 - 1][2 * u + 1] = y.w;
+                } else {
+                  v[0][4 * u] = y.x;
+                  v[0][4 * u + 1] = y.y;
+                  v[0][4 * u + 2] = y.z;
+                  v[0][4 * u + 3] = y.w;
                 }
               }
-              const int64_t o = ob + (t ? sm.step_pl : 0);
 #pragma unroll
               for (int pl = 0; pl < NP; ++pl) {
                 auto pp = [&](int e0) {
                   return __byte_perm(v[pl >> 1][e0], v[pl >> 1][e0 + 1], (pl & 1) ? 0x7632 : 0x5410);
                 };
-                *reinterpret_cast<uint4*>(Pl + pl * plane + o) = make_uint4(pp(0), pp(2), pp(4), pp(6));
+                *reinterpret_cast<uint4*>(Pl + pl * plane + back[t2]) = make_uint4(pp(0), pp(2), pp(4), pp(6));
               }
             }
             __syncwarp();
           } else {
-            store_planes<NP>(Pl, plane, ro, &colC[c0], vb, e);
+            store_planes<NP>(Pl + lane_row, plane, cn_lo, vb, x);
           }
         } else if (sm.on) {
 #pragma unroll
-          for (int jj = 0; jj < 16; ++jj) slots[lane_slot + col_slot(jj)] = make_float2(vr[jj], vi[jj]);
+          for (int jj = 0; jj < 16; ++jj) sts64(slot[jj], __float_as_uint(vr[jj]), __float_as_uint(vi[jj]));
           __syncwarp();
-          const int64_t ob = (int64_t)__shfl_sync(0xffffffffu, ro, 0) + colC[c0] + sm.off_c64;
+          float2* const Co = C + off;
+          uint4 y[8];  // C-order values 2 (lane + 32 t2) and the next one: two adjacent slots
 #pragma unroll
-          for (int t = 0; t < 8; ++t) {
-            // C-order values 2 (lane + 32 t) and the next one: two adjacent slots
-            const float4 x = reinterpret_cast<const float4*>(slots)[stage_slot(2 * (lane + 32 * t)) / 2];
-            const int32_t o = ((t & 1) ? sm.step_c64[0] : 0) + ((t & 2) ? sm.step_c64[1] : 0) +
-                              ((t & 4) ? sm.step_c64[2] : 0);
-            *reinterpret_cast<float4*>(C + ob + o) = x;
-          }
+          for (int t2 = 0; t2 < 8; ++t2) y[t2] = lds128(rd + t2 * (64 + 8) * 8);
+#pragma unroll
+          for (int t2 = 0; t2 < 8; ++t2) *reinterpret_cast<uint4*>(Co + back[t2]) = y[t2];
           __syncwarp();
         } else {
-          store_c64(C, ro, &colC[c0], vb, vr, vi);
+          float2* const Co = C + off + lane_row;
+#pragma unroll
+          for (int jj = 0; jj < 16; ++jj) Co[col_offset(cn_lo, jj)] = make_float2(vr[jj], vi[jj]);
         }
-        if (c0 % gw + CS >= gw && (sio.mc || sio.flag)) {
+        if (c0 % gw + CS >= gw && track) {
           // the unit's columns are done: its largest stored component,
           // exponent and filter flag (launch unit ulo + (uhi + f) units_lo)
           const int un = fold > 1 ? ulo + (uhi + f) * d.units_lo : unit;
-          for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-          const bool any_bad = __any_sync(0xffffffffu, bad);
+          const float wmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(vmax)));
+          const bool bad = __any_sync(0xffffffffu, planes && !(fin[0] + fin[1] == 0.f));
           if (lane == 0) {
-            if (sio.mc && c_planes) atomicMax(sio.mc + un, __float_as_uint(vmax));
-            if (sio.ec && c_planes && q == 0 && m0 == 0 && n0 == 0) sio.ec[un] = ea + eb + r;
-            if (sio.flag && (any_bad || weak)) sio.flag[sio.flag_by_lo ? ulo : un] = 1;
+            if (sio.mc && planes) atomicMax(sio.mc + un, __float_as_uint(wmax));
+            if (sio.ec && planes && q == 0 && m0 == 0 && n0 == 0) sio.ec[un] = ea + eb + r;
+            if (sio.flag && (bad || weak)) sio.flag[sio.flag_by_lo ? ulo : un] = 1;
           }
         }
       }
-      // R read out: the MMA warp may start a later tile's chunks in it
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[rb])) : "memory");
-      // every epilogue thread is done with colC before the next item rewrites it
-      asm volatile("bar.sync 1, %0;" ::"r"(ET) : "memory");
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1001,7 +1003,7 @@ int sm_count() {
 
 template <int TN, int NP, int ROWB, int EW>
 cudaError_t launch_chunked_ew(const CUtensorMap& ma, const CUtensorMap& mb, float2* C, const GemmDesc& d, int kp,
-                              const int z[4], int c_planes, const ScaleIO& sio, int fold, bool bf16, int* err,
+                              const int z[4], int out_flags, const ScaleIO& sio, int fold, bool bf16, int* err,
                               cudaStream_t s, const BulkPlanes& ba, const BulkPlanes& bb) {
   using CC = ChunkCfg<TN, NP, ROWB, EW>;
   static bool attr = false;
@@ -1018,7 +1020,7 @@ cudaError_t launch_chunked_ew(const CUtensorMap& ma, const CUtensorMap& mb, floa
   const int chunk = NP == 4 ? split_chunk() : 1 << 30;
   const unsigned grid = (unsigned)std::min<int64_t>(items, sms);
   gemm_tma_chunked<TN, NP, ROWB, EW><<<grid, CC::THREADS, CC::SMEM, s>>>(ma, mb, C, d, kp, z[0], z[1], z[2], z[3],
-                                                                          c_planes, sio, chunk, fold, bf16, err, ba, bb);
+                                                                          out_flags, sio, chunk, fold, bf16, err, ba, bb);
   return cudaGetLastError();
 }
 
@@ -1028,11 +1030,11 @@ cudaError_t launch_chunked_ew(const CUtensorMap& ma, const CUtensorMap& mb, floa
 // does and the extra operand stage matters.
 template <int TN, int NP>
 cudaError_t launch_chunked(const CUtensorMap& ma, const CUtensorMap& mb, float2* C, const GemmDesc& d, int kp,
-                           const int z[4], int c_planes, const ScaleIO& sio, int fold, bool bf16, int* err,
+                           const int z[4], int out_flags, const ScaleIO& sio, int fold, bool bf16, int* err,
                            cudaStream_t s, const BulkPlanes& ba, const BulkPlanes& bb) {
   constexpr int EWS = TN >= 64 ? 8 : 4;  // a single K stage or a few
   auto go = [&](auto rowb, auto ew) {
-    return launch_chunked_ew<TN, NP, decltype(rowb)::value, decltype(ew)::value>(ma, mb, C, d, kp, z, c_planes, sio,
+    return launch_chunked_ew<TN, NP, decltype(rowb)::value, decltype(ew)::value>(ma, mb, C, d, kp, z, out_flags, sio,
                                                                                 fold, bf16, err, s, ba, bb);
   };
   using std::integral_constant;
@@ -1100,7 +1102,9 @@ cudaError_t launch_gemm_tma(const PlaneOperand& a, const PlaneOperand& b, float2
   if (!encode_planes(&ma, a, TM) || !encode_planes(&mb, b, b_rows, fold > 1 ? 1 : 0)) return cudaErrorInvalidValue;
   const int kpi = (int)a.kp;
   const int z[4] = {a.nlo > 1, a.nhi > 1, b.nlo > 1, b.nhi > 1};
-  const int cp = c_planes ? 1 : 0;
+  // bit 0: plane output; bit 1: every even element of C on a 16-byte boundary
+  const int cp = (c_planes ? 1 : 0) |
+                 ((reinterpret_cast<uintptr_t>(C) & 15) == 0 && (d.c_lo & 1) == 0 && (d.c_hi & 1) == 0 ? 2 : 0);
   // K = 8: the operands' 16-byte rows go by contiguous bulk copies (one per
   // plane) instead of tensor-map boxes of 16-byte rows; every address and
   // size must be a multiple of 16 bytes, else the tensor maps serve
