@@ -245,6 +245,22 @@ void make_gemm_desc(const std::vector<int>& la, const std::vector<int>& lb, cons
   d.units = d.units_lo = 1;
 }
 
+// Renumbers the M and the N bits by the output's memory order (bit 0 = C's
+// fastest index of that group).  A GEMM tile takes the low bits of both, so its
+// elements then cover C's fastest indices whatever their order, and its stores
+// form long runs; values and their summation order do not change.
+void order_by_output(GemmDesc& d) {
+  auto sort2 = [](int n, int32_t* key, int32_t* other) {
+    for (int i = 1; i < n; ++i)
+      for (int j = i; j > 0 && key[j - 1] > key[j]; --j) {
+        std::swap(key[j - 1], key[j]);
+        std::swap(other[j - 1], other[j]);
+      }
+  };
+  sort2(d.nm, d.cm, d.am);
+  sort2(d.nn, d.cn, d.bn);
+}
+
 // Leaf store of a plan: every leaf in complex64 at its store offset.
 static tn_status upload_leaves(const Plan& P, float2** store) {
   const Network& N = P.net;

@@ -14,6 +14,7 @@
 
 #include <algorithm>
 
+#include "device_common.h"
 #include "kernels.h"
 
 namespace tn {
@@ -29,60 +30,38 @@ __device__ __forceinline__ float from16(uint16_t h, bool bf16) {
   return bf16 ? __bfloat162float(__ushort_as_bfloat16(h)) : __half2float(__ushort_as_half(h));
 }
 
-__device__ __forceinline__ int64_t src_offset_row(const SplitDesc& d, int64_t r) {
-  int32_t ro = 0;
-  for (int i = 0; i < d.nrow; ++i)
-    if ((r >> i) & 1) ro += d.row_st[i];
-  return ro;
-}
-
-// Load 8 consecutive K values (zero beyond K) of row r.
-__device__ __forceinline__ void load8(const float2* __restrict__ src, const SplitDesc& d, bool rok, int64_t ro,
-                                      int64_t c, float2* v) {
-  const int64_t K = int64_t(1) << d.nk;
-  if (d.kvec && rok && c * 8 < K) {
-    // 8 consecutive K values are contiguous: one 64-byte run
-    int32_t ko = 0;
-    const int64_t k0 = c * 8;
-    for (int i = 3; i < d.nk; ++i)
-      if ((k0 >> i) & 1) ko += d.k_st[i];
-    const float4* p = reinterpret_cast<const float4*>(src + ro + ko);
+// Largest |component| of each distinct tensor z (float bits, atomicMax).  The
+// operand is a dense block of 2^bits elements whatever its index order, so the
+// pass reads it front to back, 16 bytes per load.
+__global__ void __launch_bounds__(NT) max_kernel(const float2* __restrict__ src, int bits, int nlo, int64_t lo,
+                                                 int64_t hi, int vec, unsigned* __restrict__ maxbits) {
+  const int64_t z = blockIdx.y;
+  src += (z % nlo) * lo + (z / nlo) * hi;
+  float m = 0.f;
+  const int64_t step = (int64_t)gridDim.x * NT;
+  const int64_t at = (int64_t)blockIdx.x * NT + threadIdx.x;
+  if (vec) {
+    const float4* p = reinterpret_cast<const float4*>(src);
+    const int64_t n = int64_t(1) << (bits - 1);
+    int64_t e = at;
+    for (; e + 7 * step < n; e += 8 * step) {
+      float4 v[8];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float4 x = __ldg(p + q);
-      v[2 * q] = make_float2(x.x, x.y);
-      v[2 * q + 1] = make_float2(x.z, x.w);
+      for (int j = 0; j < 8; ++j) v[j] = __ldg(p + e + j * step);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        m = fmaxf(m, fmaxf(fmaxf(fabsf(v[j].x), fabsf(v[j].y)), fmaxf(fabsf(v[j].z), fabsf(v[j].w))));
+    }
+    for (; e < n; e += step) {
+      const float4 v = __ldg(p + e);
+      m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
     }
   } else {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int64_t k = c * 8 + j;
-      v[j] = make_float2(0.f, 0.f);
-      if (rok && k < K) {
-        int32_t ko = 0;
-        for (int i = 0; i < d.nk; ++i)
-          if ((k >> i) & 1) ko += d.k_st[i];
-        v[j] = __ldg(src + ro + ko);
-      }
+    const int64_t n = int64_t(1) << bits;
+    for (int64_t e = at; e < n; e += step) {
+      const float2 v = __ldg(src + e);
+      m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
     }
-  }
-}
-
-// Largest |component| of each distinct tensor z (float bits, atomicMax).
-__global__ void __launch_bounds__(NT) max_kernel(const float2* __restrict__ src, const SplitDesc d,
-                                                 unsigned* __restrict__ maxbits) {
-  const int64_t rows = int64_t(1) << d.nrow;
-  const int64_t chunks = d.kp / 8;
-  const int64_t z = blockIdx.y;
-  src += (z % d.nlo) * d.lo + (z / d.nlo) * d.hi;
-  float m = 0.f;
-  const int64_t total = rows * chunks;
-  for (int64_t e = (int64_t)blockIdx.x * NT + threadIdx.x; e < total; e += (int64_t)gridDim.x * NT) {
-    const int64_t r = e / chunks, c = e % chunks;
-    float2 v[8];
-    load8(src, d, true, src_offset_row(d, r), c, v);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) m = fmaxf(m, fmaxf(fabsf(v[j].x), fabsf(v[j].y)));
   }
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   __shared__ float wm[NT / 32];
@@ -102,16 +81,65 @@ __device__ __forceinline__ int scale_exponent(float mx) {
   return x - 14;
 }
 
-// One thread: one row and one chunk of 8 K values -> one 16-byte store per plane.
+// Eight elements (scaled, consecutive in K order) as one 16-byte store per plane.
 template <int NP>
+__device__ __forceinline__ void store8(uint16_t* out, int64_t plane, const float2* v, const Pow2& sc, bool bf16) {
+  uint16_t h[NP][8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const float re = sc(v[j].x), im = sc(v[j].y);
+    if (NP == 4) {
+      h[0][j] = to16(re, bf16);
+      h[1][j] = to16(re - from16(h[0][j], bf16), bf16);
+      h[NP / 2][j] = to16(im, bf16);
+      h[NP / 2 + 1][j] = to16(im - from16(h[NP / 2][j], bf16), bf16);
+    } else {
+      h[0][j] = to16(re, bf16);
+      h[1][j] = to16(im, bf16);
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    uint4 w;
+    w.x = (uint32_t)h[p][0] | ((uint32_t)h[p][1] << 16);
+    w.y = (uint32_t)h[p][2] | ((uint32_t)h[p][3] << 16);
+    w.z = (uint32_t)h[p][4] | ((uint32_t)h[p][5] << 16);
+    w.w = (uint32_t)h[p][6] | ((uint32_t)h[p][7] << 16);
+    *reinterpret_cast<uint4*>(out + p * plane) = w;
+  }
+}
+
+// The split pass as a tiled transpose.  An operand is a dense block of 2^R
+// elements and so is each plane; they differ in the order of their R index
+// bits.  A tile is the 2^T elements spanned by T of those bits, chosen to hold
+// both the output's fastest bits and the input's fastest ones, so whatever the
+// order, a CTA reads runs of 2^(T/2) input elements and writes runs of
+// 2^(T/2) values per plane, and turns the tile in shared memory.  (Reading 8
+// values per thread through the index strides touched a 32-byte sector per
+// 8-byte element on random orders: a 2^29-element operand took 2.8 ms for its
+// maximum and 3.4 ms for its split, whose bytes move in 0.64 and 1.3 ms; the
+// (16, 6, 13) contraction it belongs to went from 7.3 to 3.4 ms with this.)
+struct TileMap {
+  int nout;                 // index bits outside the tile
+  int32_t out_src[kMaxBits];   // their strides in the input ..
+  int8_t out_dst[kMaxBits];    // .. and their bit positions in a plane
+  // the tile's bits in input order (fastest first): input stride, and what the
+  // bit flips in the element's shared-memory slot
+  int32_t in_src[12], in_slot[12];
+  // .. and in output order: what the bit flips in the slot, bit position in a plane
+  int32_t out_slot[12];
+  int8_t dst[12];
+};
+
+template <int NP, int T>
 __global__ void __launch_bounds__(NT) split_kernel(const float2* __restrict__ src, uint16_t* __restrict__ dst,
-                                                   const SplitDesc d, bool bf16, const unsigned* __restrict__ maxbits,
+                                                   const __grid_constant__ TileMap tm, int bits, int nlo, int64_t lo,
+                                                   int64_t hi, int vec, bool bf16, const unsigned* __restrict__ maxbits,
                                                    int* __restrict__ e_out, float* __restrict__ m_out) {
-  const int64_t rows = int64_t(1) << d.nrow;
-  const int64_t kp = d.kp;
-  const int64_t chunks = kp / 8;
+  constexpr int E = 1 << T;
+  __shared__ __align__(16) float2 tile[E];
   const int64_t z = blockIdx.y;
-  src += (z % d.nlo) * d.lo + (z / d.nlo) * d.hi;
+  src += (z % nlo) * lo + (z / nlo) * hi;
   int e = 0;
   if (maxbits) {
     const float mx = __uint_as_float(maxbits[z]);
@@ -121,58 +149,196 @@ __global__ void __launch_bounds__(NT) split_kernel(const float2* __restrict__ sr
       m_out[z] = ldexpf(mx, -e);
     }
   }
-  const int64_t plane = (int64_t)d.rows_pad * kp;
+  const Pow2 sc(-e);
+  const int64_t plane = int64_t(1) << bits;
   uint16_t* out = dst + z * NP * plane;
-  const int64_t total = (int64_t)d.rows_pad * chunks;
-  for (int64_t q = (int64_t)blockIdx.x * NT + threadIdx.x; q < total; q += (int64_t)gridDim.x * NT) {
-    const int64_t r = q / chunks, c = q % chunks;
-    const bool rok = r < rows;
-    float2 v[8];
-    load8(src, d, rok, rok ? src_offset_row(d, r) : 0, c, v);
-    uint16_t h[NP][8];
+  {
+    int32_t so = 0;
+    int64_t dofs = 0;
+    for (int b = 0; b < tm.nout; ++b)
+      if ((blockIdx.x >> b) & 1) {
+        so += tm.out_src[b];
+        dofs += int64_t(1) << tm.out_dst[b];
+      }
+    src += so;
+    out += dofs;
+  }
+  const int t = threadIdx.x;
+  // load: pairs of input-adjacent elements, pair q = t + NT j (bits 1.. of the input order)
+  constexpr int PAIRS = E / 2, PL = PAIRS < NT ? PAIRS : NT, NJ = PAIRS / PL;
+  constexpr int TB = PL == 256 ? 8 : PL == 128 ? 7 : 6;  // bits of t in a pair index
+  static_assert(PL == (1 << TB), "tile size");
+  if (t < PL) {
+    int32_t so = 0, slot = 0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float re = ldexpf(v[j].x, -e), im = ldexpf(v[j].y, -e);
-      if (NP == 4) {
-        h[0][j] = to16(re, bf16);
-        h[1][j] = to16(re - from16(h[0][j], bf16), bf16);
-        h[NP / 2][j] = to16(im, bf16);
-        h[NP / 2 + 1][j] = to16(im - from16(h[NP / 2][j], bf16), bf16);
+    for (int b = 0; b < TB; ++b)
+      if ((t >> b) & 1) {
+        so += tm.in_src[1 + b];
+        slot ^= tm.in_slot[1 + b];
+      }
+    float2 v[NJ][2];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      int32_t o = so;
+#pragma unroll
+      for (int b = 0; b < T - 1 - TB; ++b)
+        if ((j >> b) & 1) o += tm.in_src[1 + TB + b];
+      if (vec) {
+        const float4 x = __ldg(reinterpret_cast<const float4*>(src + o));
+        v[j][0] = make_float2(x.x, x.y);
+        v[j][1] = make_float2(x.z, x.w);
       } else {
-        h[0][j] = to16(re, bf16);
-        h[1][j] = to16(im, bf16);
+        v[j][0] = __ldg(src + o);
+        v[j][1] = __ldg(src + o + 1);
       }
     }
-    const int64_t o = r * kp + c * 8;
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      uint4 w;
-      w.x = (uint32_t)h[p][0] | ((uint32_t)h[p][1] << 16);
-      w.y = (uint32_t)h[p][2] | ((uint32_t)h[p][3] << 16);
-      w.z = (uint32_t)h[p][4] | ((uint32_t)h[p][5] << 16);
-      w.w = (uint32_t)h[p][6] | ((uint32_t)h[p][7] << 16);
-      *reinterpret_cast<uint4*>(out + p * plane + o) = w;
+    for (int j = 0; j < NJ; ++j) {
+      int32_t p = slot;
+#pragma unroll
+      for (int b = 0; b < T - 1 - TB; ++b)
+        if ((j >> b) & 1) p ^= tm.in_slot[1 + TB + b];
+      tile[p] = v[j][0];
+      tile[p ^ tm.in_slot[0]] = v[j][1];
     }
   }
+  __syncthreads();
+  // store: eight consecutive output elements per thread
+  constexpr int GROUPS = E / 8, GL = GROUPS < NT ? GROUPS : NT;
+  if (t < GL) {
+#pragma unroll
+    for (int g0 = 0; g0 < GROUPS; g0 += GL) {
+      const int g = g0 + t;
+      int32_t slot = 0;
+      int64_t o = 0;
+#pragma unroll
+      for (int b = 3; b < T; ++b)
+        if ((g >> (b - 3)) & 1) {
+          slot ^= tm.out_slot[b];
+          o += int64_t(1) << tm.dst[b];
+        }
+      float2 v[8];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float4 y = *reinterpret_cast<const float4*>(&tile[slot ^ (2 * c)]);
+        v[2 * c] = make_float2(y.x, y.y);
+        v[2 * c + 1] = make_float2(y.z, y.w);
+      }
+      store8<NP>(out + o, plane, v, sc, bf16);
+    }
+  }
+}
+
+// The tile of T bits for an operand whose output bit i (K bits, then row bits)
+// has input stride st[i], R bits in all.
+//
+// Slots: the element with output-order index x sits at x with bits 4 and 5
+// folded onto bits 1 and 2 -- a thread reads its 8 elements as four 16-byte
+// loads, lanes 64 bytes apart, and the fold spreads every quarter-warp over all
+// banks -- and with bits 6.. folded onto bits 1..3 where that makes the slots
+// of a half-warp's stores (input bits 1..4 vary) independent in the 16 banks.
+template <int T>
+TileMap split_tile_map(const SplitDesc& d) {
+  TileMap m{};
+  const int R = d.nk + d.nrow;
+  int32_t st[kMaxBits];
+  for (int i = 0; i < R; ++i) st[i] = i < d.nk ? d.k_st[i] : d.row_st[i - d.nk];
+  bool in[kMaxBits] = {};
+  int count = 0;
+  auto take = [&](int i) {
+    if (!in[i] && count < T) {
+      in[i] = true;
+      ++count;
+    }
+  };
+  for (int i = 0; i < T / 2; ++i) take(i);
+  for (int i = 0; i < R; ++i)
+    if (st[i] < (int32_t(1) << ((T + 1) / 2))) take(i);
+  for (int i = 0; i < R; ++i) take(i);
+  int pos[kMaxBits];  // output-order position in the tile
+  int nd = 0;
+  for (int i = 0; i < R; ++i) {
+    if (in[i]) {
+      pos[i] = nd;
+      m.dst[nd++] = (int8_t)i;
+    } else {
+      m.out_src[m.nout] = st[i];
+      m.out_dst[m.nout++] = (int8_t)i;
+    }
+  }
+  int order[12], n = 0;  // the tile's output bits by input stride
+  for (int i = 0; i < R; ++i)
+    if (in[i]) {
+      int j = n++;
+      for (; j > 0 && st[order[j - 1]] > st[i]; --j) order[j] = order[j - 1];
+      order[j] = i;
+    }
+  for (int b = 0; b < T; ++b) m.out_slot[b] = (1 << b) ^ (b == 4 ? 2 : b == 5 ? 4 : 0);
+  // span of the chosen lane bits' low four slot bits (bitmap of the 16 vectors)
+  unsigned span = 1;
+  auto add = [&](int v) {
+    unsigned s = span;
+    for (int x = 0; x < 16; ++x)
+      if ((span >> x) & 1) s |= 1u << (x ^ v);
+    span = s;
+  };
+  for (int l = 1; l <= 4; ++l)
+    if (pos[order[l]] < 6) add(m.out_slot[pos[order[l]]] & 15);
+  for (int l = 1; l <= 4; ++l) {
+    const int p = pos[order[l]];
+    if (p < 6) continue;
+    for (int v = 2; v < 16; v += 2)
+      if (!((span >> v) & 1)) {
+        m.out_slot[p] ^= v;
+        add(v);
+        break;
+      }
+  }
+  for (int l = 0; l < T; ++l) {
+    m.in_src[l] = st[order[l]];
+    m.in_slot[l] = m.out_slot[pos[order[l]]];
+  }
+  return m;
+}
+
+template <int NP, int T>
+cudaError_t launch_tiles(const float2* src, uint16_t* dst, const SplitDesc& d, int nz, bool vec, bool bf16,
+                         const unsigned* maxbits, int* e_out, float* m_out, cudaStream_t s) {
+  const int R = d.nk + d.nrow;
+  split_kernel<NP, T><<<dim3(1u << (R - T), (unsigned)nz), NT, 0, s>>>(src, dst, split_tile_map<T>(d), R, d.nlo, d.lo,
+                                                                       d.hi, vec, bf16, maxbits, e_out, m_out);
+  return cudaGetLastError();
+}
+
+// 2^12-element tiles once they fill the chip a few times over (152 SMs, six
+// such CTAs each); smaller ones spread a small operand over more SMs.
+template <int NP>
+cudaError_t launch_np(const float2* src, uint16_t* dst, const SplitDesc& d, int nz, bool vec, bool bf16,
+                      const unsigned* maxbits, int* e_out, float* m_out, cudaStream_t s) {
+  const int R = d.nk + d.nrow;
+  if (R >= 12 && (int64_t(1) << (R - 12)) * nz >= 152 * 4)
+    return launch_tiles<NP, 12>(src, dst, d, nz, vec, bf16, maxbits, e_out, m_out, s);
+  if (R >= 10) return launch_tiles<NP, 10>(src, dst, d, nz, vec, bf16, maxbits, e_out, m_out, s);
+  return launch_tiles<NP, 7>(src, dst, d, nz, vec, bf16, maxbits, e_out, m_out, s);
 }
 
 }  // namespace
 
 cudaError_t launch_split(const float2* src, uint16_t* dst, const SplitDesc& d, int nz, bool bf16, int np,
                          unsigned* maxbits, int* e_out, float* m_out, cudaStream_t s, bool max_ready) {
-  if (nz < 1 || nz > 65535 || d.kp % 8 != 0 || (np != 2 && np != 4)) return cudaErrorInvalidValue;
-  const int64_t total = (int64_t)d.rows_pad * (d.kp / 8);
-  const int64_t blocks = std::min<int64_t>((total + NT - 1) / NT, 152 * 8);
+  const int R = d.nk + d.nrow;
+  if (nz < 1 || nz > 65535 || R < 7 || R > 30 || (np != 2 && np != 4)) return cudaErrorInvalidValue;
+  const bool vec = (reinterpret_cast<uintptr_t>(src) & 15) == 0 && (d.lo & 1) == 0 && (d.hi & 1) == 0;
   if (maxbits && !max_ready) {
-    max_kernel<<<dim3((unsigned)blocks, (unsigned)nz), NT, 0, s>>>(src, d, maxbits);
-    cudaError_t e = cudaGetLastError();
+    // 8 loads of 16 bytes per thread where there is enough to fill the chip
+    const int64_t n = int64_t(1) << (R - 1);
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(n / (NT * 8), 152 * 8));
+    max_kernel<<<dim3((unsigned)blocks, (unsigned)nz), NT, 0, s>>>(src, R, d.nlo, d.lo, d.hi, vec, maxbits);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  if (np == 4)
-    split_kernel<4><<<dim3((unsigned)blocks, (unsigned)nz), NT, 0, s>>>(src, dst, d, bf16, maxbits, e_out, m_out);
-  else
-    split_kernel<2><<<dim3((unsigned)blocks, (unsigned)nz), NT, 0, s>>>(src, dst, d, bf16, maxbits, e_out, m_out);
-  return cudaGetLastError();
+  return np == 4 ? launch_np<4>(src, dst, d, nz, vec, bf16, maxbits, e_out, m_out, s)
+                 : launch_np<2>(src, dst, d, nz, vec, bf16, maxbits, e_out, m_out, s);
 }
 
 namespace {
@@ -180,17 +346,11 @@ void split_desc(int nrow, const int32_t* row_st, int nk, const int32_t* k_st, in
                 SplitDesc& sd) {
   sd.nrow = nrow;
   sd.nk = nk;
-  sd.rows_pad = 1 << nrow;
-  sd.kp = 1 << nk;  // tensor-core shapes have K >= 8: whole 16-byte chunks, no padding
   sd.nlo = nlo;
   sd.lo = lo;
   sd.hi = hi;
   for (int i = 0; i < nrow; ++i) sd.row_st[i] = row_st[i];
   for (int i = 0; i < nk; ++i) sd.k_st[i] = k_st[i];
-  // vector path: K >= 8 with its three lowest bits contiguous, 16-byte aligned rows
-  bool rows_aligned = true;
-  for (int i = 0; i < nrow; ++i) rows_aligned &= (row_st[i] % 2) == 0;
-  sd.kvec = nk >= 3 && k_st[0] == 1 && k_st[1] == 2 && k_st[2] == 4 && rows_aligned && (lo % 2) == 0 && (hi % 2) == 0;
 }
 int distinct(const GemmDesc& d, int64_t lo, int64_t hi) {
   return (lo ? d.units_lo : 1) * (hi ? d.units / d.units_lo : 1);
@@ -213,10 +373,11 @@ cudaError_t split_operand(const float2* src, const GemmDesc& d, bool which_b, bo
   split_desc(nrow, which_b ? d.bn : d.am, d.nk, which_b ? d.bk : d.ak, lo ? d.units_lo : 1, lo, hi, sd);
   const int nz = distinct(d, lo, hi);
   cudaError_t e = launch_split(src, scratch, sd, nz, bf16, np, scaled ? maxbits : nullptr, e_out, m_out, s, max_ready);
-  const int64_t set = (int64_t)np * (int64_t(1) << nrow) * sd.kp * 2;
+  const int64_t K = int64_t(1) << d.nk;  // tensor-core shapes have K >= 8: whole 16-byte chunks, no padding
+  const int64_t set = (int64_t)np * (int64_t(1) << nrow) * K * 2;
   out.base = scratch;
   out.np = np;
-  out.kp = sd.kp;
+  out.kp = K;
   out.rows = int64_t(1) << nrow;
   out.nlo = lo ? d.units_lo : 1;
   out.nhi = hi ? d.units / d.units_lo : 1;

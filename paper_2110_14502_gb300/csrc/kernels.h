@@ -73,13 +73,12 @@ cudaError_t launch_gemm_tc(const float2* A, const float2* B, float2* C, const Ge
 // Operand preparation for the TMA-fed GEMM: rows = M (A) or N (B), each row a
 // K run; element (r, k) at sum bit_i(r) row_st[i] + sum bit_l(k) k_st[l] of
 // the source tensor number z, whose base is src + (z % nlo) * lo + (z / nlo) * hi.
-// Output: per z four planes {re_hi, re_lo, im_hi, im_lo} of rows_pad x kp
-// 16-bit values (kp = K >= 8; the GEMM's TMA copies read past a short K as zeros).
+// Output: per z four planes {re_hi, re_lo, im_hi, im_lo}, or two {re, im}, of
+// 2^nrow rows x 2^nk 16-bit values.  The strides of one tensor's indices are
+// 1, 2, 4, .. in some order (a dense block).
 struct SplitDesc {
   int nrow, nk;
-  int rows_pad, kp;
   int nlo;
-  int kvec;  // 8 consecutive K values contiguous and 16-byte aligned: vector loads
   int64_t lo, hi;
   int32_t row_st[kMaxBits], k_st[kMaxBits];
 };
@@ -195,5 +194,7 @@ struct Step;
 // kernel) instead of A's (GEMM kernels, whose A rows follow A's layout).
 void make_gemm_desc(const std::vector<int>& la, const std::vector<int>& lb, const std::vector<int>& lc,
                     GemmDesc& d, bool m_by_output = false);
+// M and N bits renumbered by the output's memory order.
+void order_by_output(GemmDesc& d);
 
 }  // namespace tn
