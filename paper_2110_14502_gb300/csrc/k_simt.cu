@@ -7,29 +7,35 @@
 // the operand's per-bit strides (the analogue of the paper's pre-computed
 // position array): a row's offset is computed once per CTA, and a K offset
 // splits into the chunk's high bits (once per chunk) plus a per-thread
-// constant for the low four bits.
+// constant for the low bits.
 //
-// Tiling: a CTA of 256 threads computes a 128 x BN tile of C (BN = 64 or 128)
-// over K chunks of 16.  Each thread owns an 8-row x (BN / 16)-column complex
-// micro-tile: per chunk and k it reads 8 A values (4 x 16-byte shared loads,
-// broadcast across the warp) and BN/16 B values, and issues 8 * BN/16 complex
-// multiply-adds of 4 FFMA each.  The tiles are staged in shared memory k-major
-// ([k][row], rows contiguous) with two buffers: the global loads of chunk c+1
-// are in flight in registers while chunk c is computed, then stored to the
-// other buffer; one barrier per chunk.
+// Tiling: 256 threads compute a BM x BN tile of C over K chunks of BK, each
+// thread an RM-row x RN-column complex micro-tile.  The tiles are staged in
+// shared memory k-major ([k][row], rows contiguous) with two buffers: the
+// global loads of chunk c+1 are in flight in registers while chunk c is
+// computed, then stored to the other buffer; one barrier per chunk.
+//
+// Arithmetic: packed FP32 (fma.rn.f32x2), one instruction for two of a complex
+// multiply-add's four FMAs: (re, im) += (ar, ar) (br, bi), then += (-ai, ai)
+// (bi, br).  The same four roundings in the same order as scalar FMAs, k
+// ascending, so every tile shape gives the same bits.  A sits in shared memory
+// already as (ar, ar, -ai, ai), so its operands are one 16-byte load; B's
+// swapped pair costs a register move, which issues beside the packed FMAs.
 //
 // Global loads: when the operand's two fastest indices are its first two K
 // bits (the planner's layouts put contracted indices innermost), a thread
-// reads 4 consecutive K values of one row as two 16-byte loads and the 32
-// lanes of a warp read 32 rows at the same K quad (one 32-byte sector per
+// reads 4 consecutive K values of one row as two 16-byte loads and the lanes
+// of a warp read consecutive rows at the same K quad (one 32-byte sector per
 // row); otherwise each lane reads one element, lanes on consecutive rows.
+#include <algorithm>
+
 #include "kernels.h"
 
 namespace tn {
 
 namespace {
 
-constexpr int BM = 128, BK = 16, NT = 256;
+constexpr int NT = 256;
 
 __device__ __forceinline__ int32_t bit_offset(int64_t x, int nb, const int32_t* st) {
   int32_t o = 0;
@@ -38,53 +44,68 @@ __device__ __forceinline__ int32_t bit_offset(int64_t x, int nb, const int32_t* 
   return o;
 }
 
-// Offset of the K bits at and above bit 4 of k0 (a multiple of 16).
+__host__ __device__ constexpr int ilog2(int x) { return x <= 1 ? 0 : 1 + ilog2(x / 2); }
+
+// Offset of the K bits at and above bit LOW of k0 (a multiple of 2^LOW).
+template <int LOW>
 __device__ __forceinline__ int32_t k_high_offset(int64_t k0, int nk, const int32_t* st) {
   int32_t o = 0;
-  for (int i = 4; i < nk; ++i)
+  for (int i = LOW; i < nk; ++i)
     if ((k0 >> i) & 1) o += st[i];
   return o;
 }
 
-// One operand tile of R rows (128 or 64) x 16 K values: what this thread
-// loads, where from and where it goes in shared memory.
-template <int R>
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 swap2(f32x2 v) {
+  const float2 r = unpack2(v);
+  return pack2(r.y, r.x);
+}
+__device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+
+// One operand tile of R rows x BK K values: what this thread loads, where from
+// and where it goes in shared memory.  Thread t takes row t % R at K positions
+// (t / R) + (256 / R) j -- single values, or quads of 4 (vec).
+template <int R, int BK>
 struct TileLoader {
-  static constexpr int NQ = R / 64;        // K quads per thread (vector path)
-  static constexpr int NE = R / 16;        // elements per thread (scalar path)
-  static constexpr int STEP = NT / R;      // K distance between a thread's scalar elements
+  static constexpr int NE = R * BK / NT;   // elements per thread
+  static constexpr int NQ = NE / 4;        // quads per thread (vector path)
+  static constexpr int STEP = NT / R;
+  static_assert(NE >= 4, "tile too small");
   bool vec;
   int64_t K;
-  int kq;                 // vector path: K quad of this thread
-  int32_t row_off[NQ > 0 ? NQ : 1];
-  int row[NQ > 0 ? NQ : 1];
-  int32_t low_q;          // offset of K = 4 kq within a chunk
-  int srow;               // scalar path: this thread's row
-  int32_t srow_off;
-  int32_t low_s[NE];      // offsets of K = kk0 + STEP j within a chunk
-  int kk0;
+  int row, kk0;
+  int32_t row_off;
+  int32_t low[NE];        // offsets of this thread's K positions within a chunk (vector path: of its quads)
   float2 v[NE];           // staged values (vector path: quad q's 4 values at 4 q ..)
 
   __device__ void init(const GemmDesc& d, int nrow_bits, const int32_t* rst, const int32_t* kst, int64_t r0,
                        bool vector_ok) {
     const int t = threadIdx.x;
+    constexpr int LOW = ilog2(BK);
     K = int64_t(1) << d.nk;
-    const int64_t nrows = int64_t(1) << nrow_bits;
     vec = vector_ok;
+    row = t % R;
+    kk0 = t / R;
+    row_off = r0 + row < (int64_t(1) << nrow_bits) ? bit_offset(r0 + row, nrow_bits, rst) : -1;
+    const int lb = d.nk < LOW ? d.nk : LOW;
     if (vec) {
-      kq = (t >> 5) & 3;
-      low_q = bit_offset(4 * kq, d.nk < 4 ? d.nk : 4, kst);
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        row[q] = (t & 31) + 32 * (t >> 7) + 64 * q;
-        row_off[q] = r0 + row[q] < nrows ? bit_offset(r0 + row[q], nrow_bits, rst) : -1;
-      }
+      for (int j = 0; j < NQ; ++j) low[j] = bit_offset(4 * (kk0 + STEP * j), lb, kst);
     } else {
-      srow = t % R;
-      kk0 = t / R;
-      srow_off = r0 + srow < nrows ? bit_offset(r0 + srow, nrow_bits, rst) : -1;
 #pragma unroll
-      for (int j = 0; j < NE; ++j) low_s[j] = bit_offset(kk0 + STEP * j, d.nk < 4 ? d.nk : 4, kst);
+      for (int j = 0; j < NE; ++j) low[j] = bit_offset(kk0 + STEP * j, lb, kst);
     }
   }
 
@@ -93,8 +114,8 @@ struct TileLoader {
 #pragma unroll
       for (int q = 0; q < NQ; ++q) {
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
-        if (row_off[q] >= 0 && k0 + 4 * kq < K) {
-          const float4* p = reinterpret_cast<const float4*>(src + row_off[q] + khi + low_q);
+        if (row_off >= 0 && k0 + 4 * (kk0 + STEP * q) < K) {
+          const float4* p = reinterpret_cast<const float4*>(src + row_off + khi + low[q]);
           x = __ldg(p);
           y = __ldg(p + 1);
         }
@@ -107,35 +128,45 @@ struct TileLoader {
 #pragma unroll
       for (int j = 0; j < NE; ++j) {
         float2 x = make_float2(0.f, 0.f);
-        if (srow_off >= 0 && k0 + kk0 + STEP * j < K) x = __ldg(src + srow_off + khi + low_s[j]);
+        if (row_off >= 0 && k0 + kk0 + STEP * j < K) x = __ldg(src + row_off + khi + low[j]);
         v[j] = x;
       }
     }
   }
 
-  // tile [BK][R] in shared memory
-  __device__ __forceinline__ void store(float2* tile) const {
+  // every staged value with its tile position [BK][R]
+  template <class F>
+  __device__ __forceinline__ void store(F&& put) const {
     if (vec) {
 #pragma unroll
       for (int q = 0; q < NQ; ++q)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) tile[(4 * kq + j) * R + row[q]] = v[4 * q + j];
+        for (int j = 0; j < 4; ++j) put((4 * (kk0 + STEP * q) + j) * R + row, v[4 * q + j]);
     } else {
 #pragma unroll
-      for (int j = 0; j < NE; ++j) tile[(kk0 + STEP * j) * R + srow] = v[j];
+      for (int j = 0; j < NE; ++j) put((kk0 + STEP * j) * R + row, v[j]);
     }
   }
 };
 
+template <int BM, int BN, int BK, int RM, int RN>
+struct SimtCfg {
+  static_assert(BM / RM * (BN / RN) == NT, "256 threads");
+  static constexpr int A_BUF = BK * BM * 16, B_BUF = BK * BN * 8;
+  static constexpr int SMEM = 2 * (A_BUF + B_BUF);
+};
+
 // flags: bit 0 A vector loads, bit 1 B vector loads, bit 2 C pair stores
-template <int BN>
-__global__ void __launch_bounds__(NT, 1) gemm_simt_kernel(const float2* __restrict__ A,
+template <int BM, int BN, int BK, int RM, int RN>
+__global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_kernel(const float2* __restrict__ A,
                                                            const float2* __restrict__ B,
                                                            float2* __restrict__ C, const GemmDesc d, int flags) {
-  constexpr int WN = BN / 16;  // complex columns per thread
-  extern __shared__ __align__(16) float2 smem[];
-  float2* As = smem;                 // [2][BK][BM]
-  float2* Bs = smem + 2 * BK * BM;   // [2][BK][BN]
+  using CF = SimtCfg<BM, BN, BK, RM, RN>;
+  constexpr int CG = BN / RN;        // column groups
+  constexpr int BAND = 2 * CG;       // columns 2 tn, 2 tn + 1 of each band of BAND columns (RN = 1: column tn)
+  extern __shared__ __align__(16) uint8_t smem[];
+  float4* As = reinterpret_cast<float4*>(smem);                    // [2][BK][BM] of (ar, ar, -ai, ai)
+  float2* Bs = reinterpret_cast<float2*>(smem + 2 * CF::A_BUF);    // [2][BK][BN]
   const int64_t K = int64_t(1) << d.nk;
   const int64_t m0 = (int64_t)blockIdx.x * BM, n0 = (int64_t)blockIdx.y * BN;
   const int64_t ulo = blockIdx.z % d.units_lo, uhi = blockIdx.z / d.units_lo;
@@ -143,110 +174,115 @@ __global__ void __launch_bounds__(NT, 1) gemm_simt_kernel(const float2* __restri
   B += ulo * d.b_lo + uhi * d.b_hi;
   C += ulo * d.c_lo + uhi * d.c_hi;
   const int tid = threadIdx.x;
-  const int tn = tid & 15, tm = tid >> 4;  // 16 column groups x 16 row groups
+  const int tn = tid % CG, tm = tid / CG;
 
-  TileLoader<BM> la;
-  TileLoader<BN> lb;
+  TileLoader<BM, BK> la;
+  TileLoader<BN, BK> lb;
   la.init(d, d.nm, d.am, d.ak, m0, (flags & 1) != 0);
   lb.init(d, d.nn, d.bn, d.bk, n0, (flags & 2) != 0);
 
-  float accr[8][WN], acci[8][WN];
+  f32x2 acc[RM][RN];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < WN; ++j) accr[i][j] = acci[i][j] = 0.f;
+    for (int j = 0; j < RN; ++j) acc[i][j] = 0ull;
 
+  auto store_tiles = [&](int buf) {
+    float4* at = As + buf * BK * BM;
+    float2* bt = Bs + buf * BK * BN;
+    la.store([&](int p, float2 x) { at[p] = make_float4(x.x, x.x, -x.y, x.y); });
+    lb.store([&](int p, float2 x) { bt[p] = x; });
+  };
   const int64_t nch = (K + BK - 1) / BK;
+  const int kn = K < BK ? (int)K : BK;  // K values of a chunk
   la.load(A, 0, 0);
   lb.load(B, 0, 0);
-  la.store(As);
-  lb.store(Bs);
+  store_tiles(0);
   __syncthreads();
   for (int64_t c = 0; c < nch; ++c) {
     const int buf = (int)(c & 1);
     if (c + 1 < nch) {
       const int64_t k1 = (c + 1) * BK;
-      la.load(A, k1, k_high_offset(k1, d.nk, d.ak));
-      lb.load(B, k1, k_high_offset(k1, d.nk, d.bk));
+      la.load(A, k1, k_high_offset<ilog2(BK)>(k1, d.nk, d.ak));
+      lb.load(B, k1, k_high_offset<ilog2(BK)>(k1, d.nk, d.bk));
     }
-    const float2* at = As + buf * BK * BM;
+    const ulonglong2* at = reinterpret_cast<const ulonglong2*>(As + buf * BK * BM) + RM * tm;
     const float2* bt = Bs + buf * BK * BN;
+    auto step = [&](int kk) {
+      f32x2 b[RN], bs[RN];
+      if constexpr (RN == 1) {
+        b[0] = *reinterpret_cast<const f32x2*>(bt + kk * BN + tn);
+      } else {
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float ar[8], ai[8], br[WN], bi[WN];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float4 x = *reinterpret_cast<const float4*>(at + kk * BM + 8 * tm + 2 * i);
-        ar[2 * i] = x.x;
-        ai[2 * i] = x.y;
-        ar[2 * i + 1] = x.z;
-        ai[2 * i + 1] = x.w;
-      }
-#pragma unroll
-      for (int j = 0; j < WN / 2; ++j) {
-        // columns 2 tn, 2 tn + 1 of each 32-column band
-        const float4 x = *reinterpret_cast<const float4*>(bt + kk * BN + 32 * j + 2 * tn);
-        br[2 * j] = x.x;
-        bi[2 * j] = x.y;
-        br[2 * j + 1] = x.z;
-        bi[2 * j + 1] = x.w;
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < WN; ++j) {
-          accr[i][j] = fmaf(ar[i], br[j], accr[i][j]);
-          accr[i][j] = fmaf(-ai[i], bi[j], accr[i][j]);
-          acci[i][j] = fmaf(ar[i], bi[j], acci[i][j]);
-          acci[i][j] = fmaf(ai[i], br[j], acci[i][j]);
+        for (int j = 0; j < RN / 2; ++j) {
+          const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(bt + kk * BN + BAND * j + 2 * tn);
+          b[2 * j] = x.x;
+          b[2 * j + 1] = x.y;
         }
+      }
+#pragma unroll
+      for (int j = 0; j < RN; ++j) bs[j] = swap2(b[j]);
+#pragma unroll
+      for (int i = 0; i < RM; ++i) {
+        const ulonglong2 a = at[kk * BM + i];
+#pragma unroll
+        for (int j = 0; j < RN; ++j) fma2(acc[i][j], a.x, b[j]);
+#pragma unroll
+        for (int j = 0; j < RN; ++j) fma2(acc[i][j], a.y, bs[j]);
+      }
+    };
+    if (kn == BK) {
+#pragma unroll 16
+      for (int kk = 0; kk < BK; ++kk) step(kk);
+    } else {
+      for (int kk = 0; kk < kn; ++kk) step(kk);
     }
-    if (c + 1 < nch) {
-      la.store(As + (buf ^ 1) * BK * BM);
-      lb.store(Bs + (buf ^ 1) * BK * BN);
-    }
+    if (c + 1 < nch) store_tiles(buf ^ 1);
     __syncthreads();
   }
 
   // epilogue: C offsets of this thread's rows and columns
   const int64_t M = int64_t(1) << d.nm, N = int64_t(1) << d.nn;
-  int32_t cc[WN];
+  int32_t cc[RN];
 #pragma unroll
-  for (int j = 0; j < WN; ++j) {
-    const int64_t n = n0 + 32 * (j >> 1) + 2 * tn + (j & 1);
+  for (int j = 0; j < RN; ++j) {
+    const int64_t n = n0 + (RN == 1 ? tn : BAND * (j >> 1) + 2 * tn + (j & 1));
     cc[j] = n < N ? bit_offset(n, d.nn, d.cn) : -1;
   }
-  const bool pairs = (flags & 4) != 0;  // columns 2 tn, 2 tn + 1 adjacent in C (16-byte store)
+  const bool pairs = RN > 1 && (flags & 4) != 0;  // columns 2 tn, 2 tn + 1 adjacent in C (16-byte store)
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int64_t m = m0 + 8 * tm + i;
+  for (int i = 0; i < RM; ++i) {
+    const int64_t m = m0 + RM * tm + i;
     if (m >= M) continue;
     const int32_t rc = bit_offset(m, d.nm, d.cm);
     if (pairs) {
 #pragma unroll
-      for (int j = 0; j < WN; j += 2)
-        if (cc[j] >= 0)
-          *reinterpret_cast<float4*>(C + rc + cc[j]) = make_float4(accr[i][j], acci[i][j], accr[i][j + 1], acci[i][j + 1]);
+      for (int j = 0; j < RN; j += 2)
+        if (cc[j] >= 0) {
+          const float2 x = unpack2(acc[i][j]), y = unpack2(acc[i][RN > 1 ? j + 1 : j]);
+          *reinterpret_cast<float4*>(C + rc + cc[j]) = make_float4(x.x, x.y, y.x, y.y);
+        }
     } else {
 #pragma unroll
-      for (int j = 0; j < WN; ++j)
-        if (cc[j] >= 0) C[rc + cc[j]] = make_float2(accr[i][j], acci[i][j]);
+      for (int j = 0; j < RN; ++j)
+        if (cc[j] >= 0) C[rc + cc[j]] = unpack2(acc[i][j]);
     }
   }
 }
 
-template <int BN>
-cudaError_t launch_bn(const float2* A, const float2* B, float2* C, const GemmDesc& d, int flags, cudaStream_t s) {
-  constexpr int SMEM = 2 * BK * (BM + BN) * (int)sizeof(float2);
+template <int BM, int BN, int BK, int RM, int RN>
+cudaError_t launch_tile(const float2* A, const float2* B, float2* C, const GemmDesc& d, int flags, cudaStream_t s) {
+  constexpr int SMEM = SimtCfg<BM, BN, BK, RM, RN>::SMEM;
   static bool attr = false;
   if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, BN, BK, RM, RN>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     if (e != cudaSuccess) return e;
     attr = true;
   }
   const int64_t M = int64_t(1) << d.nm, N = int64_t(1) << d.nn;
   dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), (unsigned)d.units);
-  gemm_simt_kernel<BN><<<grid, NT, SMEM, s>>>(A, B, C, d, flags);
+  gemm_simt_kernel<BM, BN, BK, RM, RN><<<grid, NT, SMEM, s>>>(A, B, C, d, flags);
   return cudaGetLastError();
 }
 
@@ -261,6 +297,12 @@ bool quad_ok(const float2* base, int nk, const int32_t* kst, int64_t lo, int64_t
 
 }  // namespace
 
+// Tile choice: the estimated time of each tile shape, waves over 152 SMs times
+// the tile's multiply-adds (padding included) over the shape's rate relative to
+// the largest (46 TFLOP/s on (12, 12, 9); scalar FMAs reached 44).  The small
+// shapes matter where the large one would leave SMs idle or compute padding:
+// (5, 4, 7) 41 -> 12 us, (5, 3, 8) x 2 units 82 -> 18 us, (6, 4, 12) x 128 units
+// 1.08 -> 0.57 ms.  Every shape gives the same bits, so this is speed alone.
 cudaError_t launch_gemm_simt(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s) {
   int flags = 0;
   if (quad_ok(A, d.nk, d.ak, d.a_lo, d.a_hi)) flags |= 1;
@@ -270,8 +312,17 @@ cudaError_t launch_gemm_simt(const float2* A, const float2* B, float2* C, const 
   if (d.nn >= 1 && d.cn[0] == 1 && (reinterpret_cast<uintptr_t>(C) & 15) == 0 && (d.c_lo & 1) == 0 &&
       (d.c_hi & 1) == 0)
     flags |= 4;
-  if (d.nn >= 7) return launch_bn<128>(A, B, C, d, flags, s);
-  return launch_bn<64>(A, B, C, d, flags, s);
+  const int64_t M = int64_t(1) << d.nm, N = int64_t(1) << d.nn;
+  auto cost = [&](int bm, int bn, double rate) {
+    const double tiles = (double)((M + bm - 1) / bm) * (double)((N + bn - 1) / bn) * d.units;
+    return (double)((int64_t)((tiles + 151) / 152)) * bm * bn / rate;
+  };
+  const double c128 = cost(128, 128, 1.0), c64 = cost(128, 64, 0.85), cm = cost(64, 32, 0.55), cs = cost(32, 16, 0.25);
+  const double best = std::min(std::min(c128, c64), std::min(cm, cs));
+  if (best == c128) return launch_tile<128, 128, 16, 8, 8>(A, B, C, d, flags, s);
+  if (best == c64) return launch_tile<128, 64, 16, 8, 4>(A, B, C, d, flags, s);
+  if (best == cm) return launch_tile<64, 32, 32, 4, 2>(A, B, C, d, flags, s);
+  return launch_tile<32, 16, 64, 2, 1>(A, B, C, d, flags, s);
 }
 
 }  // namespace tn
