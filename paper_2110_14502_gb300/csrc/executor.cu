@@ -130,6 +130,8 @@ struct Executor {
   std::vector<Tune> tuned;
   bool tune_loaded = false;
   std::vector<GemmDesc> desc;  // per step, unit strides filled at launch
+  ChainStep* chain = nullptr;  // per step, grouped by phase: its view for a run of small steps in one launch
+  std::vector<int> chain_pos;  // step -> entry of `chain`
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   std::vector<cudaEvent_t> pev;  // profiling event pool
 };
@@ -148,6 +150,7 @@ void destroy_executor(Executor* e) {
   cudaFree(e->parena);
   cudaFree(e->gather);
   cudaFree(e->perm);
+  cudaFree(e->chain);
   cudaFree(e->bits);
   cudaFree(e->acc);
   cudaFree(e->err);
@@ -399,6 +402,35 @@ static tn_status setup(Plan& P, Executor& E) {
         vector_shape_ok(E.desc[s]))
       make_gemm_desc(P.steps[s].la, P.steps[s].lb, P.steps[s].lc, E.desc[s], true);
   }
+  {
+    std::vector<ChainStep> table(P.steps.size());
+    E.chain_pos.assign(P.steps.size(), 0);
+    int at = 0;
+    auto place = [&](int x, int& space, int64_t& off) {
+      const int ph = x < L ? P.leaf_use[x].phase : P.steps[x - L].phase;
+      space = ph == 0 ? (x < L ? 0 : 1) : ph + 1;
+      off = x < L ? P.leaf_use[x].off : P.steps[x - L].off_c;
+    };
+    for (int ph = 0; ph < 3; ++ph)
+      for (size_t s = 0; s < P.steps.size(); ++s) {
+        if (P.steps[s].phase != ph) continue;
+        E.chain_pos[s] = at;
+        const GemmDesc& d = E.desc[s];
+        if (chain_shape_ok(d, 1)) {
+          int space[3];
+          int64_t off[3];
+          place(P.steps[s].a, space[0], off[0]);
+          place(P.steps[s].b, space[1], off[1]);
+          place(L + (int)s, space[2], off[2]);
+          make_chain_step(d, space, off, table[at]);
+        }
+        ++at;
+      }
+    if (!table.empty()) {
+      CK(dev_alloc(&E.chain, table.size() * sizeof(ChainStep)));
+      CK(cudaMemcpy(E.chain, table.data(), table.size() * sizeof(ChainStep), cudaMemcpyHostToDevice));
+    }
+  }
   CK(cudaEventCreate(&E.ev0));
   CK(cudaEventCreate(&E.ev1));
   CK(dev_alloc(&E.err, sizeof(int)));
@@ -510,31 +542,58 @@ tn_status run_step(Ctx& c, size_t s, const Geo& g) {
   return r;
 }
 
+// A step inside a launch: its GEMM view with unit strides, and its tensors.
+struct StepView {
+  GemmDesc d;
+  const float2 *A, *B;
+  float2* C;
+};
+StepView step_view(const Ctx& c, size_t s, const Geo& g) {
+  const Step& S = c.P.steps[s];
+  StepView v;
+  v.d = c.E.desc[s];
+  const float2* out;
+  operand(c.P, c.E, S.a, S.phase, g, v.A, v.d.a_lo, v.d.a_hi);
+  operand(c.P, c.E, S.b, S.phase, g, v.B, v.d.b_lo, v.d.b_hi);
+  operand(c.P, c.E, (int)c.P.net.leaves.size() + (int)s, S.phase, g, out, v.d.c_lo, v.d.c_hi);
+  v.C = const_cast<float2*>(out);
+  v.d.units_lo = S.phase == 0 ? 1 : g.gs;
+  v.d.units = S.phase == 0 ? 1 : S.phase == 1 ? g.gs : g.gs * g.gb;
+  return v;
+}
+
+// Kernel class of a step (tc: it runs in a tensor-core precision); `reduce`:
+// few outputs with a long contracted index, the bandwidth-bound reduction.
+int step_class(const Step& S, const GemmDesc& d, bool tc, bool& reduce) {
+  int klass = S.klass == SC_VECTOR ? TN_KCLASS_VECTOR : TN_KCLASS_GEMM_SIMT;
+  if (S.klass != SC_VECTOR && tc && tc_shape_ok(d) && !stream_preferred(d)) klass = TN_KCLASS_GEMM_TC;
+  else if (klass == TN_KCLASS_GEMM_SIMT && (!tc_shape_ok(d) || stream_preferred(d)) && vector_shape_ok(d))
+    klass = TN_KCLASS_VECTOR;
+  reduce = klass == TN_KCLASS_GEMM_SIMT && reduce_shape_ok(d);
+  return reduce ? TN_KCLASS_VECTOR : klass;
+}
+
+// Algorithmic bytes of a step: each distinct operand read once, each output written once.
+double step_bytes(const GemmDesc& d) {
+  const double M = std::ldexp(1.0, d.nm), N = std::ldexp(1.0, d.nn), K = std::ldexp(1.0, d.nk), U = d.units;
+  auto distinct = [&](int64_t lo, int64_t hi) { return (lo ? (double)d.units_lo : 1.0) * (hi ? U / d.units_lo : 1.0); };
+  return 8.0 * (M * K * distinct(d.a_lo, d.a_hi) + K * N * distinct(d.b_lo, d.b_hi) + M * N * U);
+}
+double step_flops(const GemmDesc& d) { return std::ldexp(8.0, d.nm + d.nn + d.nk) * d.units; }
+
 tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
   const Plan& P = c.P;
   Executor& E = c.E;
   const Step& S = P.steps[s];
-  GemmDesc d = E.desc[s];
-  const float2 *A, *B, *Cc;
-  int64_t clo, chi;
-  operand(P, E, S.a, S.phase, g, A, d.a_lo, d.a_hi);
-  operand(P, E, S.b, S.phase, g, B, d.b_lo, d.b_hi);
-  operand(P, E, (int)P.net.leaves.size() + (int)s, S.phase, g, Cc, clo, chi);
-  d.c_lo = clo;
-  d.c_hi = chi;
-  float2* C = const_cast<float2*>(Cc);
-  d.units_lo = S.phase == 0 ? 1 : g.gs;
-  d.units = S.phase == 0 ? 1 : S.phase == 1 ? g.gs : g.gs * g.gb;
+  const StepView view = step_view(c, s, g);
+  GemmDesc d = view.d;
+  const float2 *A = view.A, *B = view.B;
+  float2* C = view.C;
   size_t e0 = 0, e1 = 0;
   if (c.profile && !c.sizing) { tn_status r = c.event(e0); if (r) return r; }
   cudaError_t e;
-  int klass = S.klass == SC_VECTOR ? TN_KCLASS_VECTOR : TN_KCLASS_GEMM_SIMT;
-  if (S.klass != SC_VECTOR && c.tc && tc_shape_ok(d) && !stream_preferred(d)) klass = TN_KCLASS_GEMM_TC;
-  else if (klass == TN_KCLASS_GEMM_SIMT && (!tc_shape_ok(d) || stream_preferred(d)) && vector_shape_ok(d))
-    klass = TN_KCLASS_VECTOR;
-  // few outputs with a long contracted index: the bandwidth-bound reduction
-  const bool reduce = klass == TN_KCLASS_GEMM_SIMT && reduce_shape_ok(d);
-  if (reduce) klass = TN_KCLASS_VECTOR;
+  bool reduce;
+  const int klass = step_class(S, d, c.tc, reduce);
   if (c.sizing && klass != TN_KCLASS_GEMM_TC) return TN_OK;
   if (reduce) e = launch_reduce(A, B, C, d, c.st);
   else if (klass == TN_KCLASS_VECTOR) {
@@ -668,12 +727,6 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
   if (c.profile) {
     tn_status r = c.event(e1);
     if (r) return r;
-    const double M = std::ldexp(1.0, d.nm), N = std::ldexp(1.0, d.nn), K = std::ldexp(1.0, d.nk);
-    const double U = d.units;
-    auto distinct = [&](int64_t lo, int64_t hi) {
-      return (lo ? (double)d.units_lo : 1.0) * (hi ? U / d.units_lo : 1.0);
-    };
-    double bytes = 8.0 * (M * K * distinct(d.a_lo, d.a_hi) + K * N * distinct(d.b_lo, d.b_hi) + M * N * U);
     // diagnostics: C's unit-stride index (row bit i -> i, column bit j -> 100 + j), plane output,
     // 16-column vector stores, which operands vary with the lo / hi unit index
     // C's four fastest indices: row bit i -> i, column bit j -> 100 + j (base-1000 digits)
@@ -686,7 +739,7 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
     }
     const int n16 = d.nn >= 4 && d.cn[0] == 1 && d.cn[1] == 2 && d.cn[2] == 4 && d.cn[3] == 8;
     const int ulo = (d.a_lo ? 1 : 0) | (d.b_lo ? 2 : 0), uhi = (d.a_hi ? 1 : 0) | (d.b_hi ? 2 : 0);
-    c.recs.push_back({klass, 8.0 * M * N * K * U, bytes, e0, (int)s, d.nm, d.nn, d.nk, d.units, cfast,
+    c.recs.push_back({klass, step_flops(d), step_bytes(d), e0, (int)s, d.nm, d.nn, d.nk, d.units, cfast,
                       (int)(s < c.planes_out.size() && c.planes_out[s]), n16, ulo, uhi});
   }
   return TN_OK;
@@ -696,6 +749,92 @@ tn_status run_misc(Ctx& c, cudaError_t e, const char* what) {
   ++c.launches;
   if (e != cudaSuccess) return fail(TN_ECUDA, "%s launch: %s", what, cudaGetErrorString(e));
   return TN_OK;
+}
+
+}  // namespace
+
+namespace {
+
+// Leaf gather of a phase's units (count 0: none).
+struct PhaseLeaves {
+  const LeafGather* descs = nullptr;
+  int count = 0;
+  float2* arena = nullptr;
+  int64_t stride = 0;
+  const GroupInfo* slot = nullptr;
+  int units = 0;
+};
+
+// The steps of one phase in order, after the gather of its leaves.  Consecutive
+// small steps that write plain complex64 go out as one launch (launch_chain),
+// with the gather in front when they open the phase; the others as their own.
+tn_status run_phase(Ctx& c, int phase, const Geo& g, const PhaseLeaves& leaves) {
+  const Plan& P = c.P;
+  Executor& E = c.E;
+  bool gathered = leaves.count == 0;
+  auto gather = [&]() -> tn_status {
+    if (gathered) return TN_OK;
+    gathered = true;
+    return run_misc(c, launch_gather(E.store, leaves.arena, leaves.stride, leaves.descs, leaves.count, leaves.slot,
+                                     leaves.units, c.st),
+                    "gather");
+  };
+  size_t first = 0, last = 0;  // the pending run's first and last step
+  ChainRun run;
+  int units = 1;
+  double flops = 0, bytes = 0;
+  auto flush = [&]() -> tn_status {
+    const ChainRun now = run;
+    run = ChainRun{};
+    if (now.count == 0) return TN_OK;
+    if (now.count == 1 && gathered) return run_step(c, first, g);
+    size_t e0 = 0, e1 = 0;
+    if (c.profile) { tn_status r = c.event(e0); if (r) return r; }
+    const ChainBase base{E.store, E.inv, E.sarena, E.parena, P.slice_arena_elems, P.unit_arena_elems,
+                         phase == 0 ? 1 : (int64_t)g.gs};
+    tn_status r = run_misc(c, launch_chain(E.chain + E.chain_pos[first], now, base, units, E.store,
+                                           leaves.descs, gathered ? 0 : leaves.count, leaves.arena, leaves.stride,
+                                           leaves.slot, c.st),
+                           "chain");
+    if (r) return r;
+    gathered = true;
+    if (c.profile) {
+      r = c.event(e1);
+      if (r) return r;
+      const GemmDesc& d = E.desc[last];
+      c.recs.push_back({TN_KCLASS_VECTOR, flops, bytes, e0, (int)last, d.nm, d.nn, d.nk, units, 0, 0, 0, 0, 0});
+    }
+    return TN_OK;
+  };
+  for (size_t s = 0; s < P.steps.size(); ++s) {
+    if (P.steps[s].phase != phase) continue;
+    const StepView v = step_view(c, s, g);
+    const bool tc = phase != 0 && (c.step_prec ? (c.step_prec[s] >= 0 ? (int)c.step_prec[s] : c.call_precision) !=
+                                                     TN_PREC_C64
+                                               : c.tc);
+    bool reduce;
+    const int klass = step_class(P.steps[s], v.d, tc, reduce);
+    const bool plain = !(s < c.max_out.size() && c.max_out[s]) && !(s < c.planes_out.size() && c.planes_out[s]);
+    if (klass != TN_KCLASS_GEMM_TC && !reduce && plain && chain_shape_ok(v.d, v.d.units)) {
+      if (run.count == 64) { tn_status r = flush(); if (r) return r; }
+      if (run.count == 0) {
+        first = s;
+        flops = bytes = 0;
+      }
+      chain_add(run, v.d, klass == TN_KCLASS_VECTOR && vector_sums_im_first(v.A, v.d));
+      units = v.d.units;
+      flops += step_flops(v.d);
+      bytes += step_bytes(v.d);
+      last = s;
+      continue;
+    }
+    tn_status r = flush();
+    if (!r) r = gather();
+    if (!r) r = run_step(c, s, g);
+    if (r) return r;
+  }
+  tn_status r = flush();
+  return r ? r : gather();
 }
 
 }  // namespace
@@ -922,11 +1061,8 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
       const bool keep_tc = c.tc;
       c.precision = TN_PREC_C64;
       c.tc = false;
-      for (size_t s = 0; s < P.steps.size(); ++s)
-        if (P.steps[s].phase == 0) {
-          tn_status r = run_step(c, s, g);
-          if (r != TN_OK) return r;
-        }
+      tn_status r = run_phase(c, 0, g, PhaseLeaves{});
+      if (r != TN_OK) return r;
       c.precision = keep;
       c.tc = keep_tc;
       if (E.stem) {
@@ -988,29 +1124,21 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
                       !o.step_precision;
   // One launch sequence (the slice-only steps of a group, or the per-unit
   // steps of a group and its accumulation), replayed from a graph when allowed.
+  bool slice_only = scaled || E.ngather1 > 0;  // anything to do once per slice
+  for (const Step& S : P.steps) slice_only |= S.phase == 1;
   auto sequence = [&](int phase, const Geo& gg) -> tn_status {
+    if (phase == 1 && !slice_only) return TN_OK;
     auto body = [&]() -> tn_status {
+      PhaseLeaves lv;
       if (phase == 1) {
         if (scaled) CK(cudaMemsetAsync(c.flag1, 0, Gs * sizeof(int), st));
-        if (E.ngather1) {
-          tn_status r = run_misc(c, launch_gather(E.store, E.sarena, Se, E.gather, E.ngather1, E.gslot, gg.gs, st),
-                                 "gather");
-          if (r) return r;
-        }
+        lv = {E.gather, E.ngather1, E.sarena, Se, E.gslot, gg.gs};
       } else {
         if (scaled) CK(cudaMemsetAsync(c.flag2, 0, c.U * sizeof(int), st));
-        if (E.ngather2) {
-          tn_status r = run_misc(
-              c, launch_gather(E.store, E.parena, Pe, E.gather + E.ngather1, E.ngather2, E.gslot + 1, gg.gs * gg.gb, st),
-              "gather");
-          if (r) return r;
-        }
+        lv = {E.gather + E.ngather1, E.ngather2, E.parena, Pe, E.gslot + 1, gg.gs * gg.gb};
       }
-      for (size_t s = 0; s < P.steps.size(); ++s)
-        if (P.steps[s].phase == phase) {
-          tn_status r = run_step(c, s, gg);
-          if (r != TN_OK) return r;
-        }
+      tn_status rp = run_phase(c, phase, gg, lv);
+      if (rp != TN_OK) return rp;
       if (phase == 2) {
         const float2* root;
         int64_t rlo, rhi;
@@ -1062,7 +1190,7 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
     gi.units = g.gs;
     gi.bits = d_bits;
     gi.acc = d_acc;
-    {
+    if (E.ngather1) {  // (only the slice-only gather reads this slot)
       tn_status r = run_misc(c, launch_set_group(E.gslot, gi, st), "set_group");
       if (r) return r;
     }

@@ -9,6 +9,7 @@
 // FP64 in unit order, so the sum order is fixed for a given call.
 #include <algorithm>
 
+#include "device_common.h"
 #include "kernels.h"
 
 namespace tn {
@@ -20,31 +21,13 @@ __global__ void set_group_kernel(GroupInfo* slot, GroupInfo g) { *slot = g; }
 __global__ void gather_kernel(const float2* __restrict__ store, float2* __restrict__ arena, int64_t arena_stride,
                               const LeafGather* __restrict__ descs, const GroupInfo* __restrict__ slot) {
   const GroupInfo g = *slot;
-  const uint64_t* bits = g.bits;
   const LeafGather& L = descs[blockIdx.x];
   const int u = blockIdx.y;
   if (u >= g.units) return;
-  const int64_t s = g.slice0 + u % g.nslice;
-  const int64_t b = g.b0 + u / g.nslice;
-  int64_t fixed_off = L.store_off;
-  for (int f = 0; f < L.nfixed; ++f) {
-    int src = L.fixed_src[f];
-    int v;
-    if (src >= 0) v = (int)((s >> src) & 1);
-    else {
-      int q = -src - 2;
-      v = (int)((bits[b * g.words + (q >> 6)] >> (q & 63)) & 1);
-    }
-    if (v) fixed_off += L.fixed_stride[f];
-  }
+  const int64_t from = leaf_fixed_offset(L, g, u);
   const int sub = 1 << L.nkept;
   float2* dst = arena + (int64_t)u * arena_stride + L.dst_off;
-  for (int e = threadIdx.x; e < sub; e += blockDim.x) {
-    int64_t o = fixed_off;
-    for (int p = 0; p < L.nkept; ++p)
-      if ((e >> (L.nkept - 1 - p)) & 1) o += L.kept_stride[p];
-    dst[e] = store[o];
-  }
+  for (int e = threadIdx.x; e < sub; e += blockDim.x) dst[e] = store[leaf_kept_offset(L, from, e)];
 }
 
 // The filter of the scaled precisions (Sec. "A Mixed-Precision Computation

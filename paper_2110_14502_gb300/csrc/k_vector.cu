@@ -545,6 +545,10 @@ cudaError_t launch_wide(const float2* A, const float2* B, float2* C, const GemmD
   }
 }
 
+bool vector_sums_im_first(const float2* A, const GemmDesc& d) {
+  return d.nn <= 4 && (d.nk > 4 || staged_ok(A, d));
+}
+
 cudaError_t launch_vector(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s,
                           const VecOut& maxbits) {
   if (!vector_shape_ok(d) || d.units > 65535) return cudaErrorInvalidValue;

@@ -168,6 +168,45 @@ cudaError_t launch_vector(const float2* A, const float2* B, float2* C, const Gem
 // unit, K spread over the threads, warp-shuffle reduction (k_reduce.cu).
 bool reduce_shape_ok(const GemmDesc& d);
 cudaError_t launch_reduce(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s);
+// Streaming kernels add a product's imaginary-times-imaginary term first when
+// this holds (the kernels that consume K into running sums), last otherwise.
+bool vector_sums_im_first(const float2* A, const GemmDesc& d);
+
+// Runs of small steps in one launch, one CTA per unit (k_chain.cu).  A step's
+// view for it: operand and output i sit in memory space[i] (0 leaf store, 1
+// invariant store, 2 slice arena, 3 pair arena) at element offset off[i]; a
+// thread item has `items` index bits, bit b of it moving C by oc[b] and the
+// operands' shared-memory slots by ha[b], hb[b] (combined by XOR); with `tile`
+// the item is a 2 x 2 block of outputs over the N bit oc[items] and the M bit
+// oc[items + 1].  Contracted bit l moves the slots by ka[l], kb[l].
+constexpr int kChainMaxC = 14, kChainMaxK = 8, kChainMaxOperand = 12;
+struct ChainStep {
+  int64_t off[3];
+  int32_t space[3];
+  int32_t items, tile, nk, abits, bbits;
+  int32_t oc[kChainMaxC], ha[kChainMaxC], hb[kChainMaxC];
+  int32_t ka[kChainMaxK], kb[kChainMaxK];
+};
+struct ChainBase {
+  float2 *store, *inv, *sarena, *parena;
+  int64_t slice_elems, unit_elems;  // arena strides per slice / per unit
+  int64_t gs;                       // slices of the group (units u = slice + gs * bitstring)
+};
+bool chain_shape_ok(const GemmDesc& d, int64_t units);
+void make_chain_step(const GemmDesc& d, const int space[3], const int64_t off[3], ChainStep& s);
+// What a run's launch is sized by: its widest step.
+struct ChainRun {
+  int count = 0;       // steps, at most 64
+  uint64_t forms = 0;  // bit i: step i adds the im * im terms first
+  int items = 0;       // largest log2 number of thread items
+  int elems = 0;       // largest number of operand elements (A and B)
+};
+void chain_add(ChainRun& run, const GemmDesc& d, bool im_first);
+// Steps steps[0 .. run.count-1] (device table) for every unit.  With nleaves >
+// 0 each unit first gathers its leaves, as launch_gather.
+cudaError_t launch_chain(const ChainStep* steps, const ChainRun& run, const ChainBase& base, int units,
+                         const float2* leaf_store, const LeafGather* leaves, int nleaves, float2* gather_arena,
+                         int64_t gather_stride, const GroupInfo* slot, cudaStream_t s);
 cudaError_t launch_set_group(GroupInfo* slot, const GroupInfo& g, cudaStream_t s);
 // grid covers `units` units (the slot's count may be lower for a partial group)
 cudaError_t launch_gather(const float2* store, float2* arena, int64_t arena_stride, const LeafGather* descs,
