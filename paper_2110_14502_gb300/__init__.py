@@ -10,7 +10,8 @@ import ctypes as C
 import numpy as np
 
 from ._abi import (PAIR_ALGO, PREC, ExecOpts, Gate, NetworkInfo, PlanInfo, PlanOpts, PrecisionReport, Report, Request,
-                   RequestStats, ServerOpts, TensorLayout, TnError, check, i32array, lib, require_buffer)
+                   RequestStats, ServerOpts, TensorLayout, TnError, check, i32array, is_device_buffer, labels, lib,
+                   require_buffer)
 
 __all__ = ["Circuit", "Network", "Plan", "random_circuit", "circuit_from_gates", "build_network", "plan", "select_plan",
            "contract_pair", "contract_pair_noalloc", "set_wait_limit", "Server", "TnError", "PREC", "version"]
@@ -119,6 +120,7 @@ class Plan:
     def __init__(self, handle, network):
         self._h = handle
         self.network = network
+        self._sizes = None  # (qubits, open qubits, steps), which never change
 
     def __del__(self):
         if getattr(self, "_h", None):
@@ -202,8 +204,10 @@ class Plan:
         (device I/O: `out` must be a CUDA float64 tensor of nb*2^k*2 entries;
         work is queued on `stream`, a torch.cuda.Stream or raw handle).
         """
-        info = self.info()
-        k = info["num_open"]
+        if self._sizes is None:
+            info = self.info()
+            self._sizes = info["num_qubits"], info["num_open"], info["num_steps"]
+        n, k, num_steps = self._sizes
         o = ExecOpts()
         o.precision = PREC[precision] if isinstance(precision, str) else int(precision)
         o.slice_begin = slice_begin
@@ -217,14 +221,14 @@ class Plan:
         o.handover = handover
         if step_precision is not None:
             sp = np.ascontiguousarray(np.asarray(step_precision, dtype=np.int8))
-            if sp.shape != (info["num_steps"],):
-                raise TnError(1, f"step_precision needs one entry per step ({info['num_steps']}), got {sp.shape}")
+            if sp.shape != (num_steps,):
+                raise TnError(1, f"step_precision needs one entry per step ({num_steps}), got {sp.shape}")
             o.step_precision = sp.ctypes.data
         if stream is not None:
             o.stream = C.c_void_p(getattr(stream, "cuda_stream", stream))
         rep = Report()
         device = hasattr(bitstrings, "is_cuda") and bitstrings.is_cuda
-        words = (info["num_qubits"] + 63) // 64
+        words = (n + 63) // 64
         if device:
             nb = bitstrings.shape[0]
             if out is None:
@@ -248,7 +252,9 @@ class Plan:
             else:
                 require_buffer(out, "out", 16 * (nb << k), False, ("complex128",))
                 res = out
-            check(lib().tn_contract_amplitudes(self._h, _ptr(b), nb, _ptr(res), C.byref(o), C.byref(rep)))
+            # (a host call waits for its result with or without a report)
+            check(lib().tn_contract_amplitudes(self._h, _ptr(b), nb, _ptr(res), C.byref(o),
+                                               C.byref(rep) if report or profile else None))
         if report:
             r = {}
             for f, _ in Report._fields_:
@@ -304,16 +310,16 @@ def _require_pair_operands(A, la, B, lb, Cout, lc):
     """Each operand is a contiguous CUDA complex64 tensor of 2^rank elements
     (ranks above 30 are left to the library to reject)."""
     for x, ls, what in ((A, la, "A"), (B, lb, "B"), (Cout, lc, "C")):
-        if len(ls) <= 30:
+        if len(ls) <= 30 and not is_device_buffer(x, "complex64", 1 << len(ls)):
             require_buffer(x, what, 8 << len(ls), True, ("complex64",))
 
 
 def contract_pair(A, a_labels, B, b_labels, Cout, c_labels, precision="c64", algo="auto", stream=None):
     """C[c_labels] = sum over shared labels of A[a_labels] * B[b_labels] on the
     GPU; A, B, C are CUDA complex64 torch tensors (contiguous)."""
-    la, pa = i32array(a_labels)
-    lb, pb = i32array(b_labels)
-    lc, pc = i32array(c_labels)
+    la, pa = labels(a_labels)
+    lb, pb = labels(b_labels)
+    lc, pc = labels(c_labels)
     _require_pair_operands(A, la, B, lb, Cout, lc)
     s = C.c_void_p(getattr(stream, "cuda_stream", stream) if stream is not None else None)
     prec = PREC[precision] if isinstance(precision, str) else int(precision)
@@ -328,9 +334,9 @@ def contract_pair_noalloc(A, a_labels, B, b_labels, Cout, c_labels, stream=None)
     scratch taken from the library's static device array instead of an
     allocation; for callers that cannot let the library allocate.  Calls on
     one GPU share the array, so overlapping calls race."""
-    la, pa = i32array(a_labels)
-    lb, pb = i32array(b_labels)
-    lc, pc = i32array(c_labels)
+    la, pa = labels(a_labels)
+    lb, pb = labels(b_labels)
+    lc, pc = labels(c_labels)
     _require_pair_operands(A, la, B, lb, Cout, lc)
     s = C.c_void_p(getattr(stream, "cuda_stream", stream) if stream is not None else None)
     check(lib().tn_contract_pair_noalloc(_ptr(A), pa, len(la), _ptr(B), pb, len(lb), _ptr(Cout), pc, len(lc), s))

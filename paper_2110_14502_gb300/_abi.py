@@ -7,6 +7,8 @@ CPU fallback.
 """
 import ctypes as C
 import os
+import sys
+from array import array
 
 import numpy as np
 
@@ -126,15 +128,16 @@ SIGNATURES = {
     "tn_free_plan": (None, [P]),
     "tn_contract_amplitudes": (C.c_int, [P, C.c_void_p, C.c_int64, C.c_void_p, C.POINTER(ExecOpts),
                                          C.POINTER(Report)]),
-    "tn_contract_pair": (C.c_int, [C.c_void_p, I32P, C.c_int32, C.c_void_p, I32P, C.c_int32,
-                                   C.c_void_p, I32P, C.c_int32, C.c_int32, C.c_int32, C.c_void_p]),
+    # (the pair calls take their label arrays as addresses: see labels())
+    "tn_contract_pair": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p, C.c_int32,
+                                   C.c_void_p, C.c_void_p, C.c_int32, C.c_int32, C.c_int32, C.c_void_p]),
     "tn_server_create": (C.c_int, [C.POINTER(ServerOpts), C.POINTER(P)]),
     "tn_submit": (C.c_int, [P, C.POINTER(Request), C.POINTER(C.c_int64)]),
     "tn_poll": (C.c_int, [P, C.c_int64, C.POINTER(C.c_int32)]),
     "tn_wait": (C.c_int, [P, C.c_int64, C.c_void_p, C.c_int64, C.POINTER(RequestStats), C.c_double]),
     "tn_server_destroy": (None, [P]),
-    "tn_contract_pair_noalloc": (C.c_int, [C.c_void_p, I32P, C.c_int32, C.c_void_p, I32P, C.c_int32,
-                                           C.c_void_p, I32P, C.c_int32, C.c_void_p]),
+    "tn_contract_pair_noalloc": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p, C.c_int32,
+                                           C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p]),
     "tn_set_wait_limit": (C.c_int, [C.c_int64]),
     "tn_precision_analysis": (C.c_int, [P, C.c_void_p, C.c_int64, C.c_int64, C.c_int32, C.c_int32, C.c_double,
                                         C.c_void_p, C.POINTER(PrecisionReport)]),
@@ -182,3 +185,24 @@ def require_buffer(x, what, nbytes, device, dtypes):
 def i32array(xs):
     a = np.ascontiguousarray(np.asarray(list(xs), dtype=np.int32))
     return a, (a.ctypes.data_as(I32P) if a.size else None)
+
+
+def labels(xs):
+    """(array, address or None) of index labels.  array.array takes any sequence
+    of integers several times faster than NumPy plus a ctypes pointer; what it
+    rejects goes through i32array, with its conversions and errors."""
+    xs = list(xs)
+    try:
+        a = array("i", xs)
+    except (TypeError, OverflowError):
+        a, _ = i32array(xs)
+        return a, a.ctypes.data if a.size else None
+    return a, a.buffer_info()[0] if a else None
+
+
+def is_device_buffer(x, dtype, count):
+    """Whether `x` is a contiguous CUDA torch tensor of `dtype` (a name) with at
+    least `count` elements: the quick form of require_buffer, without its error."""
+    torch = sys.modules.get("torch")
+    return (torch is not None and isinstance(x, torch.Tensor) and x.dtype is getattr(torch, dtype) and x.is_cuda
+            and x.is_contiguous() and x.numel() >= count)

@@ -39,6 +39,9 @@
 namespace tn {
 
 constexpr int kFlaggedCap = 1 << 16;  // listed flagged units per call
+// Host results up to this size come back through pinned memory (a copy into
+// pageable memory costs the call about 10 us more).
+constexpr size_t kStageBytes = 64 * 1024;
 // Default of the plane handover per precision (c64, split bf16, split fp16,
 // scaled fp16, scaled bf16).  A handed-over 16-bit tensor is scaled by the
 // bound 2 K maxA maxB predicted before its values exist, so its stored
@@ -94,6 +97,39 @@ StemCacheStats stem_cache_stats(StemCache& c) {
   return {(int64_t)c.m.size(), c.bytes, c.hits, c.misses};
 }
 
+// Pinned host blocks of the executors: 64 bytes for the error word and a
+// staging area.  Allocating one takes long enough to matter to a serving
+// request, so up to kPinnedKept freed blocks are kept for the next executor.
+constexpr size_t kPinnedKept = 16;
+struct PinnedPool {
+  std::mutex mu;
+  std::vector<void*> blocks;
+};
+static PinnedPool g_pinned;
+
+static cudaError_t pinned_take(void** p) {
+  {
+    std::lock_guard<std::mutex> g(g_pinned.mu);
+    if (!g_pinned.blocks.empty()) {
+      *p = g_pinned.blocks.back();
+      g_pinned.blocks.pop_back();
+      return cudaSuccess;
+    }
+  }
+  return cudaHostAlloc(p, 64 + kStageBytes, cudaHostAllocMapped | cudaHostAllocPortable);
+}
+static void pinned_give(void* p) {
+  if (!p) return;
+  {
+    std::lock_guard<std::mutex> g(g_pinned.mu);
+    if (g_pinned.blocks.size() < kPinnedKept) {
+      g_pinned.blocks.push_back(p);
+      return;
+    }
+  }
+  cudaFreeHost(p);
+}
+
 struct Executor {
   int device = -1;
   float2* store = nullptr;
@@ -111,7 +147,12 @@ struct Executor {
   int64_t bits_cap = 0;
   double2* acc = nullptr;
   int64_t acc_cap = 0;
-  int* err = nullptr;          // device error word of bounded waits
+  // pinned host block: the error word of bounded waits, which the kernels
+  // write through its device address, then a staging area for small results
+  void* pinned = nullptr;
+  int* err = nullptr;
+  volatile int* err_host = nullptr;
+  void* stage = nullptr;
   uint16_t* scratch = nullptr; // split operand planes of the tensor-core steps
   int64_t scratch_cap = 0;     // in 16-bit elements
   // scaled precisions: per step and launch unit, exponent and stored maximum
@@ -153,7 +194,6 @@ void destroy_executor(Executor* e) {
   cudaFree(e->chain);
   cudaFree(e->bits);
   cudaFree(e->acc);
-  cudaFree(e->err);
   cudaFree(e->scratch);
   cudaFree(e->spool);
   cudaFree(e->flagged);
@@ -163,6 +203,7 @@ void destroy_executor(Executor* e) {
   if (e->ev0) cudaEventDestroy(e->ev0);
   if (e->ev1) cudaEventDestroy(e->ev1);
   for (auto ev : e->pev) cudaEventDestroy(ev);
+  pinned_give(e->pinned);  // the frees above waited for the device
   if (cur >= 0) cudaSetDevice(cur);
   delete e;
 }
@@ -433,8 +474,13 @@ static tn_status setup(Plan& P, Executor& E) {
   }
   CK(cudaEventCreate(&E.ev0));
   CK(cudaEventCreate(&E.ev1));
-  CK(dev_alloc(&E.err, sizeof(int)));
-  CK(cudaMemset(E.err, 0, sizeof(int)));
+  CK(pinned_take(&E.pinned));
+  E.err_host = static_cast<volatile int*>(E.pinned);
+  *E.err_host = 0;
+  E.stage = static_cast<char*>(E.pinned) + 64;
+  void* perr = nullptr;
+  CK(cudaHostGetDevicePointer(&perr, E.pinned, 0));
+  E.err = static_cast<int*>(perr);
   CK(dev_alloc(&E.flagged, kFlaggedCap * sizeof(int64_t)));
   CK(dev_alloc(&E.gslot, 2 * sizeof(GroupInfo)));
   CK(dev_alloc(&E.nflagged, sizeof(unsigned long long)));
@@ -899,7 +945,13 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
   const int64_t Se = P.slice_arena_elems, Pe = P.unit_arena_elems;
   int64_t Gb = std::max<int64_t>(1, std::min<int64_t>(nb, 256));
   int64_t Gs = o.units_per_group;
-  if (Gs <= 0) {
+  // the most slices a launch may take; if the arenas already hold that many
+  // there is no need to ask for the free memory (tens of microseconds)
+  const int64_t most = std::min<int64_t>(std::min<int64_t>(1024, std::max<int64_t>(ns, 1)), 65535 / Gb);
+  if (Gs <= 0 && most >= 1 && E.sarena_cap >= most * Se && E.parena_cap >= most * Gb * Pe &&
+      8.0 * most * ((double)Se + (double)Gb * Pe) <= 120.0 * (1ull << 30)) {
+    Gs = most;
+  } else if (Gs <= 0) {
     size_t freeb = 0, totb = 0;
     CK(cudaMemGetInfo(&freeb, &totb));
     double have = (double)(E.sarena_cap + E.parena_cap) * 8.0;
@@ -1042,7 +1094,7 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
     c.flag1 = (int*)q;                       q += 4 * Gs;
     c.flag2 = (int*)q;
   }
-  if (clear_out) CK(cudaEventRecord(E.ev0, st));  // a nested recompute call is timed by its caller
+  if (clear_out && rep) CK(cudaEventRecord(E.ev0, st));  // a nested recompute call is timed by its caller
   if (!o.device_io && nb > 0)
     CK(cudaMemcpyAsync((void*)d_bits, bits, nb * words * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
   if (nout > 0 && clear_out) CK(cudaMemsetAsync(d_acc, 0, nout * sizeof(double2), st));
@@ -1265,15 +1317,17 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
       }
     }
   }
-  if (!o.device_io && nout > 0) CK(cudaMemcpyAsync(out, d_acc, nout * sizeof(double2), cudaMemcpyDeviceToHost, st));
+  const bool staged = !o.device_io && nout > 0 && clear_out && nout * sizeof(double2) <= kStageBytes;
+  if (!o.device_io && nout > 0)
+    CK(cudaMemcpyAsync(staged ? E.stage : (void*)out, d_acc, nout * sizeof(double2), cudaMemcpyDeviceToHost, st));
   if (!clear_out) return TN_OK;
-  CK(cudaEventRecord(E.ev1, st));
+  if (rep) CK(cudaEventRecord(E.ev1, st));
   if (!o.device_io || rep) {
-    CK(cudaEventSynchronize(E.ev1));
-    int herr = 0;
-    CK(cudaMemcpy(&herr, E.err, sizeof(int), cudaMemcpyDeviceToHost));
+    CK(cudaStreamSynchronize(st));
+    if (staged) std::memcpy(out, E.stage, nout * sizeof(double2));
+    const int herr = *E.err_host;
     if (herr) {
-      CK(cudaMemset(E.err, 0, sizeof(int)));
+      *E.err_host = 0;
       return fail(TN_ETIMEOUT, "tn_contract_amplitudes: a tensor-core pipeline wait expired (code %d)", herr);
     }
   }

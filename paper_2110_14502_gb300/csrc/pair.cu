@@ -44,11 +44,13 @@ static cublasHandle_t cublas_handle(int dev) {
 }
 
 // Device state of the tensor-core algorithms, one per device: the kernels'
-// error word and a grow-only buffer for the operand planes.  A call holds the
+// error word (in host memory that the kernels write only when a wait expires,
+// so a call reads it without a copy) and a grow-only buffer for the operand planes.  A call holds the
 // mutex until its kernel has finished, so calls on one device are serialised
 // and the buffer is never in use by two calls at once.
 struct PairDevState {
-  int* err = nullptr;
+  int* err = nullptr;                 // device address of the word ..
+  volatile int* err_host = nullptr;   // .. and host address
   void* scratch = nullptr;
   size_t bytes = 0;
 };
@@ -61,8 +63,16 @@ static tn_status pair_state(size_t need, PairDevState*& out) {
   if ((int)g_pair_state.size() <= dev) g_pair_state.resize(dev + 1);
   PairDevState& st = g_pair_state[dev];
   if (!st.err) {
-    if (cudaMalloc(&st.err, sizeof(int)) != cudaSuccess) return fail(TN_ECUDA, "tn_contract_pair: error word");
-    if (cudaMemset(st.err, 0, sizeof(int)) != cudaSuccess) return fail(TN_ECUDA, "tn_contract_pair: error word");
+    void *h = nullptr, *p = nullptr;
+    if (cudaHostAlloc(&h, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess)
+      return fail(TN_ECUDA, "tn_contract_pair: error word");
+    if (cudaHostGetDevicePointer(&p, h, 0) != cudaSuccess) {
+      cudaFreeHost(h);
+      return fail(TN_ECUDA, "tn_contract_pair: error word");
+    }
+    st.err_host = static_cast<volatile int*>(h);
+    *st.err_host = 0;
+    st.err = static_cast<int*>(p);
   }
   if (need > st.bytes) {
     cudaFree(st.scratch);  // the previous call on this device has finished
@@ -217,13 +227,10 @@ extern "C" tn_status tn_contract_pair(const void* A, const int32_t* a_labels, in
         e = launch_gemm_tc(a, b, c, d, true, 1.f, 1.f, err, s);
       }
       if (e == cudaSuccess) {
-        int h = 0;
-        cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s);
         e = cudaStreamSynchronize(s);
+        const int h = *ps->err_host;
         if (e == cudaSuccess && h) {
-          const cudaError_t ce = cudaMemset(err, 0, sizeof(int));
-          if (ce != cudaSuccess)
-            return fail(TN_ECUDA, "tn_contract_pair: clearing the error word: %s", cudaGetErrorString(ce));
+          *ps->err_host = 0;
           return fail(TN_ETIMEOUT, "tn_contract_pair: a tensor-core pipeline wait expired (code %d)", h);
         }
       }
