@@ -98,13 +98,17 @@ __global__ void __launch_bounds__(NT) reduce_kernel(const float2* __restrict__ A
 // are an L2 -> SM stream.  So the eight warps' shares of k go to the eight CTAs
 // of a cluster, and the outputs in 2 x 2 blocks to clusters: 128 SMs for
 // 64 outputs, each reading 4 operand rows (2 of A, 2 of B) of its k share once
-// for 4 outputs, one warp per output.  The rows arrive by 8-byte cp.async
-// (any index order) through a ring of 16-value groups, 3 of 4 in flight; the
-// CTAs' partial sums meet in the first one's shared memory.  Measured per
-// tn_contract_pair call: 2^3 x 2^3 x 2^18 with contiguous K 3260 -> 45 us (of
-// which about 25 us are the call), 2^6 x 1 x 2^16 43 us, 1 x 1 x 2^19 102 us.
+// for 4 outputs, one warp per output.  Four more warps only copy: the rows
+// arrive by cp.async through a ring of 16-value groups, 7 of 8 in flight, and
+// one barrier per group paces both, so an addition chain (16 values of two
+// dependent FMAs) runs while the copies of a later group are issued.  The copies
+// move 8 bytes per lane in any index order, or 16 past L1 when the five lowest
+// contracted indices are both operands' fastest.  The CTAs' partial sums meet in
+// the first one's shared memory.  Measured per
+// tn_contract_pair call, 2^3 x 2^3 x 2^18 with contiguous K: one CTA 3260 us,
+// copies and sums by the same warps 45 us, now 33 us; 1 x 1 x 2^19 102 -> 26 us.
 constexpr int SP_G = 16;                   // values of k per thread and group (bits LOW .. LOW + 3)
-constexpr int SP_RING = 4;
+constexpr int SP_RING = 8;
 constexpr int SP_ROWS = 4;                 // at most 2 rows of A and 2 of B per CTA
 constexpr int SP_SMEM = SP_RING * SP_G * SP_ROWS * 32 * (int)sizeof(float2);
 
@@ -112,10 +116,18 @@ __device__ __forceinline__ void cp_async8(uint32_t dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
 }
 
-__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(128)
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+}
+
+// WIDE: lane bits 0..4 of k have strides 1, 2, 4, 8, 16 in A and B, every
+// 32-value run starts on a 16-byte boundary, and a group has 16 values of k.
+template <bool WIDE>
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(256)
     reduce_spread_kernel(const float2* __restrict__ A, const float2* __restrict__ B, float2* __restrict__ C,
                          const GemmDesc d) {
-  extern __shared__ __align__(16) float2 ring[];  // [SP_RING][SP_G][row][32]
+  constexpr int RING = SP_RING;
+  extern __shared__ __align__(16) float2 ring[];  // [RING][SP_G][row][32]
   __shared__ float2 part[8][4];                   // first CTA of the cluster: [original warp][output]
   const int64_t ulo = blockIdx.y % d.units_lo, uhi = blockIdx.y / d.units_lo;
   A += ulo * d.a_lo + uhi * d.a_hi;
@@ -124,7 +136,7 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(128)
   // the cluster's CTAs have all started once this barrier's phase completes
   // (awaited before the first store to another CTA's shared memory)
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int share = blockIdx.x & 7, blk = blockIdx.x >> 3;  // cluster rank, output block
   const int wm = d.nm > 0 ? 1 : 0, wn = d.nn > 0 ? 1 : 0;   // the block's rows and columns (log2)
   const int nblk_n = 1 << (d.nn - wn);
@@ -135,62 +147,74 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(128)
   const int glen = 1 << gbits;
   const int64_t ngroups = int64_t(1) << (d.nk - LOW - gbits);
   const int t = share * 32 + lane;  // the thread of the 256 whose values this lane sums
-  // The warp copies rows warp, warp + nwarps (at most two).  Everything an
-  // issue needs is in registers: the offsets of a group's 16 values, and one
-  // stride of the group index per lane, summed over the warp.
-  const float2* src[2];
-  int32_t tab[2][SP_G], gst[2];
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int r = warp + q * nwarps;
+  const int sums = 1 << (wm + wn);  // warps 0 .. sums - 1 add, warp sums + r copies row r
+  float2 c = make_float2(0.f, 0.f);
+  if (warp >= sums) {
+    // everything an issue needs is in registers: the offsets of a group's 16
+    // values, and one stride of the group index per lane, summed over the warp
+    const int r = warp - sums;
     const bool isa = r < ra;
     const int32_t* ks = isa ? d.ak : d.bk;
-    src[q] = isa ? A + bit_offset(m0 + r, 0, d.nm, d.am) : B + bit_offset(n0 + r - ra, 0, d.nn, d.bn);
-    src[q] += bit_offset(t, 0, LOW, ks);
-    gst[q] = LOW + gbits + lane < d.nk ? ks[LOW + gbits + lane] : 0;
+    const float2* src = isa ? A + bit_offset(m0 + r, 0, d.nm, d.am) : B + bit_offset(n0 + r - ra, 0, d.nn, d.bn);
+    // WIDE: a lane copies values 2 (lane % 16), + 1 of the share's run, for the
+    // group's even (lanes 0..15) or odd (16..31) values of k
+    src += WIDE ? bit_offset(share * 32, 0, LOW, ks) + 2 * (lane & 15) + (lane >> 4) * ks[LOW]
+                : bit_offset(t, 0, LOW, ks);
+    const int32_t gst = LOW + gbits + lane < d.nk ? ks[LOW + gbits + lane] : 0;
+    int32_t tab[SP_G];
 #pragma unroll
     for (int i = 0; i < SP_G; ++i) {
-      tab[q][i] = 0;
+      tab[i] = 0;
 #pragma unroll
       for (int b = 0; b < 4; ++b)
-        if (((i >> b) & 1) && b < gbits) tab[q][i] += ks[LOW + b];
+        if (((i >> b) & 1) && b < gbits) tab[i] += ks[LOW + b];
     }
-  }
-  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(ring);
-  auto issue = [&](int g) {
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(ring) + (uint32_t)r * 256u +
+                          (WIDE ? (uint32_t)((lane >> 4) * SP_ROWS) * 256u + (uint32_t)(lane & 15) * 16u
+                                : (uint32_t)lane * 8u);
+    auto issue = [&](int g) {
+      const float2* p = src + (int32_t)__reduce_add_sync(0xffffffffu, (uint32_t)(((g >> lane) & 1) ? gst : 0));
+      const uint32_t slot = base + (uint32_t)((g % RING) * SP_G * SP_ROWS) * 256u;
+      if constexpr (WIDE) {
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int r = warp + q * nwarps;
-      if (r >= rows) break;
-      const float2* p = src[q] + (int32_t)__reduce_add_sync(0xffffffffu, (uint32_t)(((g >> lane) & 1) ? gst[q] : 0));
-      const uint32_t slot = sbase + (uint32_t)(((g % SP_RING) * SP_G * SP_ROWS + r) * 32 + lane) * 8u;
+        for (int i = 0; i < SP_G; i += 2) cp_async16(slot + (uint32_t)(i * SP_ROWS) * 256u, p + tab[i]);
+      } else {
 #pragma unroll
-      for (int i = 0; i < SP_G; ++i)
-        if (i < glen) cp_async8(slot + (uint32_t)(i * SP_ROWS * 32) * 8u, p + tab[q][i]);
-    }
-  };
-  for (int g = 0; g < SP_RING - 1; ++g) {
-    if (g < ngroups) issue(g);
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-  }
-  float2 c = make_float2(0.f, 0.f);
-  for (int g = 0; g < (int)ngroups; ++g) {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(SP_RING - 2) : "memory");
-    __syncthreads();  // group g landed for every warp; group g - 1's slot is free
-    if (g + SP_RING - 1 < ngroups) issue(g + SP_RING - 1);
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-    const float2* pa = ring + ((g % SP_RING) * SP_G * SP_ROWS + m_l) * 32 + lane;
-    const float2* pb = ring + ((g % SP_RING) * SP_G * SP_ROWS + ra + n_l) * 32 + lane;
-    auto mac = [&](int i) {
-      const float2 a = pa[i * SP_ROWS * 32], b = pb[i * SP_ROWS * 32];
-      c.x = fmaf(a.x, b.x, fmaf(-a.y, b.y, c.x));
-      c.y = fmaf(a.x, b.y, fmaf(a.y, b.x, c.y));
+        for (int i = 0; i < SP_G; ++i)
+          if (i < glen) cp_async8(slot + (uint32_t)(i * SP_ROWS) * 256u, p + tab[i]);
+      }
     };
-    if (glen == SP_G) {
+    for (int g = 0; g < RING - 1; ++g) {
+      if (g < ngroups) issue(g);
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+    for (int g = 0; g < (int)ngroups; ++g) {
+      asm volatile("cp.async.wait_group %0;\n" ::"n"(RING - 2) : "memory");
+      __syncthreads();  // group g landed for every warp; group g - 1's slot is free
+      if (g + RING - 1 < ngroups) issue(g + RING - 1);
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+  } else {
+    for (int g = 0; g < (int)ngroups; ++g) {
+      __syncthreads();
+      const float2* pa = ring + ((g % RING) * SP_G * SP_ROWS + m_l) * 32 + lane;
+      const float2* pb = ring + ((g % RING) * SP_G * SP_ROWS + ra + n_l) * 32 + lane;
+      auto mac = [&](float2 a, float2 b) {
+        c.x = fmaf(a.x, b.x, fmaf(-a.y, b.y, c.x));
+        c.y = fmaf(a.x, b.y, fmaf(a.y, b.x, c.y));
+      };
+      if (glen == SP_G) {
+        float2 a[SP_G], b[SP_G];
 #pragma unroll
-      for (int i = 0; i < SP_G; ++i) mac(i);
-    } else {
-      for (int i = 0; i < glen; ++i) mac(i);
+        for (int i = 0; i < SP_G; ++i) {
+          a[i] = pa[i * SP_ROWS * 32];
+          b[i] = pb[i * SP_ROWS * 32];
+        }
+#pragma unroll
+        for (int i = 0; i < SP_G; ++i) mac(a[i], b[i]);
+      } else {
+        for (int i = 0; i < glen; ++i) mac(pa[i * SP_ROWS * 32], pb[i * SP_ROWS * 32]);
+      }
     }
   }
 #pragma unroll
@@ -199,14 +223,14 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(128)
     c.y += __shfl_xor_sync(0xffffffffu, c.y, o);
   }
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  if (lane == 0) {
+  if (warp < sums && lane == 0) {
     uint32_t dst;
     asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst)
                  : "r"((uint32_t)__cvta_generic_to_shared(&part[share][warp])));
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(c.x), "f"(c.y) : "memory");
   }
   asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  if (share == 0 && lane == 0) {
+  if (share == 0 && warp < sums && lane == 0) {
     float2 s = part[0][warp];
 #pragma unroll
     for (int w = 1; w < 8; ++w) {
@@ -222,7 +246,8 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(128)
 // group of loads each).
 constexpr int SPREAD_UNITS = 152;
 
-cudaError_t launch_spread(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s) {
+template <bool WIDE>
+cudaError_t launch_spread_as(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s) {
   static std::once_flag once[64];
   static cudaError_t attr[64];
   int dev = 0;
@@ -230,13 +255,27 @@ cudaError_t launch_spread(const float2* A, const float2* B, float2* C, const Gem
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::call_once(once[dev], [&] {
-    attr[dev] = cudaFuncSetAttribute(reduce_spread_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SP_SMEM);
+    attr[dev] = cudaFuncSetAttribute(reduce_spread_kernel<WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SP_SMEM);
   });
   if (attr[dev] != cudaSuccess) return attr[dev];
   const int wm = d.nm > 0 ? 1 : 0, wn = d.nn > 0 ? 1 : 0;
   const dim3 grid(8u << (d.nm - wm + d.nn - wn), (unsigned)d.units);
-  reduce_spread_kernel<<<grid, 32u << (wm + wn), SP_SMEM, s>>>(A, B, C, d);
+  const unsigned warps = (1u << (wm + wn)) + (1u << wm) + (1u << wn);  // adding, copying
+  reduce_spread_kernel<WIDE><<<grid, 32u * warps, SP_SMEM, s>>>(A, B, C, d);
   return cudaGetLastError();
+}
+
+cudaError_t launch_spread(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s) {
+  // 16-byte copies: runs of 32 values in both operands (every other stride is
+  // then a multiple of 32), aligned bases, even unit strides, whole groups
+  auto runs = [&](const float2* p, const int32_t* ks, int64_t lo, int64_t hi) {
+    bool ok = (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (lo & 1) == 0 && (hi & 1) == 0;
+    for (int i = 0; i < 5; ++i) ok &= ks[i] == (int32_t(1) << i);
+    return ok;
+  };
+  if (d.nk - LOW >= 4 && runs(A, d.ak, d.a_lo, d.a_hi) && runs(B, d.bk, d.b_lo, d.b_hi))
+    return launch_spread_as<true>(A, B, C, d, s);
+  return launch_spread_as<false>(A, B, C, d, s);
 }
 
 template <int NM, int NN>
