@@ -23,10 +23,19 @@ namespace tn {
 namespace {
 
 constexpr int NT = 256;
-constexpr int PER = 4;                 // rows per thread
-constexpr int CH_BITS = 10;            // 1024 rows per CTA
-constexpr int CH = 1 << CH_BITS;
-static_assert(NT * PER == CH, "chunk");
+constexpr int CH_BITS = 10;            // 1024 rows per CTA (log2) ..
+constexpr int CH_BITS_FEW = 8;         // .. or 256 when that leaves SMs idle
+
+// Rows per CTA (log2).  1024 rows amortise a CTA's tables over four rows per
+// thread; with fewer such CTAs than SMs the launch is one CTA's latency, four
+// dependent rows long: (12, 4, 2) x 2 units took 17 us on 8 CTAs.
+int chunk_bits(const GemmDesc& d) {
+  const int64_t ctas = d.nm > CH_BITS ? (int64_t(1) << (d.nm - CH_BITS)) * d.units : d.units;
+  return ctas >= 152 ? CH_BITS : CH_BITS_FEW;
+}
+dim3 chunk_grid(const GemmDesc& d, int cb) {
+  return dim3(d.nm > cb ? 1u << (d.nm - cb) : 1u, (unsigned)d.units);
+}
 
 __device__ __forceinline__ int32_t bit_offset(int64_t x, int nb, const int32_t* st) {
   int32_t o = 0;
@@ -92,11 +101,13 @@ __device__ __forceinline__ void emit(const VecOut& o, float2* C, int64_t off, fl
   }
 }
 
-template <int NK, int NN>
+template <int NK, int NN, int PER>
 __global__ void __launch_bounds__(NT) vector_kernel(const float2* __restrict__ A, const float2* __restrict__ B,
                                                     float2* __restrict__ C, const GemmDesc d,
                                                     const VecOut o) {
   constexpr int K = 1 << NK, N = 1 << NN;
+  constexpr int cb = PER == 4 ? CH_BITS : CH_BITS_FEW;
+  static_assert(NT * PER == 1 << cb, "rows of a CTA");
   const int64_t M = int64_t(1) << d.nm;
   const int64_t ulo = blockIdx.y % d.units_lo, uhi = blockIdx.y / d.units_lo;
   A += ulo * d.a_lo + uhi * d.a_hi;
@@ -106,14 +117,14 @@ __global__ void __launch_bounds__(NT) vector_kernel(const float2* __restrict__ A
   __shared__ int32_t kA[K], nC[N];
   __shared__ int32_t tAlo[32], tAhi[32], tClo[32], tChi[32];
   const int tid = threadIdx.x;
-  const int64_t base = (int64_t)blockIdx.x * CH;
+  const int64_t base = (int64_t)blockIdx.x << cb;
   for (int e = tid; e < K * N; e += NT) {
     int k = e / N, n = e % N;
     Bs[e] = B[bit_offset(k, NK, d.bk) + bit_offset(n, NN, d.bn)];
   }
   if (tid < K) kA[tid] = bit_offset(tid, NK, d.ak);
   if (tid >= 64 && tid < 64 + N) nC[tid - 64] = bit_offset(tid - 64, NN, d.cn);
-  const int lb = d.nm < CH_BITS ? d.nm : CH_BITS;  // bits of m inside the chunk
+  const int lb = d.nm < cb ? d.nm : cb;  // bits of m inside the chunk
   if (tid >= 128 && tid < 160) {
     int x = tid - 128;
     int b0 = lb < 5 ? lb : 5;
@@ -130,7 +141,7 @@ __global__ void __launch_bounds__(NT) vector_kernel(const float2* __restrict__ A
   __shared__ int32_t baseA, baseC;
   if (tid == 0) {
     int32_t oa = 0, oc = 0;
-    for (int i = CH_BITS; i < d.nm; ++i)
+    for (int i = cb; i < d.nm; ++i)
       if ((base >> i) & 1) { oa += d.am[i]; oc += d.cm[i]; }
     baseA = oa;
     baseC = oc;
@@ -170,7 +181,7 @@ __global__ void __launch_bounds__(NT) vector_kernel(const float2* __restrict__ A
 template <int NK, int NN>
 __global__ void __launch_bounds__(NT) vector_wide_kernel(const float2* __restrict__ A, const float2* __restrict__ B,
                                                          float2* __restrict__ C, const GemmDesc d,
-                                                         const VecOut o, int pair_k) {
+                                                         const VecOut o, int pair_k, int cb) {
   constexpr int K = 1 << NK, N = 1 << NN;
   static_assert(K * N <= 1024, "B must fit in shared memory");
   const int64_t M = int64_t(1) << d.nm;
@@ -183,14 +194,14 @@ __global__ void __launch_bounds__(NT) vector_wide_kernel(const float2* __restric
   __shared__ int32_t tAlo[32], tAhi[32], tClo[32], tChi[32];
   __shared__ int32_t baseA, baseC;
   const int tid = threadIdx.x;
-  const int64_t base = (int64_t)blockIdx.x * CH;
+  const int64_t base = (int64_t)blockIdx.x << cb;
   for (int e = tid; e < K * N; e += NT) {
     const int k = e / N, n = e % N;
     Bs[e] = B[bit_offset(k, NK, d.bk) + bit_offset(n, NN, d.bn)];
   }
   if (tid < K) kA[tid] = bit_offset(tid, NK, d.ak);
   for (int n = tid; n < N; n += NT) nC[n] = bit_offset(n, NN, d.cn);
-  const int lb = d.nm < CH_BITS ? d.nm : CH_BITS;
+  const int lb = d.nm < cb ? d.nm : cb;
   if (tid >= 128 && tid < 160) {
     const int x = tid - 128, b0 = lb < 5 ? lb : 5;
     tAlo[x] = x < (1 << b0) ? bit_offset(x, b0, d.am) : 0;
@@ -203,7 +214,7 @@ __global__ void __launch_bounds__(NT) vector_wide_kernel(const float2* __restric
   }
   if (tid == 192) {
     int32_t oa = 0, oc = 0;
-    for (int i = CH_BITS; i < d.nm; ++i)
+    for (int i = cb; i < d.nm; ++i)
       if ((base >> i) & 1) { oa += d.am[i]; oc += d.cm[i]; }
     baseA = oa;
     baseC = oc;
@@ -211,7 +222,7 @@ __global__ void __launch_bounds__(NT) vector_wide_kernel(const float2* __restric
   __syncthreads();
   float mx = 0.f;
 #pragma unroll 1
-  for (int r = 0; r < PER; ++r) {
+  for (int r = 0; r < (1 << cb) / NT; ++r) {
     const int loc = tid + r * NT;
     if (base + loc >= M) break;
     const int32_t oa = baseA + tAlo[loc & 31] + tAhi[loc >> 5];
@@ -253,7 +264,7 @@ __global__ void __launch_bounds__(NT) vector_wide_kernel(const float2* __restric
 template <int NK, int NN>
 __global__ void __launch_bounds__(NT) vector_long_kernel(const float2* __restrict__ A, const float2* __restrict__ B,
                                                          float2* __restrict__ C, const GemmDesc d, int pair_k,
-                                                         const VecOut o) {
+                                                         const VecOut o, int cb) {
   constexpr int K = 1 << NK, N = 1 << NN;
   static_assert(K * N <= 1024, "B must fit in shared memory");
   const int64_t M = int64_t(1) << d.nm;
@@ -266,14 +277,14 @@ __global__ void __launch_bounds__(NT) vector_long_kernel(const float2* __restric
   __shared__ int32_t tAlo[32], tAhi[32], tClo[32], tChi[32];
   __shared__ int32_t baseA, baseC;
   const int tid = threadIdx.x;
-  const int64_t base = (int64_t)blockIdx.x * CH;
+  const int64_t base = (int64_t)blockIdx.x << cb;
   for (int e = tid; e < K * N; e += NT) {
     const int k = e / N, n = e % N;
     Bs[e] = B[bit_offset(k, NK, d.bk) + bit_offset(n, NN, d.bn)];
   }
   for (int k = tid; k < K; k += NT) kA[k] = bit_offset(k, NK, d.ak);
   if (tid >= 192 && tid < 192 + N) nC[tid - 192] = bit_offset(tid - 192, NN, d.cn);
-  const int lb = d.nm < CH_BITS ? d.nm : CH_BITS;
+  const int lb = d.nm < cb ? d.nm : cb;
   if (tid >= 128 && tid < 160) {
     const int x = tid - 128, b0 = lb < 5 ? lb : 5;
     tAlo[x] = x < (1 << b0) ? bit_offset(x, b0, d.am) : 0;
@@ -286,7 +297,7 @@ __global__ void __launch_bounds__(NT) vector_long_kernel(const float2* __restric
   }
   if (tid == 0) {
     int32_t oa = 0, oc = 0;
-    for (int i = CH_BITS; i < d.nm; ++i)
+    for (int i = cb; i < d.nm; ++i)
       if ((base >> i) & 1) { oa += d.am[i]; oc += d.cm[i]; }
     baseA = oa;
     baseC = oc;
@@ -294,7 +305,7 @@ __global__ void __launch_bounds__(NT) vector_long_kernel(const float2* __restric
   __syncthreads();
   float mx = 0.f;
 #pragma unroll 1
-  for (int r = 0; r < PER; ++r) {
+  for (int r = 0; r < (1 << cb) / NT; ++r) {
     const int loc = tid + r * NT;
     if (base + loc >= M) break;
     const int32_t oa = baseA + tAlo[loc & 31] + tAhi[loc >> 5];
@@ -350,7 +361,7 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 template <int NK, int NN>
 __global__ void __launch_bounds__(SNT) vector_staged_kernel(const float2* __restrict__ A, const float2* __restrict__ B,
                                                             float2* __restrict__ C, const GemmDesc d,
-                                                            const VecOut o) {
+                                                            const VecOut o, int cb) {
   constexpr int K = 1 << NK, N = 1 << NN;
   constexpr int KC = K < 16 ? K : 16;    // K values per stage
   constexpr int PITCH = KC + 2;          // complex per staged row
@@ -369,13 +380,13 @@ __global__ void __launch_bounds__(SNT) vector_staged_kernel(const float2* __rest
   __shared__ int32_t tAlo[32], tAhi[32], tClo[32], tChi[32];
   __shared__ int32_t baseA, baseC;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t base = (int64_t)blockIdx.x * CH;
+  const int64_t base = (int64_t)blockIdx.x << cb;
   for (int e = tid; e < K * N; e += SNT) {
     const int k = e / N, n = e % N;
     Bs[e] = B[bit_offset(k, NK, d.bk) + bit_offset(n, NN, d.bn)];
   }
   if (tid < N) nC[tid] = bit_offset(tid, NN, d.cn);
-  const int lb = d.nm < CH_BITS ? d.nm : CH_BITS;
+  const int lb = d.nm < cb ? d.nm : cb;
   if (tid >= 32 && tid < 64) {
     const int x = tid - 32;
     tAlo[x] = bit_offset(x, 5, d.am);  // lb >= 5
@@ -388,13 +399,13 @@ __global__ void __launch_bounds__(SNT) vector_staged_kernel(const float2* __rest
   }
   if (tid == 96) {
     int32_t oa = 0, oc = 0;
-    for (int i = CH_BITS; i < d.nm; ++i)
+    for (int i = cb; i < d.nm; ++i)
       if ((base >> i) & 1) { oa += d.am[i]; oc += d.cm[i]; }
     baseA = oa;
     baseC = oc;
   }
   __syncthreads();
-  const int64_t rows = M - base < CH ? M - base : CH;
+  const int64_t rows = M - base < (1 << cb) ? M - base : (1 << cb);
   const int ngroups = (int)(rows >> 5);
   const int nitems = ngroups > warp ? ((ngroups - 1 - warp) / SW + 1) * NCH : 0;
   float2* st = stage[warp][0];
@@ -458,15 +469,16 @@ bool staged_ok(const float2* A, const GemmDesc& d) {
 template <int NK>
 cudaError_t launch_staged(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s,
                           const VecOut& mb) {
-  const dim3 g((unsigned)(((int64_t(1) << d.nm) + CH - 1) / CH), (unsigned)d.units);
+  const int cb = chunk_bits(d);
+  const dim3 g = chunk_grid(d, cb);
   switch (d.nn) {
-    case 0: vector_staged_kernel<NK, 0><<<g, SNT, 0, s>>>(A, B, C, d, mb); break;
-    case 1: vector_staged_kernel<NK, 1><<<g, SNT, 0, s>>>(A, B, C, d, mb); break;
-    case 2: vector_staged_kernel<NK, 2><<<g, SNT, 0, s>>>(A, B, C, d, mb); break;
-    case 3: vector_staged_kernel<NK, 3><<<g, SNT, 0, s>>>(A, B, C, d, mb); break;
+    case 0: vector_staged_kernel<NK, 0><<<g, SNT, 0, s>>>(A, B, C, d, mb, cb); break;
+    case 1: vector_staged_kernel<NK, 1><<<g, SNT, 0, s>>>(A, B, C, d, mb, cb); break;
+    case 2: vector_staged_kernel<NK, 2><<<g, SNT, 0, s>>>(A, B, C, d, mb, cb); break;
+    case 3: vector_staged_kernel<NK, 3><<<g, SNT, 0, s>>>(A, B, C, d, mb, cb); break;
     case 4:
       if constexpr (NK <= 4) {
-        vector_staged_kernel<NK, 4><<<g, SNT, 0, s>>>(A, B, C, d, mb);
+        vector_staged_kernel<NK, 4><<<g, SNT, 0, s>>>(A, B, C, d, mb, cb);
         break;
       }
       return cudaErrorInvalidValue;
@@ -476,32 +488,39 @@ cudaError_t launch_staged(const float2* A, const float2* B, float2* C, const Gem
 }
 
 template <int NK>
-cudaError_t launch_long(const float2* A, const float2* B, float2* C, const GemmDesc& d, dim3 g, cudaStream_t s,
+cudaError_t launch_long(const float2* A, const float2* B, float2* C, const GemmDesc& d, int cb, cudaStream_t s,
                         const VecOut& mb) {
+  const dim3 g = chunk_grid(d, cb);
   // pairs (k, k + 1), k even, are adjacent when A's K bit 0 has stride 1;
   // every other stride of A is then even, so a pair starts on a 16-byte
   // boundary once the base and the unit strides are even
   const int pair_k = d.nk >= 1 && d.ak[0] == 1 && (reinterpret_cast<uintptr_t>(A) & 15) == 0 &&
                      (d.a_lo & 1) == 0 && (d.a_hi & 1) == 0;
   switch (d.nn) {
-    case 0: vector_long_kernel<NK, 0><<<g, NT, 0, s>>>(A, B, C, d, pair_k, mb); break;
-    case 1: vector_long_kernel<NK, 1><<<g, NT, 0, s>>>(A, B, C, d, pair_k, mb); break;
-    case 2: vector_long_kernel<NK, 2><<<g, NT, 0, s>>>(A, B, C, d, pair_k, mb); break;
-    case 3: vector_long_kernel<NK, 3><<<g, NT, 0, s>>>(A, B, C, d, pair_k, mb); break;
+    case 0: vector_long_kernel<NK, 0><<<g, NT, 0, s>>>(A, B, C, d, pair_k, mb, cb); break;
+    case 1: vector_long_kernel<NK, 1><<<g, NT, 0, s>>>(A, B, C, d, pair_k, mb, cb); break;
+    case 2: vector_long_kernel<NK, 2><<<g, NT, 0, s>>>(A, B, C, d, pair_k, mb, cb); break;
+    case 3: vector_long_kernel<NK, 3><<<g, NT, 0, s>>>(A, B, C, d, pair_k, mb, cb); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
 
 template <int NK>
-cudaError_t launch_nn(const float2* A, const float2* B, float2* C, const GemmDesc& d, dim3 g, cudaStream_t s,
+cudaError_t launch_nn(const float2* A, const float2* B, float2* C, const GemmDesc& d, int cb, cudaStream_t s,
                       const VecOut& mb) {
+  const dim3 g = chunk_grid(d, cb);
+  auto one = [&](auto nn) {
+    constexpr int NN = decltype(nn)::value;
+    if (cb == CH_BITS) vector_kernel<NK, NN, 4><<<g, NT, 0, s>>>(A, B, C, d, mb);
+    else vector_kernel<NK, NN, 1><<<g, NT, 0, s>>>(A, B, C, d, mb);
+  };
   switch (d.nn) {
-    case 0: vector_kernel<NK, 0><<<g, NT, 0, s>>>(A, B, C, d, mb); break;
-    case 1: vector_kernel<NK, 1><<<g, NT, 0, s>>>(A, B, C, d, mb); break;
-    case 2: vector_kernel<NK, 2><<<g, NT, 0, s>>>(A, B, C, d, mb); break;
-    case 3: vector_kernel<NK, 3><<<g, NT, 0, s>>>(A, B, C, d, mb); break;
-    case 4: vector_kernel<NK, 4><<<g, NT, 0, s>>>(A, B, C, d, mb); break;
+    case 0: one(std::integral_constant<int, 0>{}); break;
+    case 1: one(std::integral_constant<int, 1>{}); break;
+    case 2: one(std::integral_constant<int, 2>{}); break;
+    case 3: one(std::integral_constant<int, 3>{}); break;
+    case 4: one(std::integral_constant<int, 4>{}); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -521,8 +540,9 @@ bool vector_shape_ok(const GemmDesc& d) {
 bool stream_preferred(const GemmDesc& d) { return d.nn == 5 && d.nk == 3; }
 
 template <int NK>
-cudaError_t launch_wide(const float2* A, const float2* B, float2* C, const GemmDesc& d, dim3 g, cudaStream_t s,
+cudaError_t launch_wide(const float2* A, const float2* B, float2* C, const GemmDesc& d, int cb, cudaStream_t s,
                         const VecOut& mb) {
+  const dim3 g = chunk_grid(d, cb);
   // pairs (k, k + 1), k even, adjacent and 16-byte aligned: A's K bit 0 has
   // stride 1 (every other stride of A is then even), even unit strides
   const int pair_k = NK >= 1 && d.ak[0] == 1 && (reinterpret_cast<uintptr_t>(A) & 15) == 0 && (d.a_lo & 1) == 0 &&
@@ -530,7 +550,7 @@ cudaError_t launch_wide(const float2* A, const float2* B, float2* C, const GemmD
   auto one = [&](auto nn) -> cudaError_t {
     constexpr int NN = decltype(nn)::value;
     if constexpr (((1 << NK) << NN) <= 1024) {
-      vector_wide_kernel<NK, NN><<<g, NT, 0, s>>>(A, B, C, d, mb, pair_k);
+      vector_wide_kernel<NK, NN><<<g, NT, 0, s>>>(A, B, C, d, mb, pair_k, cb);
       return cudaGetLastError();
     } else {
       return cudaErrorInvalidValue;
@@ -552,14 +572,13 @@ bool vector_sums_im_first(const float2* A, const GemmDesc& d) {
 cudaError_t launch_vector(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s,
                           const VecOut& maxbits) {
   if (!vector_shape_ok(d) || d.units > 65535) return cudaErrorInvalidValue;
-  int64_t M = int64_t(1) << d.nm;
-  dim3 g((unsigned)((M + CH - 1) / CH), (unsigned)d.units);
-  if (d.nn == 5 && d.nk == 3) return launch_wide<3>(A, B, C, d, g, s, maxbits);
+  const int cb = chunk_bits(d);
+  if (d.nn == 5 && d.nk == 3) return launch_wide<3>(A, B, C, d, cb, s, maxbits);
   if (d.nn > 4) {  // K <= 2 (vector_shape_ok)
     switch (d.nk) {
-      case 0: return launch_wide<0>(A, B, C, d, g, s, maxbits);
-      case 1: return launch_wide<1>(A, B, C, d, g, s, maxbits);
-      default: return launch_wide<2>(A, B, C, d, g, s, maxbits);
+      case 0: return launch_wide<0>(A, B, C, d, cb, s, maxbits);
+      case 1: return launch_wide<1>(A, B, C, d, cb, s, maxbits);
+      default: return launch_wide<2>(A, B, C, d, cb, s, maxbits);
     }
   }
   if (staged_ok(A, d)) {
@@ -573,17 +592,17 @@ cudaError_t launch_vector(const float2* A, const float2* B, float2* C, const Gem
   }
   if (d.nk > 4) {
     switch (d.nk) {
-      case 5: return launch_long<5>(A, B, C, d, g, s, maxbits);
-      case 6: return launch_long<6>(A, B, C, d, g, s, maxbits);
-      default: return launch_long<7>(A, B, C, d, g, s, maxbits);
+      case 5: return launch_long<5>(A, B, C, d, cb, s, maxbits);
+      case 6: return launch_long<6>(A, B, C, d, cb, s, maxbits);
+      default: return launch_long<7>(A, B, C, d, cb, s, maxbits);
     }
   }
   switch (d.nk) {
-    case 0: return launch_nn<0>(A, B, C, d, g, s, maxbits);
-    case 1: return launch_nn<1>(A, B, C, d, g, s, maxbits);
-    case 2: return launch_nn<2>(A, B, C, d, g, s, maxbits);
-    case 3: return launch_nn<3>(A, B, C, d, g, s, maxbits);
-    default: return launch_nn<4>(A, B, C, d, g, s, maxbits);
+    case 0: return launch_nn<0>(A, B, C, d, cb, s, maxbits);
+    case 1: return launch_nn<1>(A, B, C, d, cb, s, maxbits);
+    case 2: return launch_nn<2>(A, B, C, d, cb, s, maxbits);
+    case 3: return launch_nn<3>(A, B, C, d, cb, s, maxbits);
+    default: return launch_nn<4>(A, B, C, d, cb, s, maxbits);
   }
 }
 
