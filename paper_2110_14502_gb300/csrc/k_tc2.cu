@@ -1068,10 +1068,25 @@ cudaError_t set_tc_wait_limit(long long polls) {
   return cudaMemcpyToSymbol(g_wait_limit, &v, sizeof v);
 }
 
+// Tile width: 128 columns where the tiles fill the chip; narrower ones where
+// that spreads the work over more SMs, by waves over 152 SMs times the time of
+// a tile relative to 128 columns (a narrow MMA is less efficient, and a tile's
+// A copy does not shrink).  Every width gives the same bits.
 int tma_tile_n(const GemmDesc& d) {
   const int def = d.nn >= 7 ? 128 : (1 << d.nn);
   if (d.tile_n >= 16 && d.tile_n <= def) return d.tile_n;
-  return def;
+  int best = def;
+  double best_cost = 1e300;
+  for (int tn = def; tn >= (def < 32 ? def : 32); tn /= 2) {
+    const int64_t items = ((int64_t(1) << d.nm) / TM) * ((int64_t(1) << d.nn) / tn) * d.units;
+    const double rel = tn == 128 ? 1.0 : tn == 64 ? 0.55 : tn == 32 ? 0.35 : 0.3;
+    const double cost = (double)((items + 151) / 152) * rel;
+    if (cost < best_cost) {
+      best = tn;
+      best_cost = cost;
+    }
+  }
+  return best;
 }
 
 int64_t split_plane_elems(int nrow_bits, int nk_bits, int np) {
