@@ -454,6 +454,316 @@ __global__ void __launch_bounds__(SNT) vector_staged_kernel(const float2* __rest
   record_max(o.maxbits, mx);
 }
 
+// Any index order at the memory rate (N, K <= 16).  The kernels above give a
+// thread a row, so a warp's loads follow A only where A's fastest indices are
+// contracted or among C's fastest, and its stores follow C only where C's
+// fastest indices are rows; other orders move a 32-byte sector for 8 bytes.
+// Here a CTA takes the 2^8 rows spanned by eight row indices chosen to hold
+// both A's and C's fastest ones: it reads its block of A front to back into
+// shared memory ([row][k]), computes two rows per thread, and writes its block
+// of C front to back from shared memory.  B sits in shared memory as (re, im,
+// im, re), one 16-byte read for both packed products of a complex
+// multiply-add; the sums run in the order of the kernel that would otherwise
+// take the shape (IM_FIRST), so the results are the same bit for bit.
+constexpr int TILE_BITS = 8, TILE_ROWS = 1 << TILE_BITS, TNT = TILE_ROWS / 2;
+// Shared-memory slots are the element's index with its upper bits folded onto
+// bits 1..3 (16-byte units of a 128-byte line), so a slot is the XOR of its
+// index bits' images.  The block of A is indexed row 2^NK + k, that of C in C's
+// order.
+struct RowTile {
+  int nout;                                  // row indices outside the tile ..
+  int32_t out_a[kMaxBits], out_c[kMaxBits];  // .. and their strides
+  int32_t a_src[TILE_BITS + 4], a_slot[TILE_BITS + 4];  // the block of A's bits in A's order: stride, image
+  int32_t a_row[TILE_BITS];                             // images of the row bits in the block of A
+  int32_t c_dst[TILE_BITS + 4], c_slot[TILE_BITS + 4];  // the block of C's bits in C's order: stride, image
+  int32_t row_slot[TILE_BITS], col_slot[4];             // images of the row and column bits in the block of C
+};
+
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+
+template <int NK, int NN, bool IM_FIRST>
+__global__ void __launch_bounds__(TNT) vector_tile_kernel(const float2* __restrict__ A, const float2* __restrict__ B,
+                                                          float2* __restrict__ C, const GemmDesc d,
+                                                          const __grid_constant__ RowTile rt, int a_vec, int c_vec) {
+  constexpr int K = 1 << NK, N = 1 << NN;
+  constexpr int AE = TILE_ROWS * K, CE = TILE_ROWS * N;
+  __shared__ __align__(16) float2 block[AE > CE ? AE : CE];
+  __shared__ __align__(16) float4 Bs[K * N];
+  const int64_t ulo = blockIdx.y % d.units_lo, uhi = blockIdx.y / d.units_lo;
+  A += ulo * d.a_lo + uhi * d.a_hi;
+  B += ulo * d.b_lo + uhi * d.b_hi;
+  C += ulo * d.c_lo + uhi * d.c_hi;
+  for (int b = 0; b < rt.nout; ++b)
+    if ((blockIdx.x >> b) & 1) {
+      A += rt.out_a[b];
+      C += rt.out_c[b];
+    }
+  const int t = threadIdx.x;
+  for (int e = t; e < K * N; e += TNT) {
+    const int k = e / N, n = e % N;
+    const float2 b = B[bit_offset(k, NK, d.bk) + bit_offset(n, NN, d.bn)];
+    Bs[e] = make_float4(b.x, b.y, b.y, b.x);
+  }
+  // pairs of A-adjacent elements: pair t + TNT j (7 bits of t, then j)
+  {
+    constexpr int NJ = TILE_ROWS * K / 2 / TNT;
+    int32_t so = 0, slot = 0;
+#pragma unroll
+    for (int b = 0; b < 7; ++b)
+      if ((t >> b) & 1) {
+        so += rt.a_src[1 + b];
+        slot ^= rt.a_slot[1 + b];
+      }
+    float2 v[NJ][2];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      int32_t o = so;
+#pragma unroll
+      for (int b = 0; b < NK; ++b)
+        if ((j >> b) & 1) o += rt.a_src[8 + b];
+      if (a_vec) {
+        const float4 x = __ldg(reinterpret_cast<const float4*>(A + o));
+        v[j][0] = make_float2(x.x, x.y);
+        v[j][1] = make_float2(x.z, x.w);
+      } else {
+        v[j][0] = __ldg(A + o);
+        v[j][1] = __ldg(A + o + 1);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      int32_t p = slot;
+#pragma unroll
+      for (int b = 0; b < NK; ++b)
+        if ((j >> b) & 1) p ^= rt.a_slot[8 + b];
+      block[p] = v[j][0];
+      block[p ^ rt.a_slot[0]] = v[j][1];
+    }
+  }
+  __syncthreads();
+  // rows t and t + TNT
+  f32x2 acc[2][N];
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int n = 0; n < N; ++n) acc[r][n] = 0ull;
+  int32_t row0 = 0;
+#pragma unroll
+  for (int b = 0; b < 7; ++b)
+    if ((t >> b) & 1) row0 ^= rt.a_row[b];
+  const int32_t row1 = row0 ^ rt.a_row[7];
+  auto step = [&](int k, float2 a0, float2 a1) {
+    const f32x2 re0 = pack2(a0.x, a0.x), im0 = pack2(-a0.y, a0.y), re1 = pack2(a1.x, a1.x), im1 = pack2(-a1.y, a1.y);
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+      const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&Bs[k * N + n]);
+      if (IM_FIRST) {
+        fma2(acc[0][n], im0, b.y);
+        fma2(acc[1][n], im1, b.y);
+        fma2(acc[0][n], re0, b.x);
+        fma2(acc[1][n], re1, b.x);
+      } else {
+        fma2(acc[0][n], re0, b.x);
+        fma2(acc[1][n], re1, b.x);
+        fma2(acc[0][n], im0, b.y);
+        fma2(acc[1][n], im1, b.y);
+      }
+    }
+  };
+  if constexpr (K >= 2) {
+#pragma unroll 4
+    for (int k = 0; k < K; k += 2) {
+      const float4 x = *reinterpret_cast<const float4*>(&block[row0 ^ k]);
+      const float4 y = *reinterpret_cast<const float4*>(&block[row1 ^ k]);
+      step(k, make_float2(x.x, x.y), make_float2(y.x, y.y));
+      step(k + 1, make_float2(x.z, x.w), make_float2(y.z, y.w));
+    }
+  } else {
+    step(0, block[row0], block[row1]);
+  }
+  __syncthreads();  // every row is read: the block now takes C
+  {
+    int32_t slot = 0;
+#pragma unroll
+    for (int b = 0; b < 7; ++b)
+      if ((t >> b) & 1) slot ^= rt.row_slot[b];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int n = 0; n < N; ++n) {
+        int32_t p = slot ^ (r ? rt.row_slot[7] : 0);
+#pragma unroll
+        for (int b = 0; b < NN; ++b)
+          if ((n >> b) & 1) p ^= rt.col_slot[b];
+        *reinterpret_cast<f32x2*>(&block[p]) = acc[r][n];
+      }
+  }
+  __syncthreads();
+  // pairs of C-adjacent elements, front to back
+  int32_t co = 0, cs = 0;
+#pragma unroll
+  for (int b = 0; b < 7; ++b)
+    if ((t >> b) & 1) {
+      co += rt.c_dst[1 + b];
+      cs ^= rt.c_slot[1 + b];
+    }
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    int32_t o = co, p = cs;
+#pragma unroll
+    for (int b = 0; b < NN; ++b)
+      if ((j >> b) & 1) {
+        o += rt.c_dst[8 + b];
+        p ^= rt.c_slot[8 + b];
+      }
+    const float4 x = *reinterpret_cast<const float4*>(&block[p]);
+    if (c_vec) {
+      *reinterpret_cast<float4*>(C + o) = x;
+    } else {
+      C[o] = make_float2(x.x, x.y);
+      C[o + 1] = make_float2(x.z, x.w);
+    }
+  }
+}
+
+// The tile's row indices: those among A's and among C's 2^4 fastest elements'
+// indices (at most eight together), then those among the 2^5 fastest, then C's
+// next fastest.
+RowTile row_tile(const GemmDesc& d) {
+  RowTile rt{};
+  bool in[kMaxBits] = {};
+  int count = 0;
+  auto take = [&](int i) {
+    if (!in[i] && count < TILE_BITS) {
+      in[i] = true;
+      ++count;
+    }
+  };
+  for (int reach = 4; reach <= 5; ++reach)
+    for (int i = 0; i < d.nm; ++i)
+      if (d.am[i] < (1 << reach) || d.cm[i] < (1 << reach)) take(i);
+  int order[kMaxBits];  // row indices by C stride
+  for (int i = 0; i < d.nm; ++i) {
+    int j = i;
+    for (; j > 0 && d.cm[order[j - 1]] > d.cm[i]; --j) order[j] = order[j - 1];
+    order[j] = i;
+  }
+  for (int i = 0; i < d.nm; ++i) take(order[i]);
+  // images: bits 0..3 of an index stand for themselves, the others are folded
+  // below
+  struct Bit { int32_t st; int bit; };
+  Bit a[TILE_BITS + 4], c[TILE_BITS + 4];
+  auto insert = [](Bit* v, int& n, Bit b) {
+    int j = n++;
+    for (; j > 0 && v[j - 1].st > b.st; --j) v[j] = v[j - 1];
+    v[j] = b;
+  };
+  int na = 0, nc = 0, row = 0;
+  for (int i = 0; i < d.nm; ++i) {
+    const int m = order[i];
+    if (in[m]) {
+      insert(a, na, {d.am[m], d.nk + row});
+      insert(c, nc, {d.cm[m], row});  // (tagged with the row or column bit)
+      ++row;
+    } else {
+      rt.out_a[rt.nout] = d.am[m];
+      rt.out_c[rt.nout++] = d.cm[m];
+    }
+  }
+  for (int l = 0; l < d.nk; ++l) insert(a, na, {d.ak[l], l});
+  for (int n = 0; n < d.nn; ++n) insert(c, nc, {d.cn[n], TILE_BITS + n});
+  int32_t img[TILE_BITS + 4];
+  bool fixed[TILE_BITS + 4];
+  auto reset = [&](int n) {
+    for (int b = 0; b < n; ++b) {
+      img[b] = 1 << b;
+      fixed[b] = b < 4;
+    }
+  };
+  // folds bit b onto bits 1..3 outside the span of the images' low four bits collected so far
+  unsigned span = 1;
+  auto add = [&](int v) {
+    unsigned s = span;
+    for (int x = 0; x < 16; ++x)
+      if ((span >> x) & 1) s |= 1u << (x ^ v);
+    span = s;
+  };
+  auto place = [&](int b) {
+    if (!fixed[b]) {
+      fixed[b] = true;
+      for (int v = 2; v < 16; v += 2)
+        if (!((span >> v) & 1)) {
+          img[b] ^= v;
+          break;
+        }
+    }
+    add(img[b] & 15);
+  };
+  // block of A: a quarter-warp's 16-byte reads vary the three lowest row bits;
+  // then a half-warp's 8-byte stores vary A's index bits 1..4
+  reset(na);
+  for (int b = d.nk; b < d.nk + 3; ++b)
+    if (fixed[b]) add(img[b] & 15);
+  for (int b = d.nk; b < d.nk + 3; ++b)
+    if (!fixed[b]) place(b);
+  span = 1;
+  for (int l = 1; l <= 4; ++l)
+    if (fixed[a[l].bit]) add(img[a[l].bit] & 15);
+  for (int l = 1; l <= 4; ++l)
+    if (!fixed[a[l].bit]) place(a[l].bit);
+  for (int i = 0; i < na; ++i) {
+    rt.a_src[i] = a[i].st;
+    rt.a_slot[i] = img[a[i].bit];
+  }
+  for (int b = 0; b < TILE_BITS; ++b) rt.a_row[b] = img[d.nk + b];
+  // block of C, indexed in C's order: its reads go front to back; a half-warp's
+  // stores vary the four lowest row bits
+  reset(nc);
+  span = 1;
+  int at[TILE_BITS + 4];  // row or column bit -> index bit
+  for (int i = 0; i < nc; ++i) at[c[i].bit] = i;
+  for (int b = 0; b < 4; ++b)
+    if (fixed[at[b]]) add(img[at[b]] & 15);
+  for (int b = 0; b < 4; ++b)
+    if (!fixed[at[b]]) place(at[b]);
+  for (int i = 0; i < nc; ++i) {
+    rt.c_dst[i] = c[i].st;
+    rt.c_slot[i] = img[i];
+    (c[i].bit < TILE_BITS ? rt.row_slot[c[i].bit] : rt.col_slot[c[i].bit - TILE_BITS]) = img[i];
+  }
+  return rt;
+}
+
+template <int NK>
+cudaError_t launch_tiles(const float2* A, const float2* B, float2* C, const GemmDesc& d, bool im_first,
+                         cudaStream_t s) {
+  const dim3 g(1u << (d.nm - TILE_BITS), (unsigned)d.units);
+  const RowTile rt = row_tile(d);
+  const int av = (reinterpret_cast<uintptr_t>(A) & 15) == 0 && (d.a_lo & 1) == 0 && (d.a_hi & 1) == 0;
+  const int cv = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && (d.c_lo & 1) == 0 && (d.c_hi & 1) == 0;
+  auto one = [&](auto nn) -> cudaError_t {
+    constexpr int NN = decltype(nn)::value;
+    if (im_first) vector_tile_kernel<NK, NN, true><<<g, TNT, 0, s>>>(A, B, C, d, rt, av, cv);
+    else vector_tile_kernel<NK, NN, false><<<g, TNT, 0, s>>>(A, B, C, d, rt, av, cv);
+    return cudaGetLastError();
+  };
+  switch (d.nn) {
+    case 0: return one(std::integral_constant<int, 0>{});
+    case 1: return one(std::integral_constant<int, 1>{});
+    case 2: return one(std::integral_constant<int, 2>{});
+    case 3: return one(std::integral_constant<int, 3>{});
+    default: return one(std::integral_constant<int, 4>{});
+  }
+}
+
 // The staged kernel applies when A's K values of a row are contiguous, every
 // copied 16-byte piece is aligned, and M >= 32.
 bool staged_ok(const float2* A, const GemmDesc& d) {
@@ -565,6 +875,19 @@ cudaError_t launch_wide(const float2* A, const float2* B, float2* C, const GemmD
   }
 }
 
+// Where the row-tile kernel beats a thread per row: launches of at least 2^19
+// rows (below that a call is latency, and the tile's two extra passes through
+// shared memory cost 1-3 us), N K >= 4 (a tile of 256 single values is too
+// little work), and not where A's rows are contiguous runs and C's columns few
+// (the staged kernel).  Measured per call, 2^22 rows, thread per row -> tile, log2
+// N, K: random orders (3, 4) 262 -> 208 us, (0, 4) 205 -> 128, (2, 2) 92 -> 64,
+// (4, 4) 365 -> 313, (4, 0) 118 -> 107; contracted indices innermost (4, 1) 351
+// -> 122, (4, 4) 430 -> 319, but (1, 3) 75 -> 80.
+bool tile_preferred(const float2* A, const GemmDesc& d) {
+  return d.nk <= 4 && d.nn <= 4 && d.nm >= TILE_BITS && d.nn + d.nk >= 2 &&
+         (int64_t(1) << d.nm) * d.units >= (int64_t(1) << 19) && !(d.nn <= 3 && staged_ok(A, d));
+}
+
 bool vector_sums_im_first(const float2* A, const GemmDesc& d) {
   return d.nn <= 4 && (d.nk > 4 || staged_ok(A, d));
 }
@@ -572,6 +895,16 @@ bool vector_sums_im_first(const float2* A, const GemmDesc& d) {
 cudaError_t launch_vector(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s,
                           const VecOut& maxbits) {
   if (!vector_shape_ok(d) || d.units > 65535) return cudaErrorInvalidValue;
+  if (maxbits.mode == 0 && !maxbits.maxbits && tile_preferred(A, d)) {
+    const bool f = vector_sums_im_first(A, d);
+    switch (d.nk) {
+      case 0: return launch_tiles<0>(A, B, C, d, f, s);
+      case 1: return launch_tiles<1>(A, B, C, d, f, s);
+      case 2: return launch_tiles<2>(A, B, C, d, f, s);
+      case 3: return launch_tiles<3>(A, B, C, d, f, s);
+      default: return launch_tiles<4>(A, B, C, d, f, s);
+    }
+  }
   const int cb = chunk_bits(d);
   if (d.nn == 5 && d.nk == 3) return launch_wide<3>(A, B, C, d, cb, s, maxbits);
   if (d.nn > 4) {  // K <= 2 (vector_shape_ok)
