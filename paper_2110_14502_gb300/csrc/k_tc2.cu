@@ -276,6 +276,17 @@ __device__ __forceinline__ void store_planes(uint16_t* P, int64_t plane, const i
   }
 }
 
+// x0 f and x1 f in one instruction (x as register bits).
+__device__ __forceinline__ void mul2(uint32_t x0, uint32_t x1, float f, float& y0, float& y1) {
+  asm("{\n .reg .b64 a, b;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %4};\n mul.rn.f32x2 a, a, b;\n mov.b64 {%0, %1}, a;\n}\n"
+      : "=f"(y0), "=f"(y1)
+      : "r"(x0), "r"(x1), "f"(f));
+}
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 __device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
 }
@@ -739,7 +750,7 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
     // folded tile holds `fold` hi units side by side, f = column / 2^nn, with A
     // shared and B, C of their own) and the output shift r that keeps the
     // predicted bound 2 K maxA maxB below 2^15.
-    float vmax = 0.f, fin[2] = {0.f, 0.f};
+    float vmax[2] = {0.f, 0.f};
     bool weak = false;
     int ea = 0, eb = 0, r = 0, scaled_unit = -1;
     Pow2 sc(0);
@@ -817,7 +828,7 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
         const int f = fold > 1 ? (c0 >> d.nn) : 0;
         if (c0 % gw < CS) {
           if (f > 0) unit_scale(ulo, uhi, f);
-          vmax = fin[0] = fin[1] = 0.f;
+          vmax[0] = vmax[1] = 0.f;
         }
         uint32_t ur[16], ui[16];
         tmem_ld<16>(R + (uint32_t)c0, ur);
@@ -835,9 +846,9 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
         float vr[16], vi[16];
         if (sc.direct) {
 #pragma unroll
-          for (int jj = 0; jj < 16; ++jj) {
-            vr[jj] = __uint_as_float(ur[jj]) * sc.f;
-            vi[jj] = __uint_as_float(ui[jj]) * sc.f;
+          for (int jj = 0; jj < 16; jj += 2) {
+            mul2(ur[jj], ur[jj + 1], sc.f, vr[jj], vr[jj + 1]);
+            mul2(ui[jj], ui[jj + 1], sc.f, vi[jj], vi[jj + 1]);
           }
         } else {
 #pragma unroll
@@ -849,14 +860,10 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
         if (planes) {
           uint16_t* const Pl = reinterpret_cast<uint16_t*>(C) + off;
           if (track) {
-            // 0 x is 0 for a finite x and NaN for an infinity or NaN, so `fin`
-            // stays 0 until a value turns non-finite
+            // (two chains; a NaN passes through to the maximum, so a unit whose
+            // values turned non-finite ends with an infinity or a NaN)
 #pragma unroll
-            for (int jj = 0; jj < 16; ++jj) {
-              vmax = fmaxf(vmax, fmaxf(fabsf(vr[jj]), fabsf(vi[jj])));
-              fin[0] = fmaf(vr[jj], 0.f, fin[0]);
-              fin[1] = fmaf(vi[jj], 0.f, fin[1]);
-            }
+            for (int jj = 0; jj < 16; ++jj) vmax[jj & 1] = max_nan(vmax[jj & 1], max_nan(fabsf(vr[jj]), fabsf(vi[jj])));
           }
           uint32_t x[NP / 2][16];
           auto pack = [&](bool fmt) {
@@ -934,8 +941,10 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
           // the unit's columns are done: its largest stored component,
           // exponent and filter flag (launch unit ulo + (uhi + f) units_lo)
           const int un = fold > 1 ? ulo + (uhi + f) * d.units_lo : unit;
-          const float wmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(vmax)));
-          const bool bad = __any_sync(0xffffffffu, planes && !(fin[0] + fin[1] == 0.f));
+          // (as unsigned bits NaN > infinity > any finite value)
+          const float wmax = __uint_as_float(
+              __reduce_max_sync(0xffffffffu, max(__float_as_uint(vmax[0]), __float_as_uint(vmax[1]))));
+          const bool bad = planes && !(wmax < __int_as_float(0x7f800000));
           if (lane == 0) {
             if (sio.mc && planes) atomicMax(sio.mc + un, __float_as_uint(wmax));
             if (sio.ec && planes && q == 0 && m0 == 0 && n0 == 0) sio.ec[un] = ea + eb + r;
