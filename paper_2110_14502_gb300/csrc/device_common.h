@@ -49,4 +49,45 @@ struct Pow2 {
   __device__ float operator()(float x) const { return direct ? x * f : ldexpf(x, e); }
 };
 
+// Exponent putting a maximum into [2^13, 2^14) (0 for none or a non-finite one).
+__device__ __forceinline__ int scale_exponent(float mx) {
+  if (!(mx > 0.f) || !isfinite(mx)) return 0;
+  int x;
+  frexpf(mx, &x);  // mx in [2^(x-1), 2^x)
+  return x - 14;
+}
+
+// Shared-memory slots of a 2^T-element tile that is written in one index order
+// and read in another.  order[l]: the read-order bit that is the l-th of the
+// write order.  The element with read-order index x sits at x with bits 4 and 5
+// folded onto bits 1 and 2 -- a thread reads 8 elements as four 16-byte loads,
+// lanes 64 bytes apart, and the fold spreads every quarter-warp over all banks
+// -- and with bits 6.. folded onto bits 1..3 where that makes the slots of a
+// half-warp's stores (write-order bits 1..4 vary) independent in the 16 banks.
+// slot[b]: what read-order bit b flips.
+template <int T>
+inline void turn_slots(const int* order, int32_t* slot) {
+  for (int b = 0; b < T; ++b) slot[b] = (1 << b) ^ (b == 4 ? 2 : b == 5 ? 4 : 0);
+  // span of the chosen lane bits' low four slot bits (bitmap of the 16 vectors)
+  unsigned span = 1;
+  auto add = [&](int v) {
+    unsigned s = span;
+    for (int x = 0; x < 16; ++x)
+      if ((span >> x) & 1) s |= 1u << (x ^ v);
+    span = s;
+  };
+  for (int l = 1; l <= 4; ++l)
+    if (order[l] < 6) add(slot[order[l]] & 15);
+  for (int l = 1; l <= 4; ++l) {
+    const int p = order[l];
+    if (p < 6) continue;
+    for (int v = 2; v < 16; v += 2)
+      if (!((span >> v) & 1)) {
+        slot[p] ^= v;
+        add(v);
+        break;
+      }
+  }
+}
+
 }  // namespace tn

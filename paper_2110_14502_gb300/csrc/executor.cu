@@ -293,16 +293,17 @@ void make_gemm_desc(const std::vector<int>& la, const std::vector<int>& lb, cons
 // fastest index of that group).  A GEMM tile takes the low bits of both, so its
 // elements then cover C's fastest indices whatever their order, and its stores
 // form long runs; values and their summation order do not change.
-void order_by_output(GemmDesc& d) {
-  auto sort2 = [](int n, int32_t* key, int32_t* other) {
+void order_by_output(GemmDesc& d, bool* marks) {
+  auto sort2 = [](int n, int32_t* key, int32_t* other, bool* mark) {
     for (int i = 1; i < n; ++i)
       for (int j = i; j > 0 && key[j - 1] > key[j]; --j) {
         std::swap(key[j - 1], key[j]);
         std::swap(other[j - 1], other[j]);
+        if (mark) std::swap(mark[j - 1], mark[j]);
       }
   };
-  sort2(d.nm, d.cm, d.am);
-  sort2(d.nn, d.cn, d.bn);
+  sort2(d.nm, d.cm, d.am, marks);
+  sort2(d.nn, d.cn, d.bn, nullptr);
 }
 
 // Leaf store of a plan: every leaf in complex64 at its store offset.

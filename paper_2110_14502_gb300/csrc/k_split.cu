@@ -23,13 +23,6 @@ namespace {
 
 constexpr int NT = 256;
 
-__device__ __forceinline__ uint16_t to16(float x, bool bf16) {
-  return bf16 ? __bfloat16_as_ushort(__float2bfloat16_rn(x)) : __half_as_ushort(__float2half_rn(x));
-}
-__device__ __forceinline__ float from16(uint16_t h, bool bf16) {
-  return bf16 ? __bfloat162float(__ushort_as_bfloat16(h)) : __half2float(__ushort_as_half(h));
-}
-
 // Largest |component| of each distinct tensor z (float bits, atomicMax).  The
 // operand is a dense block of 2^bits elements whatever its index order, so the
 // pass reads it front to back, 16 bytes per load.
@@ -73,39 +66,45 @@ __global__ void __launch_bounds__(NT) max_kernel(const float2* __restrict__ src,
   }
 }
 
-// Exponent putting the maximum into [2^13, 2^14).
-__device__ __forceinline__ int scale_exponent(float mx) {
-  if (!(mx > 0.f) || !isfinite(mx)) return 0;
-  int x;
-  frexpf(mx, &x);  // mx in [2^(x-1), 2^x)
-  return x - 14;
-}
-
-// Eight elements (scaled, consecutive in K order) as one 16-byte store per plane.
-template <int NP>
-__device__ __forceinline__ void store8(uint16_t* out, int64_t plane, const float2* v, const Pow2& sc, bool bf16) {
-  uint16_t h[NP][8];
+// Eight elements (consecutive in K order) as one 16-byte store per plane: x = hi
+// + lo, hi = rn16(x), lo = rn16(x - hi), or x rounded once.
+template <int NP, bool BF16>
+__device__ __forceinline__ void store8(uint16_t* out, int64_t plane, const float2* v) {
+  uint32_t hi[8], lo[8];  // re | im << 16
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    const float re = sc(v[j].x), im = sc(v[j].y);
-    if (NP == 4) {
-      h[0][j] = to16(re, bf16);
-      h[1][j] = to16(re - from16(h[0][j], bf16), bf16);
-      h[NP / 2][j] = to16(im, bf16);
-      h[NP / 2 + 1][j] = to16(im - from16(h[NP / 2][j], bf16), bf16);
+    if (BF16) {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(v[j].x, v[j].y);
+      hi[j] = *reinterpret_cast<const uint32_t*>(&h);
+      if (NP == 4) {
+        const float2 f = __bfloat1622float2(h);
+        const __nv_bfloat162 l = __floats2bfloat162_rn(v[j].x - f.x, v[j].y - f.y);
+        lo[j] = *reinterpret_cast<const uint32_t*>(&l);
+      }
     } else {
-      h[0][j] = to16(re, bf16);
-      h[1][j] = to16(im, bf16);
+      const __half2 h = __floats2half2_rn(v[j].x, v[j].y);
+      hi[j] = *reinterpret_cast<const uint32_t*>(&h);
+      if (NP == 4) {
+        const float2 f = __half22float2(h);
+        const __half2 l = __floats2half2_rn(v[j].x - f.x, v[j].y - f.y);
+        lo[j] = *reinterpret_cast<const uint32_t*>(&l);
+      }
     }
   }
-#pragma unroll
-  for (int p = 0; p < NP; ++p) {
-    uint4 w;
-    w.x = (uint32_t)h[p][0] | ((uint32_t)h[p][1] << 16);
-    w.y = (uint32_t)h[p][2] | ((uint32_t)h[p][3] << 16);
-    w.z = (uint32_t)h[p][4] | ((uint32_t)h[p][5] << 16);
-    w.w = (uint32_t)h[p][6] | ((uint32_t)h[p][7] << 16);
-    *reinterpret_cast<uint4*>(out + p * plane) = w;
+  auto put = [&](int p, const uint32_t* x, unsigned half) {
+    *reinterpret_cast<uint4*>(out + p * plane) =
+        make_uint4(__byte_perm(x[0], x[1], half), __byte_perm(x[2], x[3], half), __byte_perm(x[4], x[5], half),
+                   __byte_perm(x[6], x[7], half));
+  };
+  constexpr unsigned RE = 0x5410, IM = 0x7632;
+  if (NP == 4) {
+    put(0, hi, RE);
+    put(1, lo, RE);
+    put(2, hi, IM);
+    put(3, lo, IM);
+  } else {
+    put(0, hi, RE);
+    put(1, hi, IM);
   }
 }
 
@@ -131,10 +130,10 @@ struct TileMap {
   int8_t dst[12];
 };
 
-template <int NP, int T>
+template <int NP, int T, bool BF16>
 __global__ void __launch_bounds__(NT) split_kernel(const float2* __restrict__ src, uint16_t* __restrict__ dst,
                                                    const __grid_constant__ TileMap tm, int bits, int nlo, int64_t lo,
-                                                   int64_t hi, int vec, bool bf16, const unsigned* __restrict__ maxbits,
+                                                   int64_t hi, int vec, const unsigned* __restrict__ maxbits,
                                                    int* __restrict__ e_out, float* __restrict__ m_out) {
   constexpr int E = 1 << T;
   __shared__ __align__(16) float2 tile[E];
@@ -224,19 +223,21 @@ __global__ void __launch_bounds__(NT) split_kernel(const float2* __restrict__ sr
         v[2 * c] = make_float2(y.x, y.y);
         v[2 * c + 1] = make_float2(y.z, y.w);
       }
-      store8<NP>(out + o, plane, v, sc, bf16);
+      // (one multiply but for exponents out of a float's range)
+      if (sc.direct) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = make_float2(v[j].x * sc.f, v[j].y * sc.f);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = make_float2(sc(v[j].x), sc(v[j].y));
+      }
+      store8<NP, BF16>(out + o, plane, v);
     }
   }
 }
 
 // The tile of T bits for an operand whose output bit i (K bits, then row bits)
 // has input stride st[i], R bits in all.
-//
-// Slots: the element with output-order index x sits at x with bits 4 and 5
-// folded onto bits 1 and 2 -- a thread reads its 8 elements as four 16-byte
-// loads, lanes 64 bytes apart, and the fold spreads every quarter-warp over all
-// banks -- and with bits 6.. folded onto bits 1..3 where that makes the slots
-// of a half-warp's stores (input bits 1..4 vary) independent in the 16 banks.
 template <int T>
 TileMap split_tile_map(const SplitDesc& d) {
   TileMap m{};
@@ -273,27 +274,9 @@ TileMap split_tile_map(const SplitDesc& d) {
       for (; j > 0 && st[order[j - 1]] > st[i]; --j) order[j] = order[j - 1];
       order[j] = i;
     }
-  for (int b = 0; b < T; ++b) m.out_slot[b] = (1 << b) ^ (b == 4 ? 2 : b == 5 ? 4 : 0);
-  // span of the chosen lane bits' low four slot bits (bitmap of the 16 vectors)
-  unsigned span = 1;
-  auto add = [&](int v) {
-    unsigned s = span;
-    for (int x = 0; x < 16; ++x)
-      if ((span >> x) & 1) s |= 1u << (x ^ v);
-    span = s;
-  };
-  for (int l = 1; l <= 4; ++l)
-    if (pos[order[l]] < 6) add(m.out_slot[pos[order[l]]] & 15);
-  for (int l = 1; l <= 4; ++l) {
-    const int p = pos[order[l]];
-    if (p < 6) continue;
-    for (int v = 2; v < 16; v += 2)
-      if (!((span >> v) & 1)) {
-        m.out_slot[p] ^= v;
-        add(v);
-        break;
-      }
-  }
+  int tile_order[12];
+  for (int l = 0; l < T; ++l) tile_order[l] = pos[order[l]];
+  turn_slots<T>(tile_order, m.out_slot);
   for (int l = 0; l < T; ++l) {
     m.in_src[l] = st[order[l]];
     m.in_slot[l] = m.out_slot[pos[order[l]]];
@@ -305,8 +288,10 @@ template <int NP, int T>
 cudaError_t launch_tiles(const float2* src, uint16_t* dst, const SplitDesc& d, int nz, bool vec, bool bf16,
                          const unsigned* maxbits, int* e_out, float* m_out, cudaStream_t s) {
   const int R = d.nk + d.nrow;
-  split_kernel<NP, T><<<dim3(1u << (R - T), (unsigned)nz), NT, 0, s>>>(src, dst, split_tile_map<T>(d), R, d.nlo, d.lo,
-                                                                       d.hi, vec, bf16, maxbits, e_out, m_out);
+  const dim3 grid(1u << (R - T), (unsigned)nz);
+  const TileMap m = split_tile_map<T>(d);
+  if (bf16) split_kernel<NP, T, true><<<grid, NT, 0, s>>>(src, dst, m, R, d.nlo, d.lo, d.hi, vec, maxbits, e_out, m_out);
+  else split_kernel<NP, T, false><<<grid, NT, 0, s>>>(src, dst, m, R, d.nlo, d.lo, d.hi, vec, maxbits, e_out, m_out);
   return cudaGetLastError();
 }
 
@@ -322,6 +307,15 @@ cudaError_t launch_np(const float2* src, uint16_t* dst, const SplitDesc& d, int 
   return launch_tiles<NP, 7>(src, dst, d, nz, vec, bf16, maxbits, e_out, m_out, s);
 }
 
+cudaError_t launch_max(const float2* src, int bits, int nz, int nlo, int64_t lo, int64_t hi, bool vec, unsigned* maxbits,
+                       cudaStream_t s) {
+  // 8 loads of 16 bytes per thread where there is enough to fill the chip
+  const int64_t n = int64_t(1) << (bits - 1);
+  const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(n / (NT * 8), 152 * 8));
+  max_kernel<<<dim3((unsigned)blocks, (unsigned)nz), NT, 0, s>>>(src, bits, nlo, lo, hi, vec, maxbits);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_split(const float2* src, uint16_t* dst, const SplitDesc& d, int nz, bool bf16, int np,
@@ -330,11 +324,7 @@ cudaError_t launch_split(const float2* src, uint16_t* dst, const SplitDesc& d, i
   if (nz < 1 || nz > 65535 || R < 7 || R > 30 || (np != 2 && np != 4)) return cudaErrorInvalidValue;
   const bool vec = (reinterpret_cast<uintptr_t>(src) & 15) == 0 && (d.lo & 1) == 0 && (d.hi & 1) == 0;
   if (maxbits && !max_ready) {
-    // 8 loads of 16 bytes per thread where there is enough to fill the chip
-    const int64_t n = int64_t(1) << (R - 1);
-    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(n / (NT * 8), 152 * 8));
-    max_kernel<<<dim3((unsigned)blocks, (unsigned)nz), NT, 0, s>>>(src, R, d.nlo, d.lo, d.hi, vec, maxbits);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_max(src, R, nz, d.nlo, d.lo, d.hi, vec, maxbits, s);
     if (e != cudaSuccess) return e;
   }
   return np == 4 ? launch_np<4>(src, dst, d, nz, vec, bf16, maxbits, e_out, m_out, s)
@@ -408,9 +398,22 @@ bool planes_in_place(const float2* base, const GemmDesc& d, bool which_b, int np
   return true;
 }
 
-cudaError_t run_gemm_tc2(const float2* A, const float2* B, float2* C, const GemmDesc& d, bool bf16, uint16_t* scratch,
+int64_t tc2_pair_scratch_elems(const GemmDesc& d) {
+  return direct_ok(d) ? split_scratch_elems(d, true, 4) : tc2_scratch_elems(d);
+}
+
+cudaError_t run_gemm_tc2(const float2* A, const float2* B, float2* C, const GemmDesc& d0, bool bf16, uint16_t* scratch,
                          int* err, cudaStream_t s) {
   PlaneOperand pa, pb;
+  GemmDesc d = d0;
+  if (direct_ok(d)) {
+    order_for_direct(d);
+    const cudaError_t e = split_operand(B, d, true, bf16, 4, false, nullptr, nullptr, nullptr, scratch, pb, s);
+    return e != cudaSuccess ? e : launch_gemm_direct(A, pb, C, d, bf16, nullptr, nullptr, err, s);
+  }
+  // the split pass reads any order of rows at the same speed, so they follow C
+  // (random orders, scaled bf16 (14, 14, 5): 2040 -> 832 us per call)
+  order_by_output(d);
   cudaError_t e = split_operand(A, d, false, bf16, 4, false, nullptr, nullptr, nullptr, scratch, pa, s);
   if (e != cudaSuccess) return e;
   e = split_operand(B, d, true, bf16, 4, false, nullptr, nullptr, nullptr, scratch + split_scratch_elems(d, false, 4),
@@ -420,14 +423,23 @@ cudaError_t run_gemm_tc2(const float2* A, const float2* B, float2* C, const Gemm
   return launch_gemm_tma(pa, pb, C, false, d, bf16, none, err, s);
 }
 
-cudaError_t run_gemm_tc2_scaled(const float2* A, const float2* B, float2* C, const GemmDesc& d, bool bf16, int np,
+cudaError_t run_gemm_tc2_scaled(const float2* A, const float2* B, float2* C, const GemmDesc& d0, bool bf16, int np,
                                 uint16_t* scratch, void* aux, int* err, cudaStream_t s) {
   unsigned* mx = reinterpret_cast<unsigned*>(aux);
   int* ex = reinterpret_cast<int*>(mx + 2);
   float* ms = reinterpret_cast<float*>(ex + 2);
+  GemmDesc d = d0;
   cudaError_t e = cudaMemsetAsync(mx, 0, 2 * sizeof(unsigned), s);
+  if (e != cudaSuccess) return e;
   PlaneOperand pa, pb;
-  if (e == cudaSuccess) e = split_operand(A, d, false, bf16, np, true, mx, ex, ms, scratch, pa, s);
+  if (direct_ok(d)) {
+    order_for_direct(d);
+    e = launch_max(A, d.nm + d.nk, 1, 1, 0, 0, (reinterpret_cast<uintptr_t>(A) & 15) == 0, mx, s);
+    if (e == cudaSuccess) e = split_operand(B, d, true, bf16, np, true, mx + 1, ex + 1, ms + 1, scratch, pb, s);
+    return e != cudaSuccess ? e : launch_gemm_direct(A, pb, C, d, bf16, mx, ex + 1, err, s);
+  }
+  order_by_output(d);
+  e = split_operand(A, d, false, bf16, np, true, mx, ex, ms, scratch, pa, s);
   if (e == cudaSuccess)
     e = split_operand(B, d, true, bf16, np, true, mx + 1, ex + 1, ms + 1,
                       scratch + split_scratch_elems(d, false, np), pb, s);

@@ -161,6 +161,43 @@ __device__ __forceinline__ void mma(uint32_t d, uint32_t a_lo, uint32_t b_lo, ui
       "r"(a_lo), "n"(OperandDesc<ROWB, TM>::HI), "r"(b_lo), "n"(OperandDesc<ROWB, TN>::HI), "r"(idesc), "r"(acc));
 }
 
+// The MMAs of one 16-K step: Dr (at dr) and Di (at di) += A B from the stage's
+// planes, a and b0 their descriptors' low words; `acc` 0 starts the sums.
+template <int NP, int TN, int ROWB>
+__device__ __forceinline__ void mma_step(uint32_t dr, uint32_t di, uint32_t a, uint32_t b0, int kk, uint32_t I,
+                                         uint32_t IN, uint32_t acc) {
+  using CF = Cfg2<TN, NP, ROWB>;
+  uint32_t A_[NP], B_[NP];
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    A_[p] = a + ((p * CF::A_PLANE + kk * 32) >> 4);
+    B_[p] = b0 + ((p * CF::B_PLANE + kk * 32) >> 4);
+  }
+  auto mm = [&](uint32_t dst, int pa, int pb, uint32_t id, uint32_t ac) { mma<ROWB, TN>(dst, A_[pa], B_[pb], id, ac); };
+  if constexpr (NP == 4) {
+    // planes: 0 re_hi, 1 re_lo, 2 im_hi, 3 im_lo; the chunk is short, so the
+    // hi*lo + lo*hi terms share the hi*hi accumulator
+    mm(dr, 0, 0, I, acc);
+    mm(dr, 0, 1, I, 1u);
+    mm(dr, 1, 0, I, 1u);
+    mm(dr, 2, 2, IN, 1u);
+    mm(dr, 2, 3, IN, 1u);
+    mm(dr, 3, 2, IN, 1u);
+    mm(di, 0, 2, I, acc);
+    mm(di, 0, 3, I, 1u);
+    mm(di, 1, 2, I, 1u);
+    mm(di, 2, 0, I, 1u);
+    mm(di, 2, 1, I, 1u);
+    mm(di, 3, 0, I, 1u);
+  } else {
+    // planes: 0 re, 1 im
+    mm(dr, 0, 0, I, acc);
+    mm(dr, 1, 1, IN, 1u);
+    mm(di, 0, 1, I, acc);
+    mm(di, 1, 0, I, 1u);
+  }
+}
+
 // One lane of the (converged) warp.  The compiler knows that a single thread
 // runs what this guards and keeps the operands of TMA and MMA instructions in
 // uniform registers; under `lane == 0` it cannot, and issuing an MMA took about
@@ -641,38 +678,7 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
             const uint32_t b0 = smem0 + (uint32_t)s * (CF::STAGE >> 4) + (CF::A_STAGE >> 4) + OperandDesc<ROWB, TN>::LO;
 #pragma unroll
             for (int kk = 0; kk < CF::KSTEPS; ++kk) {
-              uint32_t A_[NP], B_[NP];
-#pragma unroll
-              for (int p = 0; p < NP; ++p) {
-                A_[p] = a + ((p * CF::A_PLANE + kk * 32) >> 4);
-                B_[p] = b0 + ((p * CF::B_PLANE + kk * 32) >> 4);
-              }
-              const uint32_t acc = (kt > k0 || kk) ? 1u : 0u;
-              auto mm = [&](uint32_t dst, int pa, int pb, uint32_t id, uint32_t ac) {
-                mma<ROWB, TN>(dst, A_[pa], B_[pb], id, ac);
-              };
-              if constexpr (NP == 4) {
-                // planes: 0 re_hi, 1 re_lo, 2 im_hi, 3 im_lo; the chunk is short,
-                // so the hi*lo + lo*hi terms share the hi*hi accumulator
-                mm(dr, 0, 0, I, acc);
-                mm(dr, 0, 1, I, 1u);
-                mm(dr, 1, 0, I, 1u);
-                mm(dr, 2, 2, IN, 1u);
-                mm(dr, 2, 3, IN, 1u);
-                mm(dr, 3, 2, IN, 1u);
-                mm(di, 0, 2, I, acc);
-                mm(di, 0, 3, I, 1u);
-                mm(di, 1, 2, I, 1u);
-                mm(di, 2, 0, I, 1u);
-                mm(di, 2, 1, I, 1u);
-                mm(di, 3, 0, I, 1u);
-              } else {
-                // planes: 0 re, 1 im
-                mm(dr, 0, 0, I, acc);
-                mm(dr, 1, 1, IN, 1u);
-                mm(di, 0, 1, I, acc);
-                mm(di, 1, 0, I, 1u);
-              }
+              mma_step<NP, TN, ROWB>(dr, di, a, b0, kk, I, IN, (kt > k0 || kk) ? 1u : 0u);
             }
             commit(&empty[s]);
           }
@@ -962,6 +968,431 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
   }
 }
 
+// The same GEMM with A read as complex64 (one unit, N <= 64: one column tile,
+// so A is needed once).  Writing A's planes first and reading them back would
+// move three times its bytes, and here A is nearly all the bytes.  So the eight
+// epilogue warps also prepare A's stages: they load the 128 x 32 tile front to
+// back in A's own order (the tile holds A's fastest indices, order_for_direct),
+// turn it in shared memory, convert it as the split pass does and write the
+// swizzled plane rows, with two stages' loads in flight in registers.  Warp 0
+// copies B's planes by TMA, warp 1 issues the MMAs.
+//
+// TMEM holds the running sum R (buffer 0) and two partial buffers, so the chunk
+// of K that the workers are converting never waits for the previous chunk's
+// fold, which they do after it.  The workers decide together, at each stage's
+// barrier, whether one of them gave up a wait.
+constexpr int DTK = 32;                         // complex K per stage
+constexpr int RAW_BYTES = TM * DTK * 8;         // a stage's tile as complex64
+template <int TN, int NP>
+struct DirectCfg {
+  using CF = Cfg2<TN, NP, 64>;
+  static constexpr int THREADS = 128 + 256;
+  static constexpr int BUDGET = 227 * 1024 - 2 * RAW_BYTES - 1024 - 2048;
+  static constexpr int NS = (BUDGET / CF::STAGE) < 4 ? (BUDGET / CF::STAGE) : 4;
+  static constexpr int SMEM = NS * CF::STAGE + 2 * RAW_BYTES + 1024;
+  static constexpr uint32_t BUF = 2 * TN;       // TMEM columns of one buffer
+  static constexpr uint32_t COLS = TN == 64 ? 512 : TN == 32 ? 256 : 128;
+  static_assert(NS >= 2 && 3 * BUF <= COLS, "two stages, three accumulator buffers");
+  static_assert(8 * STAGE_SLOTS * 8 <= 2 * RAW_BYTES, "the output staging reuses the raw tiles");
+};
+
+// The tile's index bits (K bits 0..4, then row bits 0..6 of the descriptor) in
+// A's order: stride and shared slot; and the slots in tile order.
+struct DirectMap {
+  int32_t in_src[12], in_slot[12], out_slot[12];
+};
+
+__device__ __forceinline__ bool workers_any(bool failed) {  // barrier of the 256 workers
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.or.pred q, 1, 256, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)failed)
+      : "memory");
+  return r != 0;
+}
+
+template <int TN, int NP, bool BF16>
+__global__ void __launch_bounds__(DirectCfg<TN, NP>::THREADS, 1)
+    gemm_direct(const __grid_constant__ CUtensorMap mapB, const float2* __restrict__ A, float2* __restrict__ C,
+                const GemmDesc d, const __grid_constant__ DirectMap dm, const unsigned* __restrict__ maxA,
+                const int* __restrict__ exp_b, int a_vec, int out_wide, int chunk, int* __restrict__ err) {
+  using DC = DirectCfg<TN, NP>;
+  using CF = typename DC::CF;
+  constexpr int NS = DC::NS;
+  constexpr uint32_t BUF = DC::BUF;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  float2* const raw = reinterpret_cast<float2*>(smem + NS * CF::STAGE);  // [2][4096]
+  __shared__ uint64_t full_a[NS], full_b[NS], empty[NS], acc_full[3], acc_empty[3], mma_done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int abort_flag;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const long long wl = g_wait_limit;
+  const int items = 1 << (d.nm - 7), first = blockIdx.x, stride = gridDim.x;
+  const int nkt = 1 << (d.nk - 5);
+  const int nch = (nkt + chunk - 1) / chunk;
+
+  if (tid == 0) {
+    for (int s = 0; s < NS; ++s) {
+      mbar_init(&full_a[s], 8);
+      mbar_init(&full_b[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int b = 0; b < 3; ++b) {
+      mbar_init(&acc_full[b], 1);
+      mbar_init(&acc_empty[b], 8);
+    }
+    mbar_init(&mma_done, 1);
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapB)) : "memory");
+  }
+  if (warp == 2) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"(DC::COLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_slot;
+
+  if (warp == 0) {
+    // ---- B's stages
+    const bool leader = elect_one();
+    int64_t g = 0;
+    int s = 0;
+    uint32_t lap = 0;
+    bool ok = true;
+    for (int it = first; ok && it < items; it += stride) {
+      if (__any_sync(0xffffffffu, abort_flag)) break;
+      for (int kt = 0; kt < nkt; ++kt, ++g) {
+        if (lap > 0 && !mbar_wait_warp(&empty[s], (lap - 1) & 1, wl)) {
+          if (leader) {
+            atomicExch(err, 41);
+            abort_flag = 1;
+          }
+          ok = false;
+          break;
+        }
+        if (leader) {
+          mbar_expect_tx(&full_b[s], NP * CF::B_PLANE);
+          tma_load_5d(smem + s * CF::STAGE + CF::A_STAGE, &mapB, &full_b[s], kt * DTK, 0, 0, 0, 0);
+        }
+        if (++s == NS) {
+          s = 0;
+          ++lap;
+        }
+      }
+    }
+    if (leader) drain_loads(full_b, NS, g, err);
+    __syncwarp();
+  } else if (warp == 1) {
+    // ---- MMA issuer: chunk 0 of a tile into buffer 0, later ones into 1 and 2 in turn
+    const bool leader = elect_one();
+    constexpr uint32_t I = idesc2(BF16, TM, TN, false), IN = idesc2(BF16, TM, TN, true);
+    const uint32_t smem0 = smem_u32(smem) >> 4;
+    int64_t g = 0;
+    int s = 0;
+    uint32_t ph = 0;
+    uint32_t used[3] = {0u, 0u, 0u};
+    bool ok = true;
+    for (int it = first; ok && it < items; it += stride) {
+      if (__any_sync(0xffffffffu, abort_flag)) break;
+      for (int c = 0; c < nch && ok; ++c) {
+        const int b = c == 0 ? 0 : 1 + ((c - 1) & 1);
+        if (used[b] >= 1 && !mbar_wait_warp(&acc_empty[b], (used[b] - 1) & 1, wl)) {
+          if (leader) {
+            atomicExch(err, 42);
+            abort_flag = 1;
+          }
+          ok = false;
+          break;
+        }
+        ++used[b];
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t dr = tmem + (uint32_t)b * BUF, di = dr + TN;
+        const int k0 = c * chunk, k1 = min(nkt, k0 + chunk);
+        for (int kt = k0; kt < k1; ++kt, ++g) {
+          if (!mbar_wait_warp(&full_b[s], ph, wl) || !mbar_wait_warp(&full_a[s], ph, wl)) {
+            if (leader) {
+              atomicExch(err, 43);
+              abort_flag = 1;
+            }
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          if (leader) {
+            const uint32_t a = smem0 + (uint32_t)s * (CF::STAGE >> 4) + OperandDesc<64, TM>::LO;
+            const uint32_t b0 = smem0 + (uint32_t)s * (CF::STAGE >> 4) + (CF::A_STAGE >> 4) + OperandDesc<64, TN>::LO;
+#pragma unroll
+            for (int kk = 0; kk < CF::KSTEPS; ++kk)
+              mma_step<NP, TN, 64>(dr, di, a, b0, kk, I, IN, (kt > k0 || kk) ? 1u : 0u);
+            commit(&empty[s]);
+          }
+          __syncwarp();
+          if (++s == NS) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+        if (leader) commit(&acc_full[b]);
+        __syncwarp();
+      }
+    }
+    if (leader && g > 0) {
+      commit(&mma_done);
+      if (!mbar_wait(&mma_done, 0, kDrainLimit)) atomicExch(err, 46);
+    }
+    __syncwarp();
+  } else if (warp >= 4) {
+    // ---- workers
+    const int t = tid - 128, w = warp - 4, q = warp & 3, h = w >> 2;
+    int ea = 0;
+    if (maxA) ea = scale_exponent(__uint_as_float(*maxA));
+    const Pow2 sa(-ea), sc(ea + (exp_b ? *exp_b : 0));
+    // loads: pairs t + 256 j of A-adjacent elements; A's order bits 1..8 from t, 9..11 from j
+    int32_t so = 0, slot = 0;
+#pragma unroll
+    for (int b = 0; b < 8; ++b)
+      if ((t >> b) & 1) {
+        so += dm.in_src[1 + b];
+        slot ^= dm.in_slot[1 + b];
+      }
+    const int32_t my_am = lane >= 7 && lane < d.nm ? d.am[lane] : 0;
+    const int32_t my_ak = lane >= 5 && lane < d.nk ? d.ak[lane] : 0;
+    auto bit_sum = [&](int x, int32_t st) {
+      return (int32_t)__reduce_add_sync(0xffffffffu, (uint32_t)(((x >> lane) & 1) ? st : 0));
+    };
+    // two stages' loads in flight: one stage ahead left an SM waiting for their
+    // latency, 2 us per 32 KB stage
+    float4 pf0[8], pf1[8];
+    auto load = [&](float4(&pf)[8], int it, int kt) {
+      const float2* src = A + so + bit_sum(it << 7, my_am) + bit_sum(kt << 5, my_ak);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float2* p = src + ((j & 1) ? dm.in_src[9] : 0) + ((j & 2) ? dm.in_src[10] : 0) + ((j & 4) ? dm.in_src[11] : 0);
+        if (a_vec) {
+          pf[j] = __ldg(reinterpret_cast<const float4*>(p));
+        } else {
+          const float2 x = __ldg(p), y = __ldg(p + 1);
+          pf[j] = make_float4(x.x, x.y, y.x, y.y);
+        }
+      }
+    };
+    // conversions: K octets t and t + 256 of the tile: octet o = row o / 4, K chunk o % 4
+    int32_t oslot[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      oslot[u] = 0;
+#pragma unroll
+      for (int b = 0; b < 9; ++b)
+        if (((t + 256 * u) >> b) & 1) oslot[u] ^= dm.out_slot[3 + b];
+    }
+    const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
+    uint32_t seen[3] = {0u, 0u, 0u};
+    bool failed = false, stop = false;
+    auto wait_acc = [&](int b) {
+      if (!mbar_wait_warp(&acc_full[b], seen[b] & 1, wl)) {
+        failed = true;
+        if (lane == 0) {
+          atomicExch(err, 44);
+          abort_flag = 1;
+        }
+      }
+      ++seen[b];
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    };
+    auto release = [&](int b) {
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[b])) : "memory");
+    };
+    auto fold = [&](int c) {
+      const int b = 1 + ((c - 1) & 1);
+      if (c == 1) wait_acc(0);
+      wait_acc(b);
+      if (failed) return;
+      const uint32_t R = tq, P = tq + (uint32_t)b * BUF;
+#pragma unroll 1
+      for (int c0 = 16 * h; c0 < TN; c0 += 32) {
+        uint32_t pr[16], pi[16], rr[16], ri[16];
+        tmem_ld<16>(P + (uint32_t)c0, pr);
+        tmem_ld<16>(P + (uint32_t)(TN + c0), pi);
+        tmem_ld<16>(R + (uint32_t)c0, rr);
+        tmem_ld<16>(R + (uint32_t)(TN + c0), ri);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int jj = 0; jj < 16; ++jj) {
+          rr[jj] = __float_as_uint(__uint_as_float(rr[jj]) + __uint_as_float(pr[jj]));
+          ri[jj] = __float_as_uint(__uint_as_float(ri[jj]) + __uint_as_float(pi[jj]));
+        }
+        tmem_st16(R + (uint32_t)c0, rr);
+        tmem_st16(R + (uint32_t)(TN + c0), ri);
+      }
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      release(b);
+    };
+    int s = 0;
+    uint32_t lap = 0;
+    int64_t g = 0;
+    // the load position: two stages past the one being converted
+    int lit = first, lkt = 0;
+    auto load_next = [&](float4(&pf)[8]) {
+      if (lit >= items) return;
+      load(pf, lit, lkt);
+      if (++lkt == nkt) {
+        lkt = 0;
+        lit += stride;
+      }
+    };
+    load_next(pf0);
+    load_next(pf1);
+    for (int it = first; !stop && it < items; it += stride) {
+      for (int c = 0; c < nch && !stop; ++c) {
+        const int k1 = min(nkt, (c + 1) * chunk);
+        for (int kt = c * chunk; kt < k1; ++kt, ++g) {
+          float2* const tile = raw + (g & 1) * (TM * DTK);
+          auto land = [&](float4(&pf)[8]) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const int32_t p = slot ^ ((j & 1) ? dm.in_slot[9] : 0) ^ ((j & 2) ? dm.in_slot[10] : 0) ^
+                                ((j & 4) ? dm.in_slot[11] : 0);
+              tile[p] = make_float2(pf[j].x, pf[j].y);
+              tile[p ^ dm.in_slot[0]] = make_float2(pf[j].z, pf[j].w);
+            }
+            load_next(pf);
+          };
+          if (g & 1) land(pf1);
+          else land(pf0);
+          if (lap > 0 && !failed && !mbar_wait_warp(&empty[s], (lap - 1) & 1, wl)) {
+            failed = true;
+            if (lane == 0) {
+              atomicExch(err, 45);
+              abort_flag = 1;
+            }
+          }
+          // the tile is complete and its stage free; or everyone stops
+          if (workers_any(failed)) {
+            stop = true;
+            break;
+          }
+          uint8_t* const st = smem + s * CF::STAGE;
+          // (the shift is a single multiply but for exponents out of range)
+          auto convert = [&](auto scale4) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const int o = t + 256 * u, row = o >> 2;
+              uint32_t x[NP / 2][8];
+#pragma unroll
+              for (int v = 0; v < 4; ++v) {
+                const float4 y = scale4(sa, *reinterpret_cast<const float4*>(&tile[oslot[u] ^ (2 * v)]));
+                uint32_t e0[NP / 2], e1[NP / 2];
+                pack_planes<NP>(BF16, y.x, y.y, e0);
+                pack_planes<NP>(BF16, y.z, y.w, e1);
+#pragma unroll
+                for (int a = 0; a < NP / 2; ++a) {
+                  x[a][2 * v] = e0[a];
+                  x[a][2 * v + 1] = e1[a];
+                }
+              }
+              // 64-byte rows, 16-byte chunks swizzled by row bits 1, 2
+              uint8_t* const to = st + row * 64 + (((o & 3) ^ ((row >> 1) & 3)) << 4);
+#pragma unroll
+              for (int p = 0; p < NP; ++p) {
+                auto pp = [&](int e) { return __byte_perm(x[p >> 1][e], x[p >> 1][e + 1], (p & 1) ? 0x7632 : 0x5410); };
+                *reinterpret_cast<uint4*>(to + p * CF::A_PLANE) = make_uint4(pp(0), pp(2), pp(4), pp(6));
+              }
+            }
+          };
+          if (sa.direct)
+            convert([](const Pow2& m, float4 y) { return make_float4(y.x * m.f, y.y * m.f, y.z * m.f, y.w * m.f); });
+          else
+            convert([](const Pow2& m, float4 y) { return make_float4(m(y.x), m(y.y), m(y.z), m(y.w)); });
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the tensor core's reads
+          __syncwarp();
+          if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full_a[s])) : "memory");
+          if (++s == NS) {
+            s = 0;
+            ++lap;
+          }
+        }
+        if (!stop && c >= 2) fold(c - 1);
+      }
+      if (stop) break;
+      if (nch >= 2) fold(nch - 1);
+      else wait_acc(0);
+      // every worker is done with the raw tiles, whose memory now stages the output
+      if (workers_any(failed)) break;
+      // output addressing, as in gemm_tma_chunked (set up per tile: it would hold
+      // registers that the loads need)
+      const StageMap sm = stage_map(d, lane, false, out_wide != 0);
+      const uint32_t slots = smem_u32(raw) + w * STAGE_SLOTS * 8;
+      uint32_t cslot[4];
+      for (int b = 0; b < 4; ++b) cslot[b] = (uint32_t)stage_slot(1 << sm.rank_c[b]) * 8;
+      const uint32_t lslot = slots + (uint32_t)stage_slot(sm.lane_idx) * 8;
+      const uint32_t rd = slots + (uint32_t)stage_slot(2 * lane) * 8;
+      const int32_t lane_row = bit_offset(lane, 5, d.cm);
+      const int32_t cn_lo[4] = {d.cn[0], d.cn[1], d.cn[2], d.cn[3]};
+      const int32_t cn_mid[2] = {d.nn > 4 ? d.cn[4] : 0, d.nn > 5 ? d.cn[5] : 0};
+      const int32_t my_cm = lane >= 5 && lane < d.nm ? d.cm[lane] : 0;
+      const int32_t tile_off = bit_sum((it << 7) + q * 32, my_cm);
+#pragma unroll 1
+      for (int c0 = 16 * h; c0 < TN; c0 += 32) {
+        uint32_t ur[16], ui[16];
+        tmem_ld<16>(tq + (uint32_t)c0, ur);
+        tmem_ld<16>(tq + (uint32_t)(TN + c0), ui);
+        float2* const Co = C + (tile_off + ((c0 & 16) ? cn_mid[0] : 0) + ((c0 & 32) ? cn_mid[1] : 0));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        float vr[16], vi[16];
+        if (sc.direct) {
+#pragma unroll
+          for (int jj = 0; jj < 16; jj += 2) {
+            mul2(ur[jj], ur[jj + 1], sc.f, vr[jj], vr[jj + 1]);
+            mul2(ui[jj], ui[jj + 1], sc.f, vi[jj], vi[jj + 1]);
+          }
+        } else {
+#pragma unroll
+          for (int jj = 0; jj < 16; ++jj) {
+            vr[jj] = sc(__uint_as_float(ur[jj]));
+            vi[jj] = sc(__uint_as_float(ui[jj]));
+          }
+        }
+        if (sm.on) {
+#pragma unroll
+          for (int jj = 0; jj < 16; ++jj)
+            sts64(lslot + ((jj & 1) ? cslot[0] : 0) + ((jj & 2) ? cslot[1] : 0) + ((jj & 4) ? cslot[2] : 0) +
+                      ((jj & 8) ? cslot[3] : 0),
+                  __float_as_uint(vr[jj]), __float_as_uint(vi[jj]));
+          __syncwarp();
+          uint4 y[8];
+#pragma unroll
+          for (int t2 = 0; t2 < 8; ++t2) y[t2] = lds128(rd + t2 * (64 + 8) * 8);
+#pragma unroll
+          for (int t2 = 0; t2 < 8; ++t2)
+            *reinterpret_cast<uint4*>(Co + sm.off_c64 + ((t2 & 1) ? sm.step_c64[0] : 0) +
+                                      ((t2 & 2) ? sm.step_c64[1] : 0) + ((t2 & 4) ? sm.step_c64[2] : 0)) = y[t2];
+          __syncwarp();
+        } else {
+#pragma unroll
+          for (int jj = 0; jj < 16; ++jj) Co[lane_row + col_offset(cn_lo, jj)] = make_float2(vr[jj], vi[jj]);
+        }
+      }
+      release(0);
+      if (workers_any(failed)) break;  // the raw tiles' memory is free again
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 2) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(DC::COLS));
+  }
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   static std::once_flag once;
@@ -978,18 +1409,18 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 // 5-D map over one operand's planes: [hi unit][lo unit][plane][row][k] of
 // 16-bit values; box = row_bytes / 2 k x box_rows x box_planes x 1 x 1
-// (box_planes 0: all np planes).  A plane row holds K >= 8 values (16 bytes or
+// (box_planes 0: all np planes; row > 0: rows of that many bytes).  A plane row holds K >= 8 values (16 bytes or
 // more); when K = 8 the box reaches past it and the copy fills those K positions with
 // zeros (the other operand's are zero as well, so the products vanish), and
 // the stage still receives the box's full byte count.
-bool encode_planes(CUtensorMap* map, const PlaneOperand& o, int box_rows, int box_planes = 0) {
+bool encode_planes(CUtensorMap* map, const PlaneOperand& o, int box_rows, int box_planes = 0, int row = 0) {
   auto fn = encode_fn();
   if (!fn) return false;
   const int64_t set = (int64_t)o.np * o.rows * o.kp * 2;  // bytes of one plane set
   cuuint64_t dims[5] = {(cuuint64_t)o.kp, (cuuint64_t)o.rows, (cuuint64_t)o.np, (cuuint64_t)o.nlo, (cuuint64_t)o.nhi};
   cuuint64_t strides[4] = {(cuuint64_t)(o.kp * 2), (cuuint64_t)(o.rows * o.kp * 2),
                            (cuuint64_t)(o.nlo > 1 ? o.st_lo : set), (cuuint64_t)(o.nhi > 1 ? o.st_hi : set)};
-  const int rowb = row_bytes(o.kp, o.np);
+  const int rowb = row > 0 ? row : row_bytes(o.kp, o.np);
   cuuint32_t box[5] = {(cuuint32_t)(rowb / 2), (cuuint32_t)box_rows, (cuuint32_t)(box_planes > 0 ? box_planes : o.np), 1, 1};
   cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT16, 5, const_cast<uint16_t*>(o.base), dims, strides, box, estr,
@@ -1070,6 +1501,44 @@ cudaError_t launch_tn(int TNv, const CUtensorMap& ma, const CUtensorMap& mb, flo
   }
 }
 
+DirectMap direct_map(const GemmDesc& d) {
+  DirectMap m{};
+  int32_t st[12];
+  for (int b = 0; b < 12; ++b) st[b] = b < 5 ? d.ak[b] : d.am[b - 5];
+  int order[12];  // tile bits by A stride
+  for (int i = 0; i < 12; ++i) {
+    int j = i;
+    for (; j > 0 && st[order[j - 1]] > st[i]; --j) order[j] = order[j - 1];
+    order[j] = i;
+  }
+  turn_slots<12>(order, m.out_slot);
+  for (int l = 0; l < 12; ++l) {
+    m.in_src[l] = st[order[l]];
+    m.in_slot[l] = m.out_slot[order[l]];
+  }
+  return m;
+}
+
+template <int TN, int NP, bool BF16>
+cudaError_t launch_direct_as(const CUtensorMap& mb, const float2* A, float2* C, const GemmDesc& d, const unsigned* maxA,
+                             const int* exp_b, int* err, cudaStream_t s) {
+  using DC = DirectCfg<TN, NP>;
+  static bool attr = false;
+  static int sms = 0;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(gemm_direct<TN, NP, BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, DC::SMEM);
+    if (e != cudaSuccess) return e;
+    sms = sm_count();
+    attr = true;
+  }
+  const unsigned grid = (unsigned)std::min<int64_t>(int64_t(1) << (d.nm - 7), sms);
+  const int chunk = NP == 4 ? split_chunk() : 1 << 30;
+  gemm_direct<TN, NP, BF16><<<grid, DC::THREADS, DC::SMEM, s>>>(mb, A, C, d, direct_map(d), maxA, exp_b,
+                                                         (reinterpret_cast<uintptr_t>(A) & 15) == 0,
+                                                         (reinterpret_cast<uintptr_t>(C) & 15) == 0, chunk, err);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t set_tc_wait_limit(long long polls) {
@@ -1148,6 +1617,68 @@ cudaError_t launch_gemm_tma(const PlaneOperand& a, const PlaneOperand& b, float2
   if (kpi != 8 || !aligned(qa) || !aligned(qb)) qa = qb = BulkPlanes{};
   return a.np == 4 ? launch_tn<4>(TNv, ma, mb, C, d, kpi, z, cp, sio, fold, bf16, err, s, qa, qb)
                    : launch_tn<2>(TNv, ma, mb, C, d, kpi, z, cp, sio, fold, bf16, err, s, qa, qb);
+}
+
+// Where converting A in the GEMM beats a split pass: enough row tiles to fill
+// the chip most of the time, and a K long enough that a tile's output, which
+// the same warps store, is a small part of it.  Measured per call with random
+// orders, split pass -> here: (16, 6, 13) split fp16 2675 -> 2227 us, (17, 6, 9)
+// split bf16 307 -> 251, (14, 6, 12) split fp16 391 -> 329, (17, 6, 7) 152 -> 139;
+// but (17, 6, 5) 84 -> 87, (13, 6, 14) split bf16 694 -> 882.
+bool direct_ok(const GemmDesc& d) {
+  return d.units == 1 && tc_shape_ok(d) && d.nn <= 6 && d.nk >= 7 && d.nm >= 14;
+}
+
+void order_for_direct(GemmDesc& d) {
+  bool in[kMaxBits] = {};
+  int count = 0;
+  auto take = [&](int i) {
+    if (!in[i] && count < 7) {
+      in[i] = true;
+      ++count;
+    }
+  };
+  // A's fastest indices that are rows, then C's fastest rows
+  for (int i = 0; i < d.nm; ++i)
+    if (d.am[i] < 32) take(i);
+  order_by_output(d, in);
+  count = 0;
+  for (int i = 0; i < d.nm; ++i) count += in[i];
+  for (int i = 0; i < d.nm; ++i) take(i);
+  // the tile's rows first, each part in C's order
+  int32_t am[kMaxBits], cm[kMaxBits];
+  int n = 0;
+  for (int part = 1; part >= 0; --part)
+    for (int i = 0; i < d.nm; ++i)
+      if (in[i] == (part != 0)) {
+        am[n] = d.am[i];
+        cm[n++] = d.cm[i];
+      }
+  for (int i = 0; i < d.nm; ++i) {
+    d.am[i] = am[i];
+    d.cm[i] = cm[i];
+  }
+}
+
+cudaError_t launch_gemm_direct(const float2* A, const PlaneOperand& b, float2* C, const GemmDesc& d, bool bf16,
+                               const unsigned* maxA, const int* exp_b, int* err, cudaStream_t s) {
+  if (!direct_ok(d)) return cudaErrorInvalidValue;
+  const int tn = 1 << d.nn;
+  CUtensorMap mb;
+  if (!encode_planes(&mb, b, tn, 0, 64)) return cudaErrorInvalidValue;
+  auto go = [&](auto n, auto np, auto fmt) {
+    return launch_direct_as<decltype(n)::value, decltype(np)::value, decltype(fmt)::value>(mb, A, C, d, maxA, exp_b, err,
+                                                                                           s);
+  };
+  auto go_n = [&](auto n) {
+    using std::integral_constant;
+    if (b.np == 4)
+      return bf16 ? go(n, integral_constant<int, 4>{}, std::true_type{}) : go(n, integral_constant<int, 4>{}, std::false_type{});
+    return bf16 ? go(n, integral_constant<int, 2>{}, std::true_type{}) : go(n, integral_constant<int, 2>{}, std::false_type{});
+  };
+  if (tn == 64) return go_n(std::integral_constant<int, 64>{});
+  if (tn == 32) return go_n(std::integral_constant<int, 32>{});
+  return go_n(std::integral_constant<int, 16>{});
 }
 
 }  // namespace tn

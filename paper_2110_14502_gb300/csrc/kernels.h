@@ -135,9 +135,20 @@ cudaError_t split_operand(const float2* src, const GemmDesc& d, bool which_b, bo
 // Plane operand of a tensor a producer epilogue already wrote as np planes
 // (layout [rows][K], K >= 8); false when the step's view does not match.
 bool planes_in_place(const float2* base, const GemmDesc& d, bool which_b, int np, PlaneOperand& out);
-// Split both operands of d into `scratch` (>= tc2_scratch_elems(d) 16-bit
-// values) and run the TMA GEMM.
+// GEMM that converts A itself, for a contraction that needs A once (one unit,
+// N <= 64): b holds B's planes, maxA (may be null) the float bits of A's largest
+// |component| for a scaled precision, exp_b B's exponent.  The descriptor's rows
+// in order_for_direct's order.
+bool direct_ok(const GemmDesc& d);
+void order_for_direct(GemmDesc& d);
+cudaError_t launch_gemm_direct(const float2* A, const PlaneOperand& b, float2* C, const GemmDesc& d, bool bf16,
+                               const unsigned* maxA, const int* exp_b, int* err, cudaStream_t s);
+// Split both operands of d (or B alone, where the GEMM converts A) into
+// `scratch` and run the GEMM, rows and columns renumbered as suits it.
+// tc2_scratch_elems: 16-bit values of both operands' planes;
+// tc2_pair_scratch_elems: those that a call needs.
 int64_t tc2_scratch_elems(const GemmDesc& d);
+int64_t tc2_pair_scratch_elems(const GemmDesc& d);
 cudaError_t run_gemm_tc2(const float2* A, const float2* B, float2* C, const GemmDesc& d, bool bf16, uint16_t* scratch,
                          int* err, cudaStream_t s);
 // Same with both operands scaled by their exact maxima (one power-of-two
@@ -233,7 +244,8 @@ struct Step;
 // kernel) instead of A's (GEMM kernels, whose A rows follow A's layout).
 void make_gemm_desc(const std::vector<int>& la, const std::vector<int>& lb, const std::vector<int>& lc,
                     GemmDesc& d, bool m_by_output = false);
-// M and N bits renumbered by the output's memory order.
-void order_by_output(GemmDesc& d);
+// M and N bits renumbered by the output's memory order (marks, when given, move
+// with the M bits).
+void order_by_output(GemmDesc& d, bool* marks = nullptr);
 
 }  // namespace tn

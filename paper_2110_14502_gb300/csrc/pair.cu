@@ -204,12 +204,9 @@ extern "C" tn_status tn_contract_pair(const void* A, const int32_t* a_labels, in
       if (algo == TN_PAIR_GATHER_TC && precision != TN_PREC_SPLIT_BF16)
         return fail(TN_EINVAL, "tn_contract_pair: the gathering tensor-core kernel runs split bf16 only");
       if (!tc_shape_ok(d)) return fail(TN_EINVAL, "tn_contract_pair: tensor-core kernels need M >= 128, N >= 16, K >= 8");
-      // the split pass reads any order of rows at the same speed, so they follow C
-      // (random orders, scaled bf16 (14, 14, 5): 2040 -> 832 us per call)
-      if (algo == TN_PAIR_FUSED_TC) order_by_output(d);
       std::lock_guard<std::mutex> lock(g_pair_mu);
       // operand planes, then 32 bytes for the scaled modes' maxima and exponents
-      const size_t planes = algo == TN_PAIR_FUSED_TC ? (size_t)tc2_scratch_elems(d) * sizeof(uint16_t) : 0;
+      const size_t planes = algo == TN_PAIR_FUSED_TC ? (size_t)tc2_pair_scratch_elems(d) * sizeof(uint16_t) : 0;
       PairDevState* ps = nullptr;
       tn_status pst = pair_state(planes + 32, ps);
       if (pst != TN_OK) return pst;

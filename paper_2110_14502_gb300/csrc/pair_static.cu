@@ -134,7 +134,6 @@ extern "C" tn_status tn_contract_pair_noalloc(const void* A, const int32_t* a_la
   if (!tc_shape_ok(d))
     return fail(TN_EINVAL, "tn_contract_pair_noalloc: needs M >= 128, N >= 16, K >= 8 (got 2^%d, 2^%d, 2^%d)", d.nm,
                 d.nn, d.nk);
-  order_by_output(d);  // as tn_contract_pair
   const int64_t need = tc2_scratch_elems(d);
   if (need > kStaticScratchElems)
     return fail(TN_EINVAL,
