@@ -808,7 +808,7 @@ struct PhaseLeaves {
   int count = 0;
   float2* arena = nullptr;
   int64_t stride = 0;
-  const GroupInfo* slot = nullptr;
+  GroupArg group{};
   int units = 0;
 };
 
@@ -822,7 +822,7 @@ tn_status run_phase(Ctx& c, int phase, const Geo& g, const PhaseLeaves& leaves) 
   auto gather = [&]() -> tn_status {
     if (gathered) return TN_OK;
     gathered = true;
-    return run_misc(c, launch_gather(E.store, leaves.arena, leaves.stride, leaves.descs, leaves.count, leaves.slot,
+    return run_misc(c, launch_gather(E.store, leaves.arena, leaves.stride, leaves.descs, leaves.count, leaves.group,
                                      leaves.units, c.st),
                     "gather");
   };
@@ -841,7 +841,7 @@ tn_status run_phase(Ctx& c, int phase, const Geo& g, const PhaseLeaves& leaves) 
                          phase == 0 ? 1 : (int64_t)g.gs};
     tn_status r = run_misc(c, launch_chain(E.chain + E.chain_pos[first], now, base, units, E.store,
                                            leaves.descs, gathered ? 0 : leaves.count, leaves.arena, leaves.stride,
-                                           leaves.slot, c.st),
+                                           leaves.group, c.st),
                            "chain");
     if (r) return r;
     gathered = true;
@@ -1098,7 +1098,8 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
   if (clear_out && rep) CK(cudaEventRecord(E.ev0, st));  // a nested recompute call is timed by its caller
   if (!o.device_io && nb > 0)
     CK(cudaMemcpyAsync((void*)d_bits, bits, nb * words * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
-  if (nout > 0 && clear_out) CK(cudaMemsetAsync(d_acc, 0, nout * sizeof(double2), st));
+  // (the first slice group's sums start from zero; without one the result is zero)
+  if (nout > 0 && clear_out && ns == 0) CK(cudaMemsetAsync(d_acc, 0, nout * sizeof(double2), st));
   if (scaled && (flags & 1)) CK(cudaMemsetAsync(E.nflagged, 0, sizeof(unsigned long long), st));
   Geo g;
   if (!E.inv_ready) {
@@ -1179,16 +1180,25 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
   // steps of a group and its accumulation), replayed from a graph when allowed.
   bool slice_only = scaled || E.ngather1 > 0;  // anything to do once per slice
   for (const Step& S : P.steps) slice_only |= S.phase == 1;
-  auto sequence = [&](int phase, const Geo& gg) -> tn_status {
+  auto sequence = [&](int phase, const Geo& gg, const GroupInfo& gi) -> tn_status {
     if (phase == 1 && !slice_only) return TN_OK;
+    // replayed sequences read the group from its slot, others take it by value
+    GroupArg group{};
+    if (graphs) {
+      group.slot = E.gslot + (phase == 1 ? 0 : 1);
+      tn_status r = run_misc(c, launch_set_group(E.gslot + (phase == 1 ? 0 : 1), gi, st), "set_group");
+      if (r) return r;
+    } else {
+      group.now = gi;
+    }
     auto body = [&]() -> tn_status {
       PhaseLeaves lv;
       if (phase == 1) {
         if (scaled) CK(cudaMemsetAsync(c.flag1, 0, Gs * sizeof(int), st));
-        lv = {E.gather, E.ngather1, E.sarena, Se, E.gslot, gg.gs};
+        lv = {E.gather, E.ngather1, E.sarena, Se, group, gg.gs};
       } else {
         if (scaled) CK(cudaMemsetAsync(c.flag2, 0, c.U * sizeof(int), st));
-        lv = {E.gather + E.ngather1, E.ngather2, E.parena, Pe, E.gslot + 1, gg.gs * gg.gb};
+        lv = {E.gather + E.ngather1, E.ngather2, E.parena, Pe, group, gg.gs * gg.gb};
       }
       tn_status rp = run_phase(c, phase, gg, lv);
       if (rp != TN_OK) return rp;
@@ -1197,7 +1207,7 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
         int64_t rlo, rhi;
         operand(P, E, root_id, 2, gg, root, rlo, rhi);
         tn_status r = run_misc(c,
-                               launch_accumulate(root, rlo, rhi, E.perm, (int)P.root_perm.size(), E.gslot + 1, gg.gb,
+                               launch_accumulate(root, rlo, rhi, E.perm, (int)P.root_perm.size(), group, gg.gb,
                                                  scaled ? c.flag1 : nullptr, scaled ? c.flag2 : nullptr, E.flagged,
                                                  E.nflagged, kFlaggedCap, st),
                                "accumulate");
@@ -1243,21 +1253,18 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
     gi.units = g.gs;
     gi.bits = d_bits;
     gi.acc = d_acc;
-    if (E.ngather1) {  // (only the slice-only gather reads this slot)
-      tn_status r = run_misc(c, launch_set_group(E.gslot, gi, st), "set_group");
-      if (r) return r;
-    }
+    gi.fresh = clear_out && s0 == s_begin;
     if (scaled && o.test_flag_every > 0) {
       // host-side injection of filter flags (tests of the recompute / discard paths)
       CK(cudaMemsetAsync(c.flag1, 0, Gs * sizeof(int), st));
       std::vector<int> f(g.gs);
       for (int i = 0; i < g.gs; ++i) f[i] = ((s0 + i) % o.test_flag_every) == 0;
-      tn_status r = sequence(1, g);
+      tn_status r = sequence(1, g, gi);
       if (r) return r;
       CK(cudaMemcpyAsync(c.flag1, f.data(), g.gs * sizeof(int), cudaMemcpyHostToDevice, st));
       CK(cudaStreamSynchronize(st));
     } else {
-      tn_status r = sequence(1, g);
+      tn_status r = sequence(1, g, gi);
       if (r) return r;
     }
     for (int64_t b0 = 0; b0 < nb; b0 += Gb) {
@@ -1265,9 +1272,7 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
       gi.b0 = b0;
       gi.nb = g.gb;
       gi.units = g.gs * g.gb;
-      tn_status r = run_misc(c, launch_set_group(E.gslot + 1, gi, st), "set_group");
-      if (r) return r;
-      r = sequence(2, g);
+      tn_status r = sequence(2, g, gi);
       if (r) return r;
     }
     if (c.tuning) {

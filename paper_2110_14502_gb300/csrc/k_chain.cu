@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(512) chain_kernel(const ChainStep* __restrict_
                                                     const ChainBase base, const float2* __restrict__ leaf_store,
                                                     const LeafGather* __restrict__ leaves, int nleaves,
                                                     float2* gather_arena, int64_t gather_stride,
-                                                    const GroupInfo* __restrict__ slot) {
+                                                    const GroupArg group) {
   extern __shared__ float2 operands[];
   __shared__ ChainStep S[2];
   __shared__ int2 kt[1 << kChainMaxK];
@@ -114,9 +114,10 @@ __global__ void __launch_bounds__(512) chain_kernel(const ChainStep* __restrict_
   };
   fetch(0);
   // the unit's leaves first, when this run opens its phase: one warp per leaf
+  const GroupInfo grp = nleaves > 0 && group.slot ? *group.slot : group.now;
   for (int l = tid >> 5; l < nleaves; l += nt >> 5) {
     const LeafGather& L = leaves[l];
-    const int64_t from = leaf_fixed_offset(L, *slot, u);
+    const int64_t from = leaf_fixed_offset(L, grp, u);
     float2* dst = gather_arena + (int64_t)u * gather_stride + L.dst_off;
     for (int e = tid & 31; e < (1 << L.nkept); e += 32) dst[e] = leaf_store[leaf_kept_offset(L, from, e)];
   }
@@ -215,7 +216,7 @@ void chain_add(ChainRun& run, const GemmDesc& d, bool im_first) {
 
 cudaError_t launch_chain(const ChainStep* steps, const ChainRun& run, const ChainBase& base, int units,
                          const float2* leaf_store, const LeafGather* leaves, int nleaves, float2* gather_arena,
-                         int64_t gather_stride, const GroupInfo* slot, cudaStream_t s) {
+                         int64_t gather_stride, const GroupArg& group, cudaStream_t s) {
   if (run.count < 1 || run.count > 64 || units < 1) return cudaErrorInvalidValue;
   static std::once_flag once[64];
   static cudaError_t attr[64];
@@ -234,7 +235,7 @@ cudaError_t launch_chain(const ChainStep* steps, const ChainRun& run, const Chai
   while (nt < cap && (nt < (1 << run.items) || nt * 8 < run.elems)) nt *= 2;
   chain_kernel<<<(unsigned)units, nt, run.elems * sizeof(float2), s>>>(steps, run.count, run.forms, base, leaf_store,
                                                                        leaves, nleaves, gather_arena, gather_stride,
-                                                                       slot);
+                                                                       group);
   return cudaGetLastError();
 }
 

@@ -19,8 +19,8 @@ namespace {
 __global__ void set_group_kernel(GroupInfo* slot, GroupInfo g) { *slot = g; }
 
 __global__ void gather_kernel(const float2* __restrict__ store, float2* __restrict__ arena, int64_t arena_stride,
-                              const LeafGather* __restrict__ descs, const GroupInfo* __restrict__ slot) {
-  const GroupInfo g = *slot;
+                              const LeafGather* __restrict__ descs, const GroupArg group) {
+  const GroupInfo g = group.slot ? *group.slot : group.now;
   const LeafGather& L = descs[blockIdx.x];
   const int u = blockIdx.y;
   if (u >= g.units) return;
@@ -35,17 +35,17 @@ __global__ void gather_kernel(const float2* __restrict__ store, float2* __restri
 // out of the sum): a flagged unit adds nothing here and is listed for the
 // host, which recomputes it in complex64 or counts it as discarded.
 __global__ void accumulate_kernel(const float2* __restrict__ root, int64_t r_lo, int64_t r_hi,
-                                  const int64_t* __restrict__ perm, int nperm, const GroupInfo* __restrict__ slot,
+                                  const int64_t* __restrict__ perm, int nperm, const GroupArg group,
                                   const int* __restrict__ flag_s, const int* __restrict__ flag_u,
                                   int64_t* __restrict__ flagged, unsigned long long* __restrict__ nflagged,
                                   int cap) {
-  const GroupInfo g = *slot;
+  const GroupInfo g = group.slot ? *group.slot : group.now;
   double2* acc = g.acc;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)g.nb * nperm) return;
   const int bl = (int)(idx / nperm);
   const int j = (int)(idx % nperm);
-  double2 a = acc[(g.b0 + bl) * nperm + j];
+  double2 a = g.fresh ? make_double2(0.0, 0.0) : acc[(g.b0 + bl) * nperm + j];
   const float2* r = root + bl * r_hi + perm[j];
   for (int sl = 0; sl < g.nslice; ++sl) {
     if ((flag_s && flag_s[sl]) || (flag_u && flag_u[bl * g.nslice + sl])) {
@@ -82,19 +82,19 @@ cudaError_t launch_set_group(GroupInfo* slot, const GroupInfo& g, cudaStream_t s
 }
 
 cudaError_t launch_gather(const float2* store, float2* arena, int64_t arena_stride, const LeafGather* descs,
-                          int nleaves, const GroupInfo* slot, int units, cudaStream_t s) {
+                          int nleaves, const GroupArg& group, int units, cudaStream_t s) {
   if (nleaves == 0 || units == 0) return cudaSuccess;
   dim3 grid((unsigned)nleaves, (unsigned)units);
-  gather_kernel<<<grid, 64, 0, s>>>(store, arena, arena_stride, descs, slot);
+  gather_kernel<<<grid, 64, 0, s>>>(store, arena, arena_stride, descs, group);
   return cudaGetLastError();
 }
 
 cudaError_t launch_accumulate(const float2* root, int64_t r_lo, int64_t r_hi, const int64_t* perm, int nperm,
-                              const GroupInfo* slot, int nb_max, const int* flag_s, const int* flag_u,
+                              const GroupArg& group, int nb_max, const int* flag_s, const int* flag_u,
                               int64_t* flagged, unsigned long long* nflagged, int cap, cudaStream_t s) {
   const int64_t total = (int64_t)nb_max * nperm;
   const int nt = 256;
-  accumulate_kernel<<<(unsigned)((total + nt - 1) / nt), nt, 0, s>>>(root, r_lo, r_hi, perm, nperm, slot, flag_s,
+  accumulate_kernel<<<(unsigned)((total + nt - 1) / nt), nt, 0, s>>>(root, r_lo, r_hi, perm, nperm, group, flag_s,
                                                                      flag_u, flagged, nflagged, cap);
   return cudaGetLastError();
 }

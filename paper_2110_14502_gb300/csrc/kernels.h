@@ -48,8 +48,9 @@ struct LeafGather {
 
 // A group of units: `nslice` consecutive slice ids from slice0 for the
 // bitstrings b0 .. b0+nb-1; unit u = (u % nslice) slice, (u / nslice) bitstring.
-// The kernels read it from a device slot written by launch_set_group, so a
-// captured launch sequence can be replayed for any group.
+// The kernels take it by value, or from a device slot written by
+// launch_set_group, so that a captured launch sequence can be replayed for any
+// group.
 struct GroupInfo {
   int64_t slice0;
   int64_t b0;
@@ -59,6 +60,11 @@ struct GroupInfo {
   int32_t units;             // nslice * nb
   const uint64_t* bits;      // bitstrings of the call (device)
   double2* acc;              // amplitude accumulator of the call (device)
+  int32_t fresh;             // 1: the call's first sum into acc, which starts from zero
+};
+struct GroupArg {
+  const GroupInfo* slot;     // null: `now`
+  GroupInfo now;
 };
 
 // launchers (return cudaGetLastError())
@@ -217,17 +223,17 @@ void chain_add(ChainRun& run, const GemmDesc& d, bool im_first);
 // 0 each unit first gathers its leaves, as launch_gather.
 cudaError_t launch_chain(const ChainStep* steps, const ChainRun& run, const ChainBase& base, int units,
                          const float2* leaf_store, const LeafGather* leaves, int nleaves, float2* gather_arena,
-                         int64_t gather_stride, const GroupInfo* slot, cudaStream_t s);
+                         int64_t gather_stride, const GroupArg& group, cudaStream_t s);
 cudaError_t launch_set_group(GroupInfo* slot, const GroupInfo& g, cudaStream_t s);
-// grid covers `units` units (the slot's count may be lower for a partial group)
+// grid covers `units` units (the group's count may be lower for a partial group)
 cudaError_t launch_gather(const float2* store, float2* arena, int64_t arena_stride, const LeafGather* descs,
-                          int nleaves, const GroupInfo* slot, int units, cudaStream_t s);
+                          int nleaves, const GroupArg& group, int units, cudaStream_t s);
 // acc[b, j] += sum over the group's slices (in slice order) of root(b, s)[perm[j]],
 // root(b, s) = root + s_local * r_lo + b_local * r_hi.
 // Flagged units (flag_s per slice of the group, flag_u per unit; both may be
 // null) are skipped and appended as (b << 32 | s) to `flagged` (capacity cap).
 cudaError_t launch_accumulate(const float2* root, int64_t r_lo, int64_t r_hi, const int64_t* perm, int nperm,
-                              const GroupInfo* slot, int nb_max, const int* flag_s, const int* flag_u,
+                              const GroupArg& group, int nb_max, const int* flag_s, const int* flag_u,
                               int64_t* flagged, unsigned long long* nflagged, int cap, cudaStream_t s);
 // dst (dense, element e) = src[sum_p bit_p(e) * st[p]]: bit p of e is dst's
 // p-th fastest index, st[p] its element stride in src.
