@@ -13,6 +13,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "device_common.h"
 #include "kernels.h"
@@ -130,32 +131,41 @@ struct TileMap {
   int8_t dst[12];
 };
 
+// One operand of a launch: its tensors (z: number nlo per lo stride, then hi),
+// where their planes go, and the scaled formats' maxima and exponents.
+struct SplitJob {
+  const float2* src;
+  uint16_t* dst;
+  int bits, nlo, vec;
+  int64_t lo, hi;
+  const unsigned* maxbits;
+  int* e_out;
+  float* m_out;
+};
+
 template <int NP, int T, bool BF16>
-__global__ void __launch_bounds__(NT) split_kernel(const float2* __restrict__ src, uint16_t* __restrict__ dst,
-                                                   const __grid_constant__ TileMap tm, int bits, int nlo, int64_t lo,
-                                                   int64_t hi, int vec, const unsigned* __restrict__ maxbits,
-                                                   int* __restrict__ e_out, float* __restrict__ m_out) {
+__device__ __forceinline__ void split_tile(const SplitJob& job, const TileMap& tm, unsigned blk, int64_t z) {
   constexpr int E = 1 << T;
   __shared__ __align__(16) float2 tile[E];
-  const int64_t z = blockIdx.y;
-  src += (z % nlo) * lo + (z / nlo) * hi;
+  const float2* src = job.src + (z % job.nlo) * job.lo + (z / job.nlo) * job.hi;
+  const bool vec = job.vec != 0;
   int e = 0;
-  if (maxbits) {
-    const float mx = __uint_as_float(maxbits[z]);
+  if (job.maxbits) {
+    const float mx = __uint_as_float(job.maxbits[z]);
     e = scale_exponent(mx);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      e_out[z] = e;
-      m_out[z] = ldexpf(mx, -e);
+    if (blk == 0 && threadIdx.x == 0) {
+      job.e_out[z] = e;
+      job.m_out[z] = ldexpf(mx, -e);
     }
   }
   const Pow2 sc(-e);
-  const int64_t plane = int64_t(1) << bits;
-  uint16_t* out = dst + z * NP * plane;
+  const int64_t plane = int64_t(1) << job.bits;
+  uint16_t* out = job.dst + z * NP * plane;
   {
     int32_t so = 0;
     int64_t dofs = 0;
     for (int b = 0; b < tm.nout; ++b)
-      if ((blockIdx.x >> b) & 1) {
+      if ((blk >> b) & 1) {
         so += tm.out_src[b];
         dofs += int64_t(1) << tm.out_dst[b];
       }
@@ -236,6 +246,21 @@ __global__ void __launch_bounds__(NT) split_kernel(const float2* __restrict__ sr
   }
 }
 
+template <int NP, int T, bool BF16>
+__global__ void __launch_bounds__(NT) split_kernel(const SplitJob job, const __grid_constant__ TileMap tm) {
+  split_tile<NP, T, BF16>(job, tm, blockIdx.x, blockIdx.y);
+}
+
+// Both operands of one contraction in one launch: the first blocks take A's
+// tiles, the others B's.
+template <int NP, int T, bool BF16>
+__global__ void __launch_bounds__(NT) split_pair_kernel(const SplitJob a, const __grid_constant__ TileMap ta,
+                                                        const SplitJob b, const __grid_constant__ TileMap tb) {
+  const unsigned na = 1u << (a.bits - T);
+  if (blockIdx.x < na) split_tile<NP, T, BF16>(a, ta, blockIdx.x, 0);
+  else split_tile<NP, T, BF16>(b, tb, blockIdx.x - na, 0);
+}
+
 // The tile of T bits for an operand whose output bit i (K bits, then row bits)
 // has input stride st[i], R bits in all.
 template <int T>
@@ -284,28 +309,64 @@ TileMap split_tile_map(const SplitDesc& d) {
   return m;
 }
 
-template <int NP, int T>
-cudaError_t launch_tiles(const float2* src, uint16_t* dst, const SplitDesc& d, int nz, bool vec, bool bf16,
-                         const unsigned* maxbits, int* e_out, float* m_out, cudaStream_t s) {
-  const int R = d.nk + d.nrow;
-  const dim3 grid(1u << (R - T), (unsigned)nz);
-  const TileMap m = split_tile_map<T>(d);
-  if (bf16) split_kernel<NP, T, true><<<grid, NT, 0, s>>>(src, dst, m, R, d.nlo, d.lo, d.hi, vec, maxbits, e_out, m_out);
-  else split_kernel<NP, T, false><<<grid, NT, 0, s>>>(src, dst, m, R, d.nlo, d.lo, d.hi, vec, maxbits, e_out, m_out);
+// Tile size for an operand of 2^R elements, nz of them: 2^12 once that fills the
+// chip a few times over (152 SMs, six such CTAs each); smaller tiles spread a
+// small operand over more SMs.
+int tile_bits(int R, int nz) {
+  return R >= 12 && (int64_t(1) << (R - 12)) * nz >= 152 * 4 ? 12 : R >= 10 ? 10 : 7;
+}
+
+template <class F>
+cudaError_t for_format(int np, bool bf16, int T, F&& f) {
+  using std::integral_constant;
+  auto t = [&](auto n, auto fmt) {
+    if (T == 12) f(n, integral_constant<int, 12>{}, fmt);
+    else if (T == 10) f(n, integral_constant<int, 10>{}, fmt);
+    else f(n, integral_constant<int, 7>{}, fmt);
+  };
+  auto n = [&](auto fmt) {
+    if (np == 4) t(integral_constant<int, 4>{}, fmt);
+    else t(integral_constant<int, 2>{}, fmt);
+  };
+  if (bf16) n(std::true_type{});
+  else n(std::false_type{});
   return cudaGetLastError();
 }
 
-// 2^12-element tiles once they fill the chip a few times over (152 SMs, six
-// such CTAs each); smaller ones spread a small operand over more SMs.
-template <int NP>
-cudaError_t launch_np(const float2* src, uint16_t* dst, const SplitDesc& d, int nz, bool vec, bool bf16,
-                      const unsigned* maxbits, int* e_out, float* m_out, cudaStream_t s) {
-  const int R = d.nk + d.nrow;
-  if (R >= 12 && (int64_t(1) << (R - 12)) * nz >= 152 * 4)
-    return launch_tiles<NP, 12>(src, dst, d, nz, vec, bf16, maxbits, e_out, m_out, s);
-  if (R >= 10) return launch_tiles<NP, 10>(src, dst, d, nz, vec, bf16, maxbits, e_out, m_out, s);
-  return launch_tiles<NP, 7>(src, dst, d, nz, vec, bf16, maxbits, e_out, m_out, s);
+bool vec_ok(const float2* src, const SplitDesc& d) {
+  return (reinterpret_cast<uintptr_t>(src) & 15) == 0 && (d.lo & 1) == 0 && (d.hi & 1) == 0;
 }
+
+SplitJob split_job(const float2* src, uint16_t* dst, const SplitDesc& d, const unsigned* maxbits, int* e_out,
+                   float* m_out) {
+  return {src, dst, d.nk + d.nrow, d.nlo, vec_ok(src, d), d.lo, d.hi, maxbits, e_out, m_out};
+}
+
+// Both maxima of a contraction's operands by one CTA each, stored (no clearing,
+// no atomics): for operands that one CTA reads in a microsecond or two.
+constexpr int MAX_SMALL_BITS = 15;
+__global__ void __launch_bounds__(1024) max_small_kernel(const float2* __restrict__ a, int abits,
+                                                         const float2* __restrict__ b, int bbits,
+                                                         unsigned* __restrict__ maxbits) {
+  const float2* p = blockIdx.x ? b : a;
+  const int n = 1 << (blockIdx.x ? bbits : abits);
+  float m = 0.f;
+#pragma unroll 8
+  for (int e = threadIdx.x; e < n; e += 1024) {
+    const float2 v = __ldg(p + e);
+    m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
+  }
+  __shared__ unsigned wm[32];
+  const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = w;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const unsigned x = __reduce_max_sync(0xffffffffu, wm[threadIdx.x]);
+    if (threadIdx.x == 0) maxbits[blockIdx.x] = x;
+  }
+}
+
+}  // namespace
 
 cudaError_t launch_max(const float2* src, int bits, int nz, int nlo, int64_t lo, int64_t hi, bool vec, unsigned* maxbits,
                        cudaStream_t s) {
@@ -316,19 +377,20 @@ cudaError_t launch_max(const float2* src, int bits, int nz, int nlo, int64_t lo,
   return cudaGetLastError();
 }
 
-}  // namespace
-
 cudaError_t launch_split(const float2* src, uint16_t* dst, const SplitDesc& d, int nz, bool bf16, int np,
                          unsigned* maxbits, int* e_out, float* m_out, cudaStream_t s, bool max_ready) {
   const int R = d.nk + d.nrow;
   if (nz < 1 || nz > 65535 || R < 7 || R > 30 || (np != 2 && np != 4)) return cudaErrorInvalidValue;
-  const bool vec = (reinterpret_cast<uintptr_t>(src) & 15) == 0 && (d.lo & 1) == 0 && (d.hi & 1) == 0;
   if (maxbits && !max_ready) {
-    const cudaError_t e = launch_max(src, R, nz, d.nlo, d.lo, d.hi, vec, maxbits, s);
+    const cudaError_t e = launch_max(src, R, nz, d.nlo, d.lo, d.hi, vec_ok(src, d), maxbits, s);
     if (e != cudaSuccess) return e;
   }
-  return np == 4 ? launch_np<4>(src, dst, d, nz, vec, bf16, maxbits, e_out, m_out, s)
-                 : launch_np<2>(src, dst, d, nz, vec, bf16, maxbits, e_out, m_out, s);
+  const SplitJob job = split_job(src, dst, d, maxbits, e_out, m_out);
+  return for_format(np, bf16, tile_bits(R, nz), [&](auto n, auto t, auto fmt) {
+    constexpr int T = decltype(t)::value;
+    split_kernel<decltype(n)::value, T, decltype(fmt)::value>
+        <<<dim3(1u << (R - T), (unsigned)nz), NT, 0, s>>>(job, split_tile_map<T>(d));
+  });
 }
 
 namespace {
@@ -354,15 +416,14 @@ int64_t split_scratch_elems(const GemmDesc& d, bool which_b, int np) {
 
 int64_t tc2_scratch_elems(const GemmDesc& d) { return split_scratch_elems(d, false, 4) + split_scratch_elems(d, true, 4); }
 
-cudaError_t split_operand(const float2* src, const GemmDesc& d, bool which_b, bool bf16, int np, bool scaled,
-                          unsigned* maxbits, int* e_out, float* m_out, uint16_t* scratch, PlaneOperand& out,
-                          cudaStream_t s, bool max_ready) {
+namespace {
+// An operand's split view, number of distinct tensors, and its planes at `scratch`.
+SplitDesc operand_view(const GemmDesc& d, bool which_b, int np, const uint16_t* scratch, int& nz, PlaneOperand& out) {
   const int64_t lo = which_b ? d.b_lo : d.a_lo, hi = which_b ? d.b_hi : d.a_hi;
   const int nrow = which_b ? d.nn : d.nm;
   SplitDesc sd;
   split_desc(nrow, which_b ? d.bn : d.am, d.nk, which_b ? d.bk : d.ak, lo ? d.units_lo : 1, lo, hi, sd);
-  const int nz = distinct(d, lo, hi);
-  cudaError_t e = launch_split(src, scratch, sd, nz, bf16, np, scaled ? maxbits : nullptr, e_out, m_out, s, max_ready);
+  nz = distinct(d, lo, hi);
   const int64_t K = int64_t(1) << d.nk;  // tensor-core shapes have K >= 8: whole 16-byte chunks, no padding
   const int64_t set = (int64_t)np * (int64_t(1) << nrow) * K * 2;
   out.base = scratch;
@@ -373,7 +434,56 @@ cudaError_t split_operand(const float2* src, const GemmDesc& d, bool which_b, bo
   out.nhi = hi ? d.units / d.units_lo : 1;
   out.st_lo = set;
   out.st_hi = set * out.nlo;
+  return sd;
+}
+}  // namespace
+
+cudaError_t split_operand(const float2* src, const GemmDesc& d, bool which_b, bool bf16, int np, bool scaled,
+                          unsigned* maxbits, int* e_out, float* m_out, uint16_t* scratch, PlaneOperand& out,
+                          cudaStream_t s, bool max_ready) {
+  int nz;
+  const SplitDesc sd = operand_view(d, which_b, np, scratch, nz, out);
+  return launch_split(src, scratch, sd, nz, bf16, np, scaled ? maxbits : nullptr, e_out, m_out, s, max_ready);
+}
+
+// The maxima of a one-unit contraction's operands, mx[0] of A and mx[1] of B.
+static cudaError_t pair_maxima(const float2* A, const float2* B, const GemmDesc& d, unsigned* mx, cudaStream_t s) {
+  const int ra = d.nm + d.nk, rb = d.nn + d.nk;
+  if (ra <= MAX_SMALL_BITS && rb <= MAX_SMALL_BITS) {
+    max_small_kernel<<<2, 1024, 0, s>>>(A, ra, B, rb, mx);
+    return cudaGetLastError();
+  }
+  cudaError_t e = cudaMemsetAsync(mx, 0, 2 * sizeof(unsigned), s);
+  const auto vec = [](const float2* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  if (e == cudaSuccess) e = launch_max(A, ra, 1, 1, 0, 0, vec(A), mx, s);
+  if (e == cudaSuccess) e = launch_max(B, rb, 1, 1, 0, 0, vec(B), mx + 1, s);
   return e;
+}
+
+// Both operands of a one-unit contraction: one launch where one tile size suits
+// both (a launch saved is 3 us of a call that small), else one each.  mx (may be
+// null): their maxima, with ex, ms receiving the exponents and stored maxima.
+static cudaError_t split_pair(const float2* A, const float2* B, const GemmDesc& d, bool bf16, int np, unsigned* mx,
+                              int* ex, float* ms, uint16_t* scratch, PlaneOperand& pa, PlaneOperand& pb,
+                              cudaStream_t s) {
+  int nz;
+  uint16_t* const sb = scratch + split_scratch_elems(d, false, np);
+  const SplitDesc da = operand_view(d, false, np, scratch, nz, pa), db = operand_view(d, true, np, sb, nz, pb);
+  const int ra = d.nm + d.nk, rb = d.nn + d.nk;
+  const int ta = tile_bits(ra, 1), tb = tile_bits(rb, 1);
+  const SplitJob ja = split_job(A, scratch, da, mx, ex, ms);
+  const SplitJob jb = split_job(B, sb, db, mx ? mx + 1 : nullptr, ex ? ex + 1 : nullptr, ms ? ms + 1 : nullptr);
+  const int T = ta < tb ? ta : tb, large = ra > rb ? ra : rb;
+  if (ta == tb || (T == 10 && large <= 20) || (T == 7 && large <= 14))
+    return for_format(np, bf16, T, [&](auto n, auto t, auto fmt) {
+      constexpr int TT = decltype(t)::value;
+      split_pair_kernel<decltype(n)::value, TT, decltype(fmt)::value>
+          <<<(1u << (ra - TT)) + (1u << (rb - TT)), NT, 0, s>>>(ja, split_tile_map<TT>(da), jb, split_tile_map<TT>(db));
+    });
+  const cudaError_t e = launch_split(A, scratch, da, 1, bf16, np, mx, ex, ms, s, true);
+  return e != cudaSuccess ? e
+                          : launch_split(B, sb, db, 1, bf16, np, mx ? mx + 1 : nullptr, ex ? ex + 1 : nullptr,
+                                         ms ? ms + 1 : nullptr, s, true);
 }
 
 bool planes_in_place(const float2* base, const GemmDesc& d, bool which_b, int np, PlaneOperand& out) {
@@ -414,10 +524,7 @@ cudaError_t run_gemm_tc2(const float2* A, const float2* B, float2* C, const Gemm
   // the split pass reads any order of rows at the same speed, so they follow C
   // (random orders, scaled bf16 (14, 14, 5): 2040 -> 832 us per call)
   order_by_output(d);
-  cudaError_t e = split_operand(A, d, false, bf16, 4, false, nullptr, nullptr, nullptr, scratch, pa, s);
-  if (e != cudaSuccess) return e;
-  e = split_operand(B, d, true, bf16, 4, false, nullptr, nullptr, nullptr, scratch + split_scratch_elems(d, false, 4),
-                    pb, s);
+  const cudaError_t e = split_pair(A, B, d, bf16, 4, nullptr, nullptr, nullptr, scratch, pa, pb, s);
   if (e != cudaSuccess) return e;
   const ScaleIO none{};
   return launch_gemm_tma(pa, pb, C, false, d, bf16, none, err, s);
@@ -429,20 +536,16 @@ cudaError_t run_gemm_tc2_scaled(const float2* A, const float2* B, float2* C, con
   int* ex = reinterpret_cast<int*>(mx + 2);
   float* ms = reinterpret_cast<float*>(ex + 2);
   GemmDesc d = d0;
-  cudaError_t e = cudaMemsetAsync(mx, 0, 2 * sizeof(unsigned), s);
+  cudaError_t e = pair_maxima(A, B, d, mx, s);
   if (e != cudaSuccess) return e;
   PlaneOperand pa, pb;
   if (direct_ok(d)) {
     order_for_direct(d);
-    e = launch_max(A, d.nm + d.nk, 1, 1, 0, 0, (reinterpret_cast<uintptr_t>(A) & 15) == 0, mx, s);
-    if (e == cudaSuccess) e = split_operand(B, d, true, bf16, np, true, mx + 1, ex + 1, ms + 1, scratch, pb, s);
+    e = split_operand(B, d, true, bf16, np, true, mx + 1, ex + 1, ms + 1, scratch, pb, s, true);
     return e != cudaSuccess ? e : launch_gemm_direct(A, pb, C, d, bf16, mx, ex + 1, err, s);
   }
   order_by_output(d);
-  e = split_operand(A, d, false, bf16, np, true, mx, ex, ms, scratch, pa, s);
-  if (e == cudaSuccess)
-    e = split_operand(B, d, true, bf16, np, true, mx + 1, ex + 1, ms + 1,
-                      scratch + split_scratch_elems(d, false, np), pb, s);
+  e = split_pair(A, B, d, bf16, np, mx, ex, ms, scratch, pa, pb, s);
   if (e != cudaSuccess) return e;
   ScaleIO sio{};
   sio.ea = ex;
