@@ -112,7 +112,9 @@ __global__ void __launch_bounds__(512) chain_kernel(const ChainStep* __restrict_
     uint32_t* q = reinterpret_cast<uint32_t*>(&S[i & 1]);
     for (int w = tid; w < WORDS; w += nt) q[w] = p[w];
   };
-  fetch(0);
+  fetch(0);  // (the descriptors never change)
+  let_next_start();
+  after_previous();
   // the unit's leaves first, when this run opens its phase: one warp per leaf
   const GroupInfo grp = nleaves > 0 && group.slot ? *group.slot : group.now;
   for (int l = tid >> 5; l < nleaves; l += nt >> 5) {
@@ -233,10 +235,8 @@ cudaError_t launch_chain(const ChainStep* steps, const ChainRun& run, const Chai
   const int cap = units >= 304 ? 128 : 512;
   int nt = 64;
   while (nt < cap && (nt < (1 << run.items) || nt * 8 < run.elems)) nt *= 2;
-  chain_kernel<<<(unsigned)units, nt, run.elems * sizeof(float2), s>>>(steps, run.count, run.forms, base, leaf_store,
-                                                                       leaves, nleaves, gather_arena, gather_stride,
-                                                                       group);
-  return cudaGetLastError();
+  return launch_overlapped(chain_kernel, dim3((unsigned)units), dim3(nt), run.elems * sizeof(float2), s, steps, run.count,
+                           run.forms, base, leaf_store, leaves, nleaves, gather_arena, gather_stride, group);
 }
 
 }  // namespace tn

@@ -20,6 +20,8 @@ __global__ void set_group_kernel(GroupInfo* slot, GroupInfo g) { *slot = g; }
 
 __global__ void gather_kernel(const float2* __restrict__ store, float2* __restrict__ arena, int64_t arena_stride,
                               const LeafGather* __restrict__ descs, const GroupArg group) {
+  let_next_start();
+  after_previous();
   const GroupInfo g = group.slot ? *group.slot : group.now;
   const LeafGather& L = descs[blockIdx.x];
   const int u = blockIdx.y;
@@ -39,6 +41,8 @@ __global__ void accumulate_kernel(const float2* __restrict__ root, int64_t r_lo,
                                   const int* __restrict__ flag_s, const int* __restrict__ flag_u,
                                   int64_t* __restrict__ flagged, unsigned long long* __restrict__ nflagged,
                                   int cap) {
+  let_next_start();
+  after_previous();
   const GroupInfo g = group.slot ? *group.slot : group.now;
   double2* acc = g.acc;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -85,8 +89,7 @@ cudaError_t launch_gather(const float2* store, float2* arena, int64_t arena_stri
                           int nleaves, const GroupArg& group, int units, cudaStream_t s) {
   if (nleaves == 0 || units == 0) return cudaSuccess;
   dim3 grid((unsigned)nleaves, (unsigned)units);
-  gather_kernel<<<grid, 64, 0, s>>>(store, arena, arena_stride, descs, group);
-  return cudaGetLastError();
+  return launch_overlapped(gather_kernel, grid, dim3(64), 0, s, store, arena, arena_stride, descs, group);
 }
 
 cudaError_t launch_accumulate(const float2* root, int64_t r_lo, int64_t r_hi, const int64_t* perm, int nperm,
@@ -94,9 +97,8 @@ cudaError_t launch_accumulate(const float2* root, int64_t r_lo, int64_t r_hi, co
                               int64_t* flagged, unsigned long long* nflagged, int cap, cudaStream_t s) {
   const int64_t total = (int64_t)nb_max * nperm;
   const int nt = 256;
-  accumulate_kernel<<<(unsigned)((total + nt - 1) / nt), nt, 0, s>>>(root, r_lo, r_hi, perm, nperm, group, flag_s,
-                                                                     flag_u, flagged, nflagged, cap);
-  return cudaGetLastError();
+  return launch_overlapped(accumulate_kernel, dim3((unsigned)((total + nt - 1) / nt)), dim3(nt), 0, s, root, r_lo, r_hi, perm,
+                           nperm, group, flag_s, flag_u, flagged, nflagged, cap);
 }
 
 cudaError_t launch_permute(const float2* src, float2* dst, const PermDesc& pd, int64_t units, int64_t src_unit,

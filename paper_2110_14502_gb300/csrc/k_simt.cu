@@ -29,6 +29,7 @@
 // row); otherwise each lane reads one element, lanes on consecutive rows.
 #include <algorithm>
 
+#include "device_common.h"
 #include "kernels.h"
 
 namespace tn {
@@ -169,6 +170,8 @@ __global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_ker
   float2* Bs = reinterpret_cast<float2*>(smem + 2 * CF::A_BUF);    // [2][BK][BN]
   const int64_t K = int64_t(1) << d.nk;
   const int64_t m0 = (int64_t)blockIdx.x * BM, n0 = (int64_t)blockIdx.y * BN;
+  let_next_start();
+  after_previous();
   const int64_t ulo = blockIdx.z % d.units_lo, uhi = blockIdx.z / d.units_lo;
   A += ulo * d.a_lo + uhi * d.a_hi;
   B += ulo * d.b_lo + uhi * d.b_hi;
@@ -282,8 +285,8 @@ cudaError_t launch_tile(const float2* A, const float2* B, float2* C, const GemmD
   }
   const int64_t M = int64_t(1) << d.nm, N = int64_t(1) << d.nn;
   dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), (unsigned)d.units);
-  gemm_simt_kernel<BM, BN, BK, RM, RN><<<grid, NT, SMEM, s>>>(A, B, C, d, flags);
-  return cudaGetLastError();
+  return launch_overlapped(gemm_simt_kernel<BM, BN, BK, RM, RN>, grid, dim3(NT), SMEM, s, A, B,
+                           C, d, flags);
 }
 
 // Vector loads of 4 consecutive K values need the operand's two fastest

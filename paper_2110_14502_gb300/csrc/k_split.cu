@@ -145,6 +145,8 @@ struct SplitJob {
 
 template <int NP, int T, bool BF16>
 __device__ __forceinline__ void split_tile(const SplitJob& job, const TileMap& tm, unsigned blk, int64_t z) {
+  let_next_start();
+  after_previous();
   constexpr int E = 1 << T;
   __shared__ __align__(16) float2 tile[E];
   const float2* src = job.src + (z % job.nlo) * job.lo + (z / job.nlo) * job.hi;
@@ -320,17 +322,12 @@ template <class F>
 cudaError_t for_format(int np, bool bf16, int T, F&& f) {
   using std::integral_constant;
   auto t = [&](auto n, auto fmt) {
-    if (T == 12) f(n, integral_constant<int, 12>{}, fmt);
-    else if (T == 10) f(n, integral_constant<int, 10>{}, fmt);
-    else f(n, integral_constant<int, 7>{}, fmt);
+    return T == 12   ? f(n, integral_constant<int, 12>{}, fmt)
+           : T == 10 ? f(n, integral_constant<int, 10>{}, fmt)
+                     : f(n, integral_constant<int, 7>{}, fmt);
   };
-  auto n = [&](auto fmt) {
-    if (np == 4) t(integral_constant<int, 4>{}, fmt);
-    else t(integral_constant<int, 2>{}, fmt);
-  };
-  if (bf16) n(std::true_type{});
-  else n(std::false_type{});
-  return cudaGetLastError();
+  auto n = [&](auto fmt) { return np == 4 ? t(integral_constant<int, 4>{}, fmt) : t(integral_constant<int, 2>{}, fmt); };
+  return bf16 ? n(std::true_type{}) : n(std::false_type{});
 }
 
 bool vec_ok(const float2* src, const SplitDesc& d) {
@@ -348,6 +345,8 @@ constexpr int MAX_SMALL_BITS = 15;
 __global__ void __launch_bounds__(1024) max_small_kernel(const float2* __restrict__ a, int abits,
                                                          const float2* __restrict__ b, int bbits,
                                                          unsigned* __restrict__ maxbits) {
+  let_next_start();
+  after_previous();
   const float2* p = blockIdx.x ? b : a;
   const int n = 1 << (blockIdx.x ? bbits : abits);
   float m = 0.f;
@@ -388,8 +387,8 @@ cudaError_t launch_split(const float2* src, uint16_t* dst, const SplitDesc& d, i
   const SplitJob job = split_job(src, dst, d, maxbits, e_out, m_out);
   return for_format(np, bf16, tile_bits(R, nz), [&](auto n, auto t, auto fmt) {
     constexpr int T = decltype(t)::value;
-    split_kernel<decltype(n)::value, T, decltype(fmt)::value>
-        <<<dim3(1u << (R - T), (unsigned)nz), NT, 0, s>>>(job, split_tile_map<T>(d));
+    return launch_overlapped(split_kernel<decltype(n)::value, T, decltype(fmt)::value>,
+                             dim3(1u << (R - T), (unsigned)nz), dim3(NT), 0, s, job, split_tile_map<T>(d));
   });
 }
 
@@ -450,8 +449,7 @@ cudaError_t split_operand(const float2* src, const GemmDesc& d, bool which_b, bo
 static cudaError_t pair_maxima(const float2* A, const float2* B, const GemmDesc& d, unsigned* mx, cudaStream_t s) {
   const int ra = d.nm + d.nk, rb = d.nn + d.nk;
   if (ra <= MAX_SMALL_BITS && rb <= MAX_SMALL_BITS) {
-    max_small_kernel<<<2, 1024, 0, s>>>(A, ra, B, rb, mx);
-    return cudaGetLastError();
+    return launch_overlapped(max_small_kernel, dim3(2), dim3(1024), 0, s, A, ra, B, rb, mx);
   }
   cudaError_t e = cudaMemsetAsync(mx, 0, 2 * sizeof(unsigned), s);
   const auto vec = [](const float2* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
@@ -477,8 +475,9 @@ static cudaError_t split_pair(const float2* A, const float2* B, const GemmDesc& 
   if (ta == tb || (T == 10 && large <= 20) || (T == 7 && large <= 14))
     return for_format(np, bf16, T, [&](auto n, auto t, auto fmt) {
       constexpr int TT = decltype(t)::value;
-      split_pair_kernel<decltype(n)::value, TT, decltype(fmt)::value>
-          <<<(1u << (ra - TT)) + (1u << (rb - TT)), NT, 0, s>>>(ja, split_tile_map<TT>(da), jb, split_tile_map<TT>(db));
+      return launch_overlapped(split_pair_kernel<decltype(n)::value, TT, decltype(fmt)::value>,
+                               dim3((1u << (ra - TT)) + (1u << (rb - TT))), dim3(NT), 0, s, ja, split_tile_map<TT>(da),
+                               jb, split_tile_map<TT>(db));
     });
   const cudaError_t e = launch_split(A, scratch, da, 1, bf16, np, mx, ex, ms, s, true);
   return e != cudaSuccess ? e

@@ -568,6 +568,8 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
+  let_next_start();
+  after_previous();
 
   if (warp == 0) {
     // ---- TMA producer (the whole warp waits, one lane issues): the stage ring
@@ -1058,6 +1060,8 @@ __global__ void __launch_bounds__(DirectCfg<TN, NP>::THREADS, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
+  let_next_start();
+  after_previous();
 
   if (warp == 0) {
     // ---- B's stages
@@ -1459,9 +1463,8 @@ cudaError_t launch_chunked_ew(const CUtensorMap& ma, const CUtensorMap& mb, floa
   const int64_t items = (M / TM) * (fold > 1 ? 1 : N / TN) * (d.units / fold);
   const int chunk = NP == 4 ? split_chunk() : 1 << 30;
   const unsigned grid = (unsigned)std::min<int64_t>(items, sms);
-  gemm_tma_chunked<TN, NP, ROWB, EW><<<grid, CC::THREADS, CC::SMEM, s>>>(ma, mb, C, d, kp, z[0], z[1], z[2], z[3],
-                                                                          out_flags, sio, chunk, fold, bf16, err, ba, bb);
-  return cudaGetLastError();
+  return launch_overlapped(gemm_tma_chunked<TN, NP, ROWB, EW>, dim3(grid), dim3(CC::THREADS), CC::SMEM, s, ma, mb, C, d,
+                           kp, z[0], z[1], z[2], z[3], out_flags, sio, chunk, fold, bf16, err, ba, bb);
 }
 
 // Eight epilogue warps where the epilogue dominates a tile (a short K, at
@@ -1533,10 +1536,9 @@ cudaError_t launch_direct_as(const CUtensorMap& mb, const float2* A, float2* C, 
   }
   const unsigned grid = (unsigned)std::min<int64_t>(int64_t(1) << (d.nm - 7), sms);
   const int chunk = NP == 4 ? split_chunk() : 1 << 30;
-  gemm_direct<TN, NP, BF16><<<grid, DC::THREADS, DC::SMEM, s>>>(mb, A, C, d, direct_map(d), maxA, exp_b,
-                                                         (reinterpret_cast<uintptr_t>(A) & 15) == 0,
-                                                         (reinterpret_cast<uintptr_t>(C) & 15) == 0, chunk, err);
-  return cudaGetLastError();
+  const int av = (reinterpret_cast<uintptr_t>(A) & 15) == 0, cv = (reinterpret_cast<uintptr_t>(C) & 15) == 0;
+  return launch_overlapped(gemm_direct<TN, NP, BF16>, dim3(grid), dim3(DC::THREADS), DC::SMEM, s, mb, A, C, d,
+                           direct_map(d), maxA, exp_b, av, cv, chunk, err);
 }
 
 }  // namespace

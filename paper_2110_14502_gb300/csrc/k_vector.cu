@@ -16,6 +16,7 @@
 
 #include <type_traits>
 
+#include "device_common.h"
 #include "kernels.h"
 
 namespace tn {
@@ -109,6 +110,8 @@ __global__ void __launch_bounds__(NT) vector_kernel(const float2* __restrict__ A
   constexpr int cb = PER == 4 ? CH_BITS : CH_BITS_FEW;
   static_assert(NT * PER == 1 << cb, "rows of a CTA");
   const int64_t M = int64_t(1) << d.nm;
+  let_next_start();
+  after_previous();
   const int64_t ulo = blockIdx.y % d.units_lo, uhi = blockIdx.y / d.units_lo;
   A += ulo * d.a_lo + uhi * d.a_hi;
   B += ulo * d.b_lo + uhi * d.b_hi;
@@ -185,6 +188,8 @@ __global__ void __launch_bounds__(NT) vector_wide_kernel(const float2* __restric
   constexpr int K = 1 << NK, N = 1 << NN;
   static_assert(K * N <= 1024, "B must fit in shared memory");
   const int64_t M = int64_t(1) << d.nm;
+  let_next_start();
+  after_previous();
   const int64_t ulo = blockIdx.y % d.units_lo, uhi = blockIdx.y / d.units_lo;
   A += ulo * d.a_lo + uhi * d.a_hi;
   B += ulo * d.b_lo + uhi * d.b_hi;
@@ -268,6 +273,8 @@ __global__ void __launch_bounds__(NT) vector_long_kernel(const float2* __restric
   constexpr int K = 1 << NK, N = 1 << NN;
   static_assert(K * N <= 1024, "B must fit in shared memory");
   const int64_t M = int64_t(1) << d.nm;
+  let_next_start();
+  after_previous();
   const int64_t ulo = blockIdx.y % d.units_lo, uhi = blockIdx.y / d.units_lo;
   A += ulo * d.a_lo + uhi * d.a_hi;
   B += ulo * d.b_lo + uhi * d.b_hi;
@@ -370,6 +377,8 @@ __global__ void __launch_bounds__(SNT) vector_staged_kernel(const float2* __rest
   constexpr int NCH = K / KC;            // stages per row group
   static_assert(K * N <= 1024, "B must fit in shared memory");
   const int64_t M = int64_t(1) << d.nm;
+  let_next_start();
+  after_previous();
   const int64_t ulo = blockIdx.y % d.units_lo, uhi = blockIdx.y / d.units_lo;
   A += ulo * d.a_lo + uhi * d.a_hi;
   B += ulo * d.b_lo + uhi * d.b_hi;
@@ -497,6 +506,8 @@ __global__ void __launch_bounds__(TNT) vector_tile_kernel(const float2* __restri
   constexpr int AE = TILE_ROWS * K, CE = TILE_ROWS * N;
   __shared__ __align__(16) float2 block[AE > CE ? AE : CE];
   __shared__ __align__(16) float4 Bs[K * N];
+  let_next_start();
+  after_previous();
   const int64_t ulo = blockIdx.y % d.units_lo, uhi = blockIdx.y / d.units_lo;
   A += ulo * d.a_lo + uhi * d.a_hi;
   B += ulo * d.b_lo + uhi * d.b_hi;
@@ -751,8 +762,8 @@ cudaError_t launch_tiles(const float2* A, const float2* B, float2* C, const Gemm
   const int cv = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && (d.c_lo & 1) == 0 && (d.c_hi & 1) == 0;
   auto one = [&](auto nn) -> cudaError_t {
     constexpr int NN = decltype(nn)::value;
-    if (im_first) vector_tile_kernel<NK, NN, true><<<g, TNT, 0, s>>>(A, B, C, d, rt, av, cv);
-    else vector_tile_kernel<NK, NN, false><<<g, TNT, 0, s>>>(A, B, C, d, rt, av, cv);
+    if (im_first) launch_overlapped(vector_tile_kernel<NK, NN, true>, g, dim3(TNT), 0, s, A, B, C, d, rt, av, cv);
+    else launch_overlapped(vector_tile_kernel<NK, NN, false>, g, dim3(TNT), 0, s, A, B, C, d, rt, av, cv);
     return cudaGetLastError();
   };
   switch (d.nn) {
@@ -782,13 +793,13 @@ cudaError_t launch_staged(const float2* A, const float2* B, float2* C, const Gem
   const int cb = chunk_bits(d);
   const dim3 g = chunk_grid(d, cb);
   switch (d.nn) {
-    case 0: vector_staged_kernel<NK, 0><<<g, SNT, 0, s>>>(A, B, C, d, mb, cb); break;
-    case 1: vector_staged_kernel<NK, 1><<<g, SNT, 0, s>>>(A, B, C, d, mb, cb); break;
-    case 2: vector_staged_kernel<NK, 2><<<g, SNT, 0, s>>>(A, B, C, d, mb, cb); break;
-    case 3: vector_staged_kernel<NK, 3><<<g, SNT, 0, s>>>(A, B, C, d, mb, cb); break;
+    case 0: launch_overlapped(vector_staged_kernel<NK, 0>, g, dim3(SNT), 0, s, A, B, C, d, mb, cb); break;
+    case 1: launch_overlapped(vector_staged_kernel<NK, 1>, g, dim3(SNT), 0, s, A, B, C, d, mb, cb); break;
+    case 2: launch_overlapped(vector_staged_kernel<NK, 2>, g, dim3(SNT), 0, s, A, B, C, d, mb, cb); break;
+    case 3: launch_overlapped(vector_staged_kernel<NK, 3>, g, dim3(SNT), 0, s, A, B, C, d, mb, cb); break;
     case 4:
       if constexpr (NK <= 4) {
-        vector_staged_kernel<NK, 4><<<g, SNT, 0, s>>>(A, B, C, d, mb, cb);
+        launch_overlapped(vector_staged_kernel<NK, 4>, g, dim3(SNT), 0, s, A, B, C, d, mb, cb);
         break;
       }
       return cudaErrorInvalidValue;
@@ -807,10 +818,10 @@ cudaError_t launch_long(const float2* A, const float2* B, float2* C, const GemmD
   const int pair_k = d.nk >= 1 && d.ak[0] == 1 && (reinterpret_cast<uintptr_t>(A) & 15) == 0 &&
                      (d.a_lo & 1) == 0 && (d.a_hi & 1) == 0;
   switch (d.nn) {
-    case 0: vector_long_kernel<NK, 0><<<g, NT, 0, s>>>(A, B, C, d, pair_k, mb, cb); break;
-    case 1: vector_long_kernel<NK, 1><<<g, NT, 0, s>>>(A, B, C, d, pair_k, mb, cb); break;
-    case 2: vector_long_kernel<NK, 2><<<g, NT, 0, s>>>(A, B, C, d, pair_k, mb, cb); break;
-    case 3: vector_long_kernel<NK, 3><<<g, NT, 0, s>>>(A, B, C, d, pair_k, mb, cb); break;
+    case 0: launch_overlapped(vector_long_kernel<NK, 0>, g, dim3(NT), 0, s, A, B, C, d, pair_k, mb, cb); break;
+    case 1: launch_overlapped(vector_long_kernel<NK, 1>, g, dim3(NT), 0, s, A, B, C, d, pair_k, mb, cb); break;
+    case 2: launch_overlapped(vector_long_kernel<NK, 2>, g, dim3(NT), 0, s, A, B, C, d, pair_k, mb, cb); break;
+    case 3: launch_overlapped(vector_long_kernel<NK, 3>, g, dim3(NT), 0, s, A, B, C, d, pair_k, mb, cb); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -822,8 +833,8 @@ cudaError_t launch_nn(const float2* A, const float2* B, float2* C, const GemmDes
   const dim3 g = chunk_grid(d, cb);
   auto one = [&](auto nn) {
     constexpr int NN = decltype(nn)::value;
-    if (cb == CH_BITS) vector_kernel<NK, NN, 4><<<g, NT, 0, s>>>(A, B, C, d, mb);
-    else vector_kernel<NK, NN, 1><<<g, NT, 0, s>>>(A, B, C, d, mb);
+    if (cb == CH_BITS) launch_overlapped(vector_kernel<NK, NN, 4>, g, dim3(NT), 0, s, A, B, C, d, mb);
+    else launch_overlapped(vector_kernel<NK, NN, 1>, g, dim3(NT), 0, s, A, B, C, d, mb);
   };
   switch (d.nn) {
     case 0: one(std::integral_constant<int, 0>{}); break;
@@ -860,7 +871,7 @@ cudaError_t launch_wide(const float2* A, const float2* B, float2* C, const GemmD
   auto one = [&](auto nn) -> cudaError_t {
     constexpr int NN = decltype(nn)::value;
     if constexpr (((1 << NK) << NN) <= 1024) {
-      vector_wide_kernel<NK, NN><<<g, NT, 0, s>>>(A, B, C, d, mb, pair_k, cb);
+      launch_overlapped(vector_wide_kernel<NK, NN>, g, dim3(NT), 0, s, A, B, C, d, mb, pair_k, cb);
       return cudaGetLastError();
     } else {
       return cudaErrorInvalidValue;
