@@ -1,6 +1,8 @@
 // Device helpers shared by the kernels.
 #pragma once
 
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <utility>
@@ -50,6 +52,73 @@ struct Pow2 {
   }
   __device__ float operator()(float x) const { return direct ? x * f : ldexpf(x, e); }
 };
+
+// Packed FP32: two values per instruction.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Eight complex values (consecutive in K order) as NP 16-bit planes of 16 bytes:
+// four planes, x = hi + lo with hi = rn16(x) and lo = rn16(x - hi), in the order
+// re_hi, re_lo, im_hi, im_lo; or two, x rounded once, re, im.
+template <int NP, bool BF16>
+__device__ __forceinline__ void planes8(const f32x2 (&v)[8], uint4 (&out)[NP]) {
+  uint32_t hi[8], lo[8];  // re | im << 16
+  const f32x2 minus = pack2(-1.f, -1.f);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const float2 x = unpack2(v[j]);
+    float2 f;
+    if (BF16) {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(x.x, x.y);
+      hi[j] = *reinterpret_cast<const uint32_t*>(&h);
+      f = __bfloat1622float2(h);
+    } else {
+      const __half2 h = __floats2half2_rn(x.x, x.y);
+      hi[j] = *reinterpret_cast<const uint32_t*>(&h);
+      f = __half22float2(h);
+    }
+    if (NP == 4) {
+      const float2 d = unpack2(fma2(pack2(f.x, f.y), minus, v[j]));  // x - hi, rounded once
+      if (BF16) {
+        const __nv_bfloat162 l = __floats2bfloat162_rn(d.x, d.y);
+        lo[j] = *reinterpret_cast<const uint32_t*>(&l);
+      } else {
+        const __half2 l = __floats2half2_rn(d.x, d.y);
+        lo[j] = *reinterpret_cast<const uint32_t*>(&l);
+      }
+    }
+  }
+  auto row = [](const uint32_t* x, unsigned half) {
+    return make_uint4(__byte_perm(x[0], x[1], half), __byte_perm(x[2], x[3], half), __byte_perm(x[4], x[5], half),
+                      __byte_perm(x[6], x[7], half));
+  };
+  constexpr unsigned RE = 0x5410, IM = 0x7632;
+  out[0] = row(hi, RE);
+  out[NP / 2] = row(hi, IM);
+  if (NP == 4) {
+    out[1] = row(lo, RE);
+    out[NP - 1] = row(lo, IM);
+  }
+}
 
 // Exponent putting a maximum into [2^13, 2^14) (0 for none or a non-finite one).
 __device__ __forceinline__ int scale_exponent(float mx) {

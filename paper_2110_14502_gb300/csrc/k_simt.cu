@@ -56,24 +56,11 @@ __device__ __forceinline__ int32_t k_high_offset(int64_t k0, int nk, const int32
   return o;
 }
 
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 pack2(float x, float y) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ float2 unpack2(f32x2 v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
 __device__ __forceinline__ f32x2 swap2(f32x2 v) {
   const float2 r = unpack2(v);
   return pack2(r.y, r.x);
 }
-__device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
-}
+__device__ __forceinline__ void acc2(f32x2& c, f32x2 a, f32x2 b) { c = fma2(a, b, c); }
 
 // One operand tile of R rows x BK K values: what this thread loads, where from
 // and where it goes in shared memory.  Thread t takes row t % R at K positions
@@ -229,9 +216,9 @@ __global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_ker
       for (int i = 0; i < RM; ++i) {
         const ulonglong2 a = at[kk * BM + i];
 #pragma unroll
-        for (int j = 0; j < RN; ++j) fma2(acc[i][j], a.x, b[j]);
+        for (int j = 0; j < RN; ++j) acc2(acc[i][j], a.x, b[j]);
 #pragma unroll
-        for (int j = 0; j < RN; ++j) fma2(acc[i][j], a.y, bs[j]);
+        for (int j = 0; j < RN; ++j) acc2(acc[i][j], a.y, bs[j]);
       }
     };
     if (kn == BK) {

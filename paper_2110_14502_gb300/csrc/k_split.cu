@@ -9,9 +9,6 @@
 // Mixed-Precision Computation Method via Adaptive Precision Scaling" (half
 // precision operands: here each value is split as x = hi + lo,
 // hi = rn16(x), lo = rn16(x - hi)).
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
 #include <algorithm>
 #include <type_traits>
 
@@ -64,48 +61,6 @@ __global__ void __launch_bounds__(NT) max_kernel(const float2* __restrict__ src,
   if (threadIdx.x == 0) {
     for (int w = 1; w < NT / 32; ++w) m = fmaxf(m, wm[w]);
     atomicMax(maxbits + z, __float_as_uint(m));
-  }
-}
-
-// Eight elements (consecutive in K order) as one 16-byte store per plane: x = hi
-// + lo, hi = rn16(x), lo = rn16(x - hi), or x rounded once.
-template <int NP, bool BF16>
-__device__ __forceinline__ void store8(uint16_t* out, int64_t plane, const float2* v) {
-  uint32_t hi[8], lo[8];  // re | im << 16
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    if (BF16) {
-      const __nv_bfloat162 h = __floats2bfloat162_rn(v[j].x, v[j].y);
-      hi[j] = *reinterpret_cast<const uint32_t*>(&h);
-      if (NP == 4) {
-        const float2 f = __bfloat1622float2(h);
-        const __nv_bfloat162 l = __floats2bfloat162_rn(v[j].x - f.x, v[j].y - f.y);
-        lo[j] = *reinterpret_cast<const uint32_t*>(&l);
-      }
-    } else {
-      const __half2 h = __floats2half2_rn(v[j].x, v[j].y);
-      hi[j] = *reinterpret_cast<const uint32_t*>(&h);
-      if (NP == 4) {
-        const float2 f = __half22float2(h);
-        const __half2 l = __floats2half2_rn(v[j].x - f.x, v[j].y - f.y);
-        lo[j] = *reinterpret_cast<const uint32_t*>(&l);
-      }
-    }
-  }
-  auto put = [&](int p, const uint32_t* x, unsigned half) {
-    *reinterpret_cast<uint4*>(out + p * plane) =
-        make_uint4(__byte_perm(x[0], x[1], half), __byte_perm(x[2], x[3], half), __byte_perm(x[4], x[5], half),
-                   __byte_perm(x[6], x[7], half));
-  };
-  constexpr unsigned RE = 0x5410, IM = 0x7632;
-  if (NP == 4) {
-    put(0, hi, RE);
-    put(1, lo, RE);
-    put(2, hi, IM);
-    put(3, lo, IM);
-  } else {
-    put(0, hi, RE);
-    put(1, hi, IM);
   }
 }
 
@@ -228,22 +183,28 @@ __device__ __forceinline__ void split_tile(const SplitJob& job, const TileMap& t
           slot ^= tm.out_slot[b];
           o += int64_t(1) << tm.dst[b];
         }
-      float2 v[8];
+      f32x2 v[8];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const float4 y = *reinterpret_cast<const float4*>(&tile[slot ^ (2 * c)]);
-        v[2 * c] = make_float2(y.x, y.y);
-        v[2 * c + 1] = make_float2(y.z, y.w);
+        const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(&tile[slot ^ (2 * c)]);
+        v[2 * c] = y.x;
+        v[2 * c + 1] = y.y;
       }
       // (one multiply but for exponents out of a float's range)
       if (sc.direct) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = make_float2(v[j].x * sc.f, v[j].y * sc.f);
+        for (int j = 0; j < 8; ++j) v[j] = mul2(v[j], pack2(sc.f, sc.f));
       } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = make_float2(sc(v[j].x), sc(v[j].y));
+        for (int j = 0; j < 8; ++j) {
+          const float2 x = unpack2(v[j]);
+          v[j] = pack2(sc(x.x), sc(x.y));
+        }
       }
-      store8<NP, BF16>(out + o, plane, v);
+      uint4 p[NP];
+      planes8<NP, BF16>(v, p);
+#pragma unroll
+      for (int i = 0; i < NP; ++i) *reinterpret_cast<uint4*>(out + o + i * plane) = p[i];
     }
   }
 }

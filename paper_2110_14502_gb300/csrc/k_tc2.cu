@@ -314,7 +314,7 @@ __device__ __forceinline__ void store_planes(uint16_t* P, int64_t plane, const i
 }
 
 // x0 f and x1 f in one instruction (x as register bits).
-__device__ __forceinline__ void mul2(uint32_t x0, uint32_t x1, float f, float& y0, float& y1) {
+__device__ __forceinline__ void mul_pair(uint32_t x0, uint32_t x1, float f, float& y0, float& y1) {
   asm("{\n .reg .b64 a, b;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %4};\n mul.rn.f32x2 a, a, b;\n mov.b64 {%0, %1}, a;\n}\n"
       : "=f"(y0), "=f"(y1)
       : "r"(x0), "r"(x1), "f"(f));
@@ -855,8 +855,8 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
         if (sc.direct) {
 #pragma unroll
           for (int jj = 0; jj < 16; jj += 2) {
-            mul2(ur[jj], ur[jj + 1], sc.f, vr[jj], vr[jj + 1]);
-            mul2(ui[jj], ui[jj + 1], sc.f, vi[jj], vi[jj + 1]);
+            mul_pair(ur[jj], ur[jj + 1], sc.f, vr[jj], vr[jj + 1]);
+            mul_pair(ui[jj], ui[jj + 1], sc.f, vi[jj], vi[jj + 1]);
           }
         } else {
 #pragma unroll
@@ -1000,8 +1000,10 @@ struct DirectCfg {
 
 // The tile's index bits (K bits 0..4, then row bits 0..6 of the descriptor) in
 // A's order: stride and shared slot; and the slots in tile order.
+// in_off, in_put: the sums over A's order bits 9..11.
 struct DirectMap {
   int32_t in_src[12], in_slot[12], out_slot[12];
+  int32_t in_off[8], in_put[8];
 };
 
 __device__ __forceinline__ bool workers_any(bool failed) {  // barrier of the 256 workers
@@ -1178,7 +1180,7 @@ __global__ void __launch_bounds__(DirectCfg<TN, NP>::THREADS, 1)
       const float2* src = A + so + bit_sum(it << 7, my_am) + bit_sum(kt << 5, my_ak);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const float2* p = src + ((j & 1) ? dm.in_src[9] : 0) + ((j & 2) ? dm.in_src[10] : 0) + ((j & 4) ? dm.in_src[11] : 0);
+        const float2* p = src + dm.in_off[j];
         if (a_vec) {
           pf[j] = __ldg(reinterpret_cast<const float4*>(p));
         } else {
@@ -1187,7 +1189,9 @@ __global__ void __launch_bounds__(DirectCfg<TN, NP>::THREADS, 1)
         }
       }
     };
-    // conversions: K octets t and t + 256 of the tile: octet o = row o / 4, K chunk o % 4
+    // conversions: K octets t and t + 256 of the tile: octet o = row o / 4, K chunk
+    // o % 4, i.e. rows t / 4 and t / 4 + 64, whose swizzles agree
+    const int oplace = (t >> 2) * 64 + (((t & 3) ^ ((t >> 3) & 3)) << 4);
     int32_t oslot[2];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
@@ -1263,8 +1267,7 @@ __global__ void __launch_bounds__(DirectCfg<TN, NP>::THREADS, 1)
           auto land = [&](float4(&pf)[8]) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-              const int32_t p = slot ^ ((j & 1) ? dm.in_slot[9] : 0) ^ ((j & 2) ? dm.in_slot[10] : 0) ^
-                                ((j & 4) ? dm.in_slot[11] : 0);
+              const int32_t p = slot ^ dm.in_put[j];
               tile[p] = make_float2(pf[j].x, pf[j].y);
               tile[p ^ dm.in_slot[0]] = make_float2(pf[j].z, pf[j].w);
             }
@@ -1286,36 +1289,34 @@ __global__ void __launch_bounds__(DirectCfg<TN, NP>::THREADS, 1)
           }
           uint8_t* const st = smem + s * CF::STAGE;
           // (the shift is a single multiply but for exponents out of range)
-          auto convert = [&](auto scale4) {
+          auto convert = [&](auto scale) {
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-              const int o = t + 256 * u, row = o >> 2;
-              uint32_t x[NP / 2][8];
+              f32x2 x[8];
 #pragma unroll
               for (int v = 0; v < 4; ++v) {
-                const float4 y = scale4(sa, *reinterpret_cast<const float4*>(&tile[oslot[u] ^ (2 * v)]));
-                uint32_t e0[NP / 2], e1[NP / 2];
-                pack_planes<NP>(BF16, y.x, y.y, e0);
-                pack_planes<NP>(BF16, y.z, y.w, e1);
-#pragma unroll
-                for (int a = 0; a < NP / 2; ++a) {
-                  x[a][2 * v] = e0[a];
-                  x[a][2 * v + 1] = e1[a];
-                }
+                const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(&tile[oslot[u] ^ (2 * v)]);
+                x[2 * v] = scale(y.x);
+                x[2 * v + 1] = scale(y.y);
               }
+              uint4 p[NP];
+              planes8<NP, BF16>(x, p);
               // 64-byte rows, 16-byte chunks swizzled by row bits 1, 2
-              uint8_t* const to = st + row * 64 + (((o & 3) ^ ((row >> 1) & 3)) << 4);
 #pragma unroll
-              for (int p = 0; p < NP; ++p) {
-                auto pp = [&](int e) { return __byte_perm(x[p >> 1][e], x[p >> 1][e + 1], (p & 1) ? 0x7632 : 0x5410); };
-                *reinterpret_cast<uint4*>(to + p * CF::A_PLANE) = make_uint4(pp(0), pp(2), pp(4), pp(6));
-              }
+              for (int i = 0; i < NP; ++i) *reinterpret_cast<uint4*>(st + oplace + u * 64 * 64 + i * CF::A_PLANE) = p[i];
             }
           };
-          if (sa.direct)
-            convert([](const Pow2& m, float4 y) { return make_float4(y.x * m.f, y.y * m.f, y.z * m.f, y.w * m.f); });
-          else
-            convert([](const Pow2& m, float4 y) { return make_float4(m(y.x), m(y.y), m(y.z), m(y.w)); });
+          if (sa.direct && sa.f == 1.f) {
+            convert([](f32x2 y) { return y; });
+          } else if (sa.direct) {
+            const f32x2 f = pack2(sa.f, sa.f);
+            convert([&](f32x2 y) { return mul2(y, f); });
+          } else {
+            convert([&](f32x2 y) {
+              const float2 v = unpack2(y);
+              return pack2(sa(v.x), sa(v.y));
+            });
+          }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the tensor core's reads
           __syncwarp();
           if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full_a[s])) : "memory");
@@ -1355,8 +1356,8 @@ __global__ void __launch_bounds__(DirectCfg<TN, NP>::THREADS, 1)
         if (sc.direct) {
 #pragma unroll
           for (int jj = 0; jj < 16; jj += 2) {
-            mul2(ur[jj], ur[jj + 1], sc.f, vr[jj], vr[jj + 1]);
-            mul2(ui[jj], ui[jj + 1], sc.f, vi[jj], vi[jj + 1]);
+            mul_pair(ur[jj], ur[jj + 1], sc.f, vr[jj], vr[jj + 1]);
+            mul_pair(ui[jj], ui[jj + 1], sc.f, vi[jj], vi[jj + 1]);
           }
         } else {
 #pragma unroll
@@ -1519,6 +1520,12 @@ DirectMap direct_map(const GemmDesc& d) {
     m.in_src[l] = st[order[l]];
     m.in_slot[l] = m.out_slot[order[l]];
   }
+  for (int j = 0; j < 8; ++j)
+    for (int b = 0; b < 3; ++b)
+      if ((j >> b) & 1) {
+        m.in_off[j] += m.in_src[9 + b];
+        m.in_put[j] ^= m.in_slot[9 + b];
+      }
   return m;
 }
 

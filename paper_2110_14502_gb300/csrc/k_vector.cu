@@ -488,15 +488,7 @@ struct RowTile {
   int32_t row_slot[TILE_BITS], col_slot[4];             // images of the row and column bits in the block of C
 };
 
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 pack2(float x, float y) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
-}
+__device__ __forceinline__ void acc2(f32x2& c, f32x2 a, f32x2 b) { c = fma2(a, b, c); }
 
 template <int NK, int NN, bool IM_FIRST>
 __global__ void __launch_bounds__(TNT) vector_tile_kernel(const float2* __restrict__ A, const float2* __restrict__ B,
@@ -577,15 +569,15 @@ __global__ void __launch_bounds__(TNT) vector_tile_kernel(const float2* __restri
     for (int n = 0; n < N; ++n) {
       const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&Bs[k * N + n]);
       if (IM_FIRST) {
-        fma2(acc[0][n], im0, b.y);
-        fma2(acc[1][n], im1, b.y);
-        fma2(acc[0][n], re0, b.x);
-        fma2(acc[1][n], re1, b.x);
+        acc2(acc[0][n], im0, b.y);
+        acc2(acc[1][n], im1, b.y);
+        acc2(acc[0][n], re0, b.x);
+        acc2(acc[1][n], re1, b.x);
       } else {
-        fma2(acc[0][n], re0, b.x);
-        fma2(acc[1][n], re1, b.x);
-        fma2(acc[0][n], im0, b.y);
-        fma2(acc[1][n], im1, b.y);
+        acc2(acc[0][n], re0, b.x);
+        acc2(acc[1][n], re1, b.x);
+        acc2(acc[0][n], im0, b.y);
+        acc2(acc[1][n], im1, b.y);
       }
     }
   };
