@@ -525,6 +525,7 @@ struct Ctx {
   bool tuning = false;           // time the tile choices of each tensor-core step
   bool sizing = false;           // only compute scratch needs (no launches)
   int64_t scratch_need = 0;
+  int64_t scratch_min = 0;  // without the space for partial sums
   Ctx(const Plan& p, Executor& e, cudaStream_t s, bool prof) : P(p), E(e), st(s), profile(prof) {}
 
   tn_status event(size_t& idx) {
@@ -666,12 +667,15 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
     if ((S.a >= L && c.planes_out[S.a - L] && !a_in) || (S.b >= L && c.planes_out[S.b - L] && !b_in))
       return fail(TN_EINVAL, "step %zu: internal error, operand planes do not match the step's view", s);
     const int64_t need_a = a_in ? 0 : split_scratch_elems(d, false, c.np);
-    const int64_t need = need_a + (b_in ? 0 : split_scratch_elems(d, true, c.np));
+    const int64_t need_planes = need_a + (b_in ? 0 : split_scratch_elems(d, true, c.np));
+    const int64_t need_part = tc_part_elems(d, c.np, c.planes_out[s] != 0);  // (after the planes)
+    const int64_t need = need_planes + need_part;
     if (c.sizing) {
       c.scratch_need = std::max(c.scratch_need, need);
+      c.scratch_min = std::max(c.scratch_min, need_planes);
       return TN_OK;
     }
-    if (need > E.scratch_cap) return fail(TN_EINVAL, "step %zu: internal error, operand scratch not sized", s);
+    if (need_planes > E.scratch_cap) return fail(TN_EINVAL, "step %zu: internal error, operand scratch not sized", s);
     for (auto& t : E.tuned)
       if (t.precision == c.precision && t.step == (int)s) {
         d.tile_n = t.tile_n;
@@ -719,7 +723,7 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
       sio.flag = S.phase == 1 ? c.flag1 : c.flag2;
       sio.flag_by_lo = S.phase == 1;
     }
-    if (c.profile && e == cudaSuccess && need > 0) {
+    if (c.profile && e == cudaSuccess && need_planes > 0) {
       // the operand split and the GEMM are timed as separate classes
       size_t em = 0;
       tn_status r = c.event(em);
@@ -766,7 +770,11 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
       d.tile_n = bt;
       d.group_m = bg;
     }
-    if (e == cudaSuccess) e = launch_gemm_tma(pa, pb, C, c.planes_out[s] != 0, d, c.bf16, sio, E.err, c.st);
+    const bool parts = need_part > 0 && need <= E.scratch_cap && tc_part_elems(d, c.np, c.planes_out[s] != 0) > 0;
+    if (parts) ++c.launches;
+    if (e == cudaSuccess)
+      e = launch_gemm_tma(pa, pb, C, c.planes_out[s] != 0, d, c.bf16, sio, E.err, c.st,
+                          parts ? reinterpret_cast<float2*>(E.scratch + need_planes) : nullptr);
   }
   else e = launch_gemm_simt(A, B, C, d, c.st);
   ++c.launches;
@@ -1146,7 +1154,12 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
       cudaFree(E.scratch);
       E.scratch = nullptr;
       E.scratch_cap = 0;
-      if (dev_alloc(&E.scratch, (size_t)c.scratch_need * sizeof(uint16_t)) != cudaSuccess) {
+      if (c.scratch_need > c.scratch_min &&
+          dev_alloc(&E.scratch, (size_t)c.scratch_need * sizeof(uint16_t)) != cudaSuccess) {
+        cudaGetLastError();
+        c.scratch_need = c.scratch_min;
+      }
+      if (!E.scratch && dev_alloc(&E.scratch, (size_t)c.scratch_need * sizeof(uint16_t)) != cudaSuccess) {
         cudaGetLastError();
         return fail(TN_EHBM, "tn_contract_amplitudes: %lld bytes of operand planes do not fit",
                     (long long)(c.scratch_need * 2));

@@ -19,6 +19,10 @@
 // stores need no permutation.  Each output adds its products with k ascending
 // in the order of the kernel that would run the step alone, so results do not
 // depend on which steps share a launch.
+//
+// Measured on the sixteen steps of a 4 x 4 circuit, one unit: sixteen launches
+// 115 us of kernel time, this kernel 26; the whole call 160 -> 102 us (150 with
+// the operands read through their strides instead of from shared memory).
 #include <algorithm>
 #include <mutex>
 
@@ -162,9 +166,10 @@ constexpr int CHAIN_SMEM = 2 * (1 << kChainMaxOperand) * (int)sizeof(float2);
 }  // namespace
 
 bool chain_shape_ok(const GemmDesc& d, int64_t units) {
-  // One CTA runs a step alone: with few units that beats a launch (2-3 us) up
-  // to 2^16 multiply-adds; with enough units to fill the chip the step's own
-  // kernel, which tiles and streams, wins earlier.
+  // One CTA runs a step alone: with few units that beats a launch (2-3 us, and
+  // 12 us for a 2^5 x 2^4 x 2^7 step in the FP32 GEMM) up to 2^16 multiply-adds;
+  // with enough units to fill the chip the step's own kernel, which tiles and
+  // streams, wins earlier.
   const int limit = units <= 4 ? 16 : units < 152 ? 15 : 12;
   return d.nm + d.nn <= kChainMaxC && d.nk <= kChainMaxK && d.nm + d.nk <= kChainMaxOperand &&
          d.nn + d.nk <= kChainMaxOperand && d.nm + d.nn + d.nk <= limit && !reduce_shape_ok(d);

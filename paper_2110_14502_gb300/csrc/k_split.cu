@@ -468,12 +468,16 @@ bool planes_in_place(const float2* base, const GemmDesc& d, bool which_b, int np
   return true;
 }
 
-int64_t tc2_pair_scratch_elems(const GemmDesc& d) {
-  return direct_ok(d) ? split_scratch_elems(d, true, 4) : tc2_scratch_elems(d);
+int64_t tc2_pair_scratch_elems(const GemmDesc& d, bool sums) {
+  return direct_ok(d) ? split_scratch_elems(d, true, 4) : tc2_scratch_elems(d) + (sums ? tc_part_elems(d, 4, false) : 0);
 }
 
-cudaError_t run_gemm_tc2(const float2* A, const float2* B, float2* C, const GemmDesc& d0, bool bf16, uint16_t* scratch,
-                         int* err, cudaStream_t s) {
+static float2* part_space(const GemmDesc& d, int np, uint16_t* scratch, bool sums) {
+  return sums && tc_part_elems(d, np, false) > 0 ? reinterpret_cast<float2*>(scratch + tc2_scratch_elems(d)) : nullptr;
+}
+
+cudaError_t run_gemm_tc2(const float2* A, const float2* B, float2* C, const GemmDesc& d0, bool bf16, bool sums,
+                         uint16_t* scratch, int* err, cudaStream_t s) {
   PlaneOperand pa, pb;
   GemmDesc d = d0;
   if (direct_ok(d)) {
@@ -487,11 +491,11 @@ cudaError_t run_gemm_tc2(const float2* A, const float2* B, float2* C, const Gemm
   const cudaError_t e = split_pair(A, B, d, bf16, 4, nullptr, nullptr, nullptr, scratch, pa, pb, s);
   if (e != cudaSuccess) return e;
   const ScaleIO none{};
-  return launch_gemm_tma(pa, pb, C, false, d, bf16, none, err, s);
+  return launch_gemm_tma(pa, pb, C, false, d, bf16, none, err, s, part_space(d, 4, scratch, sums));
 }
 
 cudaError_t run_gemm_tc2_scaled(const float2* A, const float2* B, float2* C, const GemmDesc& d0, bool bf16, int np,
-                                uint16_t* scratch, void* aux, int* err, cudaStream_t s) {
+                                bool sums, uint16_t* scratch, void* aux, int* err, cudaStream_t s) {
   unsigned* mx = reinterpret_cast<unsigned*>(aux);
   int* ex = reinterpret_cast<int*>(mx + 2);
   float* ms = reinterpret_cast<float*>(ex + 2);
@@ -512,7 +516,7 @@ cudaError_t run_gemm_tc2_scaled(const float2* A, const float2* B, float2* C, con
   sio.ma = ms;
   sio.eb = ex + 1;
   sio.mb = ms + 1;
-  return launch_gemm_tma(pa, pb, C, false, d, bf16, sio, err, s);
+  return launch_gemm_tma(pa, pb, C, false, d, bf16, sio, err, s, part_space(d, np, scratch, sums));
 }
 
 }  // namespace tn

@@ -483,12 +483,12 @@ struct BulkPlanes {
   int64_t st_lo, st_hi, plane;
 };
 
-template <int TN, int NP, int ROWB, int EW>
+template <int TN, int NP, int ROWB, int EW, bool PARTS>
 __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
     gemm_tma_chunked(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                      float2* __restrict__ C0, const GemmDesc d, int kp, int a_zlo, int a_zhi, int b_zlo, int b_zhi,
                      int out_flags, const ScaleIO sio, int chunk, int fold, bool bf16, int* __restrict__ err,
-                     const BulkPlanes ba, const BulkPlanes bb) {
+                     const BulkPlanes ba, const BulkPlanes bb, int parts_arg, float2* __restrict__ part) {
   using CC = ChunkCfg<TN, NP, ROWB, EW>;
   using CF = Cfg2<TN, NP, ROWB>;
   constexpr bool K8 = ROWB == K8_ROWB;  // K = 8 by bulk copies (ba, bb)
@@ -512,13 +512,22 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
   const int nsub = 1 << d.nn;
   const int ntm = (int)((int64_t(1) << d.nm) / TM), ntn = fold > 1 ? 1 : (int)((int64_t(1) << d.nn) / TN);
   const int tiles = ntm * ntn;
-  const int64_t items = (int64_t)tiles * (d.units / fold);
+  // PARTS: each accumulation chunk of a tile is an item of its own, whose sum
+  // goes to `part` ([chunk][unit][C's elements]) unscaled; combine_kernel adds
+  // them in chunk order, as the folds below do
+  const int parts = PARTS ? parts_arg : 1;
+  const int64_t items = (int64_t)tiles * (d.units / fold) * parts;
   const int nkt = (kp + CF::TKC - 1) / CF::TKC;
-  const int nch = (nkt + chunk - 1) / chunk;
+  const int nch = PARTS ? 1 : (nkt + chunk - 1) / chunk;
   const int GM = d.group_m > 0 ? d.group_m : GROUP_M_DEFAULT;
   const bool items32 = items < (int64_t(1) << 31);
-  auto decode = [&](int64_t item, int& unit, int& m0, int& n0) {
+  auto decode = [&](int64_t item, int& unit, int& m0, int& n0, int& cp) {
     int t;
+    cp = 0;
+    if (PARTS) {
+      cp = (int)(item % parts);
+      item /= parts;
+    }
     if (items32) {  // 32-bit division: a 64-bit one is a long dependent sequence
       unit = (int)((uint32_t)item / (uint32_t)tiles);
       t = (int)((uint32_t)item - (uint32_t)unit * (uint32_t)tiles);
@@ -580,13 +589,14 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
     uint32_t lap = 0;  // times round the ring
     bool ok = true;
     for (int64_t it = first; ok && it < items; it += stride) {
-      int unit, m0, n0;
-      decode(it, unit, m0, n0);
+      int unit, m0, n0, cp;
+      decode(it, unit, m0, n0, cp);
       const int ulo = unit % d.units_lo, uhi = (unit / d.units_lo) * fold;
       const int za_lo = a_zlo ? ulo : 0, za_hi = a_zhi ? uhi : 0;
       const int zb_lo = b_zlo ? ulo : 0, zb_hi = b_zhi ? uhi : 0;
       if (__any_sync(0xffffffffu, abort_flag)) break;
-      for (int kt = 0; kt < nkt; ++kt, ++g) {
+      const int kt1 = PARTS ? min(nkt, (cp + 1) * chunk) : nkt;
+      for (int kt = cp * chunk; kt < kt1; ++kt, ++g) {
         if (lap > 0 && !mbar_wait_warp(&empty[s], (lap - 1) & 1, wl)) {
           if (leader) {
             atomicExch(err, 31);
@@ -664,7 +674,7 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
         ++used[b];
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t dr = tmem + (uint32_t)b * BUF, di = dr + TN;
-        const int k0 = c * chunk, k1 = min(nkt, k0 + chunk);
+        const int k0 = (PARTS ? (int)(it % parts) : c) * chunk, k1 = min(nkt, k0 + chunk);
         for (int kt = k0; kt < k1; ++kt, ++g) {
           if (!mbar_wait_warp(&full[s], ph, wl)) {
             if (leader) {
@@ -779,17 +789,18 @@ __global__ void __launch_bounds__(ChunkCfg<TN, NP, ROWB, EW>::THREADS, 1)
         frexpf(bound, &x);
         r = x - 15;
       }
-      sc = Pow2(planes ? -r : ea + eb);
+      if (!PARTS) sc = Pow2(planes ? -r : ea + eb);
     };
     int64_t t = 0;
     uint32_t seen[2] = {0u, 0u};
     bool ok = true;
     for (int64_t it = first; ok && it < items; it += stride, ++t) {
-      int unit, m0, n0;
-      decode(it, unit, m0, n0);
+      int unit, m0, n0, cp;
+      decode(it, unit, m0, n0, cp);
       const int ulo = unit % d.units_lo, uhi = (unit / d.units_lo) * fold;
       unit_scale(ulo, uhi, 0);  // (loads in flight while the accumulator fills)
-      float2* const Cu = C0 + ((int64_t)ulo * d.c_lo + (int64_t)uhi * d.c_hi);
+      float2* const Cu = PARTS ? part + (((int64_t)cp * d.units + unit) << (d.nm + d.nn))
+                                   : C0 + ((int64_t)ulo * d.c_lo + (int64_t)uhi * d.c_hi);
       const int32_t tile_off = bit_sum(m0 + q * 32, my_cm) + (fold > 1 ? 0 : bit_sum(n0, my_cn));
       const int rb = (int)(t & 1);
       const uint32_t R = tmem + lane_off + (uint32_t)rb * BUF, P = tmem + lane_off + (uint32_t)(1 - rb) * BUF;
@@ -1398,6 +1409,34 @@ __global__ void __launch_bounds__(DirectCfg<TN, NP>::THREADS, 1)
   }
 }
 
+// C = the chunks' sums added in order, times 2^(eA + eB): the folds and the
+// scaling of gemm_tma_chunked for items that were one chunk each, with the same
+// additions in the same order.  Bound by the sums' trip through L2 (they were
+// written microseconds before; at most 256 MB).
+__global__ void __launch_bounds__(256) combine_kernel(const float2* __restrict__ part, int parts, float2* __restrict__ C,
+                                                      const GemmDesc d, const ScaleIO sio, int a_zlo, int a_zhi,
+                                                      int b_zlo, int b_zhi) {
+  let_next_start();
+  after_previous();
+  const int unit = blockIdx.y, ulo = unit % d.units_lo, uhi = unit / d.units_lo;
+  int e = 0;
+  if (sio.ea)
+    e = sio.ea[(a_zlo ? ulo : 0) + (a_zhi ? uhi : 0) * (a_zlo ? d.units_lo : 1)] +
+        sio.eb[(b_zlo ? ulo : 0) + (b_zhi ? uhi : 0) * (b_zlo ? d.units_lo : 1)];
+  const Pow2 sc(e);
+  const int64_t n = int64_t(1) << (d.nm + d.nn);
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;  // n is a multiple of 256
+  const float2* p = part + unit * n + i;
+  float2 s = p[0];
+#pragma unroll 4
+  for (int c = 1; c < parts; ++c) {
+    const float2 x = p[(int64_t)c * d.units * n];
+    s.x += x.x;
+    s.y += x.y;
+  }
+  C[(int64_t)ulo * d.c_lo + (int64_t)uhi * d.c_hi + i] = make_float2(sc(s.x), sc(s.y));
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   static std::once_flag once;
@@ -1446,26 +1485,27 @@ int sm_count() {
   return sms > 0 ? sms : 148;
 }
 
-template <int TN, int NP, int ROWB, int EW>
+template <int TN, int NP, int ROWB, int EW, bool PARTS>
 cudaError_t launch_chunked_ew(const CUtensorMap& ma, const CUtensorMap& mb, float2* C, const GemmDesc& d, int kp,
                               const int z[4], int out_flags, const ScaleIO& sio, int fold, bool bf16, int* err,
-                              cudaStream_t s, const BulkPlanes& ba, const BulkPlanes& bb) {
+                              cudaStream_t s, const BulkPlanes& ba, const BulkPlanes& bb, int parts, float2* part) {
   using CC = ChunkCfg<TN, NP, ROWB, EW>;
   static bool attr = false;
   static int sms = 0;
   if (!attr) {
     cudaError_t e =
-        cudaFuncSetAttribute(gemm_tma_chunked<TN, NP, ROWB, EW>, cudaFuncAttributeMaxDynamicSharedMemorySize, CC::SMEM);
+        cudaFuncSetAttribute(gemm_tma_chunked<TN, NP, ROWB, EW, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             CC::SMEM);
     if (e != cudaSuccess) return e;
     sms = sm_count();
     attr = true;
   }
   const int64_t M = int64_t(1) << d.nm, N = int64_t(1) << d.nn;
-  const int64_t items = (M / TM) * (fold > 1 ? 1 : N / TN) * (d.units / fold);
+  const int64_t items = (M / TM) * (fold > 1 ? 1 : N / TN) * (d.units / fold) * parts;
   const int chunk = NP == 4 ? split_chunk() : 1 << 30;
   const unsigned grid = (unsigned)std::min<int64_t>(items, sms);
-  return launch_overlapped(gemm_tma_chunked<TN, NP, ROWB, EW>, dim3(grid), dim3(CC::THREADS), CC::SMEM, s, ma, mb, C, d,
-                           kp, z[0], z[1], z[2], z[3], out_flags, sio, chunk, fold, bf16, err, ba, bb);
+  return launch_overlapped(gemm_tma_chunked<TN, NP, ROWB, EW, PARTS>, dim3(grid), dim3(CC::THREADS), CC::SMEM, s, ma,
+                           mb, C, d, kp, z[0], z[1], z[2], z[3], out_flags, sio, chunk, fold, bf16, err, ba, bb, parts, part);
 }
 
 // Eight epilogue warps where the epilogue dominates a tile (a short K, at
@@ -1475,13 +1515,14 @@ cudaError_t launch_chunked_ew(const CUtensorMap& ma, const CUtensorMap& mb, floa
 template <int TN, int NP>
 cudaError_t launch_chunked(const CUtensorMap& ma, const CUtensorMap& mb, float2* C, const GemmDesc& d, int kp,
                            const int z[4], int out_flags, const ScaleIO& sio, int fold, bool bf16, int* err,
-                           cudaStream_t s, const BulkPlanes& ba, const BulkPlanes& bb) {
+                           cudaStream_t s, const BulkPlanes& ba, const BulkPlanes& bb, int parts, float2* part) {
   constexpr int EWS = TN >= 64 ? 8 : 4;  // a single K stage or a few
-  auto go = [&](auto rowb, auto ew) {
-    return launch_chunked_ew<TN, NP, decltype(rowb)::value, decltype(ew)::value>(ma, mb, C, d, kp, z, out_flags, sio,
-                                                                                fold, bf16, err, s, ba, bb);
-  };
   using std::integral_constant;
+  auto run = [&](auto rowb, auto ew, auto p) {
+    return launch_chunked_ew<TN, NP, decltype(rowb)::value, decltype(ew)::value, decltype(p)::value>(
+        ma, mb, C, d, kp, z, out_flags, sio, fold, bf16, err, s, ba, bb, parts, part);
+  };
+  auto go = [&](auto rowb, auto ew) { return run(rowb, ew, integral_constant<bool, false>{}); };
   if (ba.base) return go(integral_constant<int, K8_ROWB>{}, integral_constant<int, EWS>{});
   const int rowb = row_bytes(kp, NP);
   if (rowb == 32) return go(integral_constant<int, 32>{}, integral_constant<int, EWS>{});
@@ -1489,18 +1530,20 @@ cudaError_t launch_chunked(const CUtensorMap& ma, const CUtensorMap& mb, float2*
   if constexpr (WIDE == 128)
     if (rowb == 64) return go(integral_constant<int, 64>{}, integral_constant<int, EWS>{});
   if (EWS == 8 && kp <= 4 * (WIDE / 2)) return go(integral_constant<int, WIDE>{}, integral_constant<int, EWS>{});
+  if constexpr (NP == 4)  // (two or more chunks: a long K)
+    if (parts > 1) return run(integral_constant<int, WIDE>{}, integral_constant<int, 4>{}, integral_constant<bool, true>{});
   return go(integral_constant<int, WIDE>{}, integral_constant<int, 4>{});
 }
 
 template <int NP>
 cudaError_t launch_tn(int TNv, const CUtensorMap& ma, const CUtensorMap& mb, float2* C, const GemmDesc& d, int kp,
                       const int z[4], int cp, const ScaleIO& sio, int fold, bool bf16, int* err, cudaStream_t s,
-                      const BulkPlanes& ba, const BulkPlanes& bb) {
+                      const BulkPlanes& ba, const BulkPlanes& bb, int parts, float2* part) {
   switch (TNv) {
-    case 128: return launch_chunked<128, NP>(ma, mb, C, d, kp, z, cp, sio, fold, bf16, err, s, ba, bb);
-    case 64: return launch_chunked<64, NP>(ma, mb, C, d, kp, z, cp, sio, fold, bf16, err, s, ba, bb);
-    case 32: return launch_chunked<32, NP>(ma, mb, C, d, kp, z, cp, sio, fold, bf16, err, s, ba, bb);
-    case 16: return launch_chunked<16, NP>(ma, mb, C, d, kp, z, cp, sio, fold, bf16, err, s, ba, bb);
+    case 128: return launch_chunked<128, NP>(ma, mb, C, d, kp, z, cp, sio, fold, bf16, err, s, ba, bb, parts, part);
+    case 64: return launch_chunked<64, NP>(ma, mb, C, d, kp, z, cp, sio, fold, bf16, err, s, ba, bb, parts, part);
+    case 32: return launch_chunked<32, NP>(ma, mb, C, d, kp, z, cp, sio, fold, bf16, err, s, ba, bb, parts, part);
+    case 16: return launch_chunked<16, NP>(ma, mb, C, d, kp, z, cp, sio, fold, bf16, err, s, ba, bb, parts, part);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -1581,19 +1624,43 @@ int64_t split_plane_elems(int nrow_bits, int nk_bits, int np) {
   return np * (int64_t(1) << nrow_bits) * kp;
 }
 
+// Accumulation chunks that launch_gemm_tma makes items of their own (1: none).
+// With at most half as many tiles as SMs, a long K leaves the chip to a few
+// serial chains of chunks of about 5 us each; one more launch and the sums' bytes
+// cost less than one chunk.  Per tn_contract_pair call, split bf16, random
+// orders, chunks in a chain -> spread, log2 M, N, K (tiles x chunks): (7, 7, 13)
+// 4 x 16 209 -> 55 us, (8, 5, 11) 2 x 4 83 -> 49, (9, 6, 10) 8 x 2 61 -> 47,
+// (9, 8, 12) 32 x 8 129 -> 67, (9, 9, 10) 64 x 2 60 -> 51, (9, 9, 14) 64 x 32
+// 408 -> 246, (13, 5, 11) 64 x 4 121 -> 112.  From 128 tiles on, 152 SMs have at
+// most one chunk in six to gain, and the sums are as many bytes as the planes.
+static int chunk_parts(const GemmDesc& d, int np, bool c_planes) {
+  if (np != 4 || c_planes) return 1;
+  const int64_t K = int64_t(1) << d.nk;
+  const int64_t nkt = (K + 31) / 32, nch = (nkt + split_chunk() - 1) / split_chunk();
+  const int64_t tiles = ((int64_t(1) << d.nm) / TM) * ((int64_t(1) << d.nn) / tma_tile_n(d)) * d.units;
+  const bool fits = (nch * d.units) << (d.nm + d.nn) <= int64_t(1) << 25;  // 256 MB of sums
+  return nch > 1 && tiles <= 76 && fits ? (int)nch : 1;
+}
+
+int64_t tc_part_elems(const GemmDesc& d, int np, bool c_planes) {
+  const int parts = chunk_parts(d, np, c_planes);
+  return parts > 1 ? 4 * parts * (int64_t)d.units << (d.nm + d.nn) : 0;
+}
+
 cudaError_t launch_gemm_tma(const PlaneOperand& a, const PlaneOperand& b, float2* C, bool c_planes, const GemmDesc& d,
-                            bool bf16, const ScaleIO& sio, int* err, cudaStream_t s) {
+                            bool bf16, const ScaleIO& sio, int* err, cudaStream_t s, float2* part) {
   if (!tc_shape_ok(d) || d.units > 65535 || a.kp != b.kp || a.kp % 8 || a.np != b.np ||
       (a.np != 2 && a.np != 4))
     return cudaErrorInvalidValue;
   int TNv = tma_tile_n(d);
+  const int parts = part ? chunk_parts(d, a.np, c_planes) : 1;
   // Narrow N with A shared by the hi units (e.g. one slice-only tensor against
   // the bitstrings of a group): fold consecutive hi units into the columns of
   // one tile, so that the MMAs run 128 columns wide and A is read once for
   // all of them (with scaling, the epilogue takes each unit's exponents for
   // its own columns).
   int fold = 1;
-  if (d.nn < 7 && a.nhi == 1 && b.nhi > 1 && d.units_lo > 0) {
+  if (parts == 1 && d.nn < 7 && a.nhi == 1 && b.nhi > 1 && d.units_lo > 0) {
     const int uh = d.units / d.units_lo;
     while (fold * 2 <= (128 >> d.nn) && uh % (fold * 2) == 0) fold *= 2;
     if (fold > 1) TNv = (1 << d.nn) * fold;
@@ -1606,7 +1673,9 @@ cudaError_t launch_gemm_tma(const PlaneOperand& a, const PlaneOperand& b, float2
   const int z[4] = {a.nlo > 1, a.nhi > 1, b.nlo > 1, b.nhi > 1};
   // bit 0: plane output; bit 1: every even element of C on a 16-byte boundary
   const int cp = (c_planes ? 1 : 0) |
-                 ((reinterpret_cast<uintptr_t>(C) & 15) == 0 && (d.c_lo & 1) == 0 && (d.c_hi & 1) == 0 ? 2 : 0);
+                 (parts > 1 || ((reinterpret_cast<uintptr_t>(C) & 15) == 0 && (d.c_lo & 1) == 0 && (d.c_hi & 1) == 0)
+                      ? 2
+                      : 0);
   // K = 8: the operands' 16-byte rows go by contiguous bulk copies (one per
   // plane) instead of tensor-map boxes of 16-byte rows; every address and
   // size must be a multiple of 16 bytes, else the tensor maps serve
@@ -1624,8 +1693,12 @@ cudaError_t launch_gemm_tma(const PlaneOperand& a, const PlaneOperand& b, float2
            q.plane % 16 == 0;
   };
   if (kpi != 8 || !aligned(qa) || !aligned(qb)) qa = qb = BulkPlanes{};
-  return a.np == 4 ? launch_tn<4>(TNv, ma, mb, C, d, kpi, z, cp, sio, fold, bf16, err, s, qa, qb)
-                   : launch_tn<2>(TNv, ma, mb, C, d, kpi, z, cp, sio, fold, bf16, err, s, qa, qb);
+  const cudaError_t e =
+      a.np == 4 ? launch_tn<4>(TNv, ma, mb, C, d, kpi, z, cp, sio, fold, bf16, err, s, qa, qb, parts, part)
+                : launch_tn<2>(TNv, ma, mb, C, d, kpi, z, cp, sio, fold, bf16, err, s, qa, qb, 1, nullptr);
+  if (e != cudaSuccess || parts == 1) return e;
+  return launch_overlapped(combine_kernel, dim3((1u << (d.nm + d.nn)) / 256, (unsigned)d.units), dim3(256), 0, s, part,
+                           parts, C, d, sio, z[0], z[1], z[2], z[3]);
 }
 
 // Where converting A in the GEMM beats a split pass: enough row tiles to fill

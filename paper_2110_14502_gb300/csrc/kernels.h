@@ -128,7 +128,10 @@ int64_t split_plane_elems(int nrow_bits, int nk_bits, int np);
 // error code in the kernel's error word and the CTA winds down.
 cudaError_t set_tc_wait_limit(long long polls);
 cudaError_t launch_gemm_tma(const PlaneOperand& a, const PlaneOperand& b, float2* C, bool c_planes, const GemmDesc& d,
-                            bool bf16, const ScaleIO& sio, int* err, cudaStream_t s);
+                            bool bf16, const ScaleIO& sio, int* err, cudaStream_t s, float2* part = nullptr);
+// 16-bit elements of scratch with which launch_gemm_tma may spread a long K over
+// idle SMs (`part`; 0: it would not).  Results are the same with and without.
+int64_t tc_part_elems(const GemmDesc& d, int np, bool c_planes);
 // Split operand A (which_b = false) or B of d into `scratch` (returned planes).
 // With `scaled`, each distinct tensor z is first reduced to its largest
 // |component| (maxbits[z], cleared by the caller) and stored times 2^-e_z with
@@ -152,17 +155,18 @@ cudaError_t launch_gemm_direct(const float2* A, const PlaneOperand& b, float2* C
 // Split both operands of d (or B alone, where the GEMM converts A) into
 // `scratch` and run the GEMM, rows and columns renumbered as suits it.
 // tc2_scratch_elems: 16-bit values of both operands' planes;
-// tc2_pair_scratch_elems: those that a call needs.
+// tc2_pair_scratch_elems: those that a call needs, with the space for partial
+// sums that lets a long K use idle SMs (`sums`) or without it.
 int64_t tc2_scratch_elems(const GemmDesc& d);
-int64_t tc2_pair_scratch_elems(const GemmDesc& d);
-cudaError_t run_gemm_tc2(const float2* A, const float2* B, float2* C, const GemmDesc& d, bool bf16, uint16_t* scratch,
-                         int* err, cudaStream_t s);
+int64_t tc2_pair_scratch_elems(const GemmDesc& d, bool sums);
+cudaError_t run_gemm_tc2(const float2* A, const float2* B, float2* C, const GemmDesc& d, bool bf16, bool sums,
+                         uint16_t* scratch, int* err, cudaStream_t s);
 // Same with both operands scaled by their exact maxima (one power-of-two
 // exponent each) and split into np planes (4: split fp16/bf16, 2: scaled
 // single products); C is written in complex64 with the exponents applied.
 // aux: 24 bytes of device memory (maxima, exponents, stored maxima).
 cudaError_t run_gemm_tc2_scaled(const float2* A, const float2* B, float2* C, const GemmDesc& d, bool bf16, int np,
-                                uint16_t* scratch, void* aux, int* err, cudaStream_t s);
+                                bool sums, uint16_t* scratch, void* aux, int* err, cudaStream_t s);
 // Vector-like steps: N <= 16 and K <= 16, N <= 8 and K <= 128, N <= 256 and
 // K <= 4, or N = 32 and K = 8 (k_vector.cu).
 bool vector_shape_ok(const GemmDesc& d);

@@ -206,19 +206,26 @@ extern "C" tn_status tn_contract_pair(const void* A, const int32_t* a_labels, in
       if (!tc_shape_ok(d)) return fail(TN_EINVAL, "tn_contract_pair: tensor-core kernels need M >= 128, N >= 16, K >= 8");
       std::lock_guard<std::mutex> lock(g_pair_mu);
       // operand planes, then 32 bytes for the scaled modes' maxima and exponents
-      const size_t planes = algo == TN_PAIR_FUSED_TC ? (size_t)tc2_pair_scratch_elems(d) * sizeof(uint16_t) : 0;
+      const bool fused = algo == TN_PAIR_FUSED_TC;
+      bool sums = true;  // with space for partial sums, unless that does not fit
+      size_t planes = fused ? (size_t)tc2_pair_scratch_elems(d, true) * sizeof(uint16_t) : 0;
       PairDevState* ps = nullptr;
       tn_status pst = pair_state(planes + 32, ps);
+      if (pst == TN_EHBM && fused) {
+        sums = false;
+        planes = (size_t)tc2_pair_scratch_elems(d, false) * sizeof(uint16_t);
+        pst = pair_state(planes + 32, ps);
+      }
       if (pst != TN_OK) return pst;
       int* err = ps->err;
-      if (algo == TN_PAIR_FUSED_TC) {
+      if (fused) {
         uint16_t* scratch = static_cast<uint16_t*>(ps->scratch);
         void* aux = static_cast<char*>(ps->scratch) + planes;
         switch (precision) {
-          case TN_PREC_SPLIT_BF16: e = run_gemm_tc2(a, b, c, d, true, scratch, err, s); break;
-          case TN_PREC_SPLIT_FP16: e = run_gemm_tc2_scaled(a, b, c, d, false, 4, scratch, aux, err, s); break;
-          case TN_PREC_SCALED_FP16: e = run_gemm_tc2_scaled(a, b, c, d, false, 2, scratch, aux, err, s); break;
-          default: e = run_gemm_tc2_scaled(a, b, c, d, true, 2, scratch, aux, err, s); break;
+          case TN_PREC_SPLIT_BF16: e = run_gemm_tc2(a, b, c, d, true, sums, scratch, err, s); break;
+          case TN_PREC_SPLIT_FP16: e = run_gemm_tc2_scaled(a, b, c, d, false, 4, sums, scratch, aux, err, s); break;
+          case TN_PREC_SCALED_FP16: e = run_gemm_tc2_scaled(a, b, c, d, false, 2, sums, scratch, aux, err, s); break;
+          default: e = run_gemm_tc2_scaled(a, b, c, d, true, 2, sums, scratch, aux, err, s); break;
         }
       } else {
         e = launch_gemm_tc(a, b, c, d, true, 1.f, 1.f, err, s);

@@ -148,7 +148,7 @@ extern "C" tn_status tn_contract_pair_noalloc(const void* A, const int32_t* a_la
   cudaError_t e = cudaMemsetAsync(slots.err, 0, sizeof(int), s);
   if (e != cudaSuccess)
     return fail(TN_ECUDA, "tn_contract_pair_noalloc: clearing the error word: %s", cudaGetErrorString(e));
-  e = run_gemm_tc2((const float2*)A, (const float2*)B, (float2*)Cv, d, true, slots.scratch, slots.err, s);
+  e = run_gemm_tc2((const float2*)A, (const float2*)B, (float2*)Cv, d, true, false, slots.scratch, slots.err, s);
   if (e != cudaSuccess) return fail(TN_ECUDA, "tn_contract_pair_noalloc launch: %s", cudaGetErrorString(e));
   int h = 0;
   e = cudaMemcpyAsync(&h, slots.err, sizeof(int), cudaMemcpyDeviceToHost, s);
