@@ -20,7 +20,12 @@
 // (bi, br).  The same four roundings in the same order as scalar FMAs, k
 // ascending, so every tile shape gives the same bits.  A sits in shared memory
 // already as (ar, ar, -ai, ai), so its operands are one 16-byte load; B's
-// swapped pair costs a register move, which issues beside the packed FMAs.
+// swapped pair costs a register move, which issues beside the packed FMAs.  The
+// 128 x 64 tile (8 x 4 outputs per thread) keeps scalar FMAs: per multiply-add it
+// reads twice the shared memory of the 128 x 128 tile, and the doubled A costs
+// more than packing saves (log2 M, N, K, scalar and packed: (16, 6, 11) 1781 and
+// 2014 us, (14, 6, 12) 1037 and 1125, (17, 6, 8) 466 and 507; packed with two
+// CTAs per SM and spills 1872, 1381, 469).
 //
 // Global loads: when the operand's two fastest indices are its first two K
 // bits (the planner's layouts put contracted indices innermost), a thread
@@ -28,6 +33,7 @@
 // of a warp read consecutive rows at the same K quad (one 32-byte sector per
 // row); otherwise each lane reads one element, lanes on consecutive rows.
 #include <algorithm>
+#include <type_traits>
 
 #include "device_common.h"
 #include "kernels.h"
@@ -137,23 +143,24 @@ struct TileLoader {
   }
 };
 
-template <int BM, int BN, int BK, int RM, int RN>
+template <int BM, int BN, int BK, int RM, int RN, bool PACKED>
 struct SimtCfg {
   static_assert(BM / RM * (BN / RN) == NT, "256 threads");
-  static constexpr int A_BUF = BK * BM * 16, B_BUF = BK * BN * 8;
+  static constexpr int A_BUF = BK * BM * (PACKED ? 16 : 8), B_BUF = BK * BN * 8;
   static constexpr int SMEM = 2 * (A_BUF + B_BUF);
 };
 
 // flags: bit 0 A vector loads, bit 1 B vector loads, bit 2 C pair stores
-template <int BM, int BN, int BK, int RM, int RN>
+template <int BM, int BN, int BK, int RM, int RN, bool PACKED>
 __global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_kernel(const float2* __restrict__ A,
                                                            const float2* __restrict__ B,
                                                            float2* __restrict__ C, const GemmDesc d, int flags) {
-  using CF = SimtCfg<BM, BN, BK, RM, RN>;
+  using CF = SimtCfg<BM, BN, BK, RM, RN, PACKED>;
   constexpr int CG = BN / RN;        // column groups
   constexpr int BAND = 2 * CG;       // columns 2 tn, 2 tn + 1 of each band of BAND columns (RN = 1: column tn)
   extern __shared__ __align__(16) uint8_t smem[];
-  float4* As = reinterpret_cast<float4*>(smem);                    // [2][BK][BM] of (ar, ar, -ai, ai)
+  using AT = std::conditional_t<PACKED, float4, float2>;           // (ar, ar, -ai, ai), or (ar, ai)
+  AT* As = reinterpret_cast<AT*>(smem);                            // [2][BK][BM]
   float2* Bs = reinterpret_cast<float2*>(smem + 2 * CF::A_BUF);    // [2][BK][BN]
   const int64_t K = int64_t(1) << d.nk;
   const int64_t m0 = (int64_t)blockIdx.x * BM, n0 = (int64_t)blockIdx.y * BN;
@@ -171,16 +178,27 @@ __global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_ker
   la.init(d, d.nm, d.am, d.ak, m0, (flags & 1) != 0);
   lb.init(d, d.nn, d.bn, d.bk, n0, (flags & 2) != 0);
 
-  f32x2 acc[RM][RN];
+  f32x2 acc[RM][RN];   // PACKED
+  float accr[RM][RN], acci[RM][RN];
 #pragma unroll
   for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < RN; ++j) acc[i][j] = 0ull;
+    for (int j = 0; j < RN; ++j) {
+      acc[i][j] = 0ull;
+      accr[i][j] = acci[i][j] = 0.f;
+    }
+  auto result = [&](int i, int j) {
+    if constexpr (PACKED) return unpack2(acc[i][j]);
+    else return make_float2(accr[i][j], acci[i][j]);
+  };
 
   auto store_tiles = [&](int buf) {
-    float4* at = As + buf * BK * BM;
+    AT* at = As + buf * BK * BM;
     float2* bt = Bs + buf * BK * BN;
-    la.store([&](int p, float2 x) { at[p] = make_float4(x.x, x.x, -x.y, x.y); });
+    la.store([&](int p, float2 x) {
+      if constexpr (PACKED) at[p] = make_float4(x.x, x.x, -x.y, x.y);
+      else at[p] = x;
+    });
     lb.store([&](int p, float2 x) { bt[p] = x; });
   };
   const int64_t nch = (K + BK - 1) / BK;
@@ -196,9 +214,38 @@ __global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_ker
       la.load(A, k1, k_high_offset<ilog2(BK)>(k1, d.nk, d.ak));
       lb.load(B, k1, k_high_offset<ilog2(BK)>(k1, d.nk, d.bk));
     }
-    const ulonglong2* at = reinterpret_cast<const ulonglong2*>(As + buf * BK * BM) + RM * tm;
+    const AT* const a0 = As + buf * BK * BM + RM * tm;
+    const ulonglong2* at = reinterpret_cast<const ulonglong2*>(a0);
     const float2* bt = Bs + buf * BK * BN;
-    auto step = [&](int kk) {
+    auto scalar_step = [&](int kk) {
+      float ar[RM], ai[RM], br[RN], bi[RN];
+#pragma unroll
+      for (int i = 0; i < RM; i += 2) {
+        const float4 x = *reinterpret_cast<const float4*>(a0 + kk * BM + i);
+        ar[i] = x.x;
+        ai[i] = x.y;
+        ar[i + 1] = x.z;
+        ai[i + 1] = x.w;
+      }
+#pragma unroll
+      for (int j = 0; j < RN; j += 2) {
+        const float4 x = *reinterpret_cast<const float4*>(bt + kk * BN + BAND / 2 * j + 2 * tn);
+        br[j] = x.x;
+        bi[j] = x.y;
+        br[j + 1] = x.z;
+        bi[j + 1] = x.w;
+      }
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < RN; ++j) {
+          accr[i][j] = fmaf(ar[i], br[j], accr[i][j]);
+          accr[i][j] = fmaf(-ai[i], bi[j], accr[i][j]);
+          acci[i][j] = fmaf(ar[i], bi[j], acci[i][j]);
+          acci[i][j] = fmaf(ai[i], br[j], acci[i][j]);
+        }
+    };
+    auto packed_step = [&](int kk) {
       f32x2 b[RN], bs[RN];
       if constexpr (RN == 1) {
         b[0] = *reinterpret_cast<const f32x2*>(bt + kk * BN + tn);
@@ -220,6 +267,10 @@ __global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_ker
 #pragma unroll
         for (int j = 0; j < RN; ++j) acc2(acc[i][j], a.y, bs[j]);
       }
+    };
+    auto step = [&](int kk) {
+      if constexpr (PACKED) packed_step(kk);
+      else scalar_step(kk);
     };
     if (kn == BK) {
 #pragma unroll 16
@@ -249,30 +300,30 @@ __global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_ker
 #pragma unroll
       for (int j = 0; j < RN; j += 2)
         if (cc[j] >= 0) {
-          const float2 x = unpack2(acc[i][j]), y = unpack2(acc[i][RN > 1 ? j + 1 : j]);
+          const float2 x = result(i, j), y = result(i, RN > 1 ? j + 1 : j);
           *reinterpret_cast<float4*>(C + rc + cc[j]) = make_float4(x.x, x.y, y.x, y.y);
         }
     } else {
 #pragma unroll
       for (int j = 0; j < RN; ++j)
-        if (cc[j] >= 0) C[rc + cc[j]] = unpack2(acc[i][j]);
+        if (cc[j] >= 0) C[rc + cc[j]] = result(i, j);
     }
   }
 }
 
-template <int BM, int BN, int BK, int RM, int RN>
+template <int BM, int BN, int BK, int RM, int RN, bool PACKED = true>
 cudaError_t launch_tile(const float2* A, const float2* B, float2* C, const GemmDesc& d, int flags, cudaStream_t s) {
-  constexpr int SMEM = SimtCfg<BM, BN, BK, RM, RN>::SMEM;
+  constexpr int SMEM = SimtCfg<BM, BN, BK, RM, RN, PACKED>::SMEM;
   static bool attr = false;
   if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, BN, BK, RM, RN>,
+    const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, BN, BK, RM, RN, PACKED>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     if (e != cudaSuccess) return e;
     attr = true;
   }
   const int64_t M = int64_t(1) << d.nm, N = int64_t(1) << d.nn;
   dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), (unsigned)d.units);
-  return launch_overlapped(gemm_simt_kernel<BM, BN, BK, RM, RN>, grid, dim3(NT), SMEM, s, A, B,
+  return launch_overlapped(gemm_simt_kernel<BM, BN, BK, RM, RN, PACKED>, grid, dim3(NT), SMEM, s, A, B,
                            C, d, flags);
 }
 
@@ -292,7 +343,7 @@ bool quad_ok(const float2* base, int nk, const int32_t* kst, int64_t lo, int64_t
 // the largest (46 TFLOP/s on (12, 12, 9); scalar FMAs reached 44).  The small
 // shapes matter where the large one would leave SMs idle or compute padding:
 // (5, 4, 7) 41 -> 12 us, (5, 3, 8) x 2 units 82 -> 18 us, (6, 4, 12) x 128 units
-// 1.08 -> 0.57 ms.  Every shape gives the same bits, so this is speed alone.
+// 1.08 -> 0.57 ms, (16, 5, 10) 901 -> 558 us.  Every shape gives the same bits, so this is speed alone.
 cudaError_t launch_gemm_simt(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s) {
   int flags = 0;
   if (quad_ok(A, d.nk, d.ak, d.a_lo, d.a_hi)) flags |= 1;
@@ -310,7 +361,7 @@ cudaError_t launch_gemm_simt(const float2* A, const float2* B, float2* C, const 
   const double c128 = cost(128, 128, 1.0), c64 = cost(128, 64, 0.85), cm = cost(64, 32, 0.55), cs = cost(32, 16, 0.25);
   const double best = std::min(std::min(c128, c64), std::min(cm, cs));
   if (best == c128) return launch_tile<128, 128, 16, 8, 8>(A, B, C, d, flags, s);
-  if (best == c64) return launch_tile<128, 64, 16, 8, 4>(A, B, C, d, flags, s);
+  if (best == c64) return launch_tile<128, 64, 16, 8, 4, false>(A, B, C, d, flags, s);
   if (best == cm) return launch_tile<64, 32, 32, 4, 2>(A, B, C, d, flags, s);
   return launch_tile<32, 16, 64, 2, 1>(A, B, C, d, flags, s);
 }
