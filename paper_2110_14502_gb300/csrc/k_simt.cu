@@ -33,6 +33,7 @@
 // of a warp read consecutive rows at the same K quad (one 32-byte sector per
 // row); otherwise each lane reads one element, lanes on consecutive rows.
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "device_common.h"
@@ -344,6 +345,24 @@ bool quad_ok(const float2* base, int nk, const int32_t* kst, int64_t lo, int64_t
 // shapes matter where the large one would leave SMs idle or compute padding:
 // (5, 4, 7) 41 -> 12 us, (5, 3, 8) x 2 units 82 -> 18 us, (6, 4, 12) x 128 units
 // 1.08 -> 0.57 ms, (16, 5, 10) 901 -> 558 us.  Every shape gives the same bits, so this is speed alone.
+// Column tiles are counted by grid.y, which ends at 65535: a shape with more of
+// them (16 columns from N = 2^20 on, 32 from 2^21, 64 from 2^22) is no choice.
+SimtTile simt_tile(const GemmDesc& d) {
+  const int64_t M = int64_t(1) << d.nm, N = int64_t(1) << d.nn;
+  auto cost = [&](int bm, int bn, double rate) {
+    const int64_t rows = (M + bm - 1) / bm, cols = (N + bn - 1) / bn;
+    if (cols > 65535) return HUGE_VAL;
+    const double tiles = (double)rows * (double)cols * d.units;
+    return (double)((int64_t)((tiles + 151) / 152)) * bm * bn / rate;
+  };
+  const double c128 = cost(128, 128, 1.0), c64 = cost(128, 64, 0.85), cm = cost(64, 32, 0.55), cs = cost(32, 16, 0.25);
+  const double best = std::min(std::min(c128, c64), std::min(cm, cs));
+  if (best == c128) return {128, 128};
+  if (best == c64) return {128, 64};
+  if (best == cm) return {64, 32};
+  return {32, 16};
+}
+
 cudaError_t launch_gemm_simt(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s) {
   int flags = 0;
   if (quad_ok(A, d.nk, d.ak, d.a_lo, d.a_hi)) flags |= 1;
@@ -353,16 +372,10 @@ cudaError_t launch_gemm_simt(const float2* A, const float2* B, float2* C, const 
   if (d.nn >= 1 && d.cn[0] == 1 && (reinterpret_cast<uintptr_t>(C) & 15) == 0 && (d.c_lo & 1) == 0 &&
       (d.c_hi & 1) == 0)
     flags |= 4;
-  const int64_t M = int64_t(1) << d.nm, N = int64_t(1) << d.nn;
-  auto cost = [&](int bm, int bn, double rate) {
-    const double tiles = (double)((M + bm - 1) / bm) * (double)((N + bn - 1) / bn) * d.units;
-    return (double)((int64_t)((tiles + 151) / 152)) * bm * bn / rate;
-  };
-  const double c128 = cost(128, 128, 1.0), c64 = cost(128, 64, 0.85), cm = cost(64, 32, 0.55), cs = cost(32, 16, 0.25);
-  const double best = std::min(std::min(c128, c64), std::min(cm, cs));
-  if (best == c128) return launch_tile<128, 128, 16, 8, 8>(A, B, C, d, flags, s);
-  if (best == c64) return launch_tile<128, 64, 16, 8, 4, false>(A, B, C, d, flags, s);
-  if (best == cm) return launch_tile<64, 32, 32, 4, 2>(A, B, C, d, flags, s);
+  const SimtTile t = simt_tile(d);
+  if (t.rows == 128 && t.cols == 128) return launch_tile<128, 128, 16, 8, 8>(A, B, C, d, flags, s);
+  if (t.rows == 128) return launch_tile<128, 64, 16, 8, 4, false>(A, B, C, d, flags, s);
+  if (t.rows == 64) return launch_tile<64, 32, 32, 4, 2>(A, B, C, d, flags, s);
   return launch_tile<32, 16, 64, 2, 1>(A, B, C, d, flags, s);
 }
 

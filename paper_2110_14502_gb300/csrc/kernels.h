@@ -69,6 +69,9 @@ struct GroupArg {
 
 // launchers (return cudaGetLastError())
 cudaError_t launch_gemm_simt(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s);
+// Its tile: rows and columns of C per CTA.
+struct SimtTile { int rows, cols; };
+SimtTile simt_tile(const GemmDesc& d);
 // tcgen05 fused permute-GEMM (complex64 in/out, 16-bit hi+lo split products,
 // FP32 accumulation).  Operands are multiplied by a_scale / b_scale before the
 // split and the result divided by their product (powers of two).  *err is set
