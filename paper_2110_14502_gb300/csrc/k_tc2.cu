@@ -1529,9 +1529,10 @@ cudaError_t launch_chunked(const CUtensorMap& ma, const CUtensorMap& mb, float2*
   constexpr int WIDE = NP == 4 ? 64 : 128;
   if constexpr (WIDE == 128)
     if (rowb == 64) return go(integral_constant<int, 64>{}, integral_constant<int, EWS>{});
-  if (EWS == 8 && kp <= 4 * (WIDE / 2)) return go(integral_constant<int, WIDE>{}, integral_constant<int, EWS>{});
-  if constexpr (NP == 4)  // (two or more chunks: a long K)
+  // (chunks as items, two or more: a K of several stages, at any chunk length)
+  if constexpr (NP == 4)
     if (parts > 1) return run(integral_constant<int, WIDE>{}, integral_constant<int, 4>{}, integral_constant<bool, true>{});
+  if (EWS == 8 && kp <= 4 * (WIDE / 2)) return go(integral_constant<int, WIDE>{}, integral_constant<int, EWS>{});
   return go(integral_constant<int, WIDE>{}, integral_constant<int, 4>{});
 }
 
