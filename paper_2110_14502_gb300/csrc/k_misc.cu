@@ -36,9 +36,9 @@ __global__ void gather_kernel(const float2* __restrict__ store, float2* __restri
 // Method via Adaptive Precision Scaling": paths with under/overflow are kept
 // out of the sum): a flagged unit adds nothing here and is listed for the
 // host, which recomputes it in complex64 or counts it as discarded.
-__global__ void accumulate_kernel(const float2* __restrict__ root, int64_t r_lo, int64_t r_hi,
+__global__ void accumulate_kernel(const float2* root, int64_t r_lo, int64_t r_hi,
                                   const int64_t* __restrict__ perm, int nperm, const GroupArg group,
-                                  const int* __restrict__ flag_s, const int* __restrict__ flag_u,
+                                  const int* flag_s, const int* flag_u,
                                   int64_t* __restrict__ flagged, unsigned long long* __restrict__ nflagged,
                                   int cap) {
   let_next_start();

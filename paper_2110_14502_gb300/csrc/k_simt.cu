@@ -104,15 +104,15 @@ struct TileLoader {
     }
   }
 
-  __device__ __forceinline__ void load(const float2* __restrict__ src, int64_t k0, int32_t khi) {
+  __device__ __forceinline__ void load(const float2* src, int64_t k0, int32_t khi) {
     if (vec) {
 #pragma unroll
       for (int q = 0; q < NQ; ++q) {
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
         if (row_off >= 0 && k0 + 4 * (kk0 + STEP * q) < K) {
           const float4* p = reinterpret_cast<const float4*>(src + row_off + khi + low[q]);
-          x = __ldg(p);
-          y = __ldg(p + 1);
+          x = p[0];
+          y = p[1];
         }
         v[4 * q + 0] = make_float2(x.x, x.y);
         v[4 * q + 1] = make_float2(x.z, x.w);
@@ -123,7 +123,7 @@ struct TileLoader {
 #pragma unroll
       for (int j = 0; j < NE; ++j) {
         float2 x = make_float2(0.f, 0.f);
-        if (row_off >= 0 && k0 + kk0 + STEP * j < K) x = __ldg(src + row_off + khi + low[j]);
+        if (row_off >= 0 && k0 + kk0 + STEP * j < K) x = src[row_off + khi + low[j]];
         v[j] = x;
       }
     }
@@ -153,8 +153,8 @@ struct SimtCfg {
 
 // flags: bit 0 A vector loads, bit 1 B vector loads, bit 2 C pair stores
 template <int BM, int BN, int BK, int RM, int RN, bool PACKED>
-__global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_kernel(const float2* __restrict__ A,
-                                                           const float2* __restrict__ B,
+__global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_kernel(const float2* A,
+                                                           const float2* B,
                                                            float2* __restrict__ C, const GemmDesc d, int flags) {
   using CF = SimtCfg<BM, BN, BK, RM, RN, PACKED>;
   constexpr int CG = BN / RN;        // column groups

@@ -98,6 +98,13 @@ struct SplitJob {
   float* m_out;
 };
 
+// The passes over small operands start early; those over large ones (2^12 tiles)
+// are launched plainly and read past the coherent path, which is faster by more
+// than a launch (a 2^26-element operand for scaled fp16, (13, 6, 13): the call
+// takes 316 us, started early with ordinary loads 335).
+template <int T>
+constexpr bool kSplitEarly = T < 12;
+
 template <int NP, int T, bool BF16>
 __device__ __forceinline__ void split_tile(const SplitJob& job, const TileMap& tm, unsigned blk, int64_t z) {
   let_next_start();
@@ -150,12 +157,12 @@ __device__ __forceinline__ void split_tile(const SplitJob& job, const TileMap& t
       for (int b = 0; b < T - 1 - TB; ++b)
         if ((j >> b) & 1) o += tm.in_src[1 + TB + b];
       if (vec) {
-        const float4 x = __ldg(reinterpret_cast<const float4*>(src + o));
+        const float4 x = load<kSplitEarly<T>>(reinterpret_cast<const float4*>(src + o));
         v[j][0] = make_float2(x.x, x.y);
         v[j][1] = make_float2(x.z, x.w);
       } else {
-        v[j][0] = __ldg(src + o);
-        v[j][1] = __ldg(src + o + 1);
+        v[j][0] = load<kSplitEarly<T>>(src + o);
+        v[j][1] = load<kSplitEarly<T>>(src + o + 1);
       }
     }
 #pragma unroll
@@ -303,8 +310,7 @@ SplitJob split_job(const float2* src, uint16_t* dst, const SplitDesc& d, const u
 // Both maxima of a contraction's operands by one CTA each, stored (no clearing,
 // no atomics): for operands that one CTA reads in a microsecond or two.
 constexpr int MAX_SMALL_BITS = 15;
-__global__ void __launch_bounds__(1024) max_small_kernel(const float2* __restrict__ a, int abits,
-                                                         const float2* __restrict__ b, int bbits,
+__global__ void __launch_bounds__(1024) max_small_kernel(const float2* a, int abits, const float2* b, int bbits,
                                                          unsigned* __restrict__ maxbits) {
   let_next_start();
   after_previous();
@@ -313,7 +319,7 @@ __global__ void __launch_bounds__(1024) max_small_kernel(const float2* __restric
   float m = 0.f;
 #pragma unroll 8
   for (int e = threadIdx.x; e < n; e += 1024) {
-    const float2 v = __ldg(p + e);
+    const float2 v = p[e];
     m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
   }
   __shared__ unsigned wm[32];
@@ -348,8 +354,8 @@ cudaError_t launch_split(const float2* src, uint16_t* dst, const SplitDesc& d, i
   const SplitJob job = split_job(src, dst, d, maxbits, e_out, m_out);
   return for_format(np, bf16, tile_bits(R, nz), [&](auto n, auto t, auto fmt) {
     constexpr int T = decltype(t)::value;
-    return launch_overlapped(split_kernel<decltype(n)::value, T, decltype(fmt)::value>,
-                             dim3(1u << (R - T), (unsigned)nz), dim3(NT), 0, s, job, split_tile_map<T>(d));
+    return launch_kernel(kSplitEarly<T>, split_kernel<decltype(n)::value, T, decltype(fmt)::value>,
+                         dim3(1u << (R - T), (unsigned)nz), dim3(NT), 0, s, job, split_tile_map<T>(d));
   });
 }
 
@@ -436,9 +442,9 @@ static cudaError_t split_pair(const float2* A, const float2* B, const GemmDesc& 
   if (ta == tb || (T == 10 && large <= 20) || (T == 7 && large <= 14))
     return for_format(np, bf16, T, [&](auto n, auto t, auto fmt) {
       constexpr int TT = decltype(t)::value;
-      return launch_overlapped(split_pair_kernel<decltype(n)::value, TT, decltype(fmt)::value>,
-                               dim3((1u << (ra - TT)) + (1u << (rb - TT))), dim3(NT), 0, s, ja, split_tile_map<TT>(da),
-                               jb, split_tile_map<TT>(db));
+      return launch_kernel(kSplitEarly<TT>, split_pair_kernel<decltype(n)::value, TT, decltype(fmt)::value>,
+                           dim3((1u << (ra - TT)) + (1u << (rb - TT))), dim3(NT), 0, s, ja, split_tile_map<TT>(da), jb,
+                           split_tile_map<TT>(db));
     });
   const cudaError_t e = launch_split(A, scratch, da, 1, bf16, np, mx, ex, ms, s, true);
   return e != cudaSuccess ? e

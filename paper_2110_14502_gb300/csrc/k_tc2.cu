@@ -1029,9 +1029,9 @@ __device__ __forceinline__ bool workers_any(bool failed) {  // barrier of the 25
 
 template <int TN, int NP, bool BF16>
 __global__ void __launch_bounds__(DirectCfg<TN, NP>::THREADS, 1)
-    gemm_direct(const __grid_constant__ CUtensorMap mapB, const float2* __restrict__ A, float2* __restrict__ C,
-                const GemmDesc d, const __grid_constant__ DirectMap dm, const unsigned* __restrict__ maxA,
-                const int* __restrict__ exp_b, int a_vec, int out_wide, int chunk, int* __restrict__ err) {
+    gemm_direct(const __grid_constant__ CUtensorMap mapB, const float2* A, float2* __restrict__ C,
+                const GemmDesc d, const __grid_constant__ DirectMap dm, const unsigned* maxA,
+                const int* exp_b, int a_vec, int out_wide, int chunk, int* __restrict__ err) {
   using DC = DirectCfg<TN, NP>;
   using CF = typename DC::CF;
   constexpr int NS = DC::NS;
@@ -1193,9 +1193,9 @@ __global__ void __launch_bounds__(DirectCfg<TN, NP>::THREADS, 1)
       for (int j = 0; j < 8; ++j) {
         const float2* p = src + dm.in_off[j];
         if (a_vec) {
-          pf[j] = __ldg(reinterpret_cast<const float4*>(p));
+          pf[j] = *reinterpret_cast<const float4*>(p);
         } else {
-          const float2 x = __ldg(p), y = __ldg(p + 1);
+          const float2 x = p[0], y = p[1];
           pf[j] = make_float4(x.x, x.y, y.x, y.y);
         }
       }
@@ -1413,7 +1413,7 @@ __global__ void __launch_bounds__(DirectCfg<TN, NP>::THREADS, 1)
 // scaling of gemm_tma_chunked for items that were one chunk each, with the same
 // additions in the same order.  Bound by the sums' trip through L2 (they were
 // written microseconds before; at most 256 MB).
-__global__ void __launch_bounds__(256) combine_kernel(const float2* __restrict__ part, int parts, float2* __restrict__ C,
+__global__ void __launch_bounds__(256) combine_kernel(const float2* part, int parts, float2* __restrict__ C,
                                                       const GemmDesc d, const ScaleIO sio, int a_zlo, int a_zhi,
                                                       int b_zlo, int b_zhi) {
   let_next_start();

@@ -103,7 +103,7 @@ __device__ __forceinline__ void emit(const VecOut& o, float2* C, int64_t off, fl
 }
 
 template <int NK, int NN, int PER>
-__global__ void __launch_bounds__(NT) vector_kernel(const float2* __restrict__ A, const float2* __restrict__ B,
+__global__ void __launch_bounds__(NT) vector_kernel(const float2* A, const float2* B,
                                                     float2* __restrict__ C, const GemmDesc d,
                                                     const VecOut o) {
   constexpr int K = 1 << NK, N = 1 << NN;
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(NT) vector_kernel(const float2* __restrict__ A
     int32_t oc = baseC + tClo[loc & 31] + tChi[loc >> 5];
     float2 a[K];
 #pragma unroll
-    for (int k = 0; k < K; ++k) a[k] = __ldg(A + (int64_t)oa + kA[k]);
+    for (int k = 0; k < K; ++k) a[k] = A[(int64_t)oa + kA[k]];
 #pragma unroll
     for (int n = 0; n < N; ++n) {
       float2 acc = make_float2(0.f, 0.f);
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(NT) vector_kernel(const float2* __restrict__ A
 // registers while the thread walks the N columns, so the registers do not grow
 // with N; B (K N <= 1024 complex) sits in shared memory.
 template <int NK, int NN>
-__global__ void __launch_bounds__(NT) vector_wide_kernel(const float2* __restrict__ A, const float2* __restrict__ B,
+__global__ void __launch_bounds__(NT) vector_wide_kernel(const float2* A, const float2* B,
                                                          float2* __restrict__ C, const GemmDesc d,
                                                          const VecOut o, int pair_k, int cb) {
   constexpr int K = 1 << NK, N = 1 << NN;
@@ -236,13 +236,13 @@ __global__ void __launch_bounds__(NT) vector_wide_kernel(const float2* __restric
     if (K >= 2 && pair_k) {
 #pragma unroll
       for (int k = 0; k < K; k += 2) {
-        const float4 x = __ldg(reinterpret_cast<const float4*>(A + (int64_t)oa + kA[k]));
+        const float4 x = *reinterpret_cast<const float4*>(A + (int64_t)oa + kA[k]);
         a[k] = make_float2(x.x, x.y);
         a[k + 1 < K ? k + 1 : k] = make_float2(x.z, x.w);
       }
     } else {
 #pragma unroll
-      for (int k = 0; k < K; ++k) a[k] = __ldg(A + (int64_t)oa + kA[k]);
+      for (int k = 0; k < K; ++k) a[k] = A[(int64_t)oa + kA[k]];
     }
 #pragma unroll 8
     for (int n = 0; n < N; ++n) {
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(NT) vector_wide_kernel(const float2* __restric
 // has stride 1 and every pair starts on a 16-byte boundary) a row's K values
 // arrive two per 16-byte load.
 template <int NK, int NN>
-__global__ void __launch_bounds__(NT) vector_long_kernel(const float2* __restrict__ A, const float2* __restrict__ B,
+__global__ void __launch_bounds__(NT) vector_long_kernel(const float2* A, const float2* B,
                                                          float2* __restrict__ C, const GemmDesc d, int pair_k,
                                                          const VecOut o, int cb) {
   constexpr int K = 1 << NK, N = 1 << NN;
@@ -323,13 +323,13 @@ __global__ void __launch_bounds__(NT) vector_long_kernel(const float2* __restric
     if (pair_k) {
 #pragma unroll 4
       for (int k = 0; k < K; k += 2) {
-        const float4 x = __ldg(reinterpret_cast<const float4*>(A + (int64_t)oa + kA[k]));
+        const float4 x = *reinterpret_cast<const float4*>(A + (int64_t)oa + kA[k]);
         mac_pair<N>(acc, Bs + k * N, Bs + (k + 1) * N, make_float2(x.x, x.y), make_float2(x.z, x.w));
       }
     } else {
 #pragma unroll 8
       for (int k = 0; k < K; ++k) {
-        const float2 a = __ldg(A + (int64_t)oa + kA[k]);
+        const float2 a = A[(int64_t)oa + kA[k]];
 #pragma unroll
         for (int n = 0; n < N; ++n) {
           const float2 b = Bs[k * N + n];
@@ -366,7 +366,7 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
 template <int NK, int NN>
-__global__ void __launch_bounds__(SNT) vector_staged_kernel(const float2* __restrict__ A, const float2* __restrict__ B,
+__global__ void __launch_bounds__(SNT) vector_staged_kernel(const float2* A, const float2* B,
                                                             float2* __restrict__ C, const GemmDesc d,
                                                             const VecOut o, int cb) {
   constexpr int K = 1 << NK, N = 1 << NN;
@@ -473,7 +473,10 @@ __global__ void __launch_bounds__(SNT) vector_staged_kernel(const float2* __rest
 // of C front to back from shared memory.  B sits in shared memory as (re, im,
 // im, re), one 16-byte read for both packed products of a complex
 // multiply-add; the sums run in the order of the kernel that would otherwise
-// take the shape (IM_FIRST), so the results are the same bit for bit.
+// take the shape (IM_FIRST), so the results are the same bit for bit.  Launched
+// plainly: its read-only loads, which an early start would rule out, are worth
+// more than the start (log2 M, N, K = (22, 3, 4) 206 us per call; started early,
+// with ordinary loads 224, past L1 212, and with B's values fetched first 225).
 constexpr int TILE_BITS = 8, TILE_ROWS = 1 << TILE_BITS, TNT = TILE_ROWS / 2;
 // Shared-memory slots are the element's index with its upper bits folded onto
 // bits 1..3 (16-byte units of a 128-byte line), so a slot is the XOR of its
@@ -754,8 +757,8 @@ cudaError_t launch_tiles(const float2* A, const float2* B, float2* C, const Gemm
   const int cv = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && (d.c_lo & 1) == 0 && (d.c_hi & 1) == 0;
   auto one = [&](auto nn) -> cudaError_t {
     constexpr int NN = decltype(nn)::value;
-    if (im_first) launch_overlapped(vector_tile_kernel<NK, NN, true>, g, dim3(TNT), 0, s, A, B, C, d, rt, av, cv);
-    else launch_overlapped(vector_tile_kernel<NK, NN, false>, g, dim3(TNT), 0, s, A, B, C, d, rt, av, cv);
+    if (im_first) vector_tile_kernel<NK, NN, true><<<g, TNT, 0, s>>>(A, B, C, d, rt, av, cv);
+    else vector_tile_kernel<NK, NN, false><<<g, TNT, 0, s>>>(A, B, C, d, rt, av, cv);
     return cudaGetLastError();
   };
   switch (d.nn) {
