@@ -1,8 +1,11 @@
 """Accumulation chunks of one to three K stages (TN_SPLIT_CHUNK): a contracted index
 of two or more stages is then several chunks, each an item of its own where the
-tiles are few.  Every tile width, one tile and several, K from one stage on; the entry point with static scratch chains the same chunks, so its output
-must be equal bit for bit, and FP64 bounds it (split products, 2e-5 as in the
-pairwise tests)."""
+tiles are few.  Pairs: every tile width of the rule, one tile and several, K from
+one stage on; the entry point with static scratch chains the same chunks, so its
+output must be equal bit for bit, and FP64 bounds it (split products, 2e-5 as in
+the pairwise tests).  Amplitudes: the widest tiles, from a tuner file; every width
+adds the same chunks in the same order, so the amplitudes are those of the rule's
+own width."""
 import os
 import subprocess
 import sys
@@ -11,7 +14,7 @@ import pytest
 
 pytestmark = pytest.mark.gpu
 
-CHILD = """
+PAIRS = """
 import torch
 from _lib import tnlib
 from test_gpu_direct import _case
@@ -27,11 +30,45 @@ for nm, nn, nk in [(7, 4, 6), (8, 5, 7), (7, 6, 5), (7, 6, 6), (9, 6, 7), (7, 7,
         assert torch.equal(torch.view_as_real(C), torch.view_as_real(D)), (nm, nn, nk, order)
 """
 
+# the 4x5 circuit, depth 1+10+1, 6 open qubits: two steps of log2 M, N, K = (8, 7, 7), one unit each
+WIDE = """
+import os
+import numpy as np
+import tn_inputs as I
+from _lib import tnlib
+T = tnlib()
+net = T.build_network(T.random_circuit(4, 5, 10, 1), list(range(14, 20)))
+words = I.bitstrings(20, 1, 3)
+plans = [T.plan(net, num_sliced=0, search_trials=4, seed=1) for _ in range(2)]
+info = plans[0].info()
+tensors, _ = plans[0].layout()
+shapes = [(t["log2_m"], t["log2_n"], t["log2_k"]) for t in tensors[info["num_leaves"]:]]
+assert (8, 7, 7) in shapes, shapes
+for precision in ("split_bf16", "split_fp16"):
+    with open(os.environ["TN_AUTOTUNE_CACHE"], "a") as f:
+        for s, (m, n, k) in enumerate(shapes):
+            if m >= 7 and n >= 6 and k >= 3:
+                print("%x %d %d %d 8 1" % (info["hash"], T.PREC[precision], s, 128 if n >= 7 else 64), file=f)
+for precision in ("split_bf16", "split_fp16"):
+    ref = plans[0].contract_amplitudes(words, precision=precision, handover=2)
+    got = plans[1].contract_amplitudes(words, precision=precision, handover=2, autotune=True)
+    assert np.array_equal(got, ref), precision
+"""
+
+
+def _child(code, **env):
+    here = os.path.dirname(os.path.abspath(__file__))
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([here, os.path.dirname(here), os.environ.get("PYTHONPATH", "")]),
+               **env)
+    r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+
 
 @pytest.mark.parametrize("chunk", [1, 2, 3])
-def test_short_chunks(chunk):
-    here = os.path.dirname(os.path.abspath(__file__))
-    env = dict(os.environ, TN_SPLIT_CHUNK=str(chunk),
-               PYTHONPATH=os.pathsep.join([here, os.path.dirname(here), os.environ.get("PYTHONPATH", "")]))
-    r = subprocess.run([sys.executable, "-c", CHILD], env=env, capture_output=True, text=True, timeout=300)
-    assert r.returncode == 0, r.stdout + r.stderr
+def test_pairs(chunk):
+    _child(PAIRS, TN_SPLIT_CHUNK=str(chunk))
+
+
+@pytest.mark.parametrize("chunk", [1, 2])
+def test_wide_tiles_from_a_tuner_file(chunk, tmp_path):
+    _child(WIDE, TN_SPLIT_CHUNK=str(chunk), TN_AUTOTUNE_CACHE=str(tmp_path / "tuned"))
