@@ -24,10 +24,10 @@
 // 115 us of kernel time, this kernel 26; the whole call 160 -> 102 us (150 with
 // the operands read through their strides instead of from shared memory).
 #include <algorithm>
-#include <mutex>
 
 #include "device_common.h"
 #include "kernels.h"
+#include "per_device.h"
 
 namespace tn {
 
@@ -225,16 +225,9 @@ cudaError_t launch_chain(const ChainStep* steps, const ChainRun& run, const Chai
                          const float2* leaf_store, const LeafGather* leaves, int nleaves, float2* gather_arena,
                          int64_t gather_stride, const GroupArg& group, cudaStream_t s) {
   if (run.count < 1 || run.count > 64 || units < 1) return cudaErrorInvalidValue;
-  static std::once_flag once[64];
-  static cudaError_t attr[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static PerDevice once;
+  const cudaError_t e = allow_smem(once, chain_kernel, CHAIN_SMEM);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::call_once(once[dev], [&] {
-    attr[dev] = cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CHAIN_SMEM);
-  });
-  if (attr[dev] != cudaSuccess) return attr[dev];
   // threads for the widest step's items, and enough to copy the operands in
   // about eight loads each; fewer once the units fill the SMs by themselves
   const int cap = units >= 304 ? 128 : 512;

@@ -10,9 +10,8 @@
 // pass through shared memory.  Consecutive threads read consecutive k, so the
 // reads coalesce when the contracted indices are the operands' fastest ones
 // (the planner's layout puts them there).
-#include <mutex>
-
 #include "kernels.h"
+#include "per_device.h"
 
 namespace tn {
 
@@ -248,16 +247,9 @@ constexpr int SPREAD_UNITS = 152;
 
 template <bool WIDE>
 cudaError_t launch_spread_as(const float2* A, const float2* B, float2* C, const GemmDesc& d, cudaStream_t s) {
-  static std::once_flag once[64];
-  static cudaError_t attr[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static PerDevice once;
+  const cudaError_t e = allow_smem(once, reduce_spread_kernel<WIDE>, SP_SMEM);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::call_once(once[dev], [&] {
-    attr[dev] = cudaFuncSetAttribute(reduce_spread_kernel<WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SP_SMEM);
-  });
-  if (attr[dev] != cudaSuccess) return attr[dev];
   const int wm = d.nm > 0 ? 1 : 0, wn = d.nn > 0 ? 1 : 0;
   const dim3 grid(8u << (d.nm - wm + d.nn - wn), (unsigned)d.units);
   const unsigned warps = (1u << (wm + wn)) + (1u << wm) + (1u << wn);  // adding, copying

@@ -38,6 +38,7 @@
 
 #include "device_common.h"
 #include "kernels.h"
+#include "per_device.h"
 
 namespace tn {
 
@@ -315,13 +316,9 @@ __global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_ker
 template <int BM, int BN, int BK, int RM, int RN, bool PACKED = true>
 cudaError_t launch_tile(const float2* A, const float2* B, float2* C, const GemmDesc& d, int flags, cudaStream_t s) {
   constexpr int SMEM = SimtCfg<BM, BN, BK, RM, RN, PACKED>::SMEM;
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, BN, BK, RM, RN, PACKED>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static PerDevice once;
+  const cudaError_t e = allow_smem(once, gemm_simt_kernel<BM, BN, BK, RM, RN, PACKED>, SMEM);
+  if (e != cudaSuccess) return e;
   const int64_t M = int64_t(1) << d.nm, N = int64_t(1) << d.nn;
   dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), (unsigned)d.units);
   return launch_overlapped(gemm_simt_kernel<BM, BN, BK, RM, RN, PACKED>, grid, dim3(NT), SMEM, s, A, B,

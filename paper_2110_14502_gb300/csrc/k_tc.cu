@@ -31,6 +31,7 @@
 #include <cuda_fp16.h>
 
 #include "kernels.h"
+#include "per_device.h"
 
 namespace tn {
 
@@ -448,13 +449,9 @@ bool tc_shape_ok(const GemmDesc& d) { return d.nm >= 7 && d.nn >= 4 && d.nk >= 3
 template <bool BF16, int TN>
 static cudaError_t launch_cfg(const float2* A, const float2* B, float2* C, const GemmDesc& d, float as, float bs,
                               int* err, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BF16, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         Cfg<TN>::SMEM);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static PerDevice once;
+  const cudaError_t e = allow_smem(once, gemm_tc_kernel<BF16, TN>, Cfg<TN>::SMEM);
+  if (e != cudaSuccess) return e;
   const int64_t M = int64_t(1) << d.nm, N = int64_t(1) << d.nn;
   dim3 grid((unsigned)(M / TM), (unsigned)((N + TN - 1) / TN), (unsigned)d.units);
   gemm_tc_kernel<BF16, TN><<<grid, NTHREADS, Cfg<TN>::SMEM, s>>>(A, B, C, d, as, bs, err);

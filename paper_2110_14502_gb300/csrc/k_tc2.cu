@@ -44,12 +44,14 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 #include <mutex>
 #include <type_traits>
 
 #include "device_common.h"
 #include "kernels.h"
+#include "per_device.h"
 
 namespace tn {
 
@@ -1479,9 +1481,14 @@ bool encode_planes(CUtensorMap* map, const PlaneOperand& o, int box_rows, int bo
 
 // SM count of the current device (one CTA per SM for the persistent kernels).
 int sm_count() {
+  static std::atomic<int> known[64] = {};
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
+  const bool keep = dev >= 0 && dev < 64;
+  if (keep) sms = known[dev].load(std::memory_order_relaxed);
+  if (sms > 0) return sms;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (keep && sms > 0) known[dev].store(sms, std::memory_order_relaxed);
   return sms > 0 ? sms : 148;
 }
 
@@ -1490,20 +1497,13 @@ cudaError_t launch_chunked_ew(const CUtensorMap& ma, const CUtensorMap& mb, floa
                               const int z[4], int out_flags, const ScaleIO& sio, int fold, bool bf16, int* err,
                               cudaStream_t s, const BulkPlanes& ba, const BulkPlanes& bb, int parts, float2* part) {
   using CC = ChunkCfg<TN, NP, ROWB, EW>;
-  static bool attr = false;
-  static int sms = 0;
-  if (!attr) {
-    cudaError_t e =
-        cudaFuncSetAttribute(gemm_tma_chunked<TN, NP, ROWB, EW, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             CC::SMEM);
-    if (e != cudaSuccess) return e;
-    sms = sm_count();
-    attr = true;
-  }
+  static PerDevice once;
+  const cudaError_t e = allow_smem(once, gemm_tma_chunked<TN, NP, ROWB, EW, PARTS>, CC::SMEM);
+  if (e != cudaSuccess) return e;
   const int64_t M = int64_t(1) << d.nm, N = int64_t(1) << d.nn;
   const int64_t items = (M / TM) * (fold > 1 ? 1 : N / TN) * (d.units / fold) * parts;
   const int chunk = NP == 4 ? split_chunk() : 1 << 30;
-  const unsigned grid = (unsigned)std::min<int64_t>(items, sms);
+  const unsigned grid = (unsigned)std::min<int64_t>(items, sm_count());
   return launch_overlapped(gemm_tma_chunked<TN, NP, ROWB, EW, PARTS>, dim3(grid), dim3(CC::THREADS), CC::SMEM, s, ma,
                            mb, C, d, kp, z[0], z[1], z[2], z[3], out_flags, sio, chunk, fold, bf16, err, ba, bb, parts, part);
 }
@@ -1577,15 +1577,10 @@ template <int TN, int NP, bool BF16>
 cudaError_t launch_direct_as(const CUtensorMap& mb, const float2* A, float2* C, const GemmDesc& d, const unsigned* maxA,
                              const int* exp_b, int* err, cudaStream_t s) {
   using DC = DirectCfg<TN, NP>;
-  static bool attr = false;
-  static int sms = 0;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_direct<TN, NP, BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, DC::SMEM);
-    if (e != cudaSuccess) return e;
-    sms = sm_count();
-    attr = true;
-  }
-  const unsigned grid = (unsigned)std::min<int64_t>(int64_t(1) << (d.nm - 7), sms);
+  static PerDevice once;
+  const cudaError_t e = allow_smem(once, gemm_direct<TN, NP, BF16>, DC::SMEM);
+  if (e != cudaSuccess) return e;
+  const unsigned grid = (unsigned)std::min<int64_t>(int64_t(1) << (d.nm - 7), sm_count());
   const int chunk = NP == 4 ? split_chunk() : 1 << 30;
   const int av = (reinterpret_cast<uintptr_t>(A) & 15) == 0, cv = (reinterpret_cast<uintptr_t>(C) & 15) == 0;
   return launch_overlapped(gemm_direct<TN, NP, BF16>, dim3(grid), dim3(DC::THREADS), DC::SMEM, s, mb, A, C, d,
