@@ -166,28 +166,19 @@ inline void turn_slots(const int* order, int32_t* slot) {
 // let_next_start (or ended), and hold at after_previous until the whole previous
 // grid has finished and its writes are visible.  A kernel launched this way
 // calls after_previous before it touches memory that others write or read, and
-// reads what earlier kernels wrote by ordinary loads: no __ldg, and no `const T*
-// __restrict__` parameter, from which the compiler makes the same read-only loads.
-// Those take the memory as constant for the life of the grid, which it is not when
-// the grid starts before its producer has ended, and nothing keeps them below the
-// wait.  (What no kernel writes, descriptors and leaves, may be read that way.)  A
-// step of a small circuit is a few microseconds, of which a plain launch is one or
-// two.
+// reads what earlier kernels wrote by ordinary loads or __ldcg: no __ldg, and no
+// `const T* __restrict__` parameter, from which the compiler makes the same
+// read-only loads.  Those take the memory as constant for the life of the grid,
+// which it is not when the grid starts before its producer has ended, and nothing
+// keeps them below the wait.  (What no kernel writes, descriptors and leaves, may be
+// read that way.)  A step of a small circuit is a few microseconds, of which a plain
+// launch is one or two.
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// One element of what an earlier kernel wrote: an ordinary load in a kernel that
-// starts early, a read-only one in a kernel launched plainly.
-template <bool EARLY, class T>
-__device__ __forceinline__ T load(const T* p) {
-  if constexpr (EARLY) return *p;
-  else return __ldg(p);
-}
-
-// A launch that starts early (`early`) or plainly.
 template <class... P, class... A>
-inline cudaError_t launch_kernel(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                 A&&... args) {
+inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                     A&&... args) {
   cudaLaunchConfig_t c{};
   c.gridDim = grid;
   c.blockDim = block;
@@ -200,18 +191,12 @@ inline cudaError_t launch_kernel(bool early, void (*kernel)(P...), dim3 grid, di
   // in a captured sequence, whose replay has no launch cost to hide, plainly
   // (5x5 circuit, 24 kernels: 289 us replayed, 294 with overlapping edges)
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  if (early && cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
     cudaGetLastError();
     capture = cudaStreamCaptureStatusActive;
   }
-  c.numAttrs = early && capture == cudaStreamCaptureStatusNone ? 1 : 0;
+  c.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
   return cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
-}
-
-template <class... P, class... A>
-inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                     A&&... args) {
-  return launch_kernel(true, kernel, grid, block, smem, s, std::forward<A>(args)...);
 }
 
 }  // namespace tn

@@ -73,7 +73,9 @@ __global__ void __launch_bounds__(NT) max_kernel(const float2* __restrict__ src,
 // values per thread through the index strides touched a 32-byte sector per
 // 8-byte element on random orders: a 2^29-element operand took 2.8 ms for its
 // maximum and 3.4 ms for its split, whose bytes move in 0.64 and 1.3 ms; the
-// (16, 6, 13) contraction it belongs to went from 7.3 to 3.4 ms with this.)
+// (16, 6, 13) contraction it belongs to went from 7.3 to 3.4 ms with this.)  The
+// loads go past L1, where a line would stay for nothing: log2 M, N, K = (13, 6, 13)
+// in scaled fp16 302 us per call, through L1 about 20 us more.
 struct TileMap {
   int nout;                 // index bits outside the tile
   int32_t out_src[kMaxBits];   // their strides in the input ..
@@ -97,13 +99,6 @@ struct SplitJob {
   int* e_out;
   float* m_out;
 };
-
-// The passes over small operands start early; those over large ones (2^12 tiles)
-// are launched plainly and read past the coherent path, which is faster by more
-// than a launch (a 2^26-element operand for scaled fp16, (13, 6, 13): the call
-// takes 316 us, started early with ordinary loads 335).
-template <int T>
-constexpr bool kSplitEarly = T < 12;
 
 template <int NP, int T, bool BF16>
 __device__ __forceinline__ void split_tile(const SplitJob& job, const TileMap& tm, unsigned blk, int64_t z) {
@@ -157,12 +152,12 @@ __device__ __forceinline__ void split_tile(const SplitJob& job, const TileMap& t
       for (int b = 0; b < T - 1 - TB; ++b)
         if ((j >> b) & 1) o += tm.in_src[1 + TB + b];
       if (vec) {
-        const float4 x = load<kSplitEarly<T>>(reinterpret_cast<const float4*>(src + o));
+        const float4 x = __ldcg(reinterpret_cast<const float4*>(src + o));
         v[j][0] = make_float2(x.x, x.y);
         v[j][1] = make_float2(x.z, x.w);
       } else {
-        v[j][0] = load<kSplitEarly<T>>(src + o);
-        v[j][1] = load<kSplitEarly<T>>(src + o + 1);
+        v[j][0] = __ldcg(src + o);
+        v[j][1] = __ldcg(src + o + 1);
       }
     }
 #pragma unroll
@@ -354,8 +349,8 @@ cudaError_t launch_split(const float2* src, uint16_t* dst, const SplitDesc& d, i
   const SplitJob job = split_job(src, dst, d, maxbits, e_out, m_out);
   return for_format(np, bf16, tile_bits(R, nz), [&](auto n, auto t, auto fmt) {
     constexpr int T = decltype(t)::value;
-    return launch_kernel(kSplitEarly<T>, split_kernel<decltype(n)::value, T, decltype(fmt)::value>,
-                         dim3(1u << (R - T), (unsigned)nz), dim3(NT), 0, s, job, split_tile_map<T>(d));
+    return launch_overlapped(split_kernel<decltype(n)::value, T, decltype(fmt)::value>,
+                             dim3(1u << (R - T), (unsigned)nz), dim3(NT), 0, s, job, split_tile_map<T>(d));
   });
 }
 
@@ -442,9 +437,9 @@ static cudaError_t split_pair(const float2* A, const float2* B, const GemmDesc& 
   if (ta == tb || (T == 10 && large <= 20) || (T == 7 && large <= 14))
     return for_format(np, bf16, T, [&](auto n, auto t, auto fmt) {
       constexpr int TT = decltype(t)::value;
-      return launch_kernel(kSplitEarly<TT>, split_pair_kernel<decltype(n)::value, TT, decltype(fmt)::value>,
-                           dim3((1u << (ra - TT)) + (1u << (rb - TT))), dim3(NT), 0, s, ja, split_tile_map<TT>(da), jb,
-                           split_tile_map<TT>(db));
+      return launch_overlapped(split_pair_kernel<decltype(n)::value, TT, decltype(fmt)::value>,
+                               dim3((1u << (ra - TT)) + (1u << (rb - TT))), dim3(NT), 0, s, ja, split_tile_map<TT>(da),
+                               jb, split_tile_map<TT>(db));
     });
   const cudaError_t e = launch_split(A, scratch, da, 1, bf16, np, mx, ex, ms, s, true);
   return e != cudaSuccess ? e

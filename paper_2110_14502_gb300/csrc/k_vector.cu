@@ -473,10 +473,10 @@ __global__ void __launch_bounds__(SNT) vector_staged_kernel(const float2* A, con
 // of C front to back from shared memory.  B sits in shared memory as (re, im,
 // im, re), one 16-byte read for both packed products of a complex
 // multiply-add; the sums run in the order of the kernel that would otherwise
-// take the shape (IM_FIRST), so the results are the same bit for bit.  Launched
-// plainly: its read-only loads, which an early start would rule out, are worth
-// more than the start (log2 M, N, K = (22, 3, 4) 206 us per call; started early,
-// with ordinary loads 224, past L1 212, and with B's values fetched first 225).
+// take the shape (IM_FIRST), so the results are the same bit for bit.  A's
+// loads go past L1, where a line would stay for nothing: log2 M, N, K = (22, 3, 4)
+// 184 us per call back to back, through L1 198; (21, 4, 4) with the contracted
+// indices innermost 153 and 178.
 constexpr int TILE_BITS = 8, TILE_ROWS = 1 << TILE_BITS, TNT = TILE_ROWS / 2;
 // Shared-memory slots are the element's index with its upper bits folded onto
 // bits 1..3 (16-byte units of a 128-byte line), so a slot is the XOR of its
@@ -494,8 +494,7 @@ struct RowTile {
 __device__ __forceinline__ void acc2(f32x2& c, f32x2 a, f32x2 b) { c = fma2(a, b, c); }
 
 template <int NK, int NN, bool IM_FIRST>
-__global__ void __launch_bounds__(TNT) vector_tile_kernel(const float2* __restrict__ A, const float2* __restrict__ B,
-                                                          float2* __restrict__ C, const GemmDesc d,
+__global__ void __launch_bounds__(TNT) vector_tile_kernel(const float2* A, const float2* B, float2* __restrict__ C, const GemmDesc d,
                                                           const __grid_constant__ RowTile rt, int a_vec, int c_vec) {
   constexpr int K = 1 << NK, N = 1 << NN;
   constexpr int AE = TILE_ROWS * K, CE = TILE_ROWS * N;
@@ -536,12 +535,12 @@ __global__ void __launch_bounds__(TNT) vector_tile_kernel(const float2* __restri
       for (int b = 0; b < NK; ++b)
         if ((j >> b) & 1) o += rt.a_src[8 + b];
       if (a_vec) {
-        const float4 x = __ldg(reinterpret_cast<const float4*>(A + o));
+        const float4 x = __ldcg(reinterpret_cast<const float4*>(A + o));
         v[j][0] = make_float2(x.x, x.y);
         v[j][1] = make_float2(x.z, x.w);
       } else {
-        v[j][0] = __ldg(A + o);
-        v[j][1] = __ldg(A + o + 1);
+        v[j][0] = __ldcg(A + o);
+        v[j][1] = __ldcg(A + o + 1);
       }
     }
 #pragma unroll
@@ -757,8 +756,8 @@ cudaError_t launch_tiles(const float2* A, const float2* B, float2* C, const Gemm
   const int cv = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && (d.c_lo & 1) == 0 && (d.c_hi & 1) == 0;
   auto one = [&](auto nn) -> cudaError_t {
     constexpr int NN = decltype(nn)::value;
-    if (im_first) vector_tile_kernel<NK, NN, true><<<g, TNT, 0, s>>>(A, B, C, d, rt, av, cv);
-    else vector_tile_kernel<NK, NN, false><<<g, TNT, 0, s>>>(A, B, C, d, rt, av, cv);
+    if (im_first) launch_overlapped(vector_tile_kernel<NK, NN, true>, g, dim3(TNT), 0, s, A, B, C, d, rt, av, cv);
+    else launch_overlapped(vector_tile_kernel<NK, NN, false>, g, dim3(TNT), 0, s, A, B, C, d, rt, av, cv);
     return cudaGetLastError();
   };
   switch (d.nn) {

@@ -1,8 +1,7 @@
 """Kernels launched so that they start before the kernel in front of them has ended
 must not read its output through the read-only path (__ldg, or const T*
 __restrict__ parameters): that path takes the memory as constant while the kernel
-runs (load<early> chooses, where a rule decides the launch).  Checked on the
-sources; a race would show only now and then."""
+runs.  Checked on the sources; a race would show only now and then."""
 import glob
 import os
 import re
@@ -47,9 +46,8 @@ def test_no_read_only_loads_of_earlier_kernels_output():
     launched = set()
     for text in sources.values():
         launched |= set(re.findall(r"launch_overlapped\(\s*(\w+)", text))
-        launched |= set(re.findall(r"launch_kernel\([^;]*?(\w+_kernel)<", text))  # early or plainly, by a rule
     launched -= {"void"}  # its own declaration
-    assert {"chain_kernel", "split_kernel", "gemm_simt_kernel", "split_pair_kernel", "gemm_direct"} <= launched, launched
+    assert {"chain_kernel", "split_kernel", "gemm_simt_kernel", "vector_tile_kernel", "gemm_direct"} <= launched, launched
     seen, bad = set(), []
     for name, text in sources.items():
         if not any(k in launched for k, _, _ in _kernels(text)):
