@@ -34,6 +34,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "scratch.h"
 #include "tn_internal.h"
 
 namespace tn {
@@ -153,8 +154,7 @@ struct Executor {
   int* err = nullptr;
   volatile int* err_host = nullptr;
   void* stage = nullptr;
-  uint16_t* scratch = nullptr; // split operand planes of the tensor-core steps
-  int64_t scratch_cap = 0;     // in 16-bit elements
+  Scratch scratch;             // split operand planes of the tensor-core steps, and their partial sums
   // scaled precisions: per step and launch unit, exponent and stored maximum
   // of plane outputs; per split role the same plus the max reduction; flags
   uint8_t* spool = nullptr;
@@ -194,7 +194,7 @@ void destroy_executor(Executor* e) {
   cudaFree(e->chain);
   cudaFree(e->bits);
   cudaFree(e->acc);
-  cudaFree(e->scratch);
+  cudaFree(e->scratch.p);
   cudaFree(e->spool);
   cudaFree(e->flagged);
   cudaFree(e->nflagged);
@@ -675,7 +675,9 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
       c.scratch_min = std::max(c.scratch_min, need_planes);
       return TN_OK;
     }
-    if (need_planes > E.scratch_cap) return fail(TN_EINVAL, "step %zu: internal error, operand scratch not sized", s);
+    const int64_t scratch_cap = (int64_t)(E.scratch.bytes / sizeof(uint16_t));
+    uint16_t* const scratch = static_cast<uint16_t*>(E.scratch.p);
+    if (need_planes > scratch_cap) return fail(TN_EINVAL, "step %zu: internal error, operand scratch not sized", s);
     for (auto& t : E.tuned)
       if (t.precision == c.precision && t.step == (int)s) {
         d.tile_n = t.tile_n;
@@ -691,7 +693,7 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
       unsigned* mx = ready ? c.mc_all + (S.a - L) * U : c.mb[0];
       if (c.scaled && !ready) e = cudaMemsetAsync(c.mb[0], 0, U * sizeof(unsigned), c.st);
       if (e == cudaSuccess)
-        e = split_operand(A, d, false, c.bf16, c.np, c.scaled, mx, c.es[0], c.ms[0], E.scratch, pa, c.st, ready);
+        e = split_operand(A, d, false, c.bf16, c.np, c.scaled, mx, c.es[0], c.ms[0], scratch, pa, c.st, ready);
       c.launches += c.scaled && !ready ? 2 : 1;
       sio.ea = c.es[0];
       sio.ma = c.ms[0];
@@ -704,7 +706,7 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
       unsigned* mx = ready ? c.mc_all + (S.b - L) * U : c.mb[1];
       if (e == cudaSuccess && c.scaled && !ready) e = cudaMemsetAsync(c.mb[1], 0, U * sizeof(unsigned), c.st);
       if (e == cudaSuccess)
-        e = split_operand(B, d, true, c.bf16, c.np, c.scaled, mx, c.es[1], c.ms[1], E.scratch + need_a, pb, c.st,
+        e = split_operand(B, d, true, c.bf16, c.np, c.scaled, mx, c.es[1], c.ms[1], scratch + need_a, pb, c.st,
                           ready);
       c.launches += c.scaled && !ready ? 2 : 1;
       sio.eb = c.es[1];
@@ -770,11 +772,11 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
       d.tile_n = bt;
       d.group_m = bg;
     }
-    const bool parts = need_part > 0 && need <= E.scratch_cap && tc_part_elems(d, c.np, c.planes_out[s] != 0) > 0;
+    const bool parts = need_part > 0 && need <= scratch_cap && tc_part_elems(d, c.np, c.planes_out[s] != 0) > 0;
     if (parts) ++c.launches;
     if (e == cudaSuccess)
       e = launch_gemm_tma(pa, pb, C, c.planes_out[s] != 0, d, c.bf16, sio, E.err, c.st,
-                          parts ? reinterpret_cast<float2*>(E.scratch + need_planes) : nullptr);
+                          parts ? reinterpret_cast<float2*>(scratch + need_planes) : nullptr);
   }
   else e = launch_gemm_simt(A, B, C, d, c.st);
   ++c.launches;
@@ -910,7 +912,7 @@ tn_status contract_amplitudes_ex(Plan& P, const uint64_t* bits, int64_t nb, doub
 int64_t executor_bytes(const Plan& P) {
   const Executor* E = P.exec;
   if (!E) return 0;
-  return 8 * (E->sarena_cap + E->parena_cap + P.invariant_elems + P.leaf_store_elems) + 2 * E->scratch_cap +
+  return 8 * (E->sarena_cap + E->parena_cap + P.invariant_elems + P.leaf_store_elems) + (int64_t)E->scratch.bytes +
          E->spool_cap;
 }
 
@@ -1149,23 +1151,16 @@ static tn_status contract_core(Plan& P, const uint64_t* bits, int64_t nb, double
         if (r != TN_OK) return r;
       }
     c.sizing = false;
-    if (c.scratch_need > E.scratch_cap) {
-      drop_graphs();
-      cudaFree(E.scratch);
-      E.scratch = nullptr;
-      E.scratch_cap = 0;
-      if (c.scratch_need > c.scratch_min &&
-          dev_alloc(&E.scratch, (size_t)c.scratch_need * sizeof(uint16_t)) != cudaSuccess) {
-        cudaGetLastError();
-        c.scratch_need = c.scratch_min;
-      }
-      if (!E.scratch && dev_alloc(&E.scratch, (size_t)c.scratch_need * sizeof(uint16_t)) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(TN_EHBM, "tn_contract_amplitudes: %lld bytes of operand planes do not fit",
-                    (long long)(c.scratch_need * 2));
-      }
-      E.scratch_cap = c.scratch_need;
-    }
+    auto alloc = [](size_t bytes) {
+      void* p = nullptr;
+      if (dev_alloc(&p, bytes) == cudaSuccess) return p;
+      cudaGetLastError();
+      return (void*)nullptr;
+    };
+    if (!reserve(E.scratch, (size_t)c.scratch_min * sizeof(uint16_t), (size_t)c.scratch_need * sizeof(uint16_t), alloc,
+                 cudaFree, drop_graphs))
+      return fail(TN_EHBM, "tn_contract_amplitudes: %lld bytes of operand planes do not fit",
+                  (long long)(c.scratch_min * 2));
   }
   // autotuner: the first group of a precision times the tile choices
   if (c.tc && o.autotune) {

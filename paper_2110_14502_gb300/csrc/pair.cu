@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "scratch.h"
 #include "tn_internal.h"
 
 namespace tn {
@@ -51,13 +52,13 @@ static cublasHandle_t cublas_handle(int dev) {
 struct PairDevState {
   int* err = nullptr;                 // device address of the word ..
   volatile int* err_host = nullptr;   // .. and host address
-  void* scratch = nullptr;
-  size_t bytes = 0;
+  Scratch scratch;
 };
 static std::mutex g_pair_mu;
 static std::vector<PairDevState> g_pair_state;
 
-static tn_status pair_state(size_t need, PairDevState*& out) {
+// (want: with what a call can do without)
+static tn_status pair_state(size_t need, size_t want, PairDevState*& out) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return fail(TN_ECUDA, "tn_contract_pair: cudaGetDevice failed");
   if ((int)g_pair_state.size() <= dev) g_pair_state.resize(dev + 1);
@@ -74,16 +75,15 @@ static tn_status pair_state(size_t need, PairDevState*& out) {
     *st.err_host = 0;
     st.err = static_cast<int*>(p);
   }
-  if (need > st.bytes) {
-    cudaFree(st.scratch);  // the previous call on this device has finished
-    st.scratch = nullptr;
-    st.bytes = 0;
-    if (cudaMalloc(&st.scratch, need) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(TN_EHBM, "tn_contract_pair: operand planes do not fit");
-    }
-    st.bytes = need;
-  }
+  auto alloc = [](size_t bytes) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+    cudaGetLastError();
+    return (void*)nullptr;
+  };
+  // (the previous call on this device has finished)
+  if (!reserve(st.scratch, need, want, alloc, cudaFree, [] {}))
+    return fail(TN_EHBM, "tn_contract_pair: operand planes do not fit");
   out = &st;
   return TN_OK;
 }
@@ -207,20 +207,18 @@ extern "C" tn_status tn_contract_pair(const void* A, const int32_t* a_labels, in
       std::lock_guard<std::mutex> lock(g_pair_mu);
       // operand planes, then 32 bytes for the scaled modes' maxima and exponents
       const bool fused = algo == TN_PAIR_FUSED_TC;
-      bool sums = true;  // with space for partial sums, unless that does not fit
-      size_t planes = fused ? (size_t)tc2_pair_scratch_elems(d, true) * sizeof(uint16_t) : 0;
+      // (with space for partial sums, unless that does not fit)
+      const size_t least = fused ? (size_t)tc2_pair_scratch_elems(d, false) * sizeof(uint16_t) : 0;
+      const size_t most = fused ? (size_t)tc2_pair_scratch_elems(d, true) * sizeof(uint16_t) : 0;
       PairDevState* ps = nullptr;
-      tn_status pst = pair_state(planes + 32, ps);
-      if (pst == TN_EHBM && fused) {
-        sums = false;
-        planes = (size_t)tc2_pair_scratch_elems(d, false) * sizeof(uint16_t);
-        pst = pair_state(planes + 32, ps);
-      }
+      const tn_status pst = pair_state(least + 32, most + 32, ps);
       if (pst != TN_OK) return pst;
+      const bool sums = ps->scratch.bytes >= most + 32;
+      const size_t planes = sums ? most : least;
       int* err = ps->err;
       if (fused) {
-        uint16_t* scratch = static_cast<uint16_t*>(ps->scratch);
-        void* aux = static_cast<char*>(ps->scratch) + planes;
+        uint16_t* scratch = static_cast<uint16_t*>(ps->scratch.p);
+        void* aux = static_cast<char*>(ps->scratch.p) + planes;
         switch (precision) {
           case TN_PREC_SPLIT_BF16: e = run_gemm_tc2(a, b, c, d, true, sums, scratch, err, s); break;
           case TN_PREC_SPLIT_FP16: e = run_gemm_tc2_scaled(a, b, c, d, false, 4, sums, scratch, aux, err, s); break;
