@@ -741,23 +741,33 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
                         (a_in ? 0 : 1) | (b_in ? 0 : 2), 0, 0, 0});
       e0 = em;
     }
+    // space for partial sums: where the descriptor's tiles use it and it was had
+    auto sums = [&](const GemmDesc& g) {
+      return need_part > 0 && need <= scratch_cap && tc_part_elems(g, c.np, c.planes_out[s] != 0) > 0
+                 ? reinterpret_cast<float2*>(scratch + need_planes)
+                 : nullptr;
+    };
+    auto gemm = [&](const GemmDesc& g) {
+      return launch_gemm_tma(pa, pb, C, c.planes_out[s] != 0, g, c.bf16, sio, E.err, c.st, sums(g));
+    };
     if (e == cudaSuccess && c.tuning) {
-      // autotuner: time each tile choice once (every candidate writes the same
-      // result; the last launch below leaves it in place) and keep the fastest
-      const int def_n = d.nn >= 7 ? 128 : (1 << d.nn);
+      // autotuner: time each tile choice once, launched as it will be (every
+      // candidate writes the same result; the last launch below leaves it in
+      // place), and keep the fastest
       float best = 1e30f;
       int bt = 0, bg = 0;
-      for (int tn : {128, 64}) {
-        if (tn > def_n) continue;
+      int widths[3];
+      const int nw = tma_tile_widths(d, widths);
+      for (int i = 0; i < nw; ++i) {
         for (int gm : {8, 16, 32}) {
           GemmDesc dc = d;
-          dc.tile_n = tn;
+          dc.tile_n = widths[i];
           dc.group_m = gm;
           cudaEvent_t t0, t1;
           cudaEventCreate(&t0);
           cudaEventCreate(&t1);
           cudaEventRecord(t0, c.st);
-          e = launch_gemm_tma(pa, pb, C, c.planes_out[s] != 0, dc, c.bf16, sio, E.err, c.st);
+          e = gemm(dc);
           cudaEventRecord(t1, c.st);
           cudaEventSynchronize(t1);
           float ms = 0;
@@ -765,18 +775,15 @@ tn_status run_step_in(Ctx& c, size_t s, const Geo& g) {
           cudaEventDestroy(t0);
           cudaEventDestroy(t1);
           if (e != cudaSuccess) break;
-          if (ms < best) { best = ms; bt = tn; bg = gm; }
+          if (ms < best) { best = ms; bt = widths[i]; bg = gm; }
         }
       }
       E.tuned.push_back({c.precision, (int)s, bt, bg});
       d.tile_n = bt;
       d.group_m = bg;
     }
-    const bool parts = need_part > 0 && need <= scratch_cap && tc_part_elems(d, c.np, c.planes_out[s] != 0) > 0;
-    if (parts) ++c.launches;
-    if (e == cudaSuccess)
-      e = launch_gemm_tma(pa, pb, C, c.planes_out[s] != 0, d, c.bf16, sio, E.err, c.st,
-                          parts ? reinterpret_cast<float2*>(scratch + need_planes) : nullptr);
+    if (sums(d)) ++c.launches;
+    if (e == cudaSuccess) e = gemm(d);
   }
   else e = launch_gemm_simt(A, B, C, d, c.st);
   ++c.launches;

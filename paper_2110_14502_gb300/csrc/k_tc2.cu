@@ -1598,12 +1598,21 @@ cudaError_t set_tc_wait_limit(long long polls) {
 // that spreads the work over more SMs, by waves over 152 SMs times the time of
 // a tile relative to 128 columns (a narrow MMA is less efficient, and a tile's
 // A copy does not shrink).  Every width gives the same bits.
-int tma_tile_n(const GemmDesc& d) {
+int tma_tile_widths(const GemmDesc& d, int (&widths)[3]) {
+  int n = 0;
   const int def = d.nn >= 7 ? 128 : (1 << d.nn);
+  for (int tn = def; tn >= (def < 32 ? def : 32); tn /= 2) widths[n++] = tn;
+  return n;
+}
+
+int tma_tile_n(const GemmDesc& d) {
+  int widths[3];
+  const int n = tma_tile_widths(d, widths), def = widths[0];
   if (d.tile_n >= 16 && d.tile_n <= def) return d.tile_n;
   int best = def;
   double best_cost = 1e300;
-  for (int tn = def; tn >= (def < 32 ? def : 32); tn /= 2) {
+  for (int i = 0; i < n; ++i) {
+    const int tn = widths[i];
     const int64_t items = ((int64_t(1) << d.nm) / TM) * ((int64_t(1) << d.nn) / tn) * d.units;
     const double rel = tn == 128 ? 1.0 : tn == 64 ? 0.55 : tn == 32 ? 0.35 : 0.3;
     const double cost = (double)((items + 151) / 152) * rel;

@@ -108,7 +108,6 @@ struct PlaneOperand {
 // TMA-fed warp-specialized tcgen05 GEMM on plane operands.  With c_planes
 // the epilogue writes C as planes (for a tensor-core consumer) instead of
 // complex64.
-int tma_tile_n(const GemmDesc& d);
 // I/O of the scaled precisions; every pointer may be null (exponent 0, no
 // tracking).  ea/ma, eb/mb: per distinct operand tensor, the exponent e of
 // its stored values (stored = true * 2^-e) and their largest |component|.
@@ -132,6 +131,10 @@ int64_t split_plane_elems(int nrow_bits, int nk_bits, int np);
 cudaError_t set_tc_wait_limit(long long polls);
 cudaError_t launch_gemm_tma(const PlaneOperand& a, const PlaneOperand& b, float2* C, bool c_planes, const GemmDesc& d,
                             bool bf16, const ScaleIO& sio, int* err, cudaStream_t s, float2* part = nullptr);
+// Columns of its tiles, and the widths that the rule for them weighs, widest
+// first (their number is returned).
+int tma_tile_n(const GemmDesc& d);
+int tma_tile_widths(const GemmDesc& d, int (&widths)[3]);
 // 16-bit elements of scratch with which launch_gemm_tma may spread a long K over
 // idle SMs (`part`; 0: it would not).  Results are the same with and without.
 int64_t tc_part_elems(const GemmDesc& d, int np, bool c_planes);
