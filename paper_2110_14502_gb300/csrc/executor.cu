@@ -485,6 +485,10 @@ static tn_status setup(Plan& P, Executor& E) {
   CK(dev_alloc(&E.flagged, kFlaggedCap * sizeof(int64_t)));
   CK(dev_alloc(&E.gslot, 2 * sizeof(GroupInfo)));
   CK(dev_alloc(&E.nflagged, sizeof(unsigned long long)));
+  // The copies above are from pageable memory, so they may still be on their way
+  // from the driver's staging memory, and a caller's stream need not wait for the
+  // legacy stream that carries them.
+  CK(cudaStreamSynchronize(nullptr));
   return TN_OK;
 }
 
