@@ -274,9 +274,9 @@ TileMap split_tile_map(const SplitDesc& d) {
   return m;
 }
 
-// Tile size for an operand of 2^R elements, nz of them: 2^12 once that fills the
-// chip a few times over (152 SMs, six such CTAs each); smaller tiles spread a
-// small operand over more SMs.
+// Tile size for an operand of 2^R elements, nz of them: 2^12 once there are four
+// such tiles per SM (six CTAs fit one); smaller tiles spread a small operand over
+// more SMs.
 int tile_bits(int R, int nz) {
   return R >= 12 && (int64_t(1) << (R - 12)) * nz >= 152 * 4 ? 12 : R >= 10 ? 10 : 7;
 }

@@ -5,7 +5,7 @@ one stage on; the entry point with static scratch chains the same chunks, so its
 output must be equal bit for bit, and FP64 bounds it (split products, 2e-5 as in
 the pairwise tests).  Amplitudes: the widest tiles, from a tuner file; every width
 adds the same chunks in the same order, so the amplitudes are those of the rule's
-own width."""
+own width.  And a pipeline wait that expires in that form."""
 import os
 import subprocess
 import sys
@@ -72,3 +72,24 @@ def test_pairs(chunk):
 @pytest.mark.parametrize("chunk", [1, 2])
 def test_wide_tiles_from_a_tuner_file(chunk, tmp_path):
     _child(WIDE, TN_SPLIT_CHUNK=str(chunk), TN_AUTOTUNE_CACHE=str(tmp_path / "tuned"))
+
+
+def test_expired_wait_with_chunks_as_items_then_the_call_is_correct():
+    """One tile whose 16 chunks are items: every pipeline wait gives up at once, and
+    the pass that adds the chunks' sums still runs."""
+    import torch
+
+    from _lib import tnlib
+    from test_gpu_direct import _case
+    T = tnlib()
+    la, lb, lc, A, B, C, ref, at = _case(7, 7, 13, "random", 0, 11)
+    try:
+        T.set_wait_limit(0)
+        with pytest.raises(T.TnError) as ei:
+            T.contract_pair(A, la, B, lb, C, lc, precision="split_bf16", algo="fused_tc")
+        assert ei.value.status == 5, ei.value
+    finally:
+        T.set_wait_limit(-1)
+    torch.cuda.synchronize()
+    T.contract_pair(A, la, B, lb, C, lc, precision="split_bf16", algo="fused_tc")
+    assert float((C[at] - ref).norm()) <= 2e-5 * float(ref.norm())
