@@ -1709,8 +1709,8 @@ cudaError_t launch_gemm_tma(const PlaneOperand& a, const PlaneOperand& b, float2
 // Where converting A in the GEMM beats a split pass: enough row tiles to fill
 // the chip most of the time, and a K long enough that a tile's output, which
 // the same warps store, is a small part of it.  Measured per call with random
-// orders, split pass -> here: (16, 6, 13) split fp16 2675 -> 2227 us, (17, 6, 9)
-// split bf16 307 -> 251, (14, 6, 12) split fp16 391 -> 329, (17, 6, 7) 152 -> 139;
+// orders, split pass -> here: (16, 6, 13) split fp16 2675 -> 2064 us, (17, 6, 9)
+// split bf16 307 -> 223, (14, 6, 12) split fp16 391 -> 303, (17, 6, 7) 152 -> 128;
 // but (17, 6, 5) 84 -> 87, (13, 6, 14) split bf16 694 -> 882.
 bool direct_ok(const GemmDesc& d) {
   return d.units == 1 && tc_shape_ok(d) && d.nn <= 6 && d.nk >= 7 && d.nm >= 14;
