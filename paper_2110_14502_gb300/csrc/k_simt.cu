@@ -13,7 +13,11 @@
 // thread an RM-row x RN-column complex micro-tile.  The tiles are staged in
 // shared memory k-major ([k][row], rows contiguous) with two buffers: the
 // global loads of chunk c+1 are in flight in registers while chunk c is
-// computed, then stored to the other buffer; one barrier per chunk.
+// computed, then stored to the other buffer; one barrier per chunk.  They are
+// issued before the barrier, which holds ordinary loads back: log2 M, N, K =
+// (7, 9, 12) 317 us, after it 333; (12, 12, 9) 1399 and 1450, (13, 13, 5) 635 and
+// 694, (6, 4, 12) 182 and 196; with 128 x 64 tiles (16, 6, 11) 1747 and 1755, (14, 6,
+// 12) in planner order 910 and 914 but in random orders 1007 and 993.
 //
 // Arithmetic: packed FP32 (fma.rn.f32x2), one instruction for two of a complex
 // multiply-add's four FMAs: (re, im) += (ar, ar) (br, bi), then += (-ai, ai)
@@ -28,7 +32,8 @@
 // CTAs per SM and spills 1872, 1381, 469).
 //
 // What bounds the 128 x 128 tile: two warps per scheduler (246 registers, one CTA
-// per SM) do not cover the packed FMAs' latency.  Counters at (13, 13, 9), 5.8 ms:
+// per SM) do not cover the packed FMAs' latency.  Counters at (13, 13, 9), 5.8 ms,
+// with the loads after the barrier:
 // FMA pipe busy 61% of the cycles, an instruction issued in 39%; per issue a warp
 // waits 1.3 cycles on a fixed latency, 1.0 on the FMA pipe and 0.4 on instruction
 // fetch; shared memory 9% and DRAM 1% busy.
@@ -211,17 +216,17 @@ __global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_ker
   };
   const int64_t nch = (K + BK - 1) / BK;
   const int kn = K < BK ? (int)K : BK;  // K values of a chunk
-  la.load(A, 0, 0);
-  lb.load(B, 0, 0);
+  auto load_chunk = [&](int64_t c) {
+    const int64_t k = c * BK;
+    la.load(A, k, k_high_offset<ilog2(BK)>(k, d.nk, d.ak));
+    lb.load(B, k, k_high_offset<ilog2(BK)>(k, d.nk, d.bk));
+  };
+  load_chunk(0);
   store_tiles(0);
+  if (nch > 1) load_chunk(1);
   __syncthreads();
   for (int64_t c = 0; c < nch; ++c) {
     const int buf = (int)(c & 1);
-    if (c + 1 < nch) {
-      const int64_t k1 = (c + 1) * BK;
-      la.load(A, k1, k_high_offset<ilog2(BK)>(k1, d.nk, d.ak));
-      lb.load(B, k1, k_high_offset<ilog2(BK)>(k1, d.nk, d.bk));
-    }
     const AT* const a0 = As + buf * BK * BM + RM * tm;
     const ulonglong2* at = reinterpret_cast<const ulonglong2*>(a0);
     const float2* bt = Bs + buf * BK * BN;
@@ -287,6 +292,7 @@ __global__ void __launch_bounds__(NT, BM * BN >= 128 * 64 ? 1 : 2) gemm_simt_ker
       for (int kk = 0; kk < kn; ++kk) step(kk);
     }
     if (c + 1 < nch) store_tiles(buf ^ 1);
+    if (c + 2 < nch) load_chunk(c + 2);
     __syncthreads();
   }
 
