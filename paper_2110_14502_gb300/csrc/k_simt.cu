@@ -32,11 +32,10 @@
 // CTAs per SM and spills 1872, 1381, 469).
 //
 // What bounds the 128 x 128 tile: two warps per scheduler (246 registers, one CTA
-// per SM) do not cover the packed FMAs' latency.  Counters at (13, 13, 9), 5.8 ms,
-// with the loads after the barrier:
-// FMA pipe busy 61% of the cycles, an instruction issued in 39%; per issue a warp
-// waits 1.3 cycles on a fixed latency, 1.0 on the FMA pipe and 0.4 on instruction
-// fetch; shared memory 9% and DRAM 1% busy.
+// per SM) do not cover the packed FMAs' latency.  Counters at (13, 13, 9), 5.6 ms:
+// FMA pipe busy 63% of the cycles, an instruction issued in 41%; per issue a warp
+// waits 1.3 cycles on a fixed latency, 1.0 on the FMA pipe and 0.3 each on
+// instruction fetch and shared memory; shared memory 10% and DRAM 2% busy.
 //
 // Global loads: when the operand's two fastest indices are its first two K
 // bits (the planner's layouts put contracted indices innermost), a thread
